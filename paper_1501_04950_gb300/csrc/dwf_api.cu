@@ -222,7 +222,8 @@ struct dwf_ctx {
   double* scal = nullptr;          // per-rhs scalars, kScal doubles each
   double* partial = nullptr;       // reduction partials
   unsigned int* counter = nullptr; // reduction counters
-  int partial_stride = 0;
+  int partial_stride = 0;          // blocks a reduction may have
+  int counter_stride = 0;          // ticket counters per right-hand side
   int scal_rhs = 0;
   double* pinned = nullptr;        // host mirror of scal
   long long launches = 0;          // kernels launched through this handle
@@ -382,10 +383,15 @@ int ensure_reduce(dwf_ctx* h, int nrhs) {
   }
   h->scal_rhs = std::max(nrhs, 1);
   h->partial_stride = need_blocks;
+  // per right-hand side: one partial per block and one per group of blocks, and a
+  // ticket counter per group and one over the groups
+  const int slots = need_blocks + reduce_groups(need_blocks);
+  h->counter_stride = 1 + reduce_groups(need_blocks);
   CUCHK(h, cudaMalloc(&h->scal, sizeof(double) * kScal * h->scal_rhs));
-  CUCHK(h, cudaMalloc(&h->partial, sizeof(double) * (size_t)need_blocks * h->scal_rhs * 4));
-  CUCHK(h, cudaMalloc(&h->counter, sizeof(unsigned int) * h->scal_rhs * 4));
-  CUCHK(h, cudaMemset(h->counter, 0, sizeof(unsigned int) * h->scal_rhs * 4));
+  CUCHK(h, cudaMalloc(&h->partial, sizeof(double) * (size_t)slots * h->scal_rhs * 4));
+  const size_t cbytes = sizeof(unsigned int) * (size_t)h->counter_stride * h->scal_rhs * 4;
+  CUCHK(h, cudaMalloc(&h->counter, cbytes));
+  CUCHK(h, cudaMemset(h->counter, 0, cbytes));
   CUCHK(h, cudaMemset(h->scal, 0, sizeof(double) * kScal * h->scal_rhs));
   CUCHK(h, cudaMallocHost(&h->pinned, sizeof(double) * (kScal * h->scal_rhs + 1)));
   return DWF_OK;
@@ -394,10 +400,12 @@ int ensure_reduce(dwf_ctx* h, int nrhs) {
 // Reduction slot k (0..3) into scalar index which.
 Reduce make_reduce(dwf_ctx* h, int slot, int which) {
   Reduce r;
-  r.partial = h->partial + (size_t)slot * h->partial_stride * h->scal_rhs;
-  r.counter = h->counter + (size_t)slot * h->scal_rhs;
+  const int slots = h->partial_stride + reduce_groups(h->partial_stride);
+  r.partial = h->partial + (size_t)slot * slots * h->scal_rhs;
+  r.counter = h->counter + (size_t)slot * h->counter_stride * h->scal_rhs;
   r.result = h->scal + which;
-  r.partial_stride = h->partial_stride;
+  r.partial_stride = slots;
+  r.counter_stride = h->counter_stride;
   r.result_stride = kScal;
   return r;
 }

@@ -285,44 +285,85 @@ struct Store16 {
 };
 
 // ---------------------------------------------------------------------------
-// Deterministic two-level sum of one double per thread into red.result[rhs]:
-// warp shuffles, one partial per block (block bid of nblocks), and the last
-// block of the right-hand side to finish (ticket from red.counter) adds the
-// partials in block order.  Every thread of the block must call it (it
+// Deterministic sum of one double per thread into red.result[rhs]: warp shuffles,
+// one partial per block (block bid of nblocks), then a tree over the blocks.  The
+// last block to finish in a group of kReduceGroup (ticket from the group's
+// counter) adds the group's partials in block order, and the last group to finish
+// adds the group sums in group order.  Every thread of the block must call it (it
 // synchronises the block); works for 1D and 2D blocks.
+//
+// Bound by the latency of the last block's serial loads: one level, with a single
+// warp adding all 4096 partials of a 16^3x32, Ls = 16 hop pass, cost 128 dependent
+// rounds of L2 loads.  With groups of 128 the tail is two rounds of up to 4 loads a
+// lane, and all groups but the last are added while other blocks still run.
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ double warp_sum(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+// the same over the first `lanes` lanes of a warp that has no others
+__device__ __forceinline__ double warp_sum(double v, int lane, int lanes) {
+  const unsigned mask = lanes >= 32 ? 0xffffffffu : (1u << lanes) - 1u;
+  for (int o = 16; o > 0; o >>= 1) {
+    const double w = __shfl_down_sync(mask, v, o);
+    if (lane + o < lanes) v += w;
+  }
+  return v;
+}
+
+// Sum over part[0 .. n - 1] by one warp, n <= 128 in at most one round of 4 loads a lane
+// (they are issued together); part was written by other blocks of this launch.
+__device__ __forceinline__ double warp_sum_of(const double* part, int n, int lane) {
+  double acc = 0.0;
+  for (int b = lane; b < n; b += 128) {
+    double v[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) v[k] = b + 32 * k < n ? __ldcg(part + b + 32 * k) : 0.0;
+    acc += (v[0] + v[1]) + (v[2] + v[3]);
+  }
+  return warp_sum(acc);
+}
+
 __device__ __forceinline__ void block_sum_to(double v, const Reduce& red, int rhs, int nblocks,
                                              int bid) {
   __shared__ double wsum[32];
   const int nth = blockDim.x * blockDim.y;
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  if (lane == 0) wsum[warp] = v;
-  __syncthreads();
-  if (warp == 0) {
-    const int nw = (nth + 31) >> 5;
-    v = lane < nw ? wsum[lane] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    double* part = red.partial + (size_t)rhs * red.partial_stride;
-    unsigned int ticket = 0;
-    if (lane == 0) {
-      part[bid] = v;
-      __threadfence();
-      ticket = atomicAdd(red.counter + rhs, 1u);
-    }
-    ticket = __shfl_sync(0xffffffffu, ticket, 0);
-    if (ticket == (unsigned)(nblocks - 1)) {
-      __threadfence();
-      double acc = 0.0;
-      for (int b = lane; b < nblocks; b += 32) acc += *((volatile double*)(part + b));
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-      if (lane == 0) {
-        red.result[(size_t)rhs * red.result_stride] = acc;
-        red.counter[rhs] = 0u;
-      }
-    }
+  const int nw = (nth + 31) >> 5;
+  v = warp_sum(v, lane, nth - (warp << 5));
+  if (nw > 1) {
+    if (lane == 0) wsum[warp] = v;
+    __syncthreads();
+    if (warp > 0) return;
+    v = warp_sum(lane < nw ? wsum[lane] : 0.0);
   }
+  double* part = red.partial + (size_t)rhs * red.partial_stride;
+  unsigned int* count = red.counter + (size_t)rhs * red.counter_stride;
+  const int ngroups = reduce_groups(nblocks), group = bid / kReduceGroup;
+  const int first = group * kReduceGroup, size = min(kReduceGroup, nblocks - first);
+  unsigned int ticket = 0;
+  if (lane == 0) {
+    part[bid] = v;
+    __threadfence();
+    ticket = atomicAdd(count + 1 + group, 1u);
+  }
+  if (__shfl_sync(0xffffffffu, ticket, 0) != (unsigned)(size - 1)) return;
+  __threadfence();
+  double acc = warp_sum_of(part + first, size, lane);
+  if (lane == 0) count[1 + group] = 0u;
+  if (ngroups > 1) {
+    if (lane == 0) {
+      part[nblocks + group] = acc;
+      __threadfence();
+      ticket = atomicAdd(count, 1u);
+    }
+    if (__shfl_sync(0xffffffffu, ticket, 0) != (unsigned)(ngroups - 1)) return;
+    __threadfence();
+    acc = warp_sum_of(part + nblocks, ngroups, lane);
+    if (lane == 0) count[0] = 0u;
+  }
+  if (lane == 0) red.result[(size_t)rhs * red.result_stride] = acc;
 }
 
 // ---------------------------------------------------------------------------

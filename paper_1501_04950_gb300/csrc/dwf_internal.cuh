@@ -39,13 +39,20 @@ struct Geom {
 enum Prec { P64 = 0, P32 = 1, P16 = 2, PB16 = 3 };
 
 // Reduction target of a fused |.|^2.  Block b of right-hand side r writes
-// partial[r * partial_stride + b]; the last block of r to finish (ticket from
-// counter[r]) adds the partials in block order and stores result[r * result_stride].
+// partial[r * partial_stride + b]; the last block of a group of kReduceGroup to
+// finish (ticket from counter[r * counter_stride + 1 + group]) adds its partials
+// into partial[r * partial_stride + nblocks + group], and the last group to finish
+// (ticket from counter[r * counter_stride]) stores result[r * result_stride].
+constexpr int kReduceGroup = 128;
+__host__ __device__ constexpr int reduce_groups(int nblocks) {
+  return (nblocks + kReduceGroup - 1) / kReduceGroup;
+}
 struct Reduce {
   double* partial;
   unsigned int* counter;
   double* result;
   int partial_stride;
+  int counter_stride;
   int result_stride;
 };
 

@@ -44,6 +44,7 @@ struct MatSet {
   int Ls = 0;
   std::vector<double> host;
   void* dev[2] = {nullptr, nullptr};  // [0] double, [1] float
+  bool chain_ok = false;              // the recurrences are as accurate as the dense inverse
   // IT = I^T, SI = S I and SIT = (S I)^T for the operator forms of Eq. redblack1
   enum { K = 0, KT = 1, IINV = 2, IINVT = 3, IFULL = 4, BT = 5, IT = 6, SI = 7, SIT = 8, NMAT = 9 };
   size_t mat_off(int which) const { return (size_t)which * 2 * Ls * Ls; }
@@ -162,8 +163,9 @@ CycBidiag transpose_cb(const CycBidiag& m, int Ls) {
 }
 
 // Coefficients of the tuned kernels' recurrences in "lower" sweep order
-// (slice order reversed when dir = +1): multiply y_k = D_k v_k + O_k v_{k-1};
-// solve D_k y_k + O_k y_{k-1} = v_k by y_k = alpha_k + beta_k y_0.
+// (slice order reversed when dir = +1), 4 per step (hop2::chain_stride): multiply
+// y_k = D_k v_k + O_k v_{k-1}; solve D_k y_k + O_k y_{k-1} = v_k by
+// y_k = alpha_k + beta_k y_0.
 void chain_coeffs(const CycBidiag& m, int Ls, bool solve, double* out) {
   const bool rev = m.dir == +1;
   std::vector<double> D(Ls), O(Ls);
@@ -172,23 +174,38 @@ void chain_coeffs(const CycBidiag& m, int Ls, bool solve, double* out) {
     D[k] = m.d[s];
     O[k] = m.o[s];
   }
-  if (!solve) {
-    for (int k = 0; k < Ls; k++) {
-      out[k] = D[k];
-      out[Ls + k] = O[k];
-    }
-    return;
-  }
-  std::vector<double> beta(Ls);
-  beta[0] = 1.0;
-  for (int k = 1; k < Ls; k++) beta[k] = -(O[k] / D[k]) * beta[k - 1];
+  double beta = 1.0;
   for (int k = 0; k < Ls; k++) {
-    out[k] = 1.0 / D[k];
-    out[Ls + k] = O[k] / D[k];
-    out[2 * Ls + k] = beta[k];
+    if (k > 0) beta *= -(O[k] / D[k]);
+    out[4 * k] = solve ? 1.0 / D[k] : D[k];
+    out[4 * k + 1] = solve ? O[k] / D[k] : O[k];
+    out[4 * k + 2] = solve ? beta : 0.0;
+    out[4 * k + 3] = 0.0;
   }
-  out[3 * Ls] = 1.0 / (D[0] + O[0] * beta[Ls - 1]);
-  out[3 * Ls + 1] = O[0];
+  double* tail = out + 4 * Ls;
+  tail[0] = solve ? 1.0 / (D[0] + O[0] * beta) : 0.0;
+  tail[1] = solve ? O[0] : 0.0;
+  tail[2] = tail[3] = 0.0;
+}
+
+// Largest error of the solve recurrence over the unit vectors against the inverse
+// matrix (row-major, slice order), over the inverse's largest entry.
+double chain_solve_error(const double* c, int Ls, bool rev, const double* inv) {
+  double err = 0.0, big = 0.0;
+  std::vector<double> y(Ls);
+  for (int j = 0; j < Ls; j++) {
+    double prev = 0.0;
+    for (int k = 1; k < Ls; k++) y[k] = prev = (k == j ? c[4 * k] : 0.0) - c[4 * k + 1] * prev;
+    y[0] = ((j == 0 ? 1.0 : 0.0) - c[4 * Ls + 1] * prev) * c[4 * Ls];
+    for (int k = 0; k < Ls; k++) {
+      if (k > 0) y[k] += c[4 * k + 2] * y[0];
+      const double ref = rev ? inv[(size_t)(Ls - 1 - k) * Ls + (Ls - 1 - j)] : inv[(size_t)k * Ls + j];
+      const double d = std::fabs(y[k] - ref);
+      err = d <= err ? err : d;  // a NaN stays
+      big = std::max(big, std::fabs(ref));
+    }
+  }
+  return err / big;
 }
 
 }  // namespace
@@ -239,10 +256,10 @@ struct dwf_ctx {
   int* pinned_i = nullptr;         // host staging of the mask
   int active_cap = 0;
   struct Tuned {
-    int nb, tma, tile;  // right-hand-side block, staging variant, 4D sites per CTA (0: default)
+    int nb, tma, tile;  // right-hand-side block, staging variant, threads per CTA (0: by size)
   };
   std::map<std::string, Tuned> tune;  // autotuned launch shapes
-  int tile = 0;                      // 4D sites per CTA of the tuned hop kernels (0: default)
+  int tile = 0;                      // threads per CTA of the tuned hop kernels (0: by size)
   int env_tile = -1;                 // DWF_HOP_TILE set: tile fixed (-1: autotuned)
   double tier_eta = 1e-3;            // 16-bit solves: FP64 replacement once |r| < eta |r_64|
                                      // (DWF_TIER_ETA; <= 0: every replacement in FP64)
@@ -336,6 +353,16 @@ int build_matset(dwf_ctx* h, double alpha, double m, MatSet** out) {
     chain_coeffs(Ic, Ls, false, base + (hop2::OP_I * 2 + ch) * cs);
     chain_coeffs(Ic, Ls, true, base + (hop2::OP_ISOLVE * 2 + ch) * cs);
     chain_coeffs(transpose_cb(Ic, Ls), Ls, true, base + (hop2::OP_ITSOLVE * 2 + ch) * cs);
+    // |O_k / D_k| < 1 for Shamir, Mobius and Zolotarev coefficients, whose recurrences
+    // lose at most 3 ulp; coefficients for which they amplify rounding (or divide by
+    // zero) take the generic kernels with the dense inverse
+    const double* inv = ms.host.data() + ms.mat_off(MatSet::IINV) + ch * LL;
+    const double* invt = ms.host.data() + ms.mat_off(MatSet::IINVT) + ch * LL;
+    const double lim = 16.0 * 0x1p-53;
+    if (ch == 0) ms.chain_ok = true;
+    if (!(chain_solve_error(base + (hop2::OP_ISOLVE * 2 + ch) * cs, Ls, ch == 1, inv) <= lim) ||
+        !(chain_solve_error(base + (hop2::OP_ITSOLVE * 2 + ch) * cs, Ls, ch == 0, invt) <= lim))
+      ms.chain_ok = false;
   }
   std::vector<float> hf(ms.count());
   for (size_t k = 0; k < hf.size(); k++) hf[k] = (float)ms.host[k];
@@ -369,11 +396,12 @@ int get_ws(dwf_ctx* h, const std::string& name, size_t bytes, void** out) {
 }
 
 int ensure_reduce(dwf_ctx* h, int nrhs) {
-  int need_blocks =
-      std::max(hop_grid_blocks(h->g, P64, 0), std::max(hop_grid_blocks(h->g, P32, 0),
-                                                       blas_grid_blocks(h->g)));
-  if (h->Ls == 8 || h->Ls == 12 || h->Ls == 16)  // the small tile of the tuned kernels
-    need_blocks = std::max(need_blocks, hop_grid_blocks(h->g, P32, hop2::small_block_sites(h->Ls)));
+  int need_blocks = std::max(hop_grid_blocks(h->g, P64),
+                             std::max(hop_grid_blocks(h->g, P32), blas_grid_blocks(h->g)));
+  if (hop2::tuned_ls(h->Ls, false)) {  // the smallest tile of the tuned kernels
+    const int S = 32 / (h->Ls / 2);
+    need_blocks = std::max(need_blocks, (h->g.Vh + S - 1) / S);
+  }
   if (h->scal && h->scal_rhs >= nrhs && h->partial_stride >= need_blocks) return DWF_OK;
   if (h->scal) {
     cudaFree(h->scal);
@@ -427,7 +455,7 @@ HopLaunch base_hop(dwf_ctx* h, int prec, int p, int nrhs, size_t stride) {
   L.nbr = h->nbr;
   L.err = h->dev_err;
   L.use_tma = h->use_tma;
-  L.block_sites = h->tile;
+  L.block_threads = h->tile;
   L.wait_budget = h->wait_budget;
   L.skip_hop = &h->skip_hop;  // one-shot test hook, consumed by the first staged launch
   return L;
@@ -441,22 +469,52 @@ struct CoefView {
   const void* dev[2];
   size_t cstride;
   const int* active;
+  bool chain_ok;  // of every right-hand side's set
   const void* ptr(int prec, size_t off) const {
     const int f = prec == P64 ? 0 : 1;
     return reinterpret_cast<const char*>(dev[f]) + off * (f == 0 ? 8 : 4);
   }
+  // recurrence coefficients of the tuned kernels, or nullptr: the generic ones
+  const void* chain(int prec) const { return chain_ok ? ptr(prec, layout->chain_off()) : nullptr; }
+  bool tuned(int prec) const {
+    return chain_ok && !g_disable_tuned && hop2::tuned_ls(layout->Ls, prec == P16 || prec == PB16);
+  }
 };
-CoefView view_of(const MatSet& ms) { return CoefView{&ms, {ms.dev[0], ms.dev[1]}, 0, nullptr}; }
+CoefView view_of(const MatSet& ms) {
+  return CoefView{&ms, {ms.dev[0], ms.dev[1]}, 0, nullptr, ms.chain_ok};
+}
 
 void set_coef(HopLaunch& L, const CoefView& cv) {
   L.cstride = cv.cstride;
   L.active = cv.active;
 }
 
+int apply_dbb_bp(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* p, const void* bp,
+                 void* tmp, int nrhs, const Reduce* norm, cudaStream_t s);
+
 // out = D_bb in.  tmp: red half-field(s) of the same precision.
 int apply_dbb(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* in, void* tmp, int nrhs,
               const Reduce* norm, cudaStream_t s) {
   const MatSet& ms = *cv.layout;
+  if (prec == P64 && cv.tuned(P64)) {
+    // FP64 is bound by the FP64 pipe: B folded into the 8 hops of pass A is 384 of
+    // its ~1370 operations per 5D site, formed once it is 48.  out holds B in until
+    // pass B overwrites it.  16^3x32, Ls = 16:
+    // D_bb and D_bb^+ together 7.95 -> 7.20 ms.
+    LocalLaunch L{};
+    L.prec = P64;
+    L.out = out;
+    L.in = in;
+    L.stride = field_bytes(h->g, P64);
+    L.nrhs = nrhs;
+    L.prog = hop2::PR_B;
+    L.chain = cv.chain(P64);
+    L.c = 1.0;
+    L.cstride = cv.cstride;
+    L.active = cv.active;
+    KLAUNCH(h, launch_local(h->g, L, s));
+    return apply_dbb_bp(h, cv, P64, out, in, out, tmp, nrhs, norm, s);
+  }
   const int black = h->opt.rb_parity, red = 1 - black;
   const size_t st = field_bytes(h->g, prec);
   HopLaunch A = base_hop(h, prec, red, nrhs, st);
@@ -467,7 +525,7 @@ int apply_dbb(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* i
   A.pre_off = cv.ptr(prec, ms.boff_off());
   A.post = cv.ptr(prec, ms.mat_off(MatSet::K));
   A.post_prog = hop2::PR_K;
-  A.chain = cv.ptr(prec, ms.chain_off());
+  A.chain = cv.chain(prec);
   set_coef(A, cv);
   KLAUNCH(h, launch_hop(h->g, A, s));
   HopLaunch B = base_hop(h, prec, black, nrhs, st);
@@ -476,7 +534,7 @@ int apply_dbb(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* i
   B.w = in;
   B.post = cv.ptr(prec, ms.mat_off(MatSet::IINV));
   B.post_prog = hop2::PR_IINV;
-  B.chain = cv.ptr(prec, ms.chain_off());
+  B.chain = cv.chain(prec);
   B.loc = LOC_ID;
   B.c_hop = -0.25;
   B.c_loc = 1.0;
@@ -498,7 +556,7 @@ int apply_dbb_bp(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void
   A.v = bp;
   A.post = cv.ptr(prec, ms.mat_off(MatSet::K));
   A.post_prog = hop2::PR_K;
-  A.chain = cv.ptr(prec, ms.chain_off());
+  A.chain = cv.chain(prec);
   set_coef(A, cv);
   KLAUNCH(h, launch_hop(h->g, A, s));
   HopLaunch B = base_hop(h, prec, black, nrhs, st);
@@ -507,7 +565,7 @@ int apply_dbb_bp(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void
   B.w = p;
   B.post = cv.ptr(prec, ms.mat_off(MatSet::IINV));
   B.post_prog = hop2::PR_IINV;
-  B.chain = cv.ptr(prec, ms.chain_off());
+  B.chain = cv.chain(prec);
   B.loc = LOC_ID;
   B.c_hop = -0.25;
   B.c_loc = 1.0;
@@ -529,7 +587,7 @@ int apply_hat(dwf_ctx* h, const CoefView& cv, int prec, void* hat, const void* i
   L.nrhs = nrhs;
   L.m = cv.ptr(prec, ms.mat_off(MatSet::IINVT));
   L.prog = hop2::PR_ITINV;
-  L.chain = cv.ptr(prec, ms.chain_off());
+  L.chain = cv.chain(prec);
   L.c = 1.0;
   L.g5in = 1;
   L.cstride = cv.cstride;
@@ -549,7 +607,7 @@ int apply_dbb_dag_hat(dwf_ctx* h, const CoefView& cv, int prec, void* out, const
   A.v = hat;
   A.post = cv.ptr(prec, ms.mat_off(MatSet::KT));
   A.post_prog = hop2::PR_KT;
-  A.chain = cv.ptr(prec, ms.chain_off());
+  A.chain = cv.chain(prec);
   set_coef(A, cv);
   KLAUNCH(h, launch_hop(h->g, A, s));
   HopLaunch B = base_hop(h, prec, black, nrhs, st);
@@ -558,7 +616,7 @@ int apply_dbb_dag_hat(dwf_ctx* h, const CoefView& cv, int prec, void* out, const
   B.w = in;
   B.post = cv.ptr(prec, ms.mat_off(MatSet::BT));
   B.post_prog = hop2::PR_BT;
-  B.chain = cv.ptr(prec, ms.chain_off());
+  B.chain = cv.chain(prec);
   B.loc = LOC_ID;
   B.c_hop = -0.25;
   B.c_loc = 1.0;
@@ -739,7 +797,7 @@ int ensure_active(dwf_ctx* h, int nb) {
 //   z = D^+ r (fused |z|^2), beta = |z|^2 / |z_prev|^2, p = z + beta p,
 //   w = D p (fused |w|^2), a = |z|^2 / |w|^2, x += a p, r -= a w (fused |r|^2);
 // the first beta is 0 (|z_prev|^2 starts at +inf).  With the tuned kernels
-// (Ls in {8, 12, 16}) the BLAS steps are fused differently, same arithmetic:
+// (hop2::tuned_ls) the BLAS steps are fused differently, same arithmetic:
 // the residual update also writes r^ = I^-T gamma5 r (the first factor of the
 // next D^+ r) and stores a, and x += a p is deferred into the next p update
 // (flushed before every poll).  The check iterations
@@ -828,9 +886,7 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
     }
   }
   if ((rc = push_active())) return rc;
-  const int Ls = h->g.Ls;
-  const bool fused = form == DWF_SCHUR_PRECOND && h->fused_cg && !g_disable_tuned &&
-                     (Ls == 8 || Ls == 12 || Ls == 16);
+  const bool fused = form == DWF_SCHUR_PRECOND && h->fused_cg && cv.tuned(prec);
   if (fused && (rc = apply_hat(h, cv, prec, W.tb, W.r, nb, s))) return rc;
   // the p update also forms B p (of the stored p) for D_bb pass A; with BF16
   // fields the rounding of B p to 8 significand bits costs more iterations than
@@ -887,7 +943,7 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
     U.w = W.w;
     U.stride = fi;
     U.nrhs = nb;
-    U.chain = cv.ptr(prec, cv.layout->chain_off());
+    U.chain = cv.chain(prec);
     U.cstride = cv.cstride;
     U.num = zz_new;
     U.den = h->scal + S_WW;
@@ -1287,7 +1343,7 @@ int solver_params(dwf_ctx* h, int* prec, double* delta, bool* restart) {
 // DWF_TMA (set at dwf_create) fixes the staging.
 int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_out) {
   const int Ls = h->g.Ls;
-  const bool tuned = !g_disable_tuned && (Ls == 8 || Ls == 12 || Ls == 16);
+  const bool tuned = !g_disable_tuned && hop2::tuned_ls(Ls, prec == P16 || prec == PB16);
   const bool fixed_nb = h->opt.rhs_block > 0 || nrhs == 1;
   const int fnb = nrhs == 1 ? 1 : std::min(std::max(h->opt.rhs_block, 1), nrhs);
   if (!tuned) {  // one generic kernel shape: only the block is tuned (or fixed)
@@ -1297,7 +1353,7 @@ int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_ou
     }
   }
   std::ostringstream key;
-  key << "v2_" << h->g.L[0] << "x" << h->g.L[1] << "x" << h->g.L[2] << "x" << h->g.L[3] << "_Ls" << Ls
+  key << "v3_" << h->g.L[0] << "x" << h->g.L[1] << "x" << h->g.L[2] << "x" << h->g.L[3] << "_Ls" << Ls
       << "_p" << prec << "_n" << nrhs << "_b" << (fixed_nb ? fnb : 0) << "_t" << h->env_tma
       << "_s" << h->env_tile;
   auto it = h->tune.find(key.str());
@@ -1345,8 +1401,8 @@ int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_ou
   std::vector<int> tmas = {h->env_tma};
   std::vector<int> tiles = {h->env_tile >= 0 ? h->env_tile : 0};
   if (tuned) {
-    if (!h->env_tma) tmas.push_back(1);
-    if (h->env_tile < 0) tiles.push_back(hop2::small_block_sites(Ls));
+    if (h->env_tma) tiles = {0};  // the staged variant has one tile
+    else if (h->env_tile < 0) tiles = {128, 64, 32};
   }
   double best = 1e300;
   int best_nb = ok.front(), best_tma = tmas.front(), best_tile = 0;
@@ -1356,7 +1412,6 @@ int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_ou
   for (int nb : ok)
     for (int tma : tmas)
       for (int tile : tiles) {
-        if (tma && tile) continue;  // the staged variant has one tile
         h->use_tma = tma;
         h->tile = tile;
         if ((rc = apply_dbb(h, view_of(*ms), prec, y, x, t, nb, nullptr, st))) return rc;
@@ -1464,8 +1519,7 @@ int dwf_create(dwf_handle* out, const int lattice[4], int Ls, double M5, double 
   h->env_tma = h->use_tma;
   // DWF_HOP_TILE=small|default fixes the CTA tile of the tuned hop kernels
   if (const char* e = std::getenv("DWF_HOP_TILE")) {
-    const bool tuned_ls = Ls == 8 || Ls == 12 || Ls == 16;
-    h->env_tile = (std::string(e) == "small" && tuned_ls) ? hop2::small_block_sites(Ls) : 0;
+    h->env_tile = std::string(e) == "small" ? 64 : 128;
     h->tile = h->env_tile;
   }
   h->bp_fused = std::getenv("DWF_NO_BP_FUSED") == nullptr;
@@ -1879,7 +1933,8 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
       KLAUNCH(h, launch_hop(g, Hs, st));
     }
     std::vector<dwf_stats> sk(n);
-    CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr};
+    CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr, true};
+    for (int r = 0; r < n; r++) cv.chain_ok = cv.chain_ok && ms[blk + r]->chain_ok;
     rc = cgnr_batched(h, cv, prec, h->opt.rel_tol, h->opt.maxiter, delta, restart, W, n, sk.data(), st);
     if (rc && rc != DWF_ERR_NOT_CONVERGED && rc != DWF_ERR_BREAKDOWN) return rc;
     if (rc) result = rc;
@@ -1985,7 +2040,7 @@ int dwf_force(dwf_handle h, double* dSdU, const double* phi_half, const double* 
   Le.nrhs = 1;
   Le.m = ms->ptr(P64, ms->mat_off(MatSet::IINVT));
   Le.prog = hop2::PR_ITINV;
-  Le.chain = ms->ptr(P64, ms->chain_off());
+  Le.chain = view_of(*ms).chain(P64);
   Le.c = 1.0;
   KLAUNCH(h, launch_local(g, Le, st));
   // xi1 = I^-1 D_rb X = -1/2 I^-1 H_rb (B X)

@@ -295,7 +295,7 @@ cudaError_t run_hop(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   a.cstride = L.cstride;
   a.active = L.active;
   if (L.red) a.red = *L.red;
-  const int S = L.block_sites > 0 ? L.block_sites : default_block_sites(L.prec, g.Ls);
+  const int S = default_block_sites(L.prec, g.Ls);
   const size_t smem = hop_smem(L.prec, g.Ls, S);
   auto k = hop_kernel<SP, PRE, POST, LOC, G5, NORM>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -361,8 +361,8 @@ cudaError_t run_local(const Geom& g, const LocalLaunch& L, cudaStream_t st) {
 
 }  // namespace
 
-int hop_grid_blocks(const Geom& g, int prec, int block_sites) {
-  const int S = block_sites > 0 ? block_sites : default_block_sites(prec, g.Ls);
+int hop_grid_blocks(const Geom& g, int prec) {
+  const int S = default_block_sites(prec, g.Ls);
   return (g.Vh + S - 1) / S;
 }
 
@@ -379,14 +379,11 @@ cudaError_t launch_hop(const Geom& g, const HopLaunch& L, cudaStream_t st) {
     }
     if (e != cudaErrorNotSupported) return e;
   }
-  // block_sites is the tuned kernels' tile: the generic kernel takes its own default
-  HopLaunch G = L;
-  G.block_sites = 0;
-  switch (G.prec) {
-    case P64: return dispatch_hop<Store64>(g, G, st);
-    case P32: return dispatch_hop<Store32>(g, G, st);
-    case P16: return dispatch_hop<Store16<false>>(g, G, st);
-    case PB16: return dispatch_hop<Store16<true>>(g, G, st);
+  switch (L.prec) {
+    case P64: return dispatch_hop<Store64>(g, L, st);
+    case P32: return dispatch_hop<Store32>(g, L, st);
+    case P16: return dispatch_hop<Store16<false>>(g, L, st);
+    case PB16: return dispatch_hop<Store16<true>>(g, L, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -1,7 +1,10 @@
-// dwf_hop2.cuh -- the tuned hopping pass for Ls in {8, 12, 16} (sm_103a).
+// dwf_hop2.cuh -- the tuned hopping pass and the site-local 5th-dimension kernels for
+// the even Ls of tuned_ls() (sm_103a).
 //
 // Work split: one thread per (4D site, pair of 5th-dimension slices s0 = 2t,
-// s1 = 2t + 1); Ls / 2 threads per site, block = (Ls/2, S) with S sites.
+// s1 = 2t + 1), G = Ls / 2 threads per site; a CTA of nt threads (a multiple of 32,
+// at most 128) takes nt / G sites, and the nt mod G threads left over help with the
+// 5th-dimension operators only.
 //   * the half-fields store each spinor component of a slice pair as
 //     (re s0, re s1, im s0, im s1) (dwf_fields.cuh), so one vector load gives a
 //     thread both slices of a component in lane order, and the projection,
@@ -13,8 +16,10 @@
 //     on the FMAs of the reconstruction;
 //   * the B pre-multiplication of D_bb pass A (cyclic bidiagonal per chirality,
 //     Eq. mobius1 with D_w -> 1) is applied to the neighbour spinor before the
-//     projection: (B v)+(s) = d+ v+(s) + o+ v+(s-1), (B v)-(s) = d- v-(s) + o- v-(s+1),
-//     so v+ of the pair below and v- of the pair above are loaded in addition;
+//     projection: (B v)+(s) = d+ v+(s) + o+ v+(s-1), (B v)-(s) = d- v-(s) + o- v-(s+1).
+//     v+ of the pair below and v- of the pair above come from the registers of the
+//     neighbouring threads by shuffles where a site's threads share a warp (G a power
+//     of two), else they are loaded in addition;
 //   * the 5th-dimension post operators (I^-1, K = B I^-1, K^T, B^T) run as
 //     O(Ls) recurrences on register-resident chains after a transpose through
 //     shared memory: every cyclic bidiagonal matrix of the construction, put in
@@ -33,18 +38,30 @@
 namespace dwf {
 namespace hop2 {
 
+// The Ls whose kernels are compiled (the others take the generic kernels): the Ls of
+// the alpha study, of the benchmark and of the Mobius / Zolotarev comparison.  With
+// 16-bit storage (scaled) only the Ls of the benchmark workloads: elsewhere the
+// recurrences' FP32 rounding, as good as the dense contraction's but not the same, would
+// turn some 16-bit roundings of the intermediate fields the other way, and those
+// results are kept.
+__host__ __device__ constexpr bool tuned_ls(int Ls, bool scaled) {
+  return Ls == 8 || Ls == 12 || Ls == 16 ||
+         (!scaled && (Ls == 4 || Ls == 6 || Ls == 10 || Ls == 20 || Ls == 24 || Ls == 32));
+}
+
 // Chain coefficient block: [op][chirality][kChainStride(Ls)] in the compute type,
-// op = 0 B (mult), 1 B^T (mult), 2 I (mult), 3 I (solve), 4 I^T (solve).
-// mult:  a_k = diagonal, b_k = off-diagonal (lower form, sweep order)
-// solve: a_k = 1/D_k, b_k = O_k/D_k, c_k = beta_k, then G, O_0.
+// op = 0 B (mult), 1 B^T (mult), 2 I (mult), 3 I (solve), 4 I^T (solve).  Step k of
+// a sweep (lower form, sweep order) reads one 4-vector at 4k:
+// mult:  (diagonal, off-diagonal, 0, 0)
+// solve: (1/D_k, O_k/D_k, beta_k, 0); then (G, O_0, 0, 0) at 4 Ls.
 enum { OP_B = 0, OP_BT = 1, OP_I = 2, OP_ISOLVE = 3, OP_ITSOLVE = 4, NOPS = 5 };
-__host__ __device__ constexpr int chain_stride(int Ls) { return ((3 * Ls + 2) + 3) / 4 * 4; }
+__host__ __device__ constexpr int chain_stride(int Ls) { return 4 * Ls + 4; }
 __host__ __device__ constexpr int chain_block(int Ls) { return NOPS * 2 * chain_stride(Ls); }
 // op is transposed -> reversed sweep order for chirality 0, else for chirality 1
 __host__ __device__ constexpr bool op_transposed(int op) { return op == OP_BT || op == OP_ITSOLVE; }
 
 // Programs (sequence of ops) used as post / local operators.
-enum { PR_NONE = 0, PR_K = 1, PR_IINV = 2, PR_KT = 3, PR_BT = 4, PR_I = 5, PR_ITINV = 6 };
+enum { PR_NONE = 0, PR_K = 1, PR_IINV = 2, PR_KT = 3, PR_BT = 4, PR_I = 5, PR_ITINV = 6, PR_B = 7 };
 __host__ __device__ constexpr int prog_len(int p) { return p == PR_K || p == PR_KT ? 2 : (p ? 1 : 0); }
 __host__ __device__ constexpr int prog_op(int p, int i) {
   return p == PR_K ? (i == 0 ? OP_ISOLVE : OP_B)
@@ -52,21 +69,24 @@ __host__ __device__ constexpr int prog_op(int p, int i) {
        : p == PR_KT ? (i == 0 ? OP_BT : OP_ITSOLVE)
        : p == PR_BT ? OP_BT
        : p == PR_I ? OP_I
-       : p == PR_ITINV ? OP_ITSOLVE : -1;
+       : p == PR_ITINV ? OP_ITSOLVE
+       : p == PR_B ? OP_B : -1;
 }
+// elements of the coefficients of a program's ops, in the order of its ops
+__host__ __device__ constexpr int prog_coefs(int Ls, int p) { return prog_len(p) * 2 * chain_stride(Ls); }
 __host__ __device__ constexpr bool op_is_solve(int op) { return op == OP_ISOLVE || op == OP_ITSOLVE; }
 
-// Shared-memory layout of one 4D site for the 5th-dimension programs: the slice
-// pair of thread t at t * kPairStride, component c at 4c as (re s0, re s1, im s0,
-// im s1); 52 = 20 mod 32 spreads the eight 16-byte stores of a quarter warp
-// over all 32 banks.  Sites start 8 words apart modulo 32 banks.
+// Shared-memory layout of one 4D site for the 5th-dimension programs, per chirality in
+// the sweep order of the program (the slices of a chirality whose sweep is reversed are
+// stored last slice first): slices 2k, 2k + 1 of the sweep at k * kPairStride, real
+// component R = 2c + (0 re | 1 im) at 2R as (even slice, odd slice).  A sweep then
+// reads two slices of a component by one 8-byte (FP64: 16-byte) access at constant
+// offsets.  52 = 20 mod 32 spreads the 16-byte stores of a quarter warp over the banks
+// (two-way conflicts at G = 3, 4, 5), and sites 24 = 12 * 2 words apart modulo 32 make the
+// accesses of consecutive sweeps (12 of a chirality per site) conflict-free.
 constexpr int kPairStride = 52;
 __host__ __device__ constexpr int site_stride(int Ls) {
-  return (Ls / 2) * kPairStride + ((8 - ((Ls / 2) * kPairStride) % 32) + 32) % 32;
-}
-// element of slice s, real component r = 2c + (0 re | 1 im)
-__host__ __device__ constexpr int elem(int s, int r) {
-  return (s >> 1) * kPairStride + 4 * (r >> 1) + 2 * (r & 1) + (s & 1);
+  return (Ls / 2) * kPairStride + ((24 - ((Ls / 2) * kPairStride) % 32) + 32) % 32;
 }
 
 // ---------------------------------------------------------------------------
@@ -342,8 +362,15 @@ __device__ __forceinline__ void project_mul_acc(HalfP<typename Pr<typename SP::T
   }
 }
 
+// A site's G threads are an aligned group of one warp's lanes.
+__host__ __device__ constexpr bool warp_groups(int Ls) { return 32 % (Ls / 2) == 0; }
+
+__device__ __forceinline__ float lane_of(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+__device__ __forceinline__ double lane_of(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+
 // acc += f (1 - dir gamma_mu) U' v'(x +- mu) for the two slices of a thread,
-// U' = U_mu(x) (dir > 0) or U_mu(x - mu)^+ (dir < 0).
+// U' = U_mu(x) (dir > 0) or U_mu(x - mu)^+ (dir < 0).  With PRE_B and warp_groups(LS)
+// every thread of the warp calls it.
 template <class SP, int LS, int PRE, int MU, int DIR>
 __device__ __forceinline__ void hop_dir(int nb, int h, int t, size_t NP,
                                         const typename SP::T (&bd)[2][2],
@@ -365,24 +392,54 @@ __device__ __forceinline__ void hop_dir(int nb, int h, int t, size_t NP,
   if constexpr (PRE == PRE_B) {
     // (B v)+ needs v+(s0 - 1) = lane y of the pair below (cyclic in s),
     // (B v)- needs v-(s1 + 1) = lane x of the pair above.
-    const size_t base = (size_t)hn * HALF;
-    const size_t mp = base + (t == 0 ? HALF - 1 : t - 1), mn = base + (t + 1 == HALF ? 0 : t + 1);
-    HalfP<V> Pb, Ma;
-    IO::load6(v, mp, NP, 0, Pb.re, Pb.im);
-    IO::load6(v, mn, NP, 6, Ma.re, Ma.im);
+    const int tb = t == 0 ? HALF - 1 : t - 1, ta = t + 1 == HALF ? 0 : t + 1;
     T a1 = bd[0][0], a2 = bo[0][0], a3 = bd[0][1], a4 = bo[0][1];
     T b1 = bd[1][0], b2 = bo[1][0], b3 = bd[1][1], b4 = bo[1][1];
+    T pr[6], pi[6], mr[6], mi[6];  // v+ of the slice below, v- of the slice above
+    V sc = A::dup((T)1);
+    T sb = 1, sa = 1;
+    if constexpr (warp_groups(LS)) {
+      const int base = (threadIdx.x & 31) - t;
+#pragma unroll
+      for (int k = 0; k < 6; k++) {
+        pr[k] = lane_of(P.re[k].y, base + tb);
+        pi[k] = lane_of(P.im[k].y, base + tb);
+        mr[k] = lane_of(M.re[k].x, base + ta);
+        mi[k] = lane_of(M.im[k].x, base + ta);
+      }
+      if constexpr (SP::kScaled) {
+        sc = IO::scale(v, m, NP);
+        sb = lane_of(sc.y, base + tb);
+        sa = lane_of(sc.x, base + ta);
+      }
+    } else {
+      const size_t mp = (size_t)hn * HALF + tb, mn = (size_t)hn * HALF + ta;
+      HalfP<V> Pb, Ma;
+      IO::load6(v, mp, NP, 0, Pb.re, Pb.im);
+      IO::load6(v, mn, NP, 6, Ma.re, Ma.im);
+#pragma unroll
+      for (int k = 0; k < 6; k++) {
+        pr[k] = Pb.re[k].y;
+        pi[k] = Pb.im[k].y;
+        mr[k] = Ma.re[k].x;
+        mi[k] = Ma.im[k].x;
+      }
+      if constexpr (SP::kScaled) {
+        sc = IO::scale(v, m, NP);
+        sb = IO::scale(v, mp, NP).y;
+        sa = IO::scale(v, mn, NP).x;
+      }
+    }
     if constexpr (SP::kScaled) {
-      const V sc = IO::scale(v, m, NP), sb = IO::scale(v, mp, NP), sa = IO::scale(v, mn, NP);
-      a1 *= sc.x; a2 *= sb.y; a3 *= sc.y; a4 *= sc.x;
-      b1 *= sc.x; b2 *= sc.y; b3 *= sc.y; b4 *= sa.x;
+      a1 *= sc.x; a2 *= sb; a3 *= sc.y; a4 *= sc.x;
+      b1 *= sc.x; b2 *= sc.y; b3 *= sc.y; b4 *= sa;
     }
 #pragma unroll
     for (int k = 0; k < 6; k++) {
-      P.re[k] = A::mk(::fma(a2, Pb.re[k].y, a1 * P.re[k].x), ::fma(a4, P.re[k].x, a3 * P.re[k].y));
-      P.im[k] = A::mk(::fma(a2, Pb.im[k].y, a1 * P.im[k].x), ::fma(a4, P.im[k].x, a3 * P.im[k].y));
-      M.re[k] = A::mk(::fma(b2, M.re[k].y, b1 * M.re[k].x), ::fma(b4, Ma.re[k].x, b3 * M.re[k].y));
-      M.im[k] = A::mk(::fma(b2, M.im[k].y, b1 * M.im[k].x), ::fma(b4, Ma.im[k].x, b3 * M.im[k].y));
+      P.re[k] = A::mk(::fma(a2, pr[k], a1 * P.re[k].x), ::fma(a4, P.re[k].x, a3 * P.re[k].y));
+      P.im[k] = A::mk(::fma(a2, pi[k], a1 * P.im[k].x), ::fma(a4, P.im[k].x, a3 * P.im[k].y));
+      M.re[k] = A::mk(::fma(b2, M.re[k].y, b1 * M.re[k].x), ::fma(b4, mr[k], b3 * M.re[k].y));
+      M.im[k] = A::mk(::fma(b2, M.im[k].y, b1 * M.im[k].x), ::fma(b4, mi[k], b3 * M.im[k].y));
     }
   } else if constexpr (SP::kScaled) {
     f = A::mul(f, IO::scale(v, m, NP));  // per-slice scale of the neighbour site
@@ -393,116 +450,171 @@ __device__ __forceinline__ void hop_dir(int nb, int h, int t, size_t NP,
   project_mul_acc<SP, MU, DIR>(P, M, U, f, acc);
 }
 
+// One step's coefficients (4-vector) of a sweep.
+template <typename T>
+struct Coef4 {
+  T a, b, c, d;
+};
+__device__ __forceinline__ Coef4<float> coef4(const float* p) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  return Coef4<float>{v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ Coef4<double> coef4(const double* p) {
+  const double2 v = *reinterpret_cast<const double2*>(p), w = *reinterpret_cast<const double2*>(p + 2);
+  return Coef4<double>{v.x, v.y, w.x, w.y};
+}
+
 // Lower-form cyclic bidiagonal multiply: y_k = a_k v_k + b_k v_{k-1 mod L}.
-template <typename T, int LS, int CPT>
-__device__ __forceinline__ void chain_mult(T (&V)[CPT][LS], const T* c) {
-  T last[CPT];
+template <typename T, int LS, int NIT>
+__device__ __forceinline__ void chain_mult(T (&V)[NIT][LS], const T* c) {
+  T last[NIT];
 #pragma unroll
-  for (int q = 0; q < CPT; q++) last[q] = V[q][LS - 1];
+  for (int q = 0; q < NIT; q++) last[q] = V[q][LS - 1];
 #pragma unroll
   for (int k = LS - 1; k >= 1; k--) {
-    const T a = c[k], b = c[LS + k];
+    const Coef4<T> e = coef4(c + 4 * k);
 #pragma unroll
-    for (int q = 0; q < CPT; q++) V[q][k] = fma(b, V[q][k - 1], a * V[q][k]);
+    for (int q = 0; q < NIT; q++) V[q][k] = fma(e.b, V[q][k - 1], e.a * V[q][k]);
   }
-  const T a0 = c[0], b0 = c[LS];
+  const Coef4<T> e = coef4(c);
 #pragma unroll
-  for (int q = 0; q < CPT; q++) V[q][0] = fma(b0, last[q], a0 * V[q][0]);
+  for (int q = 0; q < NIT; q++) V[q][0] = fma(e.b, last[q], e.a * V[q][0]);
 }
 
 // Lower-form cyclic bidiagonal solve D_k y_k + O_k y_{k-1 mod L} = v_k:
 // y_k = alpha_k + beta_k t with t = y_0 from the row-0 equation.
-template <typename T, int LS, int CPT>
-__device__ __forceinline__ void chain_solve(T (&V)[CPT][LS], const T* c) {
-  T h0[CPT], prev[CPT];
+template <typename T, int LS, int NIT>
+__device__ __forceinline__ void chain_solve(T (&V)[NIT][LS], const T* c) {
+  T h0[NIT], prev[NIT];
 #pragma unroll
-  for (int q = 0; q < CPT; q++) {
+  for (int q = 0; q < NIT; q++) {
     h0[q] = V[q][0];
     prev[q] = (T)0;
   }
 #pragma unroll
   for (int k = 1; k < LS; k++) {
-    const T a = c[k], b = c[LS + k];
+    const Coef4<T> e = coef4(c + 4 * k);
 #pragma unroll
-    for (int q = 0; q < CPT; q++) {
-      prev[q] = fma(-b, prev[q], a * V[q][k]);
+    for (int q = 0; q < NIT; q++) {
+      prev[q] = fma(-e.b, prev[q], e.a * V[q][k]);
       V[q][k] = prev[q];
     }
   }
-  const T G = c[3 * LS], o0 = c[3 * LS + 1];
+  const Coef4<T> e = coef4(c + 4 * LS);  // (G, O_0)
 #pragma unroll
-  for (int q = 0; q < CPT; q++) {
-    const T t = fma(-o0, prev[q], h0[q]) * G;
+  for (int q = 0; q < NIT; q++) {
+    const T t = fma(-e.b, prev[q], h0[q]) * e.a;
     V[q][0] = t;
     prev[q] = t;
   }
 #pragma unroll
   for (int k = 1; k < LS; k++) {
-    const T bc = c[2 * LS + k];
+    const T bc = c[4 * k + 2];
 #pragma unroll
-    for (int q = 0; q < CPT; q++) V[q][k] = fma(bc, prev[q], V[q][k]);
+    for (int q = 0; q < NIT; q++) V[q][k] = fma(bc, prev[q], V[q][k]);
   }
 }
 
-// Run program PROG on the (Ls x 24) block of one 4D site in shared memory.
-// Thread t of the site owns real components cbase .. cbase + CPT - 1 (one chirality).
+// Coefficients of the ops of PROG (both chiralities) into shared memory, 16 bytes at a time.
 template <typename T, int LS, int PROG>
-__device__ __forceinline__ void run_prog(T* site, const T* coef, int t) {
-  constexpr int CPT = 48 / LS;
-  const int cbase = t * CPT;
-  const int ch = cbase / 12;
-  const bool rev = (ch == 1) != op_transposed(prog_op(PROG, 0));
-  T V[CPT][LS];
+__device__ __forceinline__ void load_coefs(T* coef, const T* chain, int tid, int nth) {
+  constexpr int n = 2 * chain_stride(LS) * (int)sizeof(T) / 16;
 #pragma unroll
-  for (int k = 0; k < LS; k++) {
-    const int s = rev ? LS - 1 - k : k;
+  for (int i = 0; i < prog_len(PROG); i++) {
+    const uint4* src = reinterpret_cast<const uint4*>(chain + prog_op(PROG, i) * 2 * chain_stride(LS));
+    uint4* dst = reinterpret_cast<uint4*>(coef) + i * n;
+    for (int k = tid; k < n; k += nth) dst[k] = __ldg(src + k);
+  }
+}
+
+// Chirality ch of PROG sweeps the slices last to first.
+__host__ __device__ constexpr bool prog_reversed(int prog, int ch) {
+  return (ch == 1) != op_transposed(prog_op(prog, 0));
+}
+
+__device__ __forceinline__ float2 pair_at(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ double2 pair_at(const double* p) { return *reinterpret_cast<const double2*>(p); }
+
+// Run program PROG on the sites of a CTA in shared memory (nsites blocks of
+// site_stride(LS)), by nth threads: one half of them takes the sweeps of chirality 0,
+// the other those of chirality 1 (12 real components each per site), so that a
+// coefficient is one broadcast load for all sweeps of a thread.
+template <typename T, int LS, int PROG>
+__device__ __forceinline__ void run_prog(T* sbuf, const T* coef, int tid, int nth, int nsites) {
+  constexpr int NIT = (48 + LS - 1) / LS;  // sweeps per thread: 24 nsites / nth <= 48 / LS
+  constexpr bool EXACT = 48 % LS == 0 && 32 % (LS / 2) == 0;
+  const int half = nth >> 1, ch = tid >= half ? 1 : 0;
+  T* p[NIT];
+  bool ok[NIT];
+  T V[NIT][LS];
 #pragma unroll
-    for (int q = 0; q < CPT; q++) V[q][k] = site[elem(s, cbase + q)];
+  for (int q = 0; q < NIT; q++) {
+    const int i = tid - ch * half + q * half;
+    ok[q] = EXACT || i < 12 * nsites;
+    const int site = i / 12;
+    p[q] = sbuf + site * site_stride(LS) + 24 * ch + 2 * (i - 12 * site);
+#pragma unroll
+    for (int k = 0; k < LS / 2; k++) {
+      if (ok[q]) {
+        const auto v = pair_at(p[q] + k * kPairStride);
+        V[q][2 * k] = v.x;
+        V[q][2 * k + 1] = v.y;
+      } else {
+        V[q][2 * k] = V[q][2 * k + 1] = (T)0;
+      }
+    }
   }
 #pragma unroll
   for (int i = 0; i < prog_len(PROG); i++) {
-    const int op = prog_op(PROG, i);
-    const T* c = coef + (op * 2 + ch) * chain_stride(LS);
-    if (op_is_solve(op)) chain_solve<T, LS, CPT>(V, c);
-    else chain_mult<T, LS, CPT>(V, c);
+    const T* c = coef + (2 * i + ch) * chain_stride(LS);
+    if (op_is_solve(prog_op(PROG, i))) chain_solve<T, LS, NIT>(V, c);
+    else chain_mult<T, LS, NIT>(V, c);
   }
 #pragma unroll
-  for (int k = 0; k < LS; k++) {
-    const int s = rev ? LS - 1 - k : k;
+  for (int q = 0; q < NIT; q++)
+    if (ok[q]) {
 #pragma unroll
-    for (int q = 0; q < CPT; q++) site[elem(s, cbase + q)] = V[q][k];
-  }
+      for (int k = 0; k < LS / 2; k++) {
+        using V2 = typename Pr<T>::V;
+        *reinterpret_cast<V2*>(p[q] + k * kPairStride) = Pr<T>::mk(V[q][2 * k], V[q][2 * k + 1]);
+      }
+    }
 }
 
-// thread t's slice pair <-> shared memory
-__device__ __forceinline__ void put(float* p, const SpinP<float2>& a) {
-  float4* q = reinterpret_cast<float4*>(p);
-#pragma unroll
-  for (int c = 0; c < 12; c++) q[c] = make_float4(a.re[c].x, a.re[c].y, a.im[c].x, a.im[c].y);
+// Slice pair t of a site <-> shared memory, in the sweep order of PROG.
+__device__ __forceinline__ void put4(float* p, float a, float b, float c, float d) {
+  *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
 }
-__device__ __forceinline__ void get(const float* p, SpinP<float2>& a) {
-  const float4* q = reinterpret_cast<const float4*>(p);
+__device__ __forceinline__ void put4(double* p, double a, double b, double c, double d) {
+  reinterpret_cast<double2*>(p)[0] = make_double2(a, b);
+  reinterpret_cast<double2*>(p)[1] = make_double2(c, d);
+}
+template <typename T, int LS, int PROG>
+__device__ __forceinline__ void put(T* site, int t, const SpinP<typename Pr<T>::V>& a) {
 #pragma unroll
-  for (int c = 0; c < 12; c++) {
-    const float4 v = q[c];
-    a.re[c] = make_float2(v.x, v.y);
-    a.im[c] = make_float2(v.z, v.w);
+  for (int ch = 0; ch < 2; ch++) {
+    constexpr bool R[2] = {prog_reversed(PROG, 0), prog_reversed(PROG, 1)};
+    T* p = site + (R[ch] ? LS / 2 - 1 - t : t) * kPairStride;
+#pragma unroll
+    for (int c = 6 * ch; c < 6 * ch + 6; c++) {
+      if (R[ch]) put4(p + 4 * c, a.re[c].y, a.re[c].x, a.im[c].y, a.im[c].x);
+      else put4(p + 4 * c, a.re[c].x, a.re[c].y, a.im[c].x, a.im[c].y);
+    }
   }
 }
-__device__ __forceinline__ void put(double* p, const SpinP<double2>& a) {
-  double2* q = reinterpret_cast<double2*>(p);
+template <typename T, int LS, int PROG>
+__device__ __forceinline__ void get(const T* site, int t, SpinP<typename Pr<T>::V>& a) {
+  using A = Pr<T>;
 #pragma unroll
-  for (int c = 0; c < 12; c++) {
-    q[2 * c] = a.re[c];
-    q[2 * c + 1] = a.im[c];
-  }
-}
-__device__ __forceinline__ void get(const double* p, SpinP<double2>& a) {
-  const double2* q = reinterpret_cast<const double2*>(p);
+  for (int ch = 0; ch < 2; ch++) {
+    constexpr bool R[2] = {prog_reversed(PROG, 0), prog_reversed(PROG, 1)};
+    const T* p = site + (R[ch] ? LS / 2 - 1 - t : t) * kPairStride;
 #pragma unroll
-  for (int c = 0; c < 12; c++) {
-    a.re[c] = q[2 * c];
-    a.im[c] = q[2 * c + 1];
+    for (int c = 6 * ch; c < 6 * ch + 6; c++) {
+      const Coef4<T> v = coef4(p + 4 * c);
+      a.re[c] = R[ch] ? A::mk(v.b, v.a) : A::mk(v.a, v.b);
+      a.im[c] = R[ch] ? A::mk(v.d, v.c) : A::mk(v.c, v.d);
+    }
   }
 }
 
@@ -536,38 +648,40 @@ template <typename T>
 constexpr int min_blocks() { return sizeof(T) == 8 ? 2 : 4; }
 
 // Common tail of the hopping kernels: 5th-dimension post program, scaling,
-// optional gamma5, local term, store and fused norm.  Every thread of the CTA
-// calls it (it contains __syncthreads); threads with part = false (no site of
-// their own) only take part in the barriers and the norm.
+// optional gamma5, local term (c_loc = 1), store and fused norm.  Every thread of the
+// CTA calls it (it contains __syncthreads); the nth threads with tid < nth run the
+// program, threads with part = false (no site of their own) store nothing.
 template <class SP, int LS, int POST, int LOC, bool G5, bool NORM>
 __device__ __forceinline__ void epilogue_g(const Args<typename SP::T>& a, const typename SP::T* coef,
-                                           typename SP::T* site, size_t NP, int h, int t, bool active,
-                                           bool part, int rhs,
+                                           typename SP::T* sbuf, int tid, int nth, int nsites, size_t NP,
+                                           int h, int j, int t, bool active, bool part, int rhs,
                                            SpinP<typename Pr<typename SP::T>::V>& acc) {
   using T = typename SP::T;
   using A = Pr<T>;
   using V = typename A::V;
-  if (POST != PR_NONE) {
-    if (part) put(site + t * kPairStride, acc);
+  if constexpr (POST != PR_NONE) {
+    T* site = sbuf + j * site_stride(LS);
+    if (part) put<T, LS, POST>(site, t, acc);
     __syncthreads();
-    if (part) run_prog<T, LS, POST>(site, coef, t);
+    if (tid < nth) run_prog<T, LS, POST>(sbuf, coef, tid, nth, nsites);
     __syncthreads();
-    if (part) get(site + t * kPairStride, acc);
+    if (part) get<T, LS, POST>(site, t, acc);
   }
   const V ch = A::dup(a.c_hop);
   const size_t off = rhs * a.stride;
   const size_t m = (size_t)h * (LS / 2) + t;
-  if (LOC == LOC_ID && active) {
-    SpinP<V> w;
-    load_spin<SP>(reinterpret_cast<const char*>(a.w) + off, m, NP, w);
-    const V cl = A::dup(a.c_loc);
+  if (LOC == LOC_ID) {
+    if (active) {
+      SpinP<V> w;
+      load_spin<SP>(reinterpret_cast<const char*>(a.w) + off, m, NP, w);
 #pragma unroll
-    for (int c = 0; c < 12; c++) {
-      const V f = (G5 && c >= 6) ? A::neg(ch) : ch;
-      acc.re[c] = A::fma(f, acc.re[c], A::mul(cl, w.re[c]));
-      acc.im[c] = A::fma(f, acc.im[c], A::mul(cl, w.im[c]));
+      for (int c = 0; c < 12; c++) {
+        const V f = (G5 && c >= 6) ? A::neg(ch) : ch;
+        acc.re[c] = A::fma(f, acc.re[c], w.re[c]);
+        acc.im[c] = A::fma(f, acc.im[c], w.im[c]);
+      }
     }
-  } else {
+  } else if (G5 || a.c_hop != (T)1) {
 #pragma unroll
     for (int c = 0; c < 12; c++) {
       const V f = (G5 && c >= 6) ? A::neg(ch) : ch;
@@ -592,32 +706,35 @@ __device__ __forceinline__ void epilogue_g(const Args<typename SP::T>& a, const 
   }
 }
 
-// out = c_hop G post(H v') + c_loc loc(w), two 5th-dimension slices per thread.
-template <class SP, int LS, int PRE, int POST, int LOC, bool G5, bool NORM, int MINB, int NT = 128>
-__global__ void __launch_bounds__(NT, MINB) hop_kernel(const Geom g, const Args<typename SP::T> a) {
+// out = c_hop G post(H v') + loc(w), two 5th-dimension slices per thread.
+template <class SP, int LS, int PRE, int POST, int LOC, bool G5, bool NORM, int MINB>
+__global__ void __launch_bounds__(128, MINB) hop_kernel(const Geom g, const Args<typename SP::T> a) {
   using T = typename SP::T;
   using V = typename Pr<T>::V;
-  constexpr int SST = site_stride(LS);
+  constexpr int G = LS / 2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* coef = reinterpret_cast<T*>(smem_raw);
-  T* sbuf = coef + chain_block(LS);
-  const int t = threadIdx.x, j = threadIdx.y;
-  const int nth = blockDim.x * blockDim.y, tid = j * blockDim.x + t;
-  const int h = blockIdx.x * blockDim.y + j;
-  const bool active = h < g.Vh;
+  T* sbuf = coef + prog_coefs(LS, POST);
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int S = nth / G, j = tid / G, t = tid - j * G;
+  const int h = blockIdx.x * S + j;
+  const bool part = warp_groups(LS) || j < S;
+  const bool active = part && h < g.Vh;
   const int rhs = blockIdx.z;
   if (a.active && !a.active[rhs]) return;
   const size_t co = (size_t)rhs * a.cstride;
   const size_t NP = (size_t)g.N5 >> 1;
   const int s0 = 2 * t;
-  if (POST != PR_NONE) {
-    for (int i = tid; i < chain_block(LS); i += nth) coef[i] = a.chain[co + i];
-  }
+  load_coefs<T, LS, POST>(coef, a.chain + co, tid, nth);
   const char* vb = reinterpret_cast<const char*>(a.v) + rhs * a.stride;
   SpinP<V> acc;
   zero(acc);
-  if (active) {
-    const int4 nb0 = __ldg(a.nbr + 2 * h), nb1 = __ldg(a.nbr + 2 * h + 1);
+  // the shuffles of the B pre-multiplication need whole warps: threads past the last
+  // site compute it again and store nothing
+  constexpr bool WHOLE = PRE == PRE_B && warp_groups(LS);
+  if (WHOLE || active) {
+    const int hl = WHOLE ? min(h, g.Vh - 1) : h;
+    const int4 nb0 = __ldg(a.nbr + 2 * hl), nb1 = __ldg(a.nbr + 2 * hl + 1);
     T bd[2][2] = {{0, 0}, {0, 0}}, bo[2][2] = {{0, 0}, {0, 0}};
     if (PRE == PRE_B) {
 #pragma unroll
@@ -629,42 +746,41 @@ __global__ void __launch_bounds__(NT, MINB) hop_kernel(const Geom g, const Args<
         }
     }
     const int nb[8] = {nb0.x, nb0.y, nb0.z, nb0.w, nb1.x, nb1.y, nb1.z, nb1.w};
-    hop_dir<SP, LS, PRE, 0, +1>(nb[0], h, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
-    hop_dir<SP, LS, PRE, 0, -1>(nb[1], h, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
-    hop_dir<SP, LS, PRE, 1, +1>(nb[2], h, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
-    hop_dir<SP, LS, PRE, 1, -1>(nb[3], h, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
-    hop_dir<SP, LS, PRE, 2, +1>(nb[4], h, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
-    hop_dir<SP, LS, PRE, 2, -1>(nb[5], h, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
-    hop_dir<SP, LS, PRE, 3, +1>(nb[6], h, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
-    hop_dir<SP, LS, PRE, 3, -1>(nb[7], h, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
+    hop_dir<SP, LS, PRE, 0, +1>(nb[0], hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
+    hop_dir<SP, LS, PRE, 0, -1>(nb[1], hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
+    hop_dir<SP, LS, PRE, 1, +1>(nb[2], hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
+    hop_dir<SP, LS, PRE, 1, -1>(nb[3], hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
+    hop_dir<SP, LS, PRE, 2, +1>(nb[4], hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
+    hop_dir<SP, LS, PRE, 2, -1>(nb[5], hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
+    hop_dir<SP, LS, PRE, 3, +1>(nb[6], hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
+    hop_dir<SP, LS, PRE, 3, -1>(nb[7], hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
   }
-  epilogue_g<SP, LS, POST, LOC, G5, NORM>(a, coef, sbuf + j * SST, NP, h, t, active, true, rhs, acc);
+  epilogue_g<SP, LS, POST, LOC, G5, NORM>(a, coef, sbuf, tid, nth, S, NP, h, j, t, active, part, rhs, acc);
 }
 
 // out = c * PROG(gamma5^g5in in), site-local, two slices per thread.
 template <class SP, int LS, int PROG>
 __global__ void __launch_bounds__(128) local_kernel(const Geom g, void* out, const void* in,
                                                     size_t stride, const typename SP::T* chain,
-                                                    typename SP::T c, int g5in, Reduce red,
-                                                    int do_norm, size_t cstride,
+                                                    typename SP::T c, int g5in, size_t cstride,
                                                     const int* rhs_on) {
   using T = typename SP::T;
   using A = Pr<T>;
   using V = typename A::V;
-  constexpr int SST = site_stride(LS);
+  constexpr int G = LS / 2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* coef = reinterpret_cast<T*>(smem_raw);
-  T* sbuf = coef + chain_block(LS);
-  const int t = threadIdx.x, j = threadIdx.y;
-  const int nth = blockDim.x * blockDim.y, tid = j * blockDim.x + t;
-  const int h = blockIdx.x * blockDim.y + j;
-  const bool active = h < g.Vh;
+  T* sbuf = coef + prog_coefs(LS, PROG);
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int S = nth / G, j = tid / G, t = tid - j * G;
+  const int h = blockIdx.x * S + j;
+  const bool active = j < S && h < g.Vh;
   const int rhs = blockIdx.z;
   if (rhs_on && !rhs_on[rhs]) return;
   const size_t NP = (size_t)g.N5 >> 1;
-  for (int i = tid; i < chain_block(LS); i += nth) coef[i] = chain[(size_t)rhs * cstride + i];
+  load_coefs<T, LS, PROG>(coef, chain + (size_t)rhs * cstride, tid, nth);
   const size_t off = rhs * stride;
-  const size_t m = (size_t)h * (LS / 2) + t;
+  const size_t m = (size_t)h * G + t;
   SpinP<V> x;
   zero(x);
   if (active) load_spin<SP>(reinterpret_cast<const char*>(in) + off, m, NP, x);
@@ -674,26 +790,14 @@ __global__ void __launch_bounds__(128) local_kernel(const Geom g, void* out, con
     x.re[k] = A::mul(k >= 6 ? cm : cp, x.re[k]);
     x.im[k] = A::mul(k >= 6 ? cm : cp, x.im[k]);
   }
-  T* site = sbuf + j * SST;
-  put(site + t * kPairStride, x);
+  T* site = sbuf + j * site_stride(LS);
+  if (j < S) put<T, LS, PROG>(site, t, x);
   __syncthreads();
-  run_prog<T, LS, PROG>(site, coef, t);
+  run_prog<T, LS, PROG>(sbuf, coef, tid, nth, S);
   __syncthreads();
-  get(site + t * kPairStride, x);
-  if (active) PairIO<SP>::store(reinterpret_cast<char*>(out) + off, m, NP, x);
-  if (do_norm) {
-    double v = 0.0;
-    if (active) {
-      if constexpr (SP::kScaled) {
-        SpinP<V> q = x;
-        PairIO<SP>::quantize(q);
-        v = sqr(q);
-      } else {
-        v = sqr(x);
-      }
-    }
-    block_sum_to(v, red, rhs, gridDim.x, blockIdx.x);
-  }
+  if (!active) return;
+  get<T, LS, PROG>(site, t, x);
+  PairIO<SP>::store(reinterpret_cast<char*>(out) + off, m, NP, x);
 }
 
 }  // namespace hop2
@@ -704,13 +808,22 @@ __global__ void __launch_bounds__(128) local_kernel(const Geom g, void* out, con
 namespace dwf {
 namespace hop2 {
 
-// 4D sites per CTA: the default tile (128 threads) and the small one (64 threads);
-// HopLaunch.block_sites selects the small tile when it equals small_block_sites.
-inline int block_sites(int Ls) { return 128 / (Ls / 2); }
-inline int small_block_sites(int Ls) { return 64 / (Ls / 2); }
+// Threads per CTA (HopLaunch.block_threads; 0: by the rule of tile_threads).
+constexpr int kTileThreads[3] = {128, 64, 32};
 
-inline size_t smem_bytes(int Ls, int S, size_t ts) {
-  return ts * ((size_t)chain_block(Ls) + (size_t)S * site_stride(Ls));
+// The largest CTA that still gives every SM four of them (FP64: eight): a small lattice
+// then spreads over the SMs, and over the sub-partitions of an SM.
+inline int tile_threads(int Ls, int Vh, int nrhs, bool f64) {
+  for (int nt : kTileThreads) {
+    const int S = nt / (Ls / 2);
+    const long long blocks = (long long)((Vh + S - 1) / S) * nrhs;
+    if (blocks >= 152 * (f64 ? 8 : 4) * 128 / nt) return nt;
+  }
+  return 32;
+}
+
+inline size_t smem_bytes(int Ls, int S, size_t ts, int prog) {
+  return prog == PR_NONE ? 0 : ts * ((size_t)prog_coefs(Ls, prog) + (size_t)S * site_stride(Ls));
 }
 
 // Raises a kernel's dynamic shared-memory limit once per process; safe when
@@ -764,7 +877,7 @@ cudaError_t run_tma(const Geom& g, const HopLaunch& L, const Args<typename SP::T
   CUtensorMap map;
   cudaError_t e = encode_field_map<SP, LS>(&map, g, L.v, L.stride, L.nrhs);
   if (e != cudaSuccess) return e;
-  const size_t smem = tma_smem_bytes<SP, LS, NST>();
+  const size_t smem = tma_smem_bytes<SP, LS, NST, POST>();
   auto k = hop_tma_kernel<SP, LS, PRE, POST, LOC, G5, NORM, NST, 1>;
   static std::atomic<bool> attr{false};
   e = smem_limit_once(k, smem, attr);
@@ -801,27 +914,17 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   a.cstride = L.cstride;
   a.active = L.active;
   a.err = L.err;
-  if (L.use_tma) return run_tma<SP, LS, PRE, POST, LOC, G5, NORM>(g, L, a, st);
-  const bool small = L.block_sites == small_block_sites(LS);
-  const int S = small ? small_block_sites(LS) : block_sites(LS);
-  dim3 block(LS / 2, S, 1);
-  dim3 grid((g.Vh + S - 1) / S, 1, L.nrhs);
-  const size_t smem = smem_bytes(LS, S, sizeof(T));
-  constexpr int MB = min_blocks<T>();
-  // dynamic shared memory limits, set once per kernel
-  if (small) {
-    auto k = hop_kernel<SP, LS, PRE, POST, LOC, G5, NORM, 2 * MB, 64>;
-    static std::atomic<bool> attr_small{false};
-    cudaError_t e = smem_limit_once(k, smem, attr_small);
-    if (e != cudaSuccess) return e;
-    k<<<grid, block, smem, st>>>(g, a);
-  } else {
-    auto k = hop_kernel<SP, LS, PRE, POST, LOC, G5, NORM, MB>;
-    static std::atomic<bool> attr{false};
-    cudaError_t e = smem_limit_once(k, smem, attr);
-    if (e != cudaSuccess) return e;
-    k<<<grid, block, smem, st>>>(g, a);
+  if constexpr (tma_ls(LS) && POST != PR_NONE) {
+    if (L.use_tma) return run_tma<SP, LS, PRE, POST, LOC, G5, NORM>(g, L, a, st);
   }
+  const int nt = L.block_threads ? L.block_threads : tile_threads(LS, g.Vh, L.nrhs, sizeof(T) == 8);
+  const int S = nt / (LS / 2);
+  dim3 grid((g.Vh + S - 1) / S, 1, L.nrhs);
+  auto k = hop_kernel<SP, LS, PRE, POST, LOC, G5, NORM, min_blocks<T>()>;
+  static std::atomic<bool> attr{false};
+  cudaError_t e = smem_limit_once(k, smem_bytes(LS, 128 / (LS / 2), sizeof(T), POST), attr);
+  if (e != cudaSuccess) return e;
+  k<<<grid, nt, smem_bytes(LS, S, sizeof(T), POST), st>>>(g, a);
   return cudaGetLastError();
 }
 
@@ -830,9 +933,12 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
 template <class SP, int LS>
 cudaError_t dispatch_ls(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   const bool norm = L.red != nullptr;
-  if (L.loc == LOC_DENSE) return cudaErrorNotSupported;
-  if (L.pre == PRE_B && L.post_prog == PR_K && L.loc == LOC_NONE && !L.g5out && !norm)
-    return run<SP, LS, PRE_B, PR_K, LOC_NONE, false, false>(g, L, st);
+  if (L.loc == LOC_DENSE || (L.loc == LOC_ID && L.c_loc != 1.0)) return cudaErrorNotSupported;
+  // FP64 is bound by the FP64 pipe: its callers form B v once (PR_B) and hop that
+  if constexpr (SP::kPrec != P64) {
+    if (L.pre == PRE_B && L.post_prog == PR_K && L.loc == LOC_NONE && !L.g5out && !norm)
+      return run<SP, LS, PRE_B, PR_K, LOC_NONE, false, false>(g, L, st);
+  }
   if (L.pre == PRE_NONE && L.post_prog == PR_K && L.loc == LOC_NONE && !L.g5out && !norm)
     return run<SP, LS, PRE_NONE, PR_K, LOC_NONE, false, false>(g, L, st);
   if (L.pre == PRE_NONE && L.post_prog == PR_IINV && L.loc == LOC_ID && !L.g5out)
@@ -849,41 +955,54 @@ cudaError_t dispatch_ls(const Geom& g, const HopLaunch& L, cudaStream_t st) {
 template <class SP, int LS, int PROG>
 cudaError_t run_local(const Geom& g, const LocalLaunch& L, cudaStream_t st) {
   using T = typename SP::T;
-  const int S = block_sites(LS);
-  const size_t smem = smem_bytes(LS, S, sizeof(T));
+  const int nt = tile_threads(LS, g.Vh, L.nrhs, sizeof(T) == 8), S = nt / (LS / 2);
+  const size_t smem = smem_bytes(LS, S, sizeof(T), PROG);
   auto k = local_kernel<SP, LS, PROG>;
   static std::atomic<bool> attr{false};
-  cudaError_t e = smem_limit_once(k, smem, attr);
+  cudaError_t e = smem_limit_once(k, smem_bytes(LS, 128 / (LS / 2), sizeof(T), PROG), attr);
   if (e != cudaSuccess) return e;
-  Reduce red{};
-  if (L.red) red = *L.red;
-  dim3 block(LS / 2, S, 1);
   dim3 grid((g.Vh + S - 1) / S, 1, L.nrhs);
-  k<<<grid, block, smem, st>>>(g, L.out, L.in, L.stride, reinterpret_cast<const T*>(L.chain),
-                               (T)L.c, L.g5in, red, L.red != nullptr, L.cstride, L.active);
+  k<<<grid, nt, smem, st>>>(g, L.out, L.in, L.stride, reinterpret_cast<const T*>(L.chain), (T)L.c,
+                            L.g5in, L.cstride, L.active);
   return cudaGetLastError();
 }
+
+// F<LS>::call(...) for the compiled Ls.
+#define DWF_LS_CASE(LS, CALL)                                      \
+  case LS:                                                         \
+    if constexpr (tuned_ls(LS, SP::kScaled)) return CALL(LS);      \
+    break;
+#define DWF_TUNED_LS(Ls, CALL)                                                              \
+  switch (Ls) {                                                                             \
+    DWF_LS_CASE(4, CALL) DWF_LS_CASE(6, CALL) DWF_LS_CASE(8, CALL) DWF_LS_CASE(10, CALL)    \
+    DWF_LS_CASE(12, CALL) DWF_LS_CASE(16, CALL) DWF_LS_CASE(20, CALL) DWF_LS_CASE(24, CALL) \
+    DWF_LS_CASE(32, CALL)                                                                   \
+  }                                                                                         \
+  return cudaErrorNotSupported;
 
 template <class SP>
 cudaError_t dispatch(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   if (L.chain == nullptr || L.nbr == nullptr) return cudaErrorNotSupported;
-  switch (g.Ls) {
-    case 8: return dispatch_ls<SP, 8>(g, L, st);
-    case 12: return dispatch_ls<SP, 12>(g, L, st);
-    case 16: return dispatch_ls<SP, 16>(g, L, st);
+#define DWF_CALL(LS) dispatch_ls<SP, LS>(g, L, st)
+  DWF_TUNED_LS(g.Ls, DWF_CALL)
+#undef DWF_CALL
+}
+
+template <class SP, int LS>
+cudaError_t dispatch_local_ls(const Geom& g, const LocalLaunch& L, cudaStream_t st) {
+  if (L.prog == PR_ITINV) return run_local<SP, LS, PR_ITINV>(g, L, st);
+  if constexpr (SP::kPrec == P64) {
+    if (L.prog == PR_B) return run_local<SP, LS, PR_B>(g, L, st);
   }
   return cudaErrorNotSupported;
 }
 
 template <class SP>
 cudaError_t dispatch_local(const Geom& g, const LocalLaunch& L, cudaStream_t st) {
-  if (L.chain == nullptr || L.prog != PR_ITINV) return cudaErrorNotSupported;
-  switch (g.Ls) {
-    case 8: return run_local<SP, 8, PR_ITINV>(g, L, st);
-    case 12: return run_local<SP, 12, PR_ITINV>(g, L, st);
-    case 16: return run_local<SP, 16, PR_ITINV>(g, L, st);
-  }
-  return cudaErrorNotSupported;
+  if (L.chain == nullptr || L.red != nullptr) return cudaErrorNotSupported;
+#define DWF_CALL(LS) dispatch_local_ls<SP, LS>(g, L, st)
+  DWF_TUNED_LS(g.Ls, DWF_CALL)
+#undef DWF_CALL
 }
 
 
@@ -900,23 +1019,23 @@ __global__ void __launch_bounds__(128) rupdate_kernel(const Geom g, void* r, voi
   using T = typename SP::T;
   using A = Pr<T>;
   using V = typename A::V;
-  constexpr int SST = site_stride(LS);
+  constexpr int G = LS / 2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* coef = reinterpret_cast<T*>(smem_raw);
-  T* sbuf = coef + chain_block(LS);
-  const int t = threadIdx.x, j = threadIdx.y;
-  const int nth = blockDim.x * blockDim.y, tid = j * blockDim.x + t;
-  const int h = blockIdx.x * blockDim.y + j;
-  const bool active = h < g.Vh;
+  T* sbuf = coef + prog_coefs(LS, PR_ITINV);
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int S = nth / G, j = tid / G, t = tid - j * G;
+  const int h = blockIdx.x * S + j;
+  const bool active = j < S && h < g.Vh;
   const int rhs = blockIdx.z;
   if (rhs_on && !rhs_on[rhs]) return;
   const size_t NP = (size_t)g.N5 >> 1;
   const double ad = num[(size_t)rhs * sstride] / den[(size_t)rhs * sstride];
   if (blockIdx.x == 0 && tid == 0) a_out[(size_t)rhs * sstride] = ad;
   const V na = A::dup(-(T)ad);
-  for (int i = tid; i < chain_block(LS); i += nth) coef[i] = chain[(size_t)rhs * cstride + i];
+  load_coefs<T, LS, PR_ITINV>(coef, chain + (size_t)rhs * cstride, tid, nth);
   const size_t off = rhs * stride;
-  const size_t m = (size_t)h * (LS / 2) + t;
+  const size_t m = (size_t)h * G + t;
   SpinP<V> x;
   zero(x);
   double nrm = 0.0;
@@ -939,40 +1058,37 @@ __global__ void __launch_bounds__(128) rupdate_kernel(const Geom g, void* r, voi
     x.re[k] = A::neg(x.re[k]);
     x.im[k] = A::neg(x.im[k]);
   }
-  T* site = sbuf + j * SST;
-  put(site + t * kPairStride, x);
+  T* site = sbuf + j * site_stride(LS);
+  if (j < S) put<T, LS, PR_ITINV>(site, t, x);
   __syncthreads();
-  run_prog<T, LS, PR_ITINV>(site, coef, t);
+  run_prog<T, LS, PR_ITINV>(sbuf, coef, tid, nth, S);
   __syncthreads();
-  get(site + t * kPairStride, x);
-  if (active) PairIO<SP>::store(reinterpret_cast<char*>(rhat) + off, m, NP, x);
+  if (active) {
+    get<T, LS, PR_ITINV>(site, t, x);
+    PairIO<SP>::store(reinterpret_cast<char*>(rhat) + off, m, NP, x);
+  }
   block_sum_to(nrm, red, rhs, gridDim.x, blockIdx.x);
 }
 
 template <class SP, int LS>
 cudaError_t run_rupdate(const Geom& g, const RUpdateLaunch& L, cudaStream_t st) {
   using T = typename SP::T;
-  const int S = block_sites(LS);
-  const size_t smem = smem_bytes(LS, S, sizeof(T));
+  const int nt = tile_threads(LS, g.Vh, L.nrhs, sizeof(T) == 8), S = nt / (LS / 2);
   auto k = rupdate_kernel<SP, LS>;
   static std::atomic<bool> attr{false};
-  cudaError_t e = smem_limit_once(k, smem, attr);
+  cudaError_t e = smem_limit_once(k, smem_bytes(LS, 128 / (LS / 2), sizeof(T), PR_ITINV), attr);
   if (e != cudaSuccess) return e;
-  dim3 block(LS / 2, S, 1);
   dim3 grid((g.Vh + S - 1) / S, 1, L.nrhs);
-  k<<<grid, block, smem, st>>>(g, L.r, L.rhat, L.w, L.stride, reinterpret_cast<const T*>(L.chain),
+  k<<<grid, nt, smem_bytes(LS, S, sizeof(T), PR_ITINV), st>>>(g, L.r, L.rhat, L.w, L.stride, reinterpret_cast<const T*>(L.chain),
                                L.cstride, L.num, L.den, L.a_out, L.sstride, *L.red, L.active);
   return cudaGetLastError();
 }
 
 template <class SP>
 cudaError_t dispatch_rupdate(const Geom& g, const RUpdateLaunch& L, cudaStream_t st) {
-  switch (g.Ls) {
-    case 8: return run_rupdate<SP, 8>(g, L, st);
-    case 12: return run_rupdate<SP, 12>(g, L, st);
-    case 16: return run_rupdate<SP, 16>(g, L, st);
-  }
-  return cudaErrorNotSupported;
+#define DWF_CALL(LS) run_rupdate<SP, LS>(g, L, st)
+  DWF_TUNED_LS(g.Ls, DWF_CALL)
+#undef DWF_CALL
 }
 }  // namespace hop2
 }  // namespace dwf

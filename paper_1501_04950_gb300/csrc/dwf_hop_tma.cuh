@@ -22,6 +22,8 @@ namespace hop2 {
 
 constexpr int kTmaConsumers = 128;
 constexpr int kTmaThreads = kTmaConsumers + 32;
+// the Ls with a staged variant
+__host__ __device__ constexpr bool tma_ls(int Ls) { return Ls == 8 || Ls == 12 || Ls == 16; }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -229,12 +231,11 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
   using ST = Stage<SP, LS>;
   constexpr int HALF = LS / 2;
   constexpr int S = kTmaConsumers / HALF;
-  constexpr int SST = site_stride(LS);
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw);
   uint64_t* empty = full + NST;
   T* coef = reinterpret_cast<T*>(smem_raw + 128);
-  unsigned char* stages = smem_raw + 128 + (chain_block(LS) * (int)sizeof(T) + 127) / 128 * 128;
+  unsigned char* stages = smem_raw + 128 + (prog_coefs(LS, POST) * (int)sizeof(T) + 127) / 128 * 128;
   const int tid = threadIdx.x;
   const bool producer = tid >= kTmaConsumers;
   const int t = tid % HALF, j = tid / HALF;
@@ -253,9 +254,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (POST != PR_NONE) {
-    for (int i = tid; i < chain_block(LS); i += kTmaThreads) coef[i] = a.chain[co + i];
-  }
+  load_coefs<T, LS, POST>(coef, a.chain + co, tid, kTmaThreads);
   __syncthreads();
   SpinP<V> acc;
   zero(acc);
@@ -348,17 +347,17 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
   // the stages are consumed (every full phase waited for): reuse them for the
   // 5th-dimension transpose of the epilogue
   __syncthreads();
-  T* site = reinterpret_cast<T*>(stages) + (size_t)(cons ? j : 0) * SST;
-  epilogue_g<SP, LS, POST, LOC, G5, NORM>(a, coef, site, NP, h, t, active, cons, rhs, acc);
+  epilogue_g<SP, LS, POST, LOC, G5, NORM>(a, coef, reinterpret_cast<T*>(stages), tid, kTmaConsumers, S, NP,
+                                          h, j, t, active, cons, rhs, acc);
 }
 
-template <class SP, int LS, int NST>
+template <class SP, int LS, int NST, int POST>
 constexpr size_t tma_smem_bytes() {
   using T = typename SP::T;
   constexpr int S = kTmaConsumers / (LS / 2);
   constexpr size_t ring = (size_t)NST * S * Stage<SP, LS>::kBytes;
   constexpr size_t tr = (size_t)S * site_stride(LS) * sizeof(T);
-  return 128 + ((size_t)chain_block(LS) * sizeof(T) + 127) / 128 * 128 + (ring > tr ? ring : tr);
+  return 128 + ((size_t)prog_coefs(LS, POST) * sizeof(T) + 127) / 128 * 128 + (ring > tr ? ring : tr);
 }
 
 }  // namespace hop2

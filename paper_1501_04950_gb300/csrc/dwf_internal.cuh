@@ -84,8 +84,8 @@ struct HopLaunch {
   double c_hop, c_loc;
   int g5out;
   const Reduce* red;        // nullptr: no norm
-  int block_sites;          // 4D sites per CTA (0: default)
-  // Tuned path (Ls in {8, 12, 16}): 5th-dimension operators as chain programs
+  int block_threads;        // threads per CTA of the tuned kernels (0: by size)
+  // Tuned path (hop2::tuned_ls): 5th-dimension operators as chain programs
   // (hop2::PR_*) over the recurrence coefficient block, and the neighbour table.
   int post_prog;
   int loc_prog;
@@ -106,7 +106,7 @@ cudaError_t launch_hop2_f64(const Geom& g, const HopLaunch& a, cudaStream_t s);
 cudaError_t launch_hop2_f32(const Geom& g, const HopLaunch& a, cudaStream_t s);
 cudaError_t launch_hop2_f16(const Geom& g, const HopLaunch& a, cudaStream_t s);
 cudaError_t launch_hop2_bf16(const Geom& g, const HopLaunch& a, cudaStream_t s);
-int hop_grid_blocks(const Geom& g, int prec, int block_sites);
+int hop_grid_blocks(const Geom& g, int prec);  // blocks of the generic kernel
 
 // ---- site-local dense contraction: out = c * M (gamma5^g5in in) ---------------
 struct LocalLaunch {
@@ -129,7 +129,7 @@ cudaError_t launch_hop2_f64_local(const Geom& g, const LocalLaunch& a, cudaStrea
 cudaError_t launch_hop2_f32_local(const Geom& g, const LocalLaunch& a, cudaStream_t s);
 cudaError_t launch_hop2_f16_local(const Geom& g, const LocalLaunch& a, cudaStream_t s);
 cudaError_t launch_hop2_bf16_local(const Geom& g, const LocalLaunch& a, cudaStream_t s);
-// Fused CG residual update of the tuned path (Ls in {8, 12, 16}):
+// Fused CG residual update of the tuned path (hop2::tuned_ls):
 // r -= a w (a = num/den, stored to a_out), |r|^2 -> red, rhat = I^-T gamma5 r.
 struct RUpdateLaunch {
   int prec;

@@ -492,6 +492,40 @@ void set_coef(HopLaunch& L, const CoefView& cv) {
 int apply_dbb_bp(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* p, const void* bp,
                  void* tmp, int nrhs, const Reduce* norm, cudaStream_t s);
 
+// out = PROG in, site-local, FP64 (B, I, K or I^-1), by the tuned kernels (cv.tuned(P64)).
+// in and out may be the same field.
+int apply_prog64(dwf_ctx* h, const CoefView& cv, int prog, void* out, const void* in, int nrhs,
+                 cudaStream_t s) {
+  LocalLaunch L{};
+  L.prec = P64;
+  L.out = out;
+  L.in = in;
+  L.stride = field_bytes(h->g, P64);
+  L.nrhs = nrhs;
+  L.prog = prog;
+  L.chain = cv.chain(P64);
+  L.c = 1.0;
+  L.cstride = cv.cstride;
+  L.active = cv.active;
+  KLAUNCH(h, launch_local(h->g, L, s));
+  return DWF_OK;
+}
+
+// out = w + c_hop H v at the sites of parity p, FP64, by the tuned kernels.  w may be out.
+int apply_hop64(dwf_ctx* h, const CoefView& cv, int p, void* out, const void* v, const void* w,
+                double c_hop, cudaStream_t s) {
+  HopLaunch L = base_hop(h, P64, p, 1, field_bytes(h->g, P64));
+  L.out = out;
+  L.v = v;
+  L.w = w;
+  L.loc = LOC_ID;
+  L.c_hop = c_hop;
+  L.c_loc = 1.0;
+  L.chain = cv.chain(P64);
+  KLAUNCH(h, launch_hop(h->g, L, s));
+  return DWF_OK;
+}
+
 // out = D_bb in.  tmp: red half-field(s) of the same precision.
 int apply_dbb(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* in, void* tmp, int nrhs,
               const Reduce* norm, cudaStream_t s) {
@@ -501,18 +535,7 @@ int apply_dbb(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* i
     // its ~1370 operations per 5D site, formed once it is 48.  out holds B in until
     // pass B overwrites it.  16^3x32, Ls = 16:
     // D_bb and D_bb^+ together 7.95 -> 7.20 ms.
-    LocalLaunch L{};
-    L.prec = P64;
-    L.out = out;
-    L.in = in;
-    L.stride = field_bytes(h->g, P64);
-    L.nrhs = nrhs;
-    L.prog = hop2::PR_B;
-    L.chain = cv.chain(P64);
-    L.c = 1.0;
-    L.cstride = cv.cstride;
-    L.active = cv.active;
-    KLAUNCH(h, launch_local(h->g, L, s));
+    if (int rc = apply_prog64(h, cv, hop2::PR_B, out, in, nrhs, s)) return rc;
     return apply_dbb_bp(h, cv, P64, out, in, out, tmp, nrhs, norm, s);
   }
   const int black = h->opt.rb_parity, red = 1 - black;
@@ -655,8 +678,23 @@ int apply_local_dense(dwf_ctx* h, const CoefView& cv, int prec, int which, void*
   return DWF_OK;
 }
 
-// (out0, out1) = D_alpha(ms) (in0, in1), FP64 internal halves by parity.
+// (out0, out1) = D_alpha(ms) (in0, in1) = I in - 1/2 H (B in), FP64 internal halves by parity.
 int apply_dalpha_halves(dwf_ctx* h, const MatSet& ms, void* out[2], const void* in[2], cudaStream_t s) {
+  const CoefView cv = view_of(ms);
+  if (cv.tuned(P64)) {
+    // I and B as recurrences (144 flops a 5D site each), once per site: folded into the
+    // hops and as a dense contraction they were 384 + 24 Ls of the ~1270 FP64
+    // operations of a site at Ls = 16
+    void* bv;
+    int rc = get_ws(h, "da_b", field_bytes(h->g, P64), &bv);
+    if (rc) return rc;
+    for (int p = 0; p < 2; p++)
+      if ((rc = apply_prog64(h, cv, hop2::PR_B, bv, in[1 - p], 1, s)) ||
+          (rc = apply_prog64(h, cv, hop2::PR_I, out[p], in[p], 1, s)) ||
+          (rc = apply_hop64(h, cv, p, out[p], bv, out[p], -0.5, s)))
+        return rc;
+    return DWF_OK;
+  }
   const size_t st = field_bytes(h->g, P64);
   for (int p = 0; p < 2; p++) {
     HopLaunch L = base_hop(h, P64, p, 1, st);
@@ -1911,7 +1949,16 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
       CUCHK(h, cudaMemcpyAsync(reinterpret_cast<char*>(bc32) + r * cnt * 4, m.dev[1], cnt * 4,
                                cudaMemcpyDeviceToDevice, st));
       if ((rc = make_rhs(blk + r))) return rc;
-      // r'_b = I^-1 rhs_b + 1/2 I^-1 H_br (K rhs_r)
+      // r'_b = I^-1 (rhs_b + 1/2 H_br (K rhs_r))
+      void* b_r = reinterpret_cast<char*>(W.b_hi) + r * f64;
+      const CoefView cm = view_of(m);
+      if (cm.tuned(P64)) {
+        if ((rc = apply_prog64(h, cm, hop2::PR_K, W.t64r, rhs[red], 1, st)) ||
+            (rc = apply_hop64(h, cm, black, b_r, W.t64r, rhs[black], 0.5, st)) ||
+            (rc = apply_prog64(h, cm, hop2::PR_IINV, b_r, b_r, 1, st)))
+          return rc;
+        continue;
+      }
       LocalLaunch Lk{};
       Lk.prec = P64;
       Lk.out = W.t64r;
@@ -1922,7 +1969,7 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
       Lk.c = 1.0;
       KLAUNCH(h, launch_local(g, Lk, st));
       HopLaunch Hs = base_hop(h, P64, black, 1, f64);
-      Hs.out = reinterpret_cast<char*>(W.b_hi) + r * f64;
+      Hs.out = b_r;
       Hs.v = W.t64r;
       Hs.w = rhs[black];
       Hs.post = m.ptr(P64, m.mat_off(MatSet::IINV));
@@ -1943,20 +1990,28 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
       const MatSet& m = *ms[k];
       void* xb = reinterpret_cast<char*>(W.x_hi) + r * f64;
       if ((rc = make_rhs(k))) return rc;
-      // psi_r = I^-1 rhs_r + 1/2 I^-1 H_rb (B psi_b)
-      HopLaunch Hr = base_hop(h, P64, red, 1, f64);
-      Hr.out = psi_r;
-      Hr.v = xb;
-      Hr.w = rhs[red];
-      Hr.pre = PRE_B;
-      Hr.pre_diag = m.ptr(P64, m.bdiag_off());
-      Hr.pre_off = m.ptr(P64, m.boff_off());
-      Hr.post = m.ptr(P64, m.mat_off(MatSet::IINV));
-      Hr.loc = LOC_DENSE;
-      Hr.locm = m.ptr(P64, m.mat_off(MatSet::IINV));
-      Hr.c_hop = 0.5;
-      Hr.c_loc = 1.0;
-      KLAUNCH(h, launch_hop(g, Hr, st));
+      // psi_r = I^-1 (rhs_r + 1/2 H_rb (B psi_b))
+      const CoefView cm = view_of(m);
+      if (cm.tuned(P64)) {
+        if ((rc = apply_prog64(h, cm, hop2::PR_B, W.t64, xb, 1, st)) ||
+            (rc = apply_hop64(h, cm, red, psi_r, W.t64, rhs[red], 0.5, st)) ||
+            (rc = apply_prog64(h, cm, hop2::PR_IINV, psi_r, psi_r, 1, st)))
+          return rc;
+      } else {
+        HopLaunch Hr = base_hop(h, P64, red, 1, f64);
+        Hr.out = psi_r;
+        Hr.v = xb;
+        Hr.w = rhs[red];
+        Hr.pre = PRE_B;
+        Hr.pre_diag = m.ptr(P64, m.bdiag_off());
+        Hr.pre_off = m.ptr(P64, m.boff_off());
+        Hr.post = m.ptr(P64, m.mat_off(MatSet::IINV));
+        Hr.loc = LOC_DENSE;
+        Hr.locm = m.ptr(P64, m.mat_off(MatSet::IINV));
+        Hr.c_hop = 0.5;
+        Hr.c_loc = 1.0;
+        KLAUNCH(h, launch_hop(g, Hr, st));
+      }
       void* psi[2];
       psi[black] = xb;
       psi[red] = psi_r;

@@ -939,6 +939,10 @@ cudaError_t dispatch_ls(const Geom& g, const HopLaunch& L, cudaStream_t st) {
     if (L.pre == PRE_B && L.post_prog == PR_K && L.loc == LOC_NONE && !L.g5out && !norm)
       return run<SP, LS, PRE_B, PR_K, LOC_NONE, false, false>(g, L, st);
   }
+  if constexpr (SP::kPrec == P64) {  // D_alpha, the Schur right-hand side, the red solution
+    if (L.pre == PRE_NONE && L.post_prog == PR_NONE && !L.post && L.loc == LOC_ID && !L.g5out && !norm)
+      return run<SP, LS, PRE_NONE, PR_NONE, LOC_ID, false, false>(g, L, st);
+  }
   if (L.pre == PRE_NONE && L.post_prog == PR_K && L.loc == LOC_NONE && !L.g5out && !norm)
     return run<SP, LS, PRE_NONE, PR_K, LOC_NONE, false, false>(g, L, st);
   if (L.pre == PRE_NONE && L.post_prog == PR_IINV && L.loc == LOC_ID && !L.g5out)
@@ -993,6 +997,9 @@ cudaError_t dispatch_local_ls(const Geom& g, const LocalLaunch& L, cudaStream_t 
   if (L.prog == PR_ITINV) return run_local<SP, LS, PR_ITINV>(g, L, st);
   if constexpr (SP::kPrec == P64) {
     if (L.prog == PR_B) return run_local<SP, LS, PR_B>(g, L, st);
+    if (L.prog == PR_I) return run_local<SP, LS, PR_I>(g, L, st);
+    if (L.prog == PR_K) return run_local<SP, LS, PR_K>(g, L, st);
+    if (L.prog == PR_IINV) return run_local<SP, LS, PR_IINV>(g, L, st);
   }
   return cudaErrorNotSupported;
 }

@@ -38,7 +38,7 @@ thread_local std::string g_create_error;
 
 // Real Ls x Ls matrices of one (alpha, m) for both chiralities, FP64 host copy
 // and device copies in FP64 and FP32.  Device layout (in elements):
-//   K[2][Ls][Ls] KT IinvM IinvT Ifull BT  then Bdiag[2][Ls] Boff[2][Ls]
+//   K[2][Ls][Ls] KT IinvM IinvT Ifull BT IT SI SIT B  then Bdiag[2][Ls] Boff[2][Ls]
 struct MatSet {
   double alpha = 1.0, m = 0.0;
   int Ls = 0;
@@ -46,7 +46,7 @@ struct MatSet {
   void* dev[2] = {nullptr, nullptr};  // [0] double, [1] float
   bool chain_ok = false;              // the recurrences are as accurate as the dense inverse
   // IT = I^T, SI = S I and SIT = (S I)^T for the operator forms of Eq. redblack1
-  enum { K = 0, KT = 1, IINV = 2, IINVT = 3, IFULL = 4, BT = 5, IT = 6, SI = 7, SIT = 8, NMAT = 9 };
+  enum { K = 0, KT = 1, IINV = 2, IINVT = 3, IFULL = 4, BT = 5, IT = 6, SI = 7, SIT = 8, B = 9, NMAT = 10 };
   size_t mat_off(int which) const { return (size_t)which * 2 * Ls * Ls; }
   size_t bdiag_off() const { return (size_t)NMAT * 2 * Ls * Ls; }
   size_t boff_off() const { return bdiag_off() + 2 * (size_t)Ls; }
@@ -325,7 +325,7 @@ int build_matset(dwf_ctx* h, double alpha, double m, MatSet** out) {
     }
     std::vector<double> mats[MatSet::NMAT] = {K, transpose(K, Ls), Iinv, transpose(Iinv, Ls), I,
                                               transpose(Bm[ch], Ls), transpose(I, Ls), SI,
-                                              transpose(SI, Ls)};
+                                              transpose(SI, Ls), Bm[ch]};
     for (int w = 0; w < MatSet::NMAT; w++)
       std::copy(mats[w].begin(), mats[w].end(), ms.host.begin() + ms.mat_off(w) + ch * LL);
     // cyclic bidiagonal form of B
@@ -2058,12 +2058,11 @@ int dwf_force(dwf_handle h, double* dSdU, const double* phi_half, const double* 
   if ((rc = build_matset(h, h->alpha, h->m, &ms))) return rc;
   const size_t f64 = field_bytes(g, P64);
   const int black = h->opt.rb_parity, red = 1 - black;
-  void *X, *Y, *eta1, *xi1, *eta2;
-  if ((rc = get_ws(h, "f_Y", f64, &Y)) || (rc = get_ws(h, "f_eta1", f64, &eta1)) ||
-      (rc = get_ws(h, "f_xi1", f64, &xi1)) || (rc = get_ws(h, "f_eta2", f64, &eta2)) ||
-      (rc = get_ws(h, "f_red", f64, &X)))
+  void *X, *Y, *bx, *u, *e1, *e2;
+  if ((rc = get_ws(h, "f_Y", f64, &Y)) || (rc = get_ws(h, "f_bx", f64, &bx)) ||
+      (rc = get_ws(h, "f_u", f64, &u)) || (rc = get_ws(h, "f_e1", f64, &e1)) ||
+      (rc = get_ws(h, "f_e2", f64, &e2)))
     return rc;
-  void* tred = X;  // red scratch of the FP64 applies
   if (X_half) {
     if ((rc = get_ws(h, "x_hi", f64, &X))) return rc;
     KLAUNCH(h, launch_pack_half(g, P64, X, X_half, 1, st));
@@ -2082,45 +2081,29 @@ int dwf_force(dwf_handle h, double* dSdU, const double* phi_half, const double* 
     rc = cgnormal_solve(h, *ms, prec, h->opt.rel_tol, h->opt.maxiter, delta, W, t64b, nullptr, st);
     if (rc) return rc;
     X = W.x_hi;
-    tred = W.t64r;
   }
-  // Y = D_bb X
-  if ((rc = apply_dbb(h, view_of(*ms), P64, Y, X, tred, 1, nullptr, st))) return rc;
-  // eta1 = I^-T Y
-  LocalLaunch Le{};
-  Le.prec = P64;
-  Le.out = eta1;
-  Le.in = Y;
-  Le.stride = f64;
-  Le.nrhs = 1;
-  Le.m = ms->ptr(P64, ms->mat_off(MatSet::IINVT));
-  Le.prog = hop2::PR_ITINV;
-  Le.chain = view_of(*ms).chain(P64);
-  Le.c = 1.0;
-  KLAUNCH(h, launch_local(g, Le, st));
-  // xi1 = I^-1 D_rb X = -1/2 I^-1 H_rb (B X)
-  HopLaunch Hx = base_hop(h, P64, red, 1, f64);
-  Hx.out = xi1;
-  Hx.v = X;
-  Hx.pre = PRE_B;
-  Hx.pre_diag = ms->ptr(P64, ms->bdiag_off());
-  Hx.pre_off = ms->ptr(P64, ms->boff_off());
-  Hx.post = ms->ptr(P64, ms->mat_off(MatSet::IINV));
-  Hx.c_hop = -0.5;
-  KLAUNCH(h, launch_hop(g, Hx, st));
-  // eta2 = I^-T D_br^+ eta1 = -1/2 K^T gamma5 H_rb (gamma5 eta1)
+  // The factors of the force (dwf_force.cu), each as it comes out of Y = D_bb X and the
+  // first half of D_bb^+ Y: bx = B X, u = K H_rb bx, e1 = gamma5 I^-T Y, e2 = K^T H_rb e1.
+  const CoefView cv = view_of(*ms);
+  if (cv.tuned(P64)) {
+    if ((rc = apply_prog64(h, cv, hop2::PR_B, bx, X, 1, st)) ||
+        (rc = apply_dbb_bp(h, cv, P64, Y, X, bx, u, 1, nullptr, st)))
+      return rc;
+  } else {
+    if ((rc = apply_local_dense(h, cv, P64, MatSet::B, bx, X, 1, nullptr, st)) ||
+        (rc = apply_dbb(h, cv, P64, Y, X, u, 1, nullptr, st)))
+      return rc;
+  }
+  if ((rc = apply_hat(h, cv, P64, e1, Y, 1, st))) return rc;
   HopLaunch He = base_hop(h, P64, red, 1, f64);
-  He.out = eta2;
-  He.v = eta1;
-  He.pre = PRE_G5;
-  He.post = ms->ptr(P64, ms->mat_off(MatSet::KT));
-  He.g5out = 1;
-  He.c_hop = -0.5;
+  He.out = e2;
+  He.v = e1;
+  He.post = cv.ptr(P64, ms->mat_off(MatSet::KT));
+  He.post_prog = hop2::PR_KT;
+  He.chain = cv.chain(P64);
   KLAUNCH(h, launch_hop(g, He, st));
-  KLAUNCH(h, launch_force(g, dSdU, eta1, xi1, eta2, X,
-                          reinterpret_cast<const double*>(ms->ptr(P64, ms->bdiag_off())),
-                          reinterpret_cast<const double*>(ms->ptr(P64, ms->boff_off())), h->gauge[0],
-                          gauge_bytes(g, P64) / 2, black, projected, st));
+  KLAUNCH(h, launch_force(g, dSdU, e1, bx, e2, u, h->nbr, h->gauge[0], gauge_bytes(g, P64) / 2, black,
+                          projected, st));
   return DWF_OK;
 }
 

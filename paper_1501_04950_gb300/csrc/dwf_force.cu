@@ -12,199 +12,213 @@
 // With the convention G_ij = dS/dRe U_ij + i dS/dIm U_ij a term Re[a^+ dU b]
 // contributes a b^+, and sum_spin a_spin (P b)_spin^+ for P = 1 -+ gamma_mu
 // reduces to the two rows of the projected half spinors: sum_k h(a)_k h(b)_k^+.
+//
+// The applies that lead here leave every factor in memory: W = B X on black sites and
+// W = K H_rb B X = -2 B xi1 on red ones (the input and the result of pass A of Y = D_bb X),
+// E = gamma5 eta1 on black and E = K^T H_rb gamma5 eta1 = -2 gamma5 eta2 on red ones
+// (the hat and pass A of D_bb^+ Y).  gamma5 turns the projector of E around, so that for
+// every link, with h-+ the half spinors of (1 -+ gamma_mu),
+//   G_mu(x) = s/2 sum_slices [ h+(E(x)) h-(W(x+mu))^+ + h+(W(x)) h-(E(x+mu))^+ ]
+// where s is the antiperiodic sign of the hop.
 #include <algorithm>
 
 #include "dwf_fields.cuh"
+#include "dwf_hop2.cuh"
 
 namespace dwf {
 
 namespace {
 
-// Half spinor of (1 - sg gamma_mu) psi (two rows of 3 colours), runtime mu.
-__device__ __forceinline__ void project_rt(const Spinor<double>& s, int mu, int sg,
-                                           cplx<double> h[2][3]) {
-  cplx<double> h0[3], h1[3];
-  switch (mu * 2 + (sg > 0 ? 0 : 1)) {
-    case 0: project<double, 0, +1>(s, h0, h1); break;
-    case 1: project<double, 0, -1>(s, h0, h1); break;
-    case 2: project<double, 1, +1>(s, h0, h1); break;
-    case 3: project<double, 1, -1>(s, h0, h1); break;
-    case 4: project<double, 2, +1>(s, h0, h1); break;
-    case 5: project<double, 2, -1>(s, h0, h1); break;
-    case 6: project<double, 3, +1>(s, h0, h1); break;
-    default: project<double, 3, -1>(s, h0, h1); break;
-  }
+using hop2::HalfP;
+using hop2::PairIO;
+
+struct ForceArgs {
+  const void* E[2];  // by parity
+  const void* W[2];
+  const int4* nbr;   // [2][Vh][2] neighbour table, bit 31: antiperiodic sign
+  const void* g64;   // internal FP64 gauge (both parities)
+  size_t gpar;       // bytes per parity
+  double* out;       // canonical [V][4][3][3] complex
+  int projected;
+};
+
+// Components c0 .. c0 + 5 of slices 2t, 2t + 1 of site h (odd Ls: no slice past the last).
+template <bool EVEN>
+__device__ __forceinline__ void load6(const Geom& g, const void* f, int h, int t, int c0, double2* re,
+                                      double2* im) {
+  if constexpr (EVEN) {
+    const int G = g.Ls >> 1;
+    PairIO<Store64>::load6(f, (size_t)h * G + t, (size_t)g.N5 >> 1, c0, re, im);
+  } else {
+    const int n = site5(h, 2 * t, g.Ls);
+    const bool two = 2 * t + 1 < g.Ls;
 #pragma unroll
-  for (int a = 0; a < 3; a++) {
-    h[0][a] = h0[a];
-    h[1][a] = h1[a];
+    for (int k = 0; k < 6; k++) {
+      const double* a = Store64::at(f, c0 + k, n, g.N5);
+      const double* b = Store64::at(f, c0 + k, two ? n + 1 : n, g.N5);
+      re[k] = make_double2(__ldg(a), two ? __ldg(b) : 0.0);
+      im[k] = make_double2(__ldg(a + 2), two ? __ldg(b + 2) : 0.0);
+    }
   }
 }
 
-// w = B xi at (site hs, slice s): B_+ row s = d+ e_s + o+ e_{s-1}, B_- row s = d- e_s + o- e_{s+1}.
-__device__ __forceinline__ void load_bxi(const Geom& g, const void* xi, int hs, int s,
-                                         const double* bd, const double* bo, Spinor<double>& w) {
-  const int Ls = g.Ls;
-  const int sp = s == 0 ? Ls - 1 : s - 1, sn = s == Ls - 1 ? 0 : s + 1;
-  Spinor<double> a, b;
-  Store64::load(xi, site5(hs, s, Ls), g.N5, w);
-  Store64::load_chir(xi, site5(hs, sp, Ls), g.N5, 0, a);
-  Store64::load_chir(xi, site5(hs, sn, Ls), g.N5, 1, b);
-  const double dp = bd[s], dm = bd[Ls + s], op = bo[s], om = bo[Ls + s];
-#pragma unroll
-  for (int k = 0; k < 6; k++) {
-    w.c[k] = cmake(dp * w.c[k].re + op * a.c[k].re, dp * w.c[k].im + op * a.c[k].im);
-    w.c[k + 6] = cmake(dm * w.c[k + 6].re + om * b.c[k + 6].re, dm * w.c[k + 6].im + om * b.c[k + 6].im);
-  }
+// Half spinors of (1 - DIR gamma_mu) f for the two slices.
+template <bool EVEN, int MU, int DIR>
+__device__ __forceinline__ void load_half(const Geom& g, const void* f, int h, int t, HalfP<double2>& P) {
+  HalfP<double2> M;
+  load6<EVEN>(g, f, h, t, 0, P.re, P.im);
+  load6<EVEN>(g, f, h, t, 6, M.re, M.im);
+  hop2::project_half<double, MU, DIR>(P, M);
 }
 
-// acc_ij += sum_k a_k,i conj(b_k,j)
-__device__ __forceinline__ void outer_add(cplx<double> acc[9], const cplx<double> a[2][3],
-                                          const cplx<double> b[2][3], int sign) {
+// G_ij += sum over rows and slices of a_i conj(b_j)
+__device__ __forceinline__ void outer_add(cplx<double> (&G)[9], const HalfP<double2>& a,
+                                          const HalfP<double2>& b) {
 #pragma unroll
   for (int k = 0; k < 2; k++)
 #pragma unroll
     for (int i = 0; i < 3; i++)
 #pragma unroll
       for (int j = 0; j < 3; j++) {
-        const cplx<double> x = a[k][i], y = b[k][j];
-        acc[3 * i + j].re += sign * (x.re * y.re + x.im * y.im);
-        acc[3 * i + j].im += sign * (x.im * y.re - x.re * y.im);
+        const double2 ar = a.re[3 * k + i], ai = a.im[3 * k + i], br = b.re[3 * k + j], bi = b.im[3 * k + j];
+        cplx<double>& c = G[3 * i + j];
+        c.re = fma(ar.x, br.x, fma(ai.x, bi.x, fma(ar.y, br.y, fma(ai.y, bi.y, c.re))));
+        c.im = fma(ai.x, br.x, fma(-ar.x, bi.x, fma(ai.y, br.y, fma(-ar.y, bi.y, c.im))));
       }
 }
 
-__device__ __forceinline__ void lex_coords(const Geom& g, int i, int& x, int& y, int& z, int& t) {
-  x = i % g.L[0];
-  int r = i / g.L[0];
-  y = r % g.L[1];
-  r /= g.L[1];
-  z = r % g.L[2];
-  t = r / g.L[2];
+template <bool EVEN, int MU>
+__device__ __forceinline__ void link_sum(const Geom& g, const ForceArgs& a, int p, int h, int hn, int t0,
+                                         int step, cplx<double> (&G)[9]) {
+  const int slots = (g.Ls + 1) >> 1;
+  for (int t = t0; t < slots; t += step) {
+    HalfP<double2> u, v;
+    load_half<EVEN, MU, -1>(g, a.E[p], h, t, u);
+    load_half<EVEN, MU, +1>(g, a.W[1 - p], hn, t, v);
+    outer_add(G, u, v);
+    load_half<EVEN, MU, -1>(g, a.W[p], h, t, u);
+    load_half<EVEN, MU, +1>(g, a.E[1 - p], hn, t, v);
+    outer_add(G, u, v);
+  }
 }
 
-struct ForceArgs {
-  const void* eta1;  // black
-  const void* xi1;   // red
-  const void* eta2;  // red
-  const void* xi2;   // black
-  const double* bd;  // B diagonal [2][Ls]
-  const double* bo;  // B off-diagonal [2][Ls]
-  const void* g64;   // internal FP64 gauge (both parities)
-  size_t gpar;       // bytes per parity
-  double* out;       // canonical [V][4][3][3] complex
-  int black;
-  int projected;
-};
-
-// One thread per link (x, mu): G = -(term1(eta_a(x), B xi_a(x+mu)) + term2(B xi_b(x), eta_b(x+mu))),
-// (a, b) = (1, 2) on black x and (2, 1) on red x.
-__global__ void force_kernel(const Geom g, const ForceArgs a) {
-  const size_t V = (size_t)g.Vh * 2;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < V * 4;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const int site = (int)(i / 4), mu = (int)(i % 4);
-    int x, y, z, t;
-    lex_coords(g, site, x, y, z, t);
-    const int q = (x + y + z + t) & 1;
-    const int h = site >> 1;
-    int c[4] = {x, y, z, t};
-    double sign = 1.0;
-    c[mu] += 1;
-    if (c[mu] == g.L[mu]) {
-      c[mu] = 0;
-      if (mu == 3) sign = g.bc_t;
-    }
-    const int hn = (c[0] >> 1) + g.Lxh * (c[1] + g.L[1] * (c[2] + g.L[2] * c[3]));
-    const bool is_black = q == a.black;
-    const void* eta_a = is_black ? a.eta1 : a.eta2;
-    const void* xi_a = is_black ? a.xi1 : a.xi2;
-    const void* eta_b = is_black ? a.eta2 : a.eta1;
-    const void* xi_b = is_black ? a.xi2 : a.xi1;
-    cplx<double> G[9];
+// One warp per direction mu (threadIdx.y) and 32 / PARTS sites of one parity (blockIdx.y);
+// the PARTS lanes of a site share its slices.  Bound by the FP64 pipe: 2 x (24 + 72)
+// operations per link and slice.  mu is the same for a whole warp, so that no lane waits
+// for another direction's projection; the four warps of a CTA read the same sites.
+// 16^3x32, Ls = 8: the whole force 8.91 -> 4.63 ms, this kernel 4.09 ms before (one
+// thread per link with the four directions of a site in one warp, B folded in again per link).
+template <bool EVEN, int PARTS>
+__global__ void __launch_bounds__(128) force_kernel(const Geom g, const ForceArgs a) {
+  constexpr int SITES = 32 / PARTS;
+  const int mu = threadIdx.y, p = blockIdx.y;
+  const int part = threadIdx.x / SITES;
+  const int h = blockIdx.x * SITES + threadIdx.x % SITES;
+  const bool active = h < g.Vh;
+  cplx<double> G[9];
 #pragma unroll
-    for (int k = 0; k < 9; k++) G[k] = cmake(0.0, 0.0);
-    for (int s = 0; s < g.Ls; s++) {
-      Spinor<double> e, w;
-      cplx<double> he[2][3], hw[2][3];
-      // term 1: eta_a(x)^+ (1 - gamma_mu) dU w_a(x+mu)
-      Store64::load(eta_a, site5(h, s, g.Ls), g.N5, e);
-      load_bxi(g, xi_a, hn, s, a.bd, a.bo, w);
-      project_rt(e, mu, +1, he);
-      project_rt(w, mu, +1, hw);
-      outer_add(G, he, hw, 1);
-      // term 2: eta_b(x+mu)^+ (1 + gamma_mu) dU^+ w_b(x)  ->  w_b(x) (proj eta_b)^+
-      Store64::load(eta_b, site5(hn, s, g.Ls), g.N5, e);
-      load_bxi(g, xi_b, h, s, a.bd, a.bo, w);
-      project_rt(e, mu, -1, he);
-      project_rt(w, mu, -1, hw);
-      outer_add(G, hw, he, 1);
-    }
-    // 2 * (-1/2) and the antiperiodic sign of a hop across the t boundary
-#pragma unroll
-    for (int k = 0; k < 9; k++) G[k] = cmake(-sign * G[k].re, -sign * G[k].im);
-    double2* o = reinterpret_cast<double2*>(a.out) + i * 9;
-    if (!a.projected) {
-#pragma unroll
-      for (int k = 0; k < 9; k++) o[k] = make_double2(G[k].re, G[k].im);
-    } else {
-      // F = TA(U G^+), TA(M) = (M - M^+)/2 - tr(M - M^+)/6
-      const double2* u = reinterpret_cast<const double2*>(reinterpret_cast<const char*>(a.g64) +
-                                                          (size_t)q * a.gpar) +
-                         ((size_t)h * 4 + mu) * 9;
-      cplx<double> M[9];
-#pragma unroll
-      for (int r = 0; r < 3; r++)
-#pragma unroll
-        for (int cc = 0; cc < 3; cc++) {
-          cplx<double> acc = cmake(0.0, 0.0);
-#pragma unroll
-          for (int k = 0; k < 3; k++) {
-            const double2 uu = u[3 * r + k];
-            const cplx<double> gg = G[3 * cc + k];  // (G^+)_{k,cc} = conj(G_{cc,k})
-            acc.re += uu.x * gg.re + uu.y * gg.im;
-            acc.im += uu.y * gg.re - uu.x * gg.im;
-          }
-          M[3 * r + cc] = acc;
-        }
-      cplx<double> F[9];
-      double tr_im = 0.0;
-#pragma unroll
-      for (int r = 0; r < 3; r++)
-#pragma unroll
-        for (int cc = 0; cc < 3; cc++) {
-          const cplx<double> m1 = M[3 * r + cc], m2 = M[3 * cc + r];
-          F[3 * r + cc] = cmake(0.5 * (m1.re - m2.re), 0.5 * (m1.im + m2.im));
-        }
-      tr_im = F[0].im + F[4].im + F[8].im;
-      F[0].im -= tr_im / 3.0;
-      F[4].im -= tr_im / 3.0;
-      F[8].im -= tr_im / 3.0;
-#pragma unroll
-      for (int k = 0; k < 9; k++) o[k] = make_double2(F[k].re, F[k].im);
+  for (int k = 0; k < 9; k++) G[k] = cmake(0.0, 0.0);
+  double sign = 0.5;
+  if (active) {
+    const int4 q = __ldg(a.nbr + ((size_t)p * g.Vh + h) * 2 + (mu >> 1));
+    const int nb = mu & 1 ? q.z : q.x;
+    const int hn = nb & 0x7fffffff;
+    if (nb < 0) sign = -0.5;
+    switch (mu) {
+      case 0: link_sum<EVEN, 0>(g, a, p, h, hn, part, PARTS, G); break;
+      case 1: link_sum<EVEN, 1>(g, a, p, h, hn, part, PARTS, G); break;
+      case 2: link_sum<EVEN, 2>(g, a, p, h, hn, part, PARTS, G); break;
+      default: link_sum<EVEN, 3>(g, a, p, h, hn, part, PARTS, G); break;
     }
   }
+  if (PARTS > 1) {
+#pragma unroll
+    for (int k = 0; k < 9; k++)
+#pragma unroll
+      for (int o = SITES; o < 32; o <<= 1) {
+        G[k].re += __shfl_xor_sync(0xffffffffu, G[k].re, o);
+        G[k].im += __shfl_xor_sync(0xffffffffu, G[k].im, o);
+      }
+  }
+  if (!active || part > 0) return;
+#pragma unroll
+  for (int k = 0; k < 9; k++) G[k] = cmake(sign * G[k].re, sign * G[k].im);
+  // canonical site index: x = 2 (h mod Lx/2) + parity offset of the row
+  const Coords c = site_coords(g, h, p);
+  const size_t link = ((size_t)c.x + (size_t)g.L[0] * (c.y + (size_t)g.L[1] * (c.z + (size_t)g.L[2] * c.t))) * 4 + mu;
+  double2* o = reinterpret_cast<double2*>(a.out) + link * 9;
+  if (!a.projected) {
+#pragma unroll
+    for (int k = 0; k < 9; k++) o[k] = make_double2(G[k].re, G[k].im);
+    return;
+  }
+  // F = TA(U G^+), TA(M) = (M - M^+)/2 - tr(M - M^+)/6
+  const double2* u = reinterpret_cast<const double2*>(reinterpret_cast<const char*>(a.g64) + (size_t)p * a.gpar) +
+                     ((size_t)h * 4 + mu) * 9;
+  cplx<double> M[9];
+#pragma unroll
+  for (int r = 0; r < 3; r++)
+#pragma unroll
+    for (int cc = 0; cc < 3; cc++) {
+      cplx<double> acc = cmake(0.0, 0.0);
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        const double2 uu = u[3 * r + k];
+        const cplx<double> gg = G[3 * cc + k];  // (G^+)_{k,cc} = conj(G_{cc,k})
+        acc.re += uu.x * gg.re + uu.y * gg.im;
+        acc.im += uu.y * gg.re - uu.x * gg.im;
+      }
+      M[3 * r + cc] = acc;
+    }
+  cplx<double> F[9];
+#pragma unroll
+  for (int r = 0; r < 3; r++)
+#pragma unroll
+    for (int cc = 0; cc < 3; cc++) {
+      const cplx<double> m1 = M[3 * r + cc], m2 = M[3 * cc + r];
+      F[3 * r + cc] = cmake(0.5 * (m1.re - m2.re), 0.5 * (m1.im + m2.im));
+    }
+  const double tr_im = F[0].im + F[4].im + F[8].im;
+  F[0].im -= tr_im / 3.0;
+  F[4].im -= tr_im / 3.0;
+  F[8].im -= tr_im / 3.0;
+#pragma unroll
+  for (int k = 0; k < 9; k++) o[k] = make_double2(F[k].re, F[k].im);
+}
+
+template <bool EVEN, int PARTS>
+void run_force(const Geom& g, const ForceArgs& a, cudaStream_t s) {
+  constexpr int SITES = 32 / PARTS;
+  const dim3 grid((g.Vh + SITES - 1) / SITES, 2), block(32, 4);
+  force_kernel<EVEN, PARTS><<<grid, block, 0, s>>>(g, a);
 }
 
 }  // namespace
 
-cudaError_t launch_force(const Geom& g, double* out, const void* eta1, const void* xi1,
-                         const void* eta2, const void* xi2, const double* bd, const double* bo,
-                         const void* g64, size_t gpar, int black, int projected, cudaStream_t s) {
+cudaError_t launch_force(const Geom& g, double* out, const void* e_black, const void* w_black,
+                         const void* e_red, const void* w_red, const int* nbr, const void* g64,
+                         size_t gpar, int black, int projected, cudaStream_t s) {
   ForceArgs a;
-  a.eta1 = eta1;
-  a.xi1 = xi1;
-  a.eta2 = eta2;
-  a.xi2 = xi2;
-  a.bd = bd;
-  a.bo = bo;
+  a.E[black] = e_black;
+  a.E[1 - black] = e_red;
+  a.W[black] = w_black;
+  a.W[1 - black] = w_red;
+  a.nbr = reinterpret_cast<const int4*>(nbr);
   a.g64 = g64;
   a.gpar = gpar;
   a.out = out;
-  a.black = black;
   a.projected = projected;
-  const size_t n = (size_t)g.Vh * 8;
-  int blocks = (int)std::min<size_t>((n + 127) / 128, 152 * 32);
-  force_kernel<<<blocks, 128, 0, s>>>(g, a);
+  // With fewer than 4 CTAs of 32 sites per SM the slices of a site are shared by 4 lanes:
+  // the FP64 pipes of idle SMs then take part (the sum over lanes adds 36 operations per
+  // link to ~190 per slice).
+  const bool split = 2 * ((size_t)g.Vh + 31) / 32 < 4 * 152;
+  if (g.Ls % 2 == 0) {
+    if (split) run_force<true, 4>(g, a, s);
+    else run_force<true, 1>(g, a, s);
+  } else {
+    if (split) run_force<false, 4>(g, a, s);
+    else run_force<false, 1>(g, a, s);
+  }
   return cudaGetLastError();
 }
 

@@ -62,9 +62,6 @@ __device__ __forceinline__ void hop_term(const Geom& g, const Coords& c, int h, 
       in.c[k + 6] = cmake(fma(bd[1], in.c[k + 6].re, bo[1] * b.c[k + 6].re),
                           fma(bd[1], in.c[k + 6].im, bo[1] * b.c[k + 6].im));
     }
-  } else if (PRE == PRE_G5) {
-#pragma unroll
-    for (int k = 6; k < 12; k++) in.c[k] = cmake(-in.c[k].re, -in.c[k].im);
   }
   cplx<T> h0[3], h1[3], c0[3], c1[3];
   project<T, MU, DIR>(in, h0, h1);
@@ -317,7 +314,6 @@ cudaError_t dispatch_hop(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   //  D_bb^+ pass B      PRE_NONE, post B^T,   LOC_ID, gamma5 out, (norm)
   //  D_alpha parity     PRE_B,    no post,    LOC_DENSE (I)
   //  Schur rhs/recon    PRE_NONE / PRE_B, post I^-1, LOC_DENSE (I^-1)
-  //  force eta2         PRE_G5,   post K^T,   gamma5 out
   if (L.pre == PRE_B && post && L.loc == LOC_NONE && !L.g5out && !norm)
     return run_hop<SP, PRE_B, true, LOC_NONE, false, false>(g, L, st);
   if (L.pre == PRE_NONE && post && L.loc == LOC_ID && !L.g5out)
@@ -334,10 +330,6 @@ cudaError_t dispatch_hop(const Geom& g, const HopLaunch& L, cudaStream_t st) {
     return run_hop<SP, PRE_NONE, true, LOC_DENSE, false, false>(g, L, st);
   if (L.pre == PRE_B && post && L.loc == LOC_DENSE && !L.g5out && !norm)
     return run_hop<SP, PRE_B, true, LOC_DENSE, false, false>(g, L, st);
-  if (L.pre == PRE_B && post && L.loc == LOC_NONE && !L.g5out && !norm)
-    return run_hop<SP, PRE_B, true, LOC_NONE, false, false>(g, L, st);
-  if (L.pre == PRE_G5 && post && L.loc == LOC_NONE && L.g5out && !norm)
-    return run_hop<SP, PRE_G5, true, LOC_NONE, true, false>(g, L, st);
   return cudaErrorInvalidValue;
 }
 

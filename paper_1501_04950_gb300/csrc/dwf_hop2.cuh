@@ -294,18 +294,11 @@ struct Args {
   int* err;             // set to 1 when a bounded wait gives up (staged variant)
 };
 
-// h = P_+ - dir A P_- (in place into P), chi_k = U' h_k, acc_upper(k) += f chi_k,
-// acc_lower(pk) += f rs (i) chi_k; U' = U (dir > 0) or U^+ (dir < 0).
-template <class SP, int MU, int DIR>
-__device__ __forceinline__ void project_mul_acc(HalfP<typename Pr<typename SP::T>::V>& P,
-                                                const HalfP<typename Pr<typename SP::T>::V>& M,
-                                                const Link<typename SP::T>& U,
-                                                typename Pr<typename SP::T>::V f,
-                                                SpinP<typename Pr<typename SP::T>::V>& acc) {
-  using T = typename SP::T;
+// h = P_+ - dir A P_- in place into P: the half spinor of (1 - DIR gamma_mu).
+template <typename T, int MU, int DIR>
+__device__ __forceinline__ void project_half(HalfP<typename Pr<T>::V>& P, const HalfP<typename Pr<T>::V>& M) {
   using A = Pr<T>;
   using V = typename A::V;
-  // projection h = P_+ - dir A P_- (in place into P)
 #pragma unroll
   for (int k = 0; k < 2; k++) {
     const int pk = partner(MU, k);
@@ -323,6 +316,20 @@ __device__ __forceinline__ void project_mul_acc(HalfP<typename Pr<typename SP::T
       }
     }
   }
+}
+
+// h = P_+ - dir A P_- (in place into P), chi_k = U' h_k, acc_upper(k) += f chi_k,
+// acc_lower(pk) += f rs (i) chi_k; U' = U (dir > 0) or U^+ (dir < 0).
+template <class SP, int MU, int DIR>
+__device__ __forceinline__ void project_mul_acc(HalfP<typename Pr<typename SP::T>::V>& P,
+                                                const HalfP<typename Pr<typename SP::T>::V>& M,
+                                                const Link<typename SP::T>& U,
+                                                typename Pr<typename SP::T>::V f,
+                                                SpinP<typename Pr<typename SP::T>::V>& acc) {
+  using T = typename SP::T;
+  using A = Pr<T>;
+  using V = typename A::V;
+  project_half<T, MU, DIR>(P, M);
   const V fn = A::neg(f);
   // chi_k = U' h_k; acc_upper(k) += f chi_k; acc_lower(pk) += f rs (i) chi_k
 #pragma unroll

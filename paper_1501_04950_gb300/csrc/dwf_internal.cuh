@@ -58,11 +58,11 @@ struct Reduce {
 
 // ---- the generic hopping pass -------------------------------------------------
 //   acc(x,s)  = sum_mu [ (1-g_mu) U_mu(x) v'(x+mu,s) + (1+g_mu) U_mu(x-mu)^+ v'(x-mu,s) ]
-//   v'        = B v (cyclic bidiagonal per chirality), gamma5 v, or v
+//   v'        = B v (cyclic bidiagonal per chirality) or v
 //   out(x,s)  = c_hop * G * post(acc) + c_loc * loc(w)
 //   post, loc: dense (s, s') contraction per chirality, or identity / none;
 //   G = gamma5 if g5out.  Optional fused |out|^2 per right-hand side.
-enum PreOp { PRE_NONE = 0, PRE_B = 1, PRE_G5 = 2 };
+enum PreOp { PRE_NONE = 0, PRE_B = 1 };
 enum LocOp { LOC_NONE = 0, LOC_ID = 1, LOC_DENSE = 2 };
 
 struct HopLaunch {
@@ -235,12 +235,12 @@ cudaError_t launch_dot_re64(const Geom& g, const void* a, const void* b, int nrh
 int blas_grid_blocks(const Geom& g);
 
 // ---- force (dwf_force.cu) -------------------------------------------------------
-// dS/dU of S = phi^+ (D_bb^+ D_bb)^-1 phi from the auxiliary FP64 fields
-// eta1 = I^-T Y (black), xi1 = I^-1 D_rb X (red), eta2 = I^-T D_br^+ eta1 (red),
-// xi2 = X (black); out: canonical [V][4][3][3] complex128, raw G or TA(U G^+).
-cudaError_t launch_force(const Geom& g, double* out, const void* eta1, const void* xi1,
-                         const void* eta2, const void* xi2, const double* bd, const double* bo,
-                         const void* g64, size_t gpar, int black, int projected, cudaStream_t s);
+// dS/dU of S = phi^+ (D_bb^+ D_bb)^-1 phi from the FP64 half-fields of dwf_force.cu:
+// w_black = B X, w_red = K H_rb B X, e_black = gamma5 I^-T D_bb X, e_red = K^T H_rb e_black;
+// nbr: neighbour table; out: canonical [V][4][3][3] complex128, raw G or TA(U G^+).
+cudaError_t launch_force(const Geom& g, double* out, const void* e_black, const void* w_black,
+                         const void* e_red, const void* w_red, const int* nbr, const void* g64,
+                         size_t gpar, int black, int projected, cudaStream_t s);
 
 }  // namespace dwf
 

@@ -23,43 +23,146 @@ __device__ __forceinline__ void cvt(Spinor<TD>& d, const Spinor<TS>& s) {
 }
 
 // ---- conversions --------------------------------------------------------------
+// Canonical fields keep the 12 components of a 5D site together and the sites of a
+// slice in a row; the half-fields keep the slice pairs of a site together, one row per
+// component.  A CTA takes kTile-sized blocks of sites with all their slices through
+// shared memory, so that both sides move whole lines: runs of (sites x 192) bytes on
+// the canonical side, of (sites x Ls/2) pairs on the other.  Bound by HBM; one thread
+// per 5D site, with 192-byte strides between the lanes on one side and Ls-strided
+// scattered words on the other, moved 16^3x32, Ls = 16 at a sixth of that.
+// 16^3x32, Ls = 16, FP32: a new gauge field, pack and unpack 550 -> 161 us (the bytes
+// alone at the copy rate: 106).
 
+// Tile element (site hl of the tile, slice s) at (hl Ls + s) kTileStride; real component
+// R = 2c + (0 re | 1 im).  26 = 24 + 2: 8-byte accesses to consecutive 5D sites spread
+// over the banks.
+constexpr int kTileStride = 26;
+
+// sites per tile: the largest power of two with at most 32 KB of tile (one tile per
+// parity of the full fields: nfields = 2)
+int tile_sites(int Ls, size_t ts, int nfields) {
+  int n = 16;
+  while (n > 2 && (size_t)n * Ls * kTileStride * ts * nfields > 32768) n /= 2;
+  return n;
+}
+size_t tile_bytes(int Ls, int sites, size_t ts, int nfields) {
+  // the tile(s), and one scale per 5D site of 16-bit storage
+  return (size_t)sites * Ls * (kTileStride * ts + sizeof(float)) * nfields;
+}
+
+// Tile -> internal half-field (n5 = 5D sites of the tile, first one at n0; both even).
 template <class SP>
-__global__ void pack_half_kernel(const Geom g, void* dst, const double* src, size_t stride,
-                                 int nrhs) {
+__device__ __forceinline__ void tile_store(void* dst, const typename SP::T* tile, float* scale, int n0,
+                                           int n5, int N5, int tid, int nth) {
   using T = typename SP::T;
-  const size_t total = (size_t)g.N5 * nrhs;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const int r = (int)(i / g.N5);
-    const int q = (int)(i % g.N5);
-    const int s = q / g.Vh, h = q % g.Vh;  // canonical order [s][h]
-    const double2* in = reinterpret_cast<const double2*>(src) + ((size_t)r * g.N5 + q) * 12;
-    Spinor<T> a;
+  const size_t NP = (size_t)N5 >> 1, m0 = (size_t)n0 >> 1;
+  const int np = n5 >> 1;
+  if constexpr (SP::kScaled) {
+    for (int n = tid; n < n5; n += nth) {
+      float mx = 0.f;
 #pragma unroll
-    for (int k = 0; k < 12; k++) {
-      double2 v = in[k];
-      a.c[k] = cmake((T)v.x, (T)v.y);
+      for (int k = 0; k < 24; k++) mx = fmaxf(mx, fabsf(tile[n * kTileStride + k]));
+      scale[n] = SP::scale_of(mx);
     }
-    SP::store(reinterpret_cast<char*>(dst) + r * stride, site5(h, s, g.Ls), g.N5, a);
+    __syncthreads();
+    for (int i = tid; i < 6 * np; i += nth) {
+      const int j = i / np, m = i - j * np;
+      const T* a = tile + 2 * m * kTileStride + 4 * j;
+      const T* b = a + kTileStride;
+      const float ia = 1.f / scale[2 * m], ib = 1.f / scale[2 * m + 1];
+      reinterpret_cast<uint4*>(dst)[j * NP + m0 + m] =
+          make_uint4(SP::from_f2(make_float2(a[0] * ia, b[0] * ib)), SP::from_f2(make_float2(a[1] * ia, b[1] * ib)),
+                     SP::from_f2(make_float2(a[2] * ia, b[2] * ib)), SP::from_f2(make_float2(a[3] * ia, b[3] * ib)));
+    }
+    for (int n = tid; n < n5; n += nth) const_cast<float*>(SP::scales(dst, N5))[n0 + n] = scale[n];
+  } else {
+    for (int i = tid; i < 12 * np; i += nth) {
+      const int c = i / np, m = i - c * np;
+      const T* a = tile + 2 * m * kTileStride + 2 * c;
+      const T* b = a + kTileStride;
+      if constexpr (sizeof(T) == 8) {
+        double2* o = reinterpret_cast<double2*>(dst) + (c * NP + m0 + m) * 2;
+        o[0] = make_double2(a[0], b[0]);
+        o[1] = make_double2(a[1], b[1]);
+      } else {
+        reinterpret_cast<float4*>(dst)[c * NP + m0 + m] = make_float4(a[0], b[0], a[1], b[1]);
+      }
+    }
   }
 }
 
+// Internal half-field -> tile.
 template <class SP>
-__global__ void unpack_half_kernel(const Geom g, double* dst, const void* src, size_t stride,
-                                   int nrhs) {
+__device__ __forceinline__ void tile_load(typename SP::T* tile, const void* src, int n0, int n5, int N5,
+                                          int tid, int nth) {
   using T = typename SP::T;
-  const size_t total = (size_t)g.N5 * nrhs;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const int r = (int)(i / g.N5);
-    const int q = (int)(i % g.N5);
-    const int s = q / g.Vh, h = q % g.Vh;
-    Spinor<T> a;
-    SP::load(reinterpret_cast<const char*>(src) + r * stride, site5(h, s, g.Ls), g.N5, a);
-    double2* out = reinterpret_cast<double2*>(dst) + ((size_t)r * g.N5 + q) * 12;
+  const size_t NP = (size_t)N5 >> 1, m0 = (size_t)n0 >> 1;
+  const int np = n5 >> 1;
+  if constexpr (SP::kScaled) {
+    for (int i = tid; i < 6 * np; i += nth) {
+      const int j = i / np, m = i - j * np;
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(src) + j * NP + m0 + m);
+      const float* sc = SP::scales(src, N5) + n0 + 2 * m;
+      const float sa = __ldg(sc), sb = __ldg(sc + 1);
+      T* a = tile + 2 * m * kTileStride + 4 * j;
+      T* b = a + kTileStride;
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int k = 0; k < 12; k++) out[k] = make_double2((double)a.c[k].re, (double)a.c[k].im);
+      for (int k = 0; k < 4; k++) {
+        const float2 q = SP::to_f2(w[k]);
+        a[k] = sa * q.x;
+        b[k] = sb * q.y;
+      }
+    }
+  } else {
+    for (int i = tid; i < 12 * np; i += nth) {
+      const int c = i / np, m = i - c * np;
+      T* a = tile + 2 * m * kTileStride + 2 * c;
+      T* b = a + kTileStride;
+      if constexpr (sizeof(T) == 8) {
+        const double2* q = reinterpret_cast<const double2*>(src) + (c * NP + m0 + m) * 2;
+        const double2 re = __ldg(q), im = __ldg(q + 1);
+        a[0] = re.x; b[0] = re.y; a[1] = im.x; b[1] = im.y;
+      } else {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(src) + c * NP + m0 + m);
+        a[0] = v.x; b[0] = v.y; a[1] = v.z; b[1] = v.w;
+      }
+    }
+  }
+}
+
+// Canonical half-field(s) [nrhs][Ls][Vh][12] <-> internal, `sites` sites per CTA.
+template <class SP, bool PACK>
+__global__ void __launch_bounds__(kBlasThreads) half_kernel(const Geom g, void* field, double* canon,
+                                                            size_t stride, int sites, int tiles) {
+  using T = typename SP::T;
+  extern __shared__ __align__(16) unsigned char tile_raw[];
+  T* tile = reinterpret_cast<T*>(tile_raw);
+  float* scale = reinterpret_cast<float*>(tile + (size_t)sites * g.Ls * kTileStride);
+  const int tid = threadIdx.x, nth = blockDim.x, rhs = blockIdx.x / tiles;
+  const int h0 = (blockIdx.x - rhs * tiles) * sites, nh = min(sites, g.Vh - h0);
+  char* f = reinterpret_cast<char*>(field) + (size_t)rhs * stride;
+  double2* c = reinterpret_cast<double2*>(canon) + (size_t)rhs * g.N5 * 12;
+  const int run = nh * 12;  // components of one slice of the tile
+  if (!PACK) {
+    tile_load<SP>(tile, f, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
+    __syncthreads();
+  }
+  for (int i = tid; i < run * g.Ls; i += nth) {
+    const int s = i / run, r = i - s * run, hl = r / 12, k = r - 12 * hl;
+    double2* q = c + ((size_t)s * g.Vh + h0) * 12 + r;
+    T* e = tile + (hl * g.Ls + s) * kTileStride + 2 * k;
+    if (PACK) {
+      const double2 v = *q;
+      e[0] = (T)v.x;
+      e[1] = (T)v.y;
+    } else {
+      *q = make_double2((double)e[0], (double)e[1]);
+    }
+  }
+  if (PACK) {
+    __syncthreads();
+    tile_store<SP>(f, tile, scale, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
   }
 }
 
@@ -72,71 +175,89 @@ __device__ __forceinline__ void lex_coords(const Geom& g, int i, int& x, int& y,
   t = r / g.L[2];
 }
 
-// full canonical [Ls][V][4][3] <-> FP64 internal halves
-__global__ void split_full_kernel(const Geom g, void* p0, void* p1, const double* full, int to_full) {
+// Parity of the even-x site of half index h (sites 2h and 2h + 1 have both parities).
+__device__ __forceinline__ int row_parity(const Geom& g, int h) {
+  int r = h / g.Lxh;
+  const int y = r % g.L[1];
+  r /= g.L[1];
+  return (y + r % g.L[2] + r / g.L[2]) & 1;
+}
+
+// full canonical [Ls][V][4][3] <-> FP64 internal halves, 2 x `sites` sites per CTA
+template <bool SPLIT>
+__global__ void __launch_bounds__(kBlasThreads) full_kernel(const Geom g, void* p0, void* p1, double* full,
+                                                            int sites) {
+  extern __shared__ __align__(16) unsigned char tile_raw[];
+  double* tile = reinterpret_cast<double*>(tile_raw);
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int h0 = blockIdx.x * sites, nh = min(sites, g.Vh - h0);
+  const int per = sites * g.Ls * kTileStride;  // tile of parity 1 after that of parity 0
+  const int run = 2 * nh * 12;
   const size_t V = (size_t)g.Vh * 2;
-  const size_t total = V * g.Ls;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const int s = (int)(i / V);
-    const int site = (int)(i % V);
-    int x, y, z, t;
-    lex_coords(g, site, x, y, z, t);
-    const int par = (x + y + z + t) & 1;
-    const int h = site >> 1;
-    void* half = par ? p1 : p0;
-    double2* cf = reinterpret_cast<double2*>(const_cast<double*>(full)) + i * 12;
-    Spinor<double> a;
-    if (!to_full) {
-#pragma unroll
-      for (int k = 0; k < 12; k++) a.c[k] = cmake(cf[k].x, cf[k].y);
-      Store64::store(half, site5(h, s, g.Ls), g.N5, a);
+  if (!SPLIT) {
+    tile_load<Store64>(tile, p0, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
+    tile_load<Store64>(tile + per, p1, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
+    __syncthreads();
+  }
+  for (int i = tid; i < run * g.Ls; i += nth) {
+    const int s = i / run, r = i - s * run, site = r / 12, k = r - 12 * site, hl = site >> 1;
+    const int par = row_parity(g, h0 + hl) ^ (site & 1);
+    double2* q = reinterpret_cast<double2*>(full) + (s * V + 2 * (size_t)h0) * 12 + r;
+    double* e = tile + par * per + (hl * g.Ls + s) * kTileStride + 2 * k;
+    if (SPLIT) {
+      const double2 v = *q;
+      e[0] = v.x;
+      e[1] = v.y;
     } else {
-      Store64::load(half, site5(h, s, g.Ls), g.N5, a);
-#pragma unroll
-      for (int k = 0; k < 12; k++) cf[k] = make_double2(a.c[k].re, a.c[k].im);
+      *q = make_double2(e[0], e[1]);
     }
+  }
+  if (SPLIT) {
+    __syncthreads();
+    tile_store<Store64>(p0, tile, nullptr, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
+    tile_store<Store64>(p1, tile + per, nullptr, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
   }
 }
 
-__global__ void gauge_convert_kernel(const Geom g, const double* U, double2* g64, float4* g32,
-                                     uint4* g16) {
-  const size_t V = (size_t)g.Vh * 2;
-  const size_t total = V * 4;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const int site = (int)(i / 4), mu = (int)(i % 4);
-    int x, y, z, t;
-    lex_coords(g, site, x, y, z, t);
-    const int par = (x + y + z + t) & 1;
-    const size_t slot = (size_t)par * g.Vh + (site >> 1);
-    const double2* u = reinterpret_cast<const double2*>(U) + i * 9;
-    double2 v[9];
+// Links U[t][z][y][x][mu][3][3] -> the per-parity FP64, FP32 and FP16 layouts.  A CTA
+// takes the 4 links of kGaugeSites neighbouring sites through shared memory: the links
+// of the sites of one parity are a contiguous run of every output.  HBM bound, like the
+// field conversions.
+constexpr int kGaugeSites = 32;
+__global__ void __launch_bounds__(kBlasThreads) gauge_convert_kernel(const Geom g, const double* U, double2* g64,
+                                                                     float4* g32, uint4* g16) {
+  __shared__ double2 tile[2][kGaugeSites / 2 * 36];
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int h0 = blockIdx.x * (kGaugeSites / 2), nh = min(kGaugeSites / 2, g.Vh - h0);
+  const double2* u = reinterpret_cast<const double2*>(U) + (size_t)h0 * 72;
+  for (int i = tid; i < nh * 72; i += nth) {
+    const int site = i / 36, hl = site >> 1;
+    tile[row_parity(g, h0 + hl) ^ (site & 1)][hl * 36 + (i - site * 36)] = u[i];
+  }
+  __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 9; k++) v[k] = u[k];
-    double2* d64 = g64 + (slot * 4 + mu) * 9;
-#pragma unroll
-    for (int k = 0; k < 9; k++) d64[k] = v[k];
-    float f[20];
-#pragma unroll
-    for (int k = 0; k < 9; k++) {
-      f[2 * k] = (float)v[k].x;
-      f[2 * k + 1] = (float)v[k].y;
+  for (int p = 0; p < 2; p++) {
+    const size_t slot = ((size_t)p * g.Vh + h0) * 4;  // first link of the run
+    for (int i = tid; i < nh * 36; i += nth) g64[slot * 9 + i] = tile[p][i];
+    for (int i = tid; i < nh * 20; i += nth) {
+      const int l = i / 5, k = 2 * (i - 5 * l);
+      const double2 a = tile[p][l * 9 + k], b = k < 8 ? tile[p][l * 9 + k + 1] : make_double2(0.0, 0.0);
+      g32[slot * 5 + i] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
     }
-    f[18] = 0.f;
-    f[19] = 0.f;
-    float4* d32 = g32 + (slot * 4 + mu) * 5;
+    for (int i = tid; i < nh * 12; i += nth) {
+      const int l = i / 3, k = 4 * (i - 3 * l);
+      uint32_t w[4];
 #pragma unroll
-    for (int k = 0; k < 5; k++) d32[k] = make_float4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
-    uint32_t w[12];
-#pragma unroll
-    for (int k = 0; k < 9; k++)
-      w[k] = (uint32_t)__half_as_ushort(__float2half_rn((float)v[k].x)) |
-             ((uint32_t)__half_as_ushort(__float2half_rn((float)v[k].y)) << 16);
-    w[9] = w[10] = w[11] = 0u;
-    uint4* d16 = g16 + (slot * 4 + mu) * 3;
-#pragma unroll
-    for (int k = 0; k < 3; k++) d16[k] = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+      for (int q = 0; q < 4; q++) {
+        w[q] = 0u;
+        if (k + q < 9) {
+          const double2 v = tile[p][l * 9 + k + q];
+          w[q] = (uint32_t)__half_as_ushort(__float2half_rn((float)v.x)) |
+                 ((uint32_t)__half_as_ushort(__float2half_rn((float)v.y)) << 16);
+        }
+      }
+      g16[slot * 3 + i] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
   }
 }
 
@@ -576,37 +697,47 @@ size_t gauge_bytes(const Geom& g, int prec) {
     default: return cudaErrorInvalidValue;             \
   }
 
+template <class SP, bool PACK>
+void run_half(const Geom& g, void* field, double* canon, int nrhs, size_t stride, cudaStream_t s) {
+  const size_t ts = sizeof(typename SP::T);
+  const int sites = tile_sites(g.Ls, ts, 1);
+  const int tiles = (g.Vh + sites - 1) / sites;
+  half_kernel<SP, PACK><<<(unsigned)tiles * nrhs, kBlasThreads, tile_bytes(g.Ls, sites, ts, 1), s>>>(
+      g, field, canon, stride, sites, tiles);
+}
+
 cudaError_t launch_pack_half(const Geom& g, int prec, void* dst, const double* src, int nrhs,
                              cudaStream_t s) {
-  const size_t stride = field_bytes(g, prec);
-  const int blocks = elementwise_blocks((size_t)g.N5 * nrhs);
-  DWF_PREC_SWITCH(prec, SP, pack_half_kernel<SP><<<blocks, kBlasThreads, 0, s>>>(g, dst, src, stride, nrhs));
+  DWF_PREC_SWITCH(prec, SP, run_half<SP, true>(g, dst, const_cast<double*>(src), nrhs, field_bytes(g, prec), s));
   return cudaGetLastError();
 }
 
 cudaError_t launch_unpack_half(const Geom& g, int prec, double* dst, const void* src, int nrhs,
                                cudaStream_t s) {
-  const size_t stride = field_bytes(g, prec);
-  const int blocks = elementwise_blocks((size_t)g.N5 * nrhs);
-  DWF_PREC_SWITCH(prec, SP, unpack_half_kernel<SP><<<blocks, kBlasThreads, 0, s>>>(g, dst, src, stride, nrhs));
+  DWF_PREC_SWITCH(prec, SP, run_half<SP, false>(g, const_cast<void*>(src), dst, nrhs, field_bytes(g, prec), s));
+  return cudaGetLastError();
+}
+
+template <bool SPLIT>
+cudaError_t run_full(const Geom& g, void* p0, void* p1, double* full, cudaStream_t s) {
+  const int sites = tile_sites(g.Ls, 8, 2);
+  full_kernel<SPLIT><<<(g.Vh + sites - 1) / sites, kBlasThreads, tile_bytes(g.Ls, sites, 8, 2), s>>>(g, p0, p1, full, sites);
   return cudaGetLastError();
 }
 
 cudaError_t launch_split_full(const Geom& g, void* p0, void* p1, const double* full, cudaStream_t s) {
-  split_full_kernel<<<elementwise_blocks((size_t)g.N5 * 2), kBlasThreads, 0, s>>>(g, p0, p1, full, 0);
-  return cudaGetLastError();
+  return run_full<true>(g, p0, p1, const_cast<double*>(full), s);
 }
 
 cudaError_t launch_merge_full(const Geom& g, double* full, const void* p0, const void* p1,
                               cudaStream_t s) {
-  split_full_kernel<<<elementwise_blocks((size_t)g.N5 * 2), kBlasThreads, 0, s>>>(
-      g, const_cast<void*>(p0), const_cast<void*>(p1), full, 1);
-  return cudaGetLastError();
+  return run_full<false>(g, const_cast<void*>(p0), const_cast<void*>(p1), full, s);
 }
 
 cudaError_t launch_gauge_convert(const Geom& g, const double* U, void* g64, void* g32, void* g16,
                                  cudaStream_t s) {
-  gauge_convert_kernel<<<elementwise_blocks((size_t)g.Vh * 8), kBlasThreads, 0, s>>>(
+  const int per = kGaugeSites / 2;
+  gauge_convert_kernel<<<(g.Vh + per - 1) / per, kBlasThreads, 0, s>>>(
       g, U, reinterpret_cast<double2*>(g64), reinterpret_cast<float4*>(g32),
       reinterpret_cast<uint4*>(g16));
   return cudaGetLastError();

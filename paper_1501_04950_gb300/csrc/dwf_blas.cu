@@ -1,5 +1,7 @@
 // dwf_blas.cu -- layout conversions, sources, propagator extraction and the
 // fused BLAS-1 kernels of the CG on the normal equations (sm_103a).
+#include <algorithm>
+
 #include "dwf_fields.cuh"
 
 namespace dwf {
@@ -166,15 +168,6 @@ __global__ void __launch_bounds__(kBlasThreads) half_kernel(const Geom g, void* 
   }
 }
 
-__device__ __forceinline__ void lex_coords(const Geom& g, int i, int& x, int& y, int& z, int& t) {
-  x = i % g.L[0];
-  int r = i / g.L[0];
-  y = r % g.L[1];
-  r /= g.L[1];
-  z = r % g.L[2];
-  t = r / g.L[2];
-}
-
 // Parity of the even-x site of half index h (sites 2h and 2h + 1 have both parities).
 __device__ __forceinline__ int row_parity(const Geom& g, int h) {
   int r = h / g.Lxh;
@@ -261,52 +254,39 @@ __global__ void __launch_bounds__(kBlasThreads) gauge_convert_kernel(const Geom 
   }
 }
 
-// (Pb)_1 = P_- b_1 (spins 2,3), (Pb)_Ls = P_+ b_1 (spins 0,1); zero elsewhere.
+// (Pb)_1 = P_- b_1 (spins 2,3), (Pb)_Ls = P_+ b_1 (spins 0,1); zero elsewhere.  One
+// thread per slice pair m of either half (blockIdx.y), whose stores are whole lines.
 __global__ void source_pb_kernel(const Geom g, void* p0, void* p1, const double* src) {
-  const size_t V = (size_t)g.Vh * 2;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < V;
-       i += (size_t)gridDim.x * blockDim.x) {
-    int x, y, z, t;
-    lex_coords(g, (int)i, x, y, z, t);
-    const int par = (x + y + z + t) & 1;
-    const int h = (int)(i >> 1);
-    void* half = par ? p1 : p0;
-    const double2* b = reinterpret_cast<const double2*>(src) + i * 12;
-    for (int s = 0; s < g.Ls; s++) {
-      Spinor<double> a;
+  const int NP = g.N5 >> 1, par = blockIdx.y;
+  void* half = par ? p1 : p0;
+  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < NP; m += gridDim.x * blockDim.x) {
+    Spinor<double> a[2];
 #pragma unroll
-      for (int k = 0; k < 12; k++) a.c[k] = cmake(0.0, 0.0);
-      if (s == 0) {
+    for (int l = 0; l < 2; l++) {
+      const int n = 2 * m + l, h = n / g.Ls, s = n - h * g.Ls;
 #pragma unroll
-        for (int k = 6; k < 12; k++) a.c[k] = cmake(b[k].x, b[k].y);
+      for (int k = 0; k < 12; k++) a[l].c[k] = cmake(0.0, 0.0);
+      if (s == 0 || s == g.Ls - 1) {
+        const int site = 2 * h + (row_parity(g, h) ^ par);
+        const double2* b = reinterpret_cast<const double2*>(src) + (size_t)site * 12;
+#pragma unroll
+        for (int k = 0; k < 12; k++)
+          if ((k >= 6 && s == 0) || (k < 6 && s == g.Ls - 1)) a[l].c[k] = cmake(b[k].x, b[k].y);
       }
-      if (s == g.Ls - 1) {
-#pragma unroll
-        for (int k = 0; k < 6; k++) a.c[k] = cmake(b[k].x, b[k].y);
-      }
-      Store64::store(half, site5(h, s, g.Ls), g.N5, a);
     }
+    Store64::store_pair(half, m, NP, a[0], a[1]);
   }
 }
 
-// z_1 = P_- psi_1 + P_+ psi_Ls
+// z_1 = P_- psi_1 + P_+ psi_Ls, one thread per component of a site
 __global__ void extract_z1_kernel(const Geom g, double* prop, const void* p0, const void* p1) {
-  const size_t V = (size_t)g.Vh * 2;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < V;
+  const size_t total = (size_t)g.Vh * 24;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
        i += (size_t)gridDim.x * blockDim.x) {
-    int x, y, z, t;
-    lex_coords(g, (int)i, x, y, z, t);
-    const int par = (x + y + z + t) & 1;
-    const int h = (int)(i >> 1);
-    const void* half = par ? p1 : p0;
-    Spinor<double> a, b;
-    Store64::load(half, site5(h, 0, g.Ls), g.N5, a);
-    Store64::load(half, site5(h, g.Ls - 1, g.Ls), g.N5, b);
-    double2* o = reinterpret_cast<double2*>(prop) + i * 12;
-#pragma unroll
-    for (int k = 0; k < 6; k++) o[k] = make_double2(b.c[k].re, b.c[k].im);
-#pragma unroll
-    for (int k = 6; k < 12; k++) o[k] = make_double2(a.c[k].re, a.c[k].im);
+    const int site = (int)(i / 12), k = (int)(i - (size_t)site * 12), h = site >> 1;
+    const void* half = (row_parity(g, h) ^ (site & 1)) ? p1 : p0;
+    const double* q = Store64::at(half, k, site5(h, k < 6 ? g.Ls - 1 : 0, g.Ls), g.N5);
+    reinterpret_cast<double2*>(prop)[i] = make_double2(__ldg(q), __ldg(q + 2));
   }
 }
 
@@ -656,16 +636,21 @@ __global__ void __launch_bounds__(kBlasThreads) dot_re64_kernel(const Geom g, co
   block_sum_to(acc, red, rhs, gridDim.x, blockIdx.x);
 }
 
-int elementwise_blocks(size_t n) {
-  size_t b = (n + kBlasThreads - 1) / kBlasThreads;
-  if (b > 152 * 16) b = 152 * 16;
-  if (b < 1) b = 1;
-  return (int)b;
+// Launch shape of n elements, one per thread up to 16 CTAs of kBlasThreads per SM.  Below
+// two CTAs of 256 per SM the CTAs are of 64 threads, so that a small lattice still
+// spreads over all SMs.
+struct Shape {
+  int blocks, threads;
+};
+Shape elementwise(size_t n) {
+  const int threads = n < (size_t)152 * 2 * kBlasThreads ? 64 : kBlasThreads;
+  const size_t b = (n + threads - 1) / threads;
+  return Shape{(int)std::min<size_t>(std::max<size_t>(b, 1), 152 * 16), threads};
 }
 
 }  // namespace
 
-int blas_grid_blocks(const Geom& g) { return elementwise_blocks((size_t)g.N5 / 2); }
+int blas_grid_blocks(const Geom& g) { return elementwise((size_t)g.N5 / 2).blocks; }
 
 size_t field_bytes(const Geom& g, int prec) {
   size_t b = 0;
@@ -744,13 +729,15 @@ cudaError_t launch_gauge_convert(const Geom& g, const double* U, void* g64, void
 }
 
 cudaError_t launch_source_pb(const Geom& g, void* p0, void* p1, const double* src, cudaStream_t s) {
-  source_pb_kernel<<<elementwise_blocks((size_t)g.Vh * 2), kBlasThreads, 0, s>>>(g, p0, p1, src);
+  const Shape sh = elementwise((size_t)g.N5 / 2);
+  source_pb_kernel<<<dim3(sh.blocks, 2), sh.threads, 0, s>>>(g, p0, p1, src);
   return cudaGetLastError();
 }
 
 cudaError_t launch_extract_z1(const Geom& g, double* prop, const void* p0, const void* p1,
                               cudaStream_t s) {
-  extract_z1_kernel<<<elementwise_blocks((size_t)g.Vh * 2), kBlasThreads, 0, s>>>(g, prop, p0, p1);
+  const Shape sh = elementwise((size_t)g.Vh * 24);
+  extract_z1_kernel<<<sh.blocks, sh.threads, 0, s>>>(g, prop, p0, p1);
   return cudaGetLastError();
 }
 
@@ -758,11 +745,12 @@ cudaError_t launch_xr_update(const Geom& g, int prec, int xprec, void* x, void* 
                              const void* w, const double* num, const double* den, int sstride,
                              int nrhs, size_t stride_x, size_t stride, const Reduce* red,
                              cudaStream_t s, const int* active) {
-  dim3 grid(elementwise_blocks((size_t)g.N5 / 2), nrhs);
+  const Shape sh = elementwise((size_t)g.N5 / 2);
+  const dim3 grid(sh.blocks, nrhs);
   if (xprec == prec) {
-    DWF_PREC_SWITCH(prec, SP, xr_update_kernel<SP, SP><<<grid, kBlasThreads, 0, s>>>(g, x, r, p, w, num, den, sstride, stride_x, stride, *red, active));
+    DWF_PREC_SWITCH(prec, SP, xr_update_kernel<SP, SP><<<grid, sh.threads, 0, s>>>(g, x, r, p, w, num, den, sstride, stride_x, stride, *red, active));
   } else if (xprec == P32) {
-    DWF_PREC_SWITCH(prec, SP, xr_update_kernel<Store32, SP><<<grid, kBlasThreads, 0, s>>>(g, x, r, p, w, num, den, sstride, stride_x, stride, *red, active));
+    DWF_PREC_SWITCH(prec, SP, xr_update_kernel<Store32, SP><<<grid, sh.threads, 0, s>>>(g, x, r, p, w, num, den, sstride, stride_x, stride, *red, active));
   } else {
     return cudaErrorInvalidValue;
   }
@@ -772,19 +760,21 @@ cudaError_t launch_xr_update(const Geom& g, int prec, int xprec, void* x, void* 
 cudaError_t launch_p_update(const Geom& g, int prec, void* p, const void* z, const double* num,
                             const double* den, int sstride, int nrhs, size_t stride,
                             cudaStream_t s, const int* active) {
-  dim3 grid(elementwise_blocks((size_t)g.N5 / 2), nrhs);
-  DWF_PREC_SWITCH(prec, SP, p_update_kernel<SP><<<grid, kBlasThreads, 0, s>>>(g, p, z, num, den, sstride, stride, active));
+  const Shape sh = elementwise((size_t)g.N5 / 2);
+  const dim3 grid(sh.blocks, nrhs);
+  DWF_PREC_SWITCH(prec, SP, p_update_kernel<SP><<<grid, sh.threads, 0, s>>>(g, p, z, num, den, sstride, stride, active));
   return cudaGetLastError();
 }
 
 template <class SPD>
 cudaError_t convert_from(const Geom& g, void* dst, int prec_s, const void* src, int nrhs, size_t sd,
                          size_t ss, const Reduce* red, cudaStream_t s, const int* active) {
-  dim3 grid(elementwise_blocks((size_t)g.N5 / 2), nrhs);
+  const Shape sh = elementwise((size_t)g.N5 / 2);
+  const dim3 grid(sh.blocks, nrhs);
   Reduce r{};
   if (red) r = *red;
   const int dn = red != nullptr;
-  DWF_PREC_SWITCH(prec_s, SPS, convert_kernel<SPD, SPS><<<grid, kBlasThreads, 0, s>>>(g, dst, src, sd, ss, r, dn, active));
+  DWF_PREC_SWITCH(prec_s, SPS, convert_kernel<SPD, SPS><<<grid, sh.threads, 0, s>>>(g, dst, src, sd, ss, r, dn, active));
   return cudaGetLastError();
 }
 
@@ -805,8 +795,9 @@ template <class SPX>
 cudaError_t px_from(const Geom& g, int prec, void* x, void* p, const void* z, const double* a_ptr,
                     const double* num, const double* den, int sstride, int nrhs, size_t sx,
                     size_t sp, cudaStream_t s, const int* active, int do_p) {
-  dim3 grid(elementwise_blocks((size_t)g.N5 / 2), nrhs);
-  DWF_PREC_SWITCH(prec, SP, px_update_kernel<SPX, SP><<<grid, kBlasThreads, 0, s>>>(g, x, p, z, a_ptr, num, den, sstride, sx, sp, active, do_p));
+  const Shape sh = elementwise((size_t)g.N5 / 2);
+  const dim3 grid(sh.blocks, nrhs);
+  DWF_PREC_SWITCH(prec, SP, px_update_kernel<SPX, SP><<<grid, sh.threads, 0, s>>>(g, x, p, z, a_ptr, num, den, sstride, sx, sp, active, do_p));
   return cudaGetLastError();
 }
 
@@ -831,25 +822,26 @@ cudaError_t launch_pxb_update(const Geom& g, int prec, int xprec, void* x, const
                               const double* den, int sstride, int nrhs, size_t sx, size_t sp,
                               const void* bdiag, const void* boff, size_t cstride, cudaStream_t s,
                               const int* active, int do_x) {
-  dim3 grid(elementwise_blocks((size_t)g.N5 / 2), nrhs);
+  const Shape sh = elementwise((size_t)g.N5 / 2);
+  const dim3 grid(sh.blocks, nrhs);
   if (prec == P32 && xprec == P32) {
-    pxb_update_kernel<Store32, Store32><<<grid, kBlasThreads, 0, s>>>(
+    pxb_update_kernel<Store32, Store32><<<grid, sh.threads, 0, s>>>(
         g, x, p, pnew, bp, z, a_ptr, num, den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
         reinterpret_cast<const float*>(boff), cstride, active, do_x);
   } else if (prec == P32 && xprec == P64) {
-    pxb_update_kernel<Store64, Store32><<<grid, kBlasThreads, 0, s>>>(
+    pxb_update_kernel<Store64, Store32><<<grid, sh.threads, 0, s>>>(
         g, x, p, pnew, bp, z, a_ptr, num, den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
         reinterpret_cast<const float*>(boff), cstride, active, do_x);
   } else if (prec == P64 && xprec == P64) {
-    pxb_update_kernel<Store64, Store64><<<grid, kBlasThreads, 0, s>>>(
+    pxb_update_kernel<Store64, Store64><<<grid, sh.threads, 0, s>>>(
         g, x, p, pnew, bp, z, a_ptr, num, den, sstride, sx, sp, reinterpret_cast<const double*>(bdiag),
         reinterpret_cast<const double*>(boff), cstride, active, do_x);
   } else if (prec == P16 && xprec == P32) {
-    pxb_update_kernel<Store32, Store16<false>><<<grid, kBlasThreads, 0, s>>>(
+    pxb_update_kernel<Store32, Store16<false>><<<grid, sh.threads, 0, s>>>(
         g, x, p, pnew, bp, z, a_ptr, num, den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
         reinterpret_cast<const float*>(boff), cstride, active, do_x);
   } else if (prec == PB16 && xprec == P32) {
-    pxb_update_kernel<Store32, Store16<true>><<<grid, kBlasThreads, 0, s>>>(
+    pxb_update_kernel<Store32, Store16<true>><<<grid, sh.threads, 0, s>>>(
         g, x, p, pnew, bp, z, a_ptr, num, den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
         reinterpret_cast<const float*>(boff), cstride, active, do_x);
   } else {
@@ -860,32 +852,35 @@ cudaError_t launch_pxb_update(const Geom& g, int prec, int xprec, void* x, const
 
 cudaError_t launch_accumulate64(const Geom& g, void* x64, int prec_s, void* src, int zero_src,
                                 int nrhs, size_t sd, size_t ss, cudaStream_t s, const int* active) {
-  dim3 grid(elementwise_blocks((size_t)g.N5 / 2), nrhs);
-  DWF_PREC_SWITCH(prec_s, SPS, accumulate64_kernel<SPS><<<grid, kBlasThreads, 0, s>>>(g, x64, src, zero_src, sd, ss, active));
+  const Shape sh = elementwise((size_t)g.N5 / 2);
+  const dim3 grid(sh.blocks, nrhs);
+  DWF_PREC_SWITCH(prec_s, SPS, accumulate64_kernel<SPS><<<grid, sh.threads, 0, s>>>(g, x64, src, zero_src, sd, ss, active));
   return cudaGetLastError();
 }
 
 cudaError_t launch_sub64_norm(const Geom& g, void* out, const void* a, const void* b, int nrhs,
                               size_t stride, const Reduce* red, cudaStream_t s, const int* active) {
-  dim3 grid(elementwise_blocks((size_t)g.N5 / 2), nrhs);
-  sub64_norm_kernel<<<grid, kBlasThreads, 0, s>>>(g, out, a, b, stride, *red, active);
+  const Shape sh = elementwise((size_t)g.N5 / 2);
+  const dim3 grid(sh.blocks, nrhs);
+  sub64_norm_kernel<<<grid, sh.threads, 0, s>>>(g, out, a, b, stride, *red, active);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sub_to(const Geom& g, int prec_d, void* dst, const void* a64, const void* b32,
                           int nrhs, size_t sd, size_t sa, size_t sb, const Reduce* red,
                           cudaStream_t s, const int* active) {
-  dim3 grid(elementwise_blocks((size_t)g.N5 / 2), nrhs);
+  const Shape sh = elementwise((size_t)g.N5 / 2);
+  const dim3 grid(sh.blocks, nrhs);
   switch (prec_d) {
     case P32:
-      sub_to_kernel<Store32><<<grid, kBlasThreads, 0, s>>>(g, dst, a64, b32, sd, sa, sb, *red, active);
+      sub_to_kernel<Store32><<<grid, sh.threads, 0, s>>>(g, dst, a64, b32, sd, sa, sb, *red, active);
       break;
     case P16:
-      sub_to_kernel<Store16<false>><<<grid, kBlasThreads, 0, s>>>(g, dst, a64, b32, sd, sa, sb, *red,
+      sub_to_kernel<Store16<false>><<<grid, sh.threads, 0, s>>>(g, dst, a64, b32, sd, sa, sb, *red,
                                                                   active);
       break;
     case PB16:
-      sub_to_kernel<Store16<true>><<<grid, kBlasThreads, 0, s>>>(g, dst, a64, b32, sd, sa, sb, *red,
+      sub_to_kernel<Store16<true>><<<grid, sh.threads, 0, s>>>(g, dst, a64, b32, sd, sa, sb, *red,
                                                                  active);
       break;
     default: return cudaErrorInvalidValue;
@@ -895,15 +890,17 @@ cudaError_t launch_sub_to(const Geom& g, int prec_d, void* dst, const void* a64,
 
 cudaError_t launch_norm(const Geom& g, int prec, const void* x, int nrhs, size_t stride,
                         const Reduce* red, cudaStream_t s) {
-  dim3 grid(elementwise_blocks((size_t)g.N5 / 2), nrhs);
-  DWF_PREC_SWITCH(prec, SP, norm_kernel<SP><<<grid, kBlasThreads, 0, s>>>(g, x, stride, *red));
+  const Shape sh = elementwise((size_t)g.N5 / 2);
+  const dim3 grid(sh.blocks, nrhs);
+  DWF_PREC_SWITCH(prec, SP, norm_kernel<SP><<<grid, sh.threads, 0, s>>>(g, x, stride, *red));
   return cudaGetLastError();
 }
 
 cudaError_t launch_dot_re64(const Geom& g, const void* a, const void* b, int nrhs, size_t stride,
                             const Reduce* red, cudaStream_t s) {
-  dim3 grid(elementwise_blocks((size_t)g.N5 / 2), nrhs);
-  dot_re64_kernel<<<grid, kBlasThreads, 0, s>>>(g, a, b, stride, *red);
+  const Shape sh = elementwise((size_t)g.N5 / 2);
+  const dim3 grid(sh.blocks, nrhs);
+  dot_re64_kernel<<<grid, sh.threads, 0, s>>>(g, a, b, stride, *red);
   return cudaGetLastError();
 }
 

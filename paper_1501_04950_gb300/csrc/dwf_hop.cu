@@ -371,6 +371,7 @@ cudaError_t launch_hop(const Geom& g, const HopLaunch& L, cudaStream_t st) {
     }
     if (e != cudaErrorNotSupported) return e;
   }
+  if (L.extra) return cudaErrorInvalidValue;
   switch (L.prec) {
     case P64: return dispatch_hop<Store64>(g, L, st);
     case P32: return dispatch_hop<Store32>(g, L, st);

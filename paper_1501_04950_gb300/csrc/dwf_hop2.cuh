@@ -292,6 +292,13 @@ struct Args {
   size_t cstride;       // elements between right-hand sides of bdiag, boff, chain
   const int* active;    // per right-hand side: 0 skips it (nullptr: all active)
   int* err;             // set to 1 when a bounded wait gives up (staged variant)
+  // EX_HAT: out2 = I^-T gamma5 out.  EX_RUPD: r = out2 is updated, r -= a out, a = *num / *den
+  // (stored to a_out, one per right-hand side sstride apart), and out itself is not stored.
+  void* out2;
+  const double* num;
+  const double* den;
+  double* a_out;
+  int sstride;
 };
 
 // h = P_+ - dir A P_- in place into P: the half spinor of (1 - DIR gamma_mu).
@@ -654,11 +661,16 @@ __device__ __forceinline__ void zero(SpinP<V>& a) {
 template <typename T>
 constexpr int min_blocks() { return sizeof(T) == 8 ? 2 : 4; }
 
+// Steps of the CG on D_bb^+ D_bb that end a hopping pass (HopLaunch.extra).
+enum { EX_NONE = 0, EX_HAT = 1, EX_RUPD = 2 };
+
 // Common tail of the hopping kernels: 5th-dimension post program, scaling,
 // optional gamma5, local term (c_loc = 1), store and fused norm.  Every thread of the
 // CTA calls it (it contains __syncthreads); the nth threads with tid < nth run the
-// program, threads with part = false (no site of their own) store nothing.
-template <class SP, int LS, int POST, int LOC, bool G5, bool NORM>
+// program, threads with part = false (no site of their own) store nothing.  With EX_HAT
+// the result also goes through PR_ITINV (coefficients after those of POST); with EX_RUPD
+// it updates the residual, whose norm is the fused one.
+template <class SP, int LS, int POST, int LOC, bool G5, bool NORM, int EX = EX_NONE>
 __device__ __forceinline__ void epilogue_g(const Args<typename SP::T>& a, const typename SP::T* coef,
                                            typename SP::T* sbuf, int tid, int nth, int nsites, size_t NP,
                                            int h, int j, int t, bool active, bool part, int rhs,
@@ -696,8 +708,44 @@ __device__ __forceinline__ void epilogue_g(const Args<typename SP::T>& a, const 
       acc.im[c] = A::mul(f, acc.im[c]);
     }
   }
-  if (active) PairIO<SP>::store(reinterpret_cast<char*>(a.out) + off, m, NP, acc);
-  if (NORM) {
+  if constexpr (EX == EX_RUPD) {
+    const double ad = a.num[(size_t)rhs * a.sstride] / a.den[(size_t)rhs * a.sstride];
+    if (blockIdx.x == 0 && tid == 0) a.a_out[(size_t)rhs * a.sstride] = ad;
+    if (active) {
+      const V na = A::dup(-(T)ad);
+      char* r = reinterpret_cast<char*>(a.out2) + off;
+      SpinP<V> x;
+      load_spin<SP>(r, m, NP, x);
+#pragma unroll
+      for (int c = 0; c < 12; c++) {
+        acc.re[c] = A::fma(na, acc.re[c], x.re[c]);
+        acc.im[c] = A::fma(na, acc.im[c], x.im[c]);
+      }
+      PairIO<SP>::store(r, m, NP, acc);
+    }
+  } else {
+    if (active) PairIO<SP>::store(reinterpret_cast<char*>(a.out) + off, m, NP, acc);
+  }
+  if constexpr (EX == EX_HAT) {
+    static_assert(!SP::kScaled && NORM, "the fused hat is for FP32 and FP64 fields");
+    const double nrm = active ? sqr(acc) : 0.0;
+#pragma unroll
+    for (int c = 6; c < 12; c++) {
+      acc.re[c] = A::neg(acc.re[c]);
+      acc.im[c] = A::neg(acc.im[c]);
+    }
+    T* site = sbuf + j * site_stride(LS);
+    __syncthreads();
+    if (part) put<T, LS, PR_ITINV>(site, t, acc);
+    __syncthreads();
+    if (tid < nth) run_prog<T, LS, PR_ITINV>(sbuf, coef + prog_coefs(LS, POST), tid, nth, nsites);
+    __syncthreads();
+    if (active) {
+      get<T, LS, PR_ITINV>(site, t, acc);
+      PairIO<SP>::store(reinterpret_cast<char*>(a.out2) + off, m, NP, acc);
+    }
+    block_sum_to(nrm, a.red, rhs, gridDim.x, blockIdx.x);
+  } else if (NORM) {
     double v = 0.0;
     if (active) {
       if constexpr (SP::kScaled) {
@@ -714,14 +762,14 @@ __device__ __forceinline__ void epilogue_g(const Args<typename SP::T>& a, const 
 }
 
 // out = c_hop G post(H v') + loc(w), two 5th-dimension slices per thread.
-template <class SP, int LS, int PRE, int POST, int LOC, bool G5, bool NORM, int MINB>
+template <class SP, int LS, int PRE, int POST, int LOC, bool G5, bool NORM, int MINB, int EX = EX_NONE>
 __global__ void __launch_bounds__(128, MINB) hop_kernel(const Geom g, const Args<typename SP::T> a) {
   using T = typename SP::T;
   using V = typename Pr<T>::V;
   constexpr int G = LS / 2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* coef = reinterpret_cast<T*>(smem_raw);
-  T* sbuf = coef + prog_coefs(LS, POST);
+  T* sbuf = coef + prog_coefs(LS, POST) + (EX == EX_HAT ? prog_coefs(LS, PR_ITINV) : 0);
   const int tid = threadIdx.x, nth = blockDim.x;
   const int S = nth / G, j = tid / G, t = tid - j * G;
   const int h = blockIdx.x * S + j;
@@ -733,6 +781,7 @@ __global__ void __launch_bounds__(128, MINB) hop_kernel(const Geom g, const Args
   const size_t NP = (size_t)g.N5 >> 1;
   const int s0 = 2 * t;
   load_coefs<T, LS, POST>(coef, a.chain + co, tid, nth);
+  if (EX == EX_HAT) load_coefs<T, LS, PR_ITINV>(coef + prog_coefs(LS, POST), a.chain + co, tid, nth);
   const char* vb = reinterpret_cast<const char*>(a.v) + rhs * a.stride;
   SpinP<V> acc;
   zero(acc);
@@ -762,7 +811,7 @@ __global__ void __launch_bounds__(128, MINB) hop_kernel(const Geom g, const Args
     hop_dir<SP, LS, PRE, 3, +1>(nb[6], hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
     hop_dir<SP, LS, PRE, 3, -1>(nb[7], hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);
   }
-  epilogue_g<SP, LS, POST, LOC, G5, NORM>(a, coef, sbuf, tid, nth, S, NP, h, j, t, active, part, rhs, acc);
+  epilogue_g<SP, LS, POST, LOC, G5, NORM, EX>(a, coef, sbuf, tid, nth, S, NP, h, j, t, active, part, rhs, acc);
 }
 
 // out = c * PROG(gamma5^g5in in), site-local, two slices per thread.
@@ -829,8 +878,9 @@ inline int tile_threads(int Ls, int Vh, int nrhs, bool f64) {
   return 32;
 }
 
-inline size_t smem_bytes(int Ls, int S, size_t ts, int prog) {
-  return prog == PR_NONE ? 0 : ts * ((size_t)prog_coefs(Ls, prog) + (size_t)S * site_stride(Ls));
+inline size_t smem_bytes(int Ls, int S, size_t ts, int prog, int extra = EX_NONE) {
+  const int coefs = prog_coefs(Ls, prog) + (extra == EX_HAT ? prog_coefs(Ls, PR_ITINV) : 0);
+  return prog == PR_NONE ? 0 : ts * ((size_t)coefs + (size_t)S * site_stride(Ls));
 }
 
 // Raises a kernel's dynamic shared-memory limit once per process; safe when
@@ -900,7 +950,7 @@ cudaError_t run_tma(const Geom& g, const HopLaunch& L, const Args<typename SP::T
   return cudaGetLastError();
 }
 
-template <class SP, int LS, int PRE, int POST, int LOC, bool G5, bool NORM>
+template <class SP, int LS, int PRE, int POST, int LOC, bool G5, bool NORM, int EX = EX_NONE>
 cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   using T = typename SP::T;
   Args<T> a;
@@ -921,17 +971,22 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   a.cstride = L.cstride;
   a.active = L.active;
   a.err = L.err;
-  if constexpr (tma_ls(LS) && POST != PR_NONE) {
+  a.out2 = L.out2;
+  a.num = L.num;
+  a.den = L.den;
+  a.a_out = L.a_out;
+  a.sstride = L.sstride;
+  if constexpr (tma_ls(LS) && POST != PR_NONE && EX == EX_NONE) {
     if (L.use_tma) return run_tma<SP, LS, PRE, POST, LOC, G5, NORM>(g, L, a, st);
   }
   const int nt = L.block_threads ? L.block_threads : tile_threads(LS, g.Vh, L.nrhs, sizeof(T) == 8);
   const int S = nt / (LS / 2);
   dim3 grid((g.Vh + S - 1) / S, 1, L.nrhs);
-  auto k = hop_kernel<SP, LS, PRE, POST, LOC, G5, NORM, min_blocks<T>()>;
+  auto k = hop_kernel<SP, LS, PRE, POST, LOC, G5, NORM, min_blocks<T>(), EX>;
   static std::atomic<bool> attr{false};
-  cudaError_t e = smem_limit_once(k, smem_bytes(LS, 128 / (LS / 2), sizeof(T), POST), attr);
+  cudaError_t e = smem_limit_once(k, smem_bytes(LS, 128 / (LS / 2), sizeof(T), POST, EX), attr);
   if (e != cudaSuccess) return e;
-  k<<<grid, nt, smem_bytes(LS, S, sizeof(T), POST), st>>>(g, a);
+  k<<<grid, nt, smem_bytes(LS, S, sizeof(T), POST, EX), st>>>(g, a);
   return cudaGetLastError();
 }
 
@@ -941,6 +996,13 @@ template <class SP, int LS>
 cudaError_t dispatch_ls(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   const bool norm = L.red != nullptr;
   if (L.loc == LOC_DENSE || (L.loc == LOC_ID && L.c_loc != 1.0)) return cudaErrorNotSupported;
+  if constexpr (!SP::kScaled) {
+    if (L.extra == EX_HAT && L.pre == PRE_NONE && L.post_prog == PR_IINV && L.loc == LOC_ID && !L.g5out && norm)
+      return run<SP, LS, PRE_NONE, PR_IINV, LOC_ID, false, true, EX_HAT>(g, L, st);
+    if (L.extra == EX_RUPD && L.pre == PRE_NONE && L.post_prog == PR_BT && L.loc == LOC_ID && L.g5out && norm)
+      return run<SP, LS, PRE_NONE, PR_BT, LOC_ID, true, true, EX_RUPD>(g, L, st);
+  }
+  if (L.extra != EX_NONE) return cudaErrorNotSupported;
   // FP64 is bound by the FP64 pipe: its callers form B v once (PR_B) and hop that
   if constexpr (SP::kPrec != P64) {
     if (L.pre == PRE_B && L.post_prog == PR_K && L.loc == LOC_NONE && !L.g5out && !norm)

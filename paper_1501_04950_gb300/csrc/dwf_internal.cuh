@@ -99,8 +99,17 @@ struct HopLaunch {
   size_t cstride;           // elements between right-hand sides of every coefficient
                             // array (pre_diag, pre_off, post, locm, chain); 0: shared
   const int* active;        // per right-hand side: 0 skips it (nullptr: all active)
+  // Tuned path, FP32 / FP64: what the pass does besides (hop2::EX_*): 1 out2 = I^-T gamma5 out;
+  // 2 out2 -= a out with a = *num / *den -> a_out (per right-hand side, sstride apart), out is
+  // not stored and red takes |out2|^2
+  int extra;
+  void* out2;
+  const double* num;
+  const double* den;
+  double* a_out;
+  int sstride;
 };
-// Tries the tuned kernel first, then the generic one.
+// Tries the tuned kernel first, then the generic one (which has no extra steps).
 cudaError_t launch_hop(const Geom& g, const HopLaunch& a, cudaStream_t s);
 cudaError_t launch_hop2_f64(const Geom& g, const HopLaunch& a, cudaStream_t s);
 cudaError_t launch_hop2_f32(const Geom& g, const HopLaunch& a, cudaStream_t s);

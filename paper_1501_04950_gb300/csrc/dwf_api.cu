@@ -398,7 +398,7 @@ int get_ws(dwf_ctx* h, const std::string& name, size_t bytes, void** out) {
 int ensure_reduce(dwf_ctx* h, int nrhs) {
   int need_blocks = std::max(hop_grid_blocks(h->g, P64),
                              std::max(hop_grid_blocks(h->g, P32), blas_grid_blocks(h->g)));
-  if (hop2::tuned_ls(h->Ls, false)) {  // the smallest tile of the tuned kernels
+  if (hop2::tuned_ls(h->Ls, false)) {  // the smallest tile of the tuned kernels (32 threads a site)
     const int S = 32 / (h->Ls / 2);
     need_blocks = std::max(need_blocks, (h->g.Vh + S - 1) / S);
   }
@@ -470,6 +470,7 @@ struct CoefView {
   size_t cstride;
   const int* active;
   bool chain_ok;  // of every right-hand side's set
+  int rule_nrhs;  // HopLaunch.rule_nrhs
   const void* ptr(int prec, size_t off) const {
     const int f = prec == P64 ? 0 : 1;
     return reinterpret_cast<const char*>(dev[f]) + off * (f == 0 ? 8 : 4);
@@ -481,12 +482,13 @@ struct CoefView {
   }
 };
 CoefView view_of(const MatSet& ms) {
-  return CoefView{&ms, {ms.dev[0], ms.dev[1]}, 0, nullptr, ms.chain_ok};
+  return CoefView{&ms, {ms.dev[0], ms.dev[1]}, 0, nullptr, ms.chain_ok, 0};
 }
 
 void set_coef(HopLaunch& L, const CoefView& cv) {
   L.cstride = cv.cstride;
   L.active = cv.active;
+  L.rule_nrhs = cv.rule_nrhs;
 }
 
 int apply_dbb_bp(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* p, const void* bp,
@@ -1545,6 +1547,8 @@ int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_ou
   CUCHK(h, cudaMemsetAsync(x, 0, fi * maxnb, st));
   MatSet* ms;
   if ((rc = build_matset(h, h->alpha, h->m, &ms))) return rc;
+  CoefView tv = view_of(*ms);
+  tv.rule_nrhs = nrhs;
   cudaEvent_t e0, e1;
   CUCHK(h, cudaEventCreate(&e0));
   CUCHK(h, cudaEventCreate(&e1));
@@ -1552,7 +1556,9 @@ int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_ou
   std::vector<int> tiles = {h->env_tile >= 0 ? h->env_tile : 0};
   if (tuned) {
     if (h->env_tma) tiles = {0};  // the staged variant has one tile
-    else if (h->env_tile < 0) tiles = {128, 64, 32};
+    else if (h->env_tile < 0 && (prec == P16 || prec == PB16 ||
+                                 !hop2::split_directions(Ls, h->g.Vh, nrhs, prec == P64)))
+      tiles = {128, 64, 32};  // all of the same bits
   }
   double best = 1e300;
   int best_nb = ok.front(), best_tma = tmas.front(), best_tile = 0;
@@ -1564,13 +1570,13 @@ int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_ou
       for (int tile : tiles) {
         h->use_tma = tma;
         h->tile = tile;
-        if ((rc = apply_dbb(h, view_of(*ms), prec, y, x, t, nb, nullptr, st))) return rc;
+        if ((rc = apply_dbb(h, tv, prec, y, x, t, nb, nullptr, st))) return rc;
         // best of two timed passes of 3 applies (one slow pass does not decide)
         double per_rhs = 1e300;
         for (int pass = 0; pass < 2; pass++) {
           CUCHK(h, cudaEventRecord(e0, st));
           for (int k = 0; k < 3; k++)
-            if ((rc = apply_dbb(h, view_of(*ms), prec, y, x, t, nb, nullptr, st))) return rc;
+            if ((rc = apply_dbb(h, tv, prec, y, x, t, nb, nullptr, st))) return rc;
           CUCHK(h, cudaEventRecord(e1, st));
           CUCHK(h, cudaEventSynchronize(e1));
           float ms_t = 0.f;
@@ -2092,7 +2098,7 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
       KLAUNCH(h, launch_hop(g, Hs, st));
     }
     std::vector<dwf_stats> sk(n);
-    CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr, true};
+    CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr, true, nrhs};
     for (int r = 0; r < n; r++) cv.chain_ok = cv.chain_ok && ms[blk + r]->chain_ok;
     rc = cgnr_batched(h, cv, prec, h->opt.rel_tol, h->opt.maxiter, delta, restart, W, n, sk.data(), st);
     if (rc && rc != DWF_ERR_NOT_CONVERGED && rc != DWF_ERR_BREAKDOWN) return rc;

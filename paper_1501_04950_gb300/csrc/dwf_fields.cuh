@@ -580,4 +580,30 @@ __device__ __forceinline__ void su3_mul(const Link<T>& U, const cplx<T> h0[3], c
   }
 }
 
+// ---------------------------------------------------------------------------
+// The tuned kernels (dwf_hop2.cuh): the Ls they are compiled for (the others take the
+// generic kernels) are the Ls of the alpha study, of the benchmark and of the Mobius /
+// Zolotarev comparison.  With 16-bit storage (scaled) only the Ls of the benchmark
+// workloads: elsewhere the recurrences' FP32 rounding, as good as the dense
+// contraction's but not the same, would turn some 16-bit roundings of the intermediate
+// fields the other way, and those results are kept.  One translation unit per storage
+// precision and group of Ls.
+// ---------------------------------------------------------------------------
+namespace hop2 {
+__host__ __device__ constexpr bool tuned_ls(int Ls, bool scaled) {
+  return Ls == 8 || Ls == 12 || Ls == 16 ||
+         (!scaled && (Ls == 4 || Ls == 6 || Ls == 10 || Ls == 20 || Ls == 24 || Ls == 32));
+}
+constexpr int kLsGroups = 4;
+__host__ __device__ constexpr int ls_group(int Ls) {
+  return Ls <= 8 ? 0 : Ls <= 12 ? 1 : Ls <= 20 ? 2 : 3;
+}
+template <class SP, int GROUP>
+cudaError_t dispatch(const Geom& g, const HopLaunch& L, cudaStream_t st);
+template <class SP, int GROUP>
+cudaError_t dispatch(const Geom& g, const LocalLaunch& L, cudaStream_t st);
+template <class SP, int GROUP>
+cudaError_t dispatch(const Geom& g, const RUpdateLaunch& L, cudaStream_t st);
+}  // namespace hop2
+
 }  // namespace dwf

@@ -360,17 +360,36 @@ int hop_grid_blocks(const Geom& g, int prec) {
 
 int g_disable_tuned = 0;
 
-cudaError_t launch_hop(const Geom& g, const HopLaunch& L, cudaStream_t st) {
-  if (!g_disable_tuned) {
-    cudaError_t e = cudaErrorNotSupported;
-    switch (L.prec) {
-      case P64: e = launch_hop2_f64(g, L, st); break;
-      case P32: e = launch_hop2_f32(g, L, st); break;
-      case P16: e = launch_hop2_f16(g, L, st); break;
-      case PB16: e = launch_hop2_bf16(g, L, st); break;
-    }
-    if (e != cudaErrorNotSupported) return e;
+namespace {
+
+// The tuned kernels of a launch's precision and Ls, or cudaErrorNotSupported.
+template <class SP, class Launch>
+cudaError_t tuned_of(const Geom& g, const Launch& L, cudaStream_t st) {
+  if (!hop2::tuned_ls(g.Ls, SP::kScaled)) return cudaErrorNotSupported;
+  switch (hop2::ls_group(g.Ls)) {
+    case 0: return hop2::dispatch<SP, 0>(g, L, st);
+    case 1: return hop2::dispatch<SP, 1>(g, L, st);
+    case 2: return hop2::dispatch<SP, 2>(g, L, st);
+    default: return hop2::dispatch<SP, 3>(g, L, st);
   }
+}
+template <class Launch>
+cudaError_t tuned(const Geom& g, const Launch& L, cudaStream_t st) {
+  if (g_disable_tuned) return cudaErrorNotSupported;
+  switch (L.prec) {
+    case P64: return tuned_of<Store64>(g, L, st);
+    case P32: return tuned_of<Store32>(g, L, st);
+    case P16: return tuned_of<Store16<false>>(g, L, st);
+    case PB16: return tuned_of<Store16<true>>(g, L, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+cudaError_t launch_hop(const Geom& g, const HopLaunch& L, cudaStream_t st) {
+  const cudaError_t e = tuned(g, L, st);
+  if (e != cudaErrorNotSupported) return e;
   if (L.extra) return cudaErrorInvalidValue;
   switch (L.prec) {
     case P64: return dispatch_hop<Store64>(g, L, st);
@@ -381,28 +400,11 @@ cudaError_t launch_hop(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_rupdate(const Geom& g, const RUpdateLaunch& L, cudaStream_t st) {
-  if (g_disable_tuned) return cudaErrorNotSupported;
-  switch (L.prec) {
-    case P64: return launch_hop2_f64_rupdate(g, L, st);
-    case P32: return launch_hop2_f32_rupdate(g, L, st);
-    case P16: return launch_hop2_f16_rupdate(g, L, st);
-    case PB16: return launch_hop2_bf16_rupdate(g, L, st);
-  }
-  return cudaErrorInvalidValue;
-}
+cudaError_t launch_rupdate(const Geom& g, const RUpdateLaunch& L, cudaStream_t st) { return tuned(g, L, st); }
 
 cudaError_t launch_local(const Geom& g, const LocalLaunch& L, cudaStream_t st) {
-  if (!g_disable_tuned) {
-    cudaError_t e = cudaErrorNotSupported;
-    switch (L.prec) {
-      case P64: e = launch_hop2_f64_local(g, L, st); break;
-      case P32: e = launch_hop2_f32_local(g, L, st); break;
-      case P16: e = launch_hop2_f16_local(g, L, st); break;
-      case PB16: e = launch_hop2_bf16_local(g, L, st); break;
-    }
-    if (e != cudaErrorNotSupported) return e;
-  }
+  const cudaError_t e = tuned(g, L, st);
+  if (e != cudaErrorNotSupported) return e;
   switch (L.prec) {
     case P64: return run_local<Store64>(g, L, st);
     case P32: return run_local<Store32>(g, L, st);

@@ -28,6 +28,7 @@
 //     for the unknown first element and one back-substitution sweep.
 #pragma once
 
+#include <algorithm>
 #include <atomic>
 #include <cstdlib>
 
@@ -37,17 +38,6 @@
 
 namespace dwf {
 namespace hop2 {
-
-// The Ls whose kernels are compiled (the others take the generic kernels): the Ls of
-// the alpha study, of the benchmark and of the Mobius / Zolotarev comparison.  With
-// 16-bit storage (scaled) only the Ls of the benchmark workloads: elsewhere the
-// recurrences' FP32 rounding, as good as the dense contraction's but not the same, would
-// turn some 16-bit roundings of the intermediate fields the other way, and those
-// results are kept.
-__host__ __device__ constexpr bool tuned_ls(int Ls, bool scaled) {
-  return Ls == 8 || Ls == 12 || Ls == 16 ||
-         (!scaled && (Ls == 4 || Ls == 6 || Ls == 10 || Ls == 20 || Ls == 24 || Ls == 32));
-}
 
 // Chain coefficient block: [op][chirality][kChainStride(Ls)] in the compute type,
 // op = 0 B (mult), 1 B^T (mult), 2 I (mult), 3 I (solve), 4 I^T (solve).  Step k of
@@ -658,6 +648,16 @@ __device__ __forceinline__ void zero(SpinP<V>& a) {
   }
 }
 
+template <typename V>
+__device__ __forceinline__ void add(SpinP<V>& a, const SpinP<V>& b) {
+  using A = Pr<decltype(a.re[0].x)>;
+#pragma unroll
+  for (int c = 0; c < 12; c++) {
+    a.re[c] = A::add(a.re[c], b.re[c]);
+    a.im[c] = A::add(a.im[c], b.im[c]);
+  }
+}
+
 template <typename T>
 constexpr int min_blocks() { return sizeof(T) == 8 ? 2 : 4; }
 
@@ -814,6 +814,202 @@ __global__ void __launch_bounds__(128, MINB) hop_kernel(const Geom g, const Args
   epilogue_g<SP, LS, POST, LOC, G5, NORM, EX>(a, coef, sbuf, tid, nth, S, NP, h, j, t, active, part, rhs, acc);
 }
 
+// --- small lattices: the directions of a site on four warps ---------------------------
+
+// One component of a slice pair (FP32 and FP64 fields).
+__device__ __forceinline__ void load_comp(const float* base, size_t m, size_t NP, int c, float2& re, float2& im) {
+  const float4 v = __ldg(reinterpret_cast<const float4*>(base) + (size_t)c * NP + m);
+  re = make_float2(v.x, v.y);
+  im = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void load_comp(const double* base, size_t m, size_t NP, int c, double2& re, double2& im) {
+  const double2* p = reinterpret_cast<const double2*>(base) + ((size_t)c * NP + m) * 2;
+  re = __ldg(p);
+  im = __ldg(p + 1);
+}
+__device__ __forceinline__ void store_comp(float* base, size_t m, size_t NP, int c, float2 re, float2 im) {
+  reinterpret_cast<float4*>(base)[(size_t)c * NP + m] = make_float4(re.x, re.y, im.x, im.y);
+}
+__device__ __forceinline__ void store_comp(double* base, size_t m, size_t NP, int c, double2 re, double2 im) {
+  double2* p = reinterpret_cast<double2*>(base) + ((size_t)c * NP + m) * 2;
+  p[0] = re;
+  p[1] = im;
+}
+
+// run_prog for 128 threads on nsites <= 32 / (LS / 2) sites whose input is the sum of
+// NPART blocks, `part_stride` apart; the result replaces the first block.
+template <typename T, int LS, int PROG, int NPART>
+__device__ __forceinline__ void run_prog_sum(T* sbuf, int part_stride, const T* coef, int tid, int nsites) {
+  constexpr int NIT = (12 * (32 / (LS / 2)) + 63) / 64;
+  const int ch = tid >> 6;
+  T V[NIT][LS];
+#pragma unroll
+  for (int q = 0; q < NIT; q++) {
+    const int i = (tid & 63) + 64 * q, site = i / 12;
+    const T* p = sbuf + site * site_stride(LS) + 24 * ch + 2 * (i - 12 * site);
+#pragma unroll
+    for (int k = 0; k < LS / 2; k++) {
+      V[q][2 * k] = V[q][2 * k + 1] = (T)0;
+      if (i < 12 * nsites) {
+        auto v = pair_at(p + k * kPairStride);
+#pragma unroll
+        for (int b = 1; b < NPART; b++) v = Pr<T>::add(v, pair_at(p + b * part_stride + k * kPairStride));
+        V[q][2 * k] = v.x;
+        V[q][2 * k + 1] = v.y;
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < prog_len(PROG); i++) {
+    const T* c = coef + (2 * i + ch) * chain_stride(LS);
+    if (op_is_solve(prog_op(PROG, i))) chain_solve<T, LS, NIT>(V, c);
+    else chain_mult<T, LS, NIT>(V, c);
+  }
+#pragma unroll
+  for (int q = 0; q < NIT; q++) {
+    const int i = (tid & 63) + 64 * q, site = i / 12;
+    T* p = sbuf + site * site_stride(LS) + 24 * ch + 2 * (i - 12 * site);
+    if (i < 12 * nsites)
+#pragma unroll
+      for (int k = 0; k < LS / 2; k++)
+        *reinterpret_cast<typename Pr<T>::V*>(p + k * kPairStride) = Pr<T>::mk(V[q][2 * k], V[q][2 * k + 1]);
+  }
+}
+
+// hop_kernel with the four directions mu of a site on the four warps of a CTA (two hops
+// each) and 32 / G sites per CTA; the warps' sums are added on the way into the
+// 5th-dimension program, and each warp finishes three of the twelve components.
+// For lattices that leave SM sub-partitions without a warp: a warp alone is bound by its
+// own chain (FP64: one instruction per 64 cycles of its sub-partition's pipe; FP32: eight
+// gathers one after the other), which this cuts to a quarter.
+template <class SP, int LS, int PRE, int POST, int LOC, bool G5, bool NORM, int MINB, int EX = EX_NONE>
+__global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, const Args<typename SP::T> a) {
+  using T = typename SP::T;
+  using A = Pr<T>;
+  using V = typename A::V;
+  constexpr int G = LS / 2, S = 32 / G, SST = site_stride(LS);
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  T* coef = reinterpret_cast<T*>(smem_raw);
+  T* sbuf = coef + prog_coefs(LS, POST) + (EX == EX_HAT ? prog_coefs(LS, PR_ITINV) : 0);
+  const int tid = threadIdx.x, mu = tid >> 5, lane = tid & 31;
+  const int j = lane / G, t = lane - j * G;
+  const int h = blockIdx.x * S + j;
+  const bool part = warp_groups(LS) || j < S;
+  const bool active = part && h < g.Vh;
+  const int rhs = blockIdx.z;
+  if (a.active && !a.active[rhs]) return;
+  const size_t co = (size_t)rhs * a.cstride;
+  const size_t NP = (size_t)g.N5 >> 1;
+  load_coefs<T, LS, POST>(coef, a.chain + co, tid, 128);
+  if (EX == EX_HAT) load_coefs<T, LS, PR_ITINV>(coef + prog_coefs(LS, POST), a.chain + co, tid, 128);
+  const char* vb = reinterpret_cast<const char*>(a.v) + rhs * a.stride;
+  SpinP<V> acc;
+  zero(acc);
+  constexpr bool WHOLE = PRE == PRE_B && warp_groups(LS);
+  if (WHOLE || active) {
+    const int hl = WHOLE ? min(h, g.Vh - 1) : h;
+    const int2 nb = __ldg(reinterpret_cast<const int2*>(a.nbr) + (size_t)hl * 4 + mu);
+    T bd[2][2] = {{0, 0}, {0, 0}}, bo[2][2] = {{0, 0}, {0, 0}};
+    if (PRE == PRE_B) {
+#pragma unroll
+      for (int c = 0; c < 2; c++)
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+          bd[c][k] = __ldg(a.bdiag + co + c * LS + 2 * t + k);
+          bo[c][k] = __ldg(a.boff + co + c * LS + 2 * t + k);
+        }
+    }
+#define DWF_SPLIT_MU(MU)                                                                          \
+  case MU:                                                                                        \
+    hop_dir<SP, LS, PRE, MU, +1>(nb.x, hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);          \
+    hop_dir<SP, LS, PRE, MU, -1>(nb.y, hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);          \
+    break;
+    switch (mu) {
+      DWF_SPLIT_MU(0)
+      DWF_SPLIT_MU(1)
+      DWF_SPLIT_MU(2)
+      DWF_SPLIT_MU(3)
+    }
+#undef DWF_SPLIT_MU
+  }
+  // this warp's components of the result: 3 mu .. 3 mu + 2, all of chirality mu / 2
+  const size_t off = rhs * a.stride, m = (size_t)h * G + t;
+  const int c0 = 3 * mu, chir = mu >> 1;
+  const T* other = reinterpret_cast<const T*>(
+      (EX == EX_RUPD ? reinterpret_cast<const char*>(a.out2) : reinterpret_cast<const char*>(a.w)) + off);
+  V wr[3], wi[3], xr[3], xi[3];
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    wr[k] = wi[k] = xr[k] = xi[k] = A::dup((T)0);
+    if (LOC == LOC_ID && active)
+      load_comp(reinterpret_cast<const T*>(reinterpret_cast<const char*>(a.w) + off), m, NP, c0 + k, wr[k], wi[k]);
+    if (EX == EX_RUPD && active) load_comp(other, m, NP, c0 + k, xr[k], xi[k]);
+  }
+  if (part) put<T, LS, POST>(sbuf + (mu * S + j) * SST, t, acc);
+  __syncthreads();
+  run_prog_sum<T, LS, POST, 4>(sbuf, S * SST, coef, tid, S);
+  __syncthreads();
+  const bool rev = prog_reversed(POST, 1) == (chir == 1);  // one of the chiralities is reversed
+  const T* p = sbuf + j * SST + (rev ? G - 1 - t : t) * kPairStride + 4 * c0;
+  const T f = G5 && chir == 1 ? -a.c_hop : a.c_hop;
+  V re[3], im[3];
+  double nrm = 0.0;
+  T na = 0;
+  if (EX == EX_RUPD) {
+    const double ad = a.num[(size_t)rhs * a.sstride] / a.den[(size_t)rhs * a.sstride];
+    if (blockIdx.x == 0 && tid == 0) a.a_out[(size_t)rhs * a.sstride] = ad;
+    na = -(T)ad;
+  }
+  if (active) {
+    V n2 = A::dup((T)0);
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      const Coef4<T> v = coef4(p + 4 * k);
+      re[k] = rev ? A::mk(v.b, v.a) : A::mk(v.a, v.b);
+      im[k] = rev ? A::mk(v.d, v.c) : A::mk(v.c, v.d);
+      re[k] = LOC == LOC_ID ? A::fma(A::dup(f), re[k], wr[k]) : A::mul(A::dup(f), re[k]);
+      im[k] = LOC == LOC_ID ? A::fma(A::dup(f), im[k], wi[k]) : A::mul(A::dup(f), im[k]);
+      if (EX == EX_RUPD) {
+        re[k] = A::fma(A::dup(na), re[k], xr[k]);
+        im[k] = A::fma(A::dup(na), im[k], xi[k]);
+      }
+      store_comp(reinterpret_cast<T*>(reinterpret_cast<char*>(EX == EX_RUPD ? a.out2 : a.out) + off), m, NP,
+                 c0 + k, re[k], im[k]);
+      n2 = A::fma(re[k], re[k], n2);
+      n2 = A::fma(im[k], im[k], n2);
+    }
+    nrm = (double)n2.x + (double)n2.y;
+  }
+  if (EX == EX_HAT) {
+    const bool hrev = prog_reversed(PR_ITINV, 1) == (chir == 1);
+    T* q = sbuf + j * SST + (hrev ? G - 1 - t : t) * kPairStride + 4 * c0;
+    __syncthreads();
+    if (active) {
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        if (chir == 1) {
+          re[k] = A::neg(re[k]);
+          im[k] = A::neg(im[k]);
+        }
+        if (hrev) put4(q + 4 * k, re[k].y, re[k].x, im[k].y, im[k].x);
+        else put4(q + 4 * k, re[k].x, re[k].y, im[k].x, im[k].y);
+      }
+    }
+    __syncthreads();
+    run_prog_sum<T, LS, PR_ITINV, 1>(sbuf, 0, coef + prog_coefs(LS, POST), tid, S);
+    __syncthreads();
+    if (active) {
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        const Coef4<T> v = coef4(q + 4 * k);
+        store_comp(reinterpret_cast<T*>(reinterpret_cast<char*>(a.out2) + off), m, NP, c0 + k,
+                   hrev ? A::mk(v.b, v.a) : A::mk(v.a, v.b), hrev ? A::mk(v.d, v.c) : A::mk(v.c, v.d));
+      }
+    }
+  }
+  if (NORM) block_sum_to(nrm, a.red, rhs, gridDim.x, blockIdx.x);
+}
+
 // out = c * PROG(gamma5^g5in in), site-local, two slices per thread.
 template <class SP, int LS, int PROG>
 __global__ void __launch_bounds__(128) local_kernel(const Geom g, void* out, const void* in,
@@ -867,10 +1063,13 @@ namespace hop2 {
 // Threads per CTA (HopLaunch.block_threads; 0: by the rule of tile_threads).
 constexpr int kTileThreads[3] = {128, 64, 32};
 
-// The largest CTA that still gives every SM four of them (FP64: eight): a small lattice
-// then spreads over the SMs, and over the sub-partitions of an SM.
+// The largest CTA that still gives every SM four of them (FP64: eight, its pipe wants the
+// warps spread evenly over the sub-partitions); 64 threads at most where a site's threads
+// straddle warps and the CTA's tail of unused lanes counts (FP32, Ls = 10, 12^3x24, D_bb +
+// D_bb^+: 103.6 us at 64, 107.4 at 128).  All of them give the same bits.
 inline int tile_threads(int Ls, int Vh, int nrhs, bool f64) {
   for (int nt : kTileThreads) {
+    if (nt == 128 && !f64 && !warp_groups(Ls)) continue;
     const int S = nt / (Ls / 2);
     const long long blocks = (long long)((Vh + S - 1) / S) * nrhs;
     if (blocks >= 152 * (f64 ? 8 : 4) * 128 / nt) return nt;
@@ -878,9 +1077,25 @@ inline int tile_threads(int Ls, int Vh, int nrhs, bool f64) {
   return 32;
 }
 
+constexpr size_t split_smem(int Ls, size_t ts, int prog, int extra) {
+  return ts * ((size_t)prog_coefs(Ls, prog) + (extra == EX_HAT ? prog_coefs(Ls, PR_ITINV) : 0) +
+               4 * (size_t)(32 / (Ls / 2)) * site_stride(Ls));
+}
+
 inline size_t smem_bytes(int Ls, int S, size_t ts, int prog, int extra = EX_NONE) {
   const int coefs = prog_coefs(Ls, prog) + (extra == EX_HAT ? prog_coefs(Ls, PR_ITINV) : 0);
   return prog == PR_NONE ? 0 : ts * ((size_t)coefs + (size_t)S * site_stride(Ls));
+}
+
+// hop_split_kernel instead of hop_kernel: while the warps of hop_kernel do not fill the 608
+// SM sub-partitions once (FP32), or fill them in a last round of FP64 work that four times
+// as many quarter-sized warps finish sooner.  D_bb + D_bb^+ at Ls = 16, us with / without
+// (CUDA graph): FP32 4^4 14.3 / 26.3, 8^4 (512 warps) 24.0 / 28.8, 12 right-hand sides of
+// 8^2x4^2 (1536 warps) 49.4 / 42.4; FP64 4^4 101 / 276, 8^3x4 (256) 175 / 277,
+// 12^2x8x12 at Ls = 4 (432) 237 / 290, 8^4 (512) 326 / 296.
+inline bool split_directions(int Ls, int Vh, int nrhs, bool f64) {
+  const int S = 32 / (Ls / 2);
+  return (long long)((Vh + S - 1) / S) * nrhs <= (f64 ? 456 : 608);
 }
 
 // Raises a kernel's dynamic shared-memory limit once per process; safe when
@@ -945,8 +1160,8 @@ cudaError_t run_tma(const Geom& g, const HopLaunch& L, const Args<typename SP::T
     skip = *L.skip_hop;
     *L.skip_hop = -1;
   }
-  k<<<grid, kTmaThreads, smem, st>>>(g, a, map, L.wait_budget > 0 ? L.wait_budget : (1LL << 31),
-                                     skip);
+  k<<<grid, kTmaThreads, smem, st>>>(g, a, map, L.wait_budget > 0 ? L.wait_budget : (1LL << 31), skip,
+                                     split_directions(LS, g.Vh, std::max(L.nrhs, L.rule_nrhs), sizeof(typename SP::T) == 8));
   return cudaGetLastError();
 }
 
@@ -978,6 +1193,18 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   a.sstride = L.sstride;
   if constexpr (tma_ls(LS) && POST != PR_NONE && EX == EX_NONE) {
     if (L.use_tma) return run_tma<SP, LS, PRE, POST, LOC, G5, NORM>(g, L, a, st);
+  }
+  if constexpr (!SP::kScaled) {
+    if (L.block_threads == 0 && split_directions(LS, g.Vh, std::max(L.nrhs, L.rule_nrhs), sizeof(T) == 8)) {
+      constexpr int S = 32 / (LS / 2);
+      constexpr size_t smem = split_smem(LS, sizeof(T), POST, EX);
+      auto k = hop_split_kernel<SP, LS, PRE, POST, LOC, G5, NORM, min_blocks<T>(), EX>;
+      static std::atomic<bool> attr{false};
+      cudaError_t e = smem_limit_once(k, smem, attr);
+      if (e != cudaSuccess) return e;
+      k<<<dim3((g.Vh + S - 1) / S, 1, L.nrhs), 128, smem, st>>>(g, a);
+      return cudaGetLastError();
+    }
   }
   const int nt = L.block_threads ? L.block_threads : tile_threads(LS, g.Vh, L.nrhs, sizeof(T) == 8);
   const int S = nt / (LS / 2);
@@ -1040,10 +1267,10 @@ cudaError_t run_local(const Geom& g, const LocalLaunch& L, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// F<LS>::call(...) for the compiled Ls.
-#define DWF_LS_CASE(LS, CALL)                                      \
-  case LS:                                                         \
-    if constexpr (tuned_ls(LS, SP::kScaled)) return CALL(LS);      \
+// CALL(Ls) for the compiled Ls of the translation unit's group.
+#define DWF_LS_CASE(LS, CALL)                                 \
+  case LS:                                                    \
+    if constexpr (ls_group(LS) == GROUP && tuned_ls(LS, SP::kScaled)) return CALL(LS); \
     break;
 #define DWF_TUNED_LS(Ls, CALL)                                                              \
   switch (Ls) {                                                                             \
@@ -1053,7 +1280,7 @@ cudaError_t run_local(const Geom& g, const LocalLaunch& L, cudaStream_t st) {
   }                                                                                         \
   return cudaErrorNotSupported;
 
-template <class SP>
+template <class SP, int GROUP>
 cudaError_t dispatch(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   if (L.chain == nullptr || L.nbr == nullptr) return cudaErrorNotSupported;
 #define DWF_CALL(LS) dispatch_ls<SP, LS>(g, L, st)
@@ -1073,8 +1300,8 @@ cudaError_t dispatch_local_ls(const Geom& g, const LocalLaunch& L, cudaStream_t 
   return cudaErrorNotSupported;
 }
 
-template <class SP>
-cudaError_t dispatch_local(const Geom& g, const LocalLaunch& L, cudaStream_t st) {
+template <class SP, int GROUP>
+cudaError_t dispatch(const Geom& g, const LocalLaunch& L, cudaStream_t st) {
   if (L.chain == nullptr || L.red != nullptr) return cudaErrorNotSupported;
 #define DWF_CALL(LS) dispatch_local_ls<SP, LS>(g, L, st)
   DWF_TUNED_LS(g.Ls, DWF_CALL)
@@ -1160,24 +1387,11 @@ cudaError_t run_rupdate(const Geom& g, const RUpdateLaunch& L, cudaStream_t st) 
   return cudaGetLastError();
 }
 
-template <class SP>
-cudaError_t dispatch_rupdate(const Geom& g, const RUpdateLaunch& L, cudaStream_t st) {
+template <class SP, int GROUP>
+cudaError_t dispatch(const Geom& g, const RUpdateLaunch& L, cudaStream_t st) {
 #define DWF_CALL(LS) run_rupdate<SP, LS>(g, L, st)
   DWF_TUNED_LS(g.Ls, DWF_CALL)
 #undef DWF_CALL
 }
 }  // namespace hop2
 }  // namespace dwf
-
-#define DWF_HOP2_INSTANTIATE(NAME, SP)                                                    \
-  namespace dwf {                                                                        \
-  cudaError_t NAME(const Geom& g, const HopLaunch& L, cudaStream_t st) {                 \
-    return hop2::dispatch<SP>(g, L, st);                                                 \
-  }                                                                                      \
-  cudaError_t NAME##_local(const Geom& g, const LocalLaunch& L, cudaStream_t st) {       \
-    return hop2::dispatch_local<SP>(g, L, st);                                           \
-  }                                                                                      \
-  cudaError_t NAME##_rupdate(const Geom& g, const RUpdateLaunch& L, cudaStream_t st) {   \
-    return hop2::dispatch_rupdate<SP>(g, L, st);                                         \
-  }                                                                                      \
-  }

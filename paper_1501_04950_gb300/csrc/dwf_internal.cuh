@@ -85,6 +85,8 @@ struct HopLaunch {
   int g5out;
   const Reduce* red;        // nullptr: no norm
   int block_threads;        // threads per CTA of the tuned kernels (0: by size)
+  int rule_nrhs;            // right-hand sides that the choice by size counts (at least nrhs): a
+                            // solve's total, so that its bits do not depend on how it is blocked
   // Tuned path (hop2::tuned_ls): 5th-dimension operators as chain programs
   // (hop2::PR_*) over the recurrence coefficient block, and the neighbour table.
   int post_prog;
@@ -111,10 +113,6 @@ struct HopLaunch {
 };
 // Tries the tuned kernel first, then the generic one (which has no extra steps).
 cudaError_t launch_hop(const Geom& g, const HopLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_f64(const Geom& g, const HopLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_f32(const Geom& g, const HopLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_f16(const Geom& g, const HopLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_bf16(const Geom& g, const HopLaunch& a, cudaStream_t s);
 int hop_grid_blocks(const Geom& g, int prec);  // blocks of the generic kernel
 
 // ---- site-local dense contraction: out = c * M (gamma5^g5in in) ---------------
@@ -134,10 +132,6 @@ struct LocalLaunch {
   const int* active;
 };
 cudaError_t launch_local(const Geom& g, const LocalLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_f64_local(const Geom& g, const LocalLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_f32_local(const Geom& g, const LocalLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_f16_local(const Geom& g, const LocalLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_bf16_local(const Geom& g, const LocalLaunch& a, cudaStream_t s);
 // Fused CG residual update of the tuned path (hop2::tuned_ls):
 // r -= a w (a = num/den, stored to a_out), |r|^2 -> red, rhat = I^-T gamma5 r.
 struct RUpdateLaunch {
@@ -157,10 +151,6 @@ struct RUpdateLaunch {
   const int* active;
 };
 cudaError_t launch_rupdate(const Geom& g, const RUpdateLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_f64_rupdate(const Geom& g, const RUpdateLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_f32_rupdate(const Geom& g, const RUpdateLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_f16_rupdate(const Geom& g, const RUpdateLaunch& a, cudaStream_t s);
-cudaError_t launch_hop2_bf16_rupdate(const Geom& g, const RUpdateLaunch& a, cudaStream_t s);
 // x += a_prev p; p = z + beta p (a_prev = *a_ptr, beta = num / den); x in xprec.
 cudaError_t launch_px_update(const Geom& g, int prec, int xprec, void* x, void* p, const void* z,
                              const double* a_ptr, const double* num, const double* den,

@@ -2107,7 +2107,8 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
       const int k = blk + r;
       const MatSet& m = *ms[k];
       void* xb = reinterpret_cast<char*>(W.x_hi) + r * f64;
-      if ((rc = make_rhs(k))) return rc;
+      // a block of one still has its right-hand side in rhs (the CG leaves it alone)
+      if (n > 1 && (rc = make_rhs(k))) return rc;
       // psi_r = I^-1 (rhs_r + 1/2 H_rb (B psi_b))
       const CoefView cm = view_of(m);
       if (cm.tuned(P64)) {

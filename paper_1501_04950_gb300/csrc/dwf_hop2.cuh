@@ -18,8 +18,8 @@
 //     Eq. mobius1 with D_w -> 1) is applied to the neighbour spinor before the
 //     projection: (B v)+(s) = d+ v+(s) + o+ v+(s-1), (B v)-(s) = d- v-(s) + o- v-(s+1).
 //     v+ of the pair below and v- of the pair above come from the registers of the
-//     neighbouring threads by shuffles where a site's threads share a warp (G a power
-//     of two), else they are loaded in addition;
+//     neighbouring threads by shuffles: a warp then takes 32 / G whole sites (FP16,
+//     24^3x48, Ls = 12: pass A 343 us, 411 with the pairs loaded in addition);
 //   * the 5th-dimension post operators (I^-1, K = B I^-1, K^T, B^T) run as
 //     O(Ls) recurrences on register-resident chains after a transpose through
 //     shared memory: every cyclic bidiagonal matrix of the construction, put in
@@ -315,18 +315,16 @@ __device__ __forceinline__ void project_half(HalfP<typename Pr<T>::V>& P, const 
   }
 }
 
-// h = P_+ - dir A P_- (in place into P), chi_k = U' h_k, acc_upper(k) += f chi_k,
-// acc_lower(pk) += f rs (i) chi_k; U' = U (dir > 0) or U^+ (dir < 0).
+// chi_k = U' h_k, acc_upper(k) += f chi_k, acc_lower(pk) += f rs (i) chi_k for the half
+// spinor h = P; U' = U (dir > 0) or U^+ (dir < 0).
 template <class SP, int MU, int DIR>
-__device__ __forceinline__ void project_mul_acc(HalfP<typename Pr<typename SP::T>::V>& P,
-                                                const HalfP<typename Pr<typename SP::T>::V>& M,
-                                                const Link<typename SP::T>& U,
-                                                typename Pr<typename SP::T>::V f,
-                                                SpinP<typename Pr<typename SP::T>::V>& acc) {
+__device__ __forceinline__ void mul_acc(const HalfP<typename Pr<typename SP::T>::V>& P,
+                                        const Link<typename SP::T>& U,
+                                        typename Pr<typename SP::T>::V f,
+                                        SpinP<typename Pr<typename SP::T>::V>& acc) {
   using T = typename SP::T;
   using A = Pr<T>;
   using V = typename A::V;
-  project_half<T, MU, DIR>(P, M);
   const V fn = A::neg(f);
   // chi_k = U' h_k; acc_upper(k) += f chi_k; acc_lower(pk) += f rs (i) chi_k
 #pragma unroll
@@ -366,92 +364,85 @@ __device__ __forceinline__ void project_mul_acc(HalfP<typename Pr<typename SP::T
   }
 }
 
-// A site's G threads are an aligned group of one warp's lanes.
+// 32 / G sites fill a warp.
 __host__ __device__ constexpr bool warp_groups(int Ls) { return 32 % (Ls / 2) == 0; }
 
 __device__ __forceinline__ float lane_of(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 __device__ __forceinline__ double lane_of(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 
+// Where a hop's neighbour spinor pair, its scale and its link come from.
+// Memory: pair m of field v, link mu of half-site hl in the parity's links.
+template <class SP>
+struct MemSrc {
+  using V = typename Pr<typename SP::T>::V;
+  const void* v;
+  size_t m, NP;
+  const void* links;
+  int hl;
+  __device__ __forceinline__ void load6(int c0, V* re, V* im) const { PairIO<SP>::load6(v, m, NP, c0, re, im); }
+  __device__ __forceinline__ V scale() const { return PairIO<SP>::scale(v, m, NP); }
+  template <int MU>
+  __device__ __forceinline__ void link(Link<typename SP::T>& U) const {
+    GaugeOf<SP>::type::load(links, hl, MU, U);
+  }
+};
+
 // acc += f (1 - dir gamma_mu) U' v'(x +- mu) for the two slices of a thread,
-// U' = U_mu(x) (dir > 0) or U_mu(x - mu)^+ (dir < 0).  With PRE_B and warp_groups(LS)
-// every thread of the warp calls it.
+// U' = U_mu(x) (dir > 0) or U_mu(x - mu)^+ (dir < 0).  With PRE_B the G threads of a site
+// are neighbouring lanes and every thread of the warp calls it.
+template <class SP, int LS, int PRE, int MU, int DIR, class Src>
+__device__ __forceinline__ void hop_from(const Src& src, bool neg, int t, const typename SP::T (&bd)[2][2],
+                                         const typename SP::T (&bo)[2][2],
+                                         SpinP<typename Pr<typename SP::T>::V>& acc) {
+  using T = typename SP::T;
+  using A = Pr<T>;
+  using V = typename A::V;
+  constexpr int HALF = LS / 2;
+  HalfP<V> P, M;
+  src.load6(0, P.re, P.im);
+  src.load6(6, M.re, M.im);
+  V f = A::dup(neg ? (T)-1 : (T)1);  // boundary sign of the hop
+  if constexpr (PRE == PRE_B) {
+    // (B v)+ needs v+(s0 - 1) = lane y of the pair below (cyclic in s),
+    // (B v)- needs v-(s1 + 1) = lane x of the pair above.
+    const int tb = t == 0 ? HALF - 1 : t - 1, ta = t + 1 == HALF ? 0 : t + 1;
+    const int base = (threadIdx.x & 31) - t;
+    T a1 = bd[0][0], a2 = bo[0][0], a3 = bd[0][1], a4 = bo[0][1];
+    T b1 = bd[1][0], b2 = bo[1][0], b3 = bd[1][1], b4 = bo[1][1];
+    if constexpr (SP::kScaled) {
+      const V sc = src.scale();
+      const T sb = lane_of(sc.y, base + tb), sa = lane_of(sc.x, base + ta);
+      a1 *= sc.x; a2 *= sb; a3 *= sc.y; a4 *= sc.x;
+      b1 *= sc.x; b2 *= sc.y; b3 *= sc.y; b4 *= sa;
+    }
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+      const T pr = lane_of(P.re[k].y, base + tb), pi = lane_of(P.im[k].y, base + tb);
+      const T mr = lane_of(M.re[k].x, base + ta), mi = lane_of(M.im[k].x, base + ta);
+      P.re[k] = A::mk(::fma(a2, pr, a1 * P.re[k].x), ::fma(a4, P.re[k].x, a3 * P.re[k].y));
+      P.im[k] = A::mk(::fma(a2, pi, a1 * P.im[k].x), ::fma(a4, P.im[k].x, a3 * P.im[k].y));
+      M.re[k] = A::mk(::fma(b2, M.re[k].y, b1 * M.re[k].x), ::fma(b4, mr, b3 * M.re[k].y));
+      M.im[k] = A::mk(::fma(b2, M.im[k].y, b1 * M.im[k].x), ::fma(b4, mi, b3 * M.im[k].y));
+    }
+  } else if constexpr (SP::kScaled) {
+    f = A::mul(f, src.scale());  // per-slice scale of the neighbour site
+  }
+  Link<T> U;
+  src.template link<MU>(U);
+  project_half<T, MU, DIR>(P, M);
+  mul_acc<SP, MU, DIR>(P, U, f, acc);
+}
+
+// The same from memory: neighbour entry nb of site h.
 template <class SP, int LS, int PRE, int MU, int DIR>
 __device__ __forceinline__ void hop_dir(int nb, int h, int t, size_t NP,
                                         const typename SP::T (&bd)[2][2],
                                         const typename SP::T (&bo)[2][2], const void* v,
                                         const void* gp, const void* gq,
                                         SpinP<typename Pr<typename SP::T>::V>& acc) {
-  using T = typename SP::T;
-  using A = Pr<T>;
-  using V = typename A::V;
-  using IO = PairIO<SP>;
-  using GP = typename GaugeOf<SP>::type;
-  constexpr int HALF = LS / 2;
   const int hn = nb & 0x7fffffff;
-  const size_t m = (size_t)hn * HALF + t;
-  HalfP<V> P, M;
-  IO::load6(v, m, NP, 0, P.re, P.im);
-  IO::load6(v, m, NP, 6, M.re, M.im);
-  V f = A::dup(nb < 0 ? (T)-1 : (T)1);  // boundary sign of the hop
-  if constexpr (PRE == PRE_B) {
-    // (B v)+ needs v+(s0 - 1) = lane y of the pair below (cyclic in s),
-    // (B v)- needs v-(s1 + 1) = lane x of the pair above.
-    const int tb = t == 0 ? HALF - 1 : t - 1, ta = t + 1 == HALF ? 0 : t + 1;
-    T a1 = bd[0][0], a2 = bo[0][0], a3 = bd[0][1], a4 = bo[0][1];
-    T b1 = bd[1][0], b2 = bo[1][0], b3 = bd[1][1], b4 = bo[1][1];
-    T pr[6], pi[6], mr[6], mi[6];  // v+ of the slice below, v- of the slice above
-    V sc = A::dup((T)1);
-    T sb = 1, sa = 1;
-    if constexpr (warp_groups(LS)) {
-      const int base = (threadIdx.x & 31) - t;
-#pragma unroll
-      for (int k = 0; k < 6; k++) {
-        pr[k] = lane_of(P.re[k].y, base + tb);
-        pi[k] = lane_of(P.im[k].y, base + tb);
-        mr[k] = lane_of(M.re[k].x, base + ta);
-        mi[k] = lane_of(M.im[k].x, base + ta);
-      }
-      if constexpr (SP::kScaled) {
-        sc = IO::scale(v, m, NP);
-        sb = lane_of(sc.y, base + tb);
-        sa = lane_of(sc.x, base + ta);
-      }
-    } else {
-      const size_t mp = (size_t)hn * HALF + tb, mn = (size_t)hn * HALF + ta;
-      HalfP<V> Pb, Ma;
-      IO::load6(v, mp, NP, 0, Pb.re, Pb.im);
-      IO::load6(v, mn, NP, 6, Ma.re, Ma.im);
-#pragma unroll
-      for (int k = 0; k < 6; k++) {
-        pr[k] = Pb.re[k].y;
-        pi[k] = Pb.im[k].y;
-        mr[k] = Ma.re[k].x;
-        mi[k] = Ma.im[k].x;
-      }
-      if constexpr (SP::kScaled) {
-        sc = IO::scale(v, m, NP);
-        sb = IO::scale(v, mp, NP).y;
-        sa = IO::scale(v, mn, NP).x;
-      }
-    }
-    if constexpr (SP::kScaled) {
-      a1 *= sc.x; a2 *= sb; a3 *= sc.y; a4 *= sc.x;
-      b1 *= sc.x; b2 *= sc.y; b3 *= sc.y; b4 *= sa;
-    }
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-      P.re[k] = A::mk(::fma(a2, pr[k], a1 * P.re[k].x), ::fma(a4, P.re[k].x, a3 * P.re[k].y));
-      P.im[k] = A::mk(::fma(a2, pi[k], a1 * P.im[k].x), ::fma(a4, P.im[k].x, a3 * P.im[k].y));
-      M.re[k] = A::mk(::fma(b2, M.re[k].y, b1 * M.re[k].x), ::fma(b4, mr[k], b3 * M.re[k].y));
-      M.im[k] = A::mk(::fma(b2, M.im[k].y, b1 * M.im[k].x), ::fma(b4, mi[k], b3 * M.im[k].y));
-    }
-  } else if constexpr (SP::kScaled) {
-    f = A::mul(f, IO::scale(v, m, NP));  // per-slice scale of the neighbour site
-  }
-  Link<T> U;
-  if (DIR > 0) GP::load(gp, h, MU, U);
-  else GP::load(gq, hn, MU, U);
-  project_mul_acc<SP, MU, DIR>(P, M, U, f, acc);
+  const MemSrc<SP> src{v, (size_t)hn * (LS / 2) + t, NP, DIR > 0 ? gp : gq, DIR > 0 ? h : hn};
+  hop_from<SP, LS, PRE, MU, DIR>(src, nb < 0, t, bd, bo, acc);
 }
 
 // One step's coefficients (4-vector) of a sweep.
@@ -761,6 +752,13 @@ __device__ __forceinline__ void epilogue_g(const Args<typename SP::T>& a, const 
   }
 }
 
+// Sites per CTA of nth threads: 32 / G per warp where a site's threads exchange registers,
+// else as many as the threads have room for.
+template <int LS, int PRE>
+__host__ __device__ constexpr int cta_sites(int nth) {
+  return PRE == PRE_B ? nth / 32 * (32 / (LS / 2)) : nth / (LS / 2);
+}
+
 // out = c_hop G post(H v') + loc(w), two 5th-dimension slices per thread.
 template <class SP, int LS, int PRE, int POST, int LOC, bool G5, bool NORM, int MINB, int EX = EX_NONE>
 __global__ void __launch_bounds__(128, MINB) hop_kernel(const Geom g, const Args<typename SP::T> a) {
@@ -770,10 +768,13 @@ __global__ void __launch_bounds__(128, MINB) hop_kernel(const Geom g, const Args
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* coef = reinterpret_cast<T*>(smem_raw);
   T* sbuf = coef + prog_coefs(LS, POST) + (EX == EX_HAT ? prog_coefs(LS, PR_ITINV) : 0);
+  constexpr bool BYWARP = PRE == PRE_B;  // a site's threads in one warp
   const int tid = threadIdx.x, nth = blockDim.x;
-  const int S = nth / G, j = tid / G, t = tid - j * G;
+  const int S = cta_sites<LS, PRE>(nth);
+  const int first = BYWARP ? tid >> 5 : 0, lane = BYWARP ? tid & 31 : tid;
+  const int jl = lane / G, t = lane - jl * G, j = first * (32 / G) + jl;
   const int h = blockIdx.x * S + j;
-  const bool part = warp_groups(LS) || j < S;
+  const bool part = warp_groups(LS) || (BYWARP ? jl < 32 / G : j < S);
   const bool active = part && h < g.Vh;
   const int rhs = blockIdx.z;
   if (a.active && !a.active[rhs]) return;
@@ -785,11 +786,10 @@ __global__ void __launch_bounds__(128, MINB) hop_kernel(const Geom g, const Args
   const char* vb = reinterpret_cast<const char*>(a.v) + rhs * a.stride;
   SpinP<V> acc;
   zero(acc);
-  // the shuffles of the B pre-multiplication need whole warps: threads past the last
-  // site compute it again and store nothing
-  constexpr bool WHOLE = PRE == PRE_B && warp_groups(LS);
-  if (WHOLE || active) {
-    const int hl = WHOLE ? min(h, g.Vh - 1) : h;
+  // whole warps take part in the shuffles of the B pre-multiplication: threads past the
+  // last site compute it again and store nothing
+  if (BYWARP || active) {
+    const int hl = BYWARP ? min(h, g.Vh - 1) : h;
     const int4 nb0 = __ldg(a.nbr + 2 * hl), nb1 = __ldg(a.nbr + 2 * hl + 1);
     T bd[2][2] = {{0, 0}, {0, 0}}, bo[2][2] = {{0, 0}, {0, 0}};
     if (PRE == PRE_B) {
@@ -905,7 +905,7 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
   const char* vb = reinterpret_cast<const char*>(a.v) + rhs * a.stride;
   SpinP<V> acc;
   zero(acc);
-  constexpr bool WHOLE = PRE == PRE_B && warp_groups(LS);
+  constexpr bool WHOLE = PRE == PRE_B;  // its shuffles need whole warps
   if (WHOLE || active) {
     const int hl = WHOLE ? min(h, g.Vh - 1) : h;
     const int2 nb = __ldg(reinterpret_cast<const int2*>(a.nbr) + (size_t)hl * 4 + mu);
@@ -1036,11 +1036,19 @@ __global__ void __launch_bounds__(128) local_kernel(const Geom g, void* out, con
   SpinP<V> x;
   zero(x);
   if (active) load_spin<SP>(reinterpret_cast<const char*>(in) + off, m, NP, x);
-  const V cp = A::dup(c), cm = A::dup(g5in ? -c : c);
+  if (c != (T)1) {
 #pragma unroll
-  for (int k = 0; k < 12; k++) {
-    x.re[k] = A::mul(k >= 6 ? cm : cp, x.re[k]);
-    x.im[k] = A::mul(k >= 6 ? cm : cp, x.im[k]);
+    for (int k = 0; k < 12; k++) {
+      x.re[k] = A::mul(A::dup(c), x.re[k]);
+      x.im[k] = A::mul(A::dup(c), x.im[k]);
+    }
+  }
+  if (g5in) {
+#pragma unroll
+    for (int k = 6; k < 12; k++) {
+      x.re[k] = A::neg(x.re[k]);
+      x.im[k] = A::neg(x.im[k]);
+    }
   }
   T* site = sbuf + j * site_stride(LS);
   if (j < S) put<T, LS, PROG>(site, t, x);
@@ -1207,13 +1215,14 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
     }
   }
   const int nt = L.block_threads ? L.block_threads : tile_threads(LS, g.Vh, L.nrhs, sizeof(T) == 8);
-  const int S = nt / (LS / 2);
+  const int S = cta_sites<LS, PRE>(nt);
+  const auto smem_of = [](int n) { return smem_bytes(LS, cta_sites<LS, PRE>(n), sizeof(T), POST, EX); };
   dim3 grid((g.Vh + S - 1) / S, 1, L.nrhs);
   auto k = hop_kernel<SP, LS, PRE, POST, LOC, G5, NORM, min_blocks<T>(), EX>;
   static std::atomic<bool> attr{false};
-  cudaError_t e = smem_limit_once(k, smem_bytes(LS, 128 / (LS / 2), sizeof(T), POST, EX), attr);
+  cudaError_t e = smem_limit_once(k, smem_of(128), attr);
   if (e != cudaSuccess) return e;
-  k<<<grid, nt, smem_bytes(LS, S, sizeof(T), POST, EX), st>>>(g, a);
+  k<<<grid, nt, smem_of(nt), st>>>(g, a);
   return cudaGetLastError();
 }
 

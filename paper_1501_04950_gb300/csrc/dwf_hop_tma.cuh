@@ -219,7 +219,8 @@ __device__ __forceinline__ void hop_staged(const unsigned char* sb, bool neg, in
   }
   Link<T> U;
   IO::link(sb + Stage<SP, LS>::kLinkOff, U);
-  project_mul_acc<SP, MU, DIR>(P, M, U, f, acc);
+  project_half<T, MU, DIR>(P, M);
+  mul_acc<SP, MU, DIR>(P, U, f, acc);
 }
 
 template <class SP, int LS, int PRE, int POST, int LOC, bool G5, bool NORM, int NST, int MINB>

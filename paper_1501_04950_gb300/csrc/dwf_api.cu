@@ -239,6 +239,7 @@ struct dwf_ctx {
   double* scal = nullptr;          // per-rhs scalars, kScal doubles each
   double* partial = nullptr;       // reduction partials
   unsigned int* counter = nullptr; // reduction counters
+  bin_t* bins = nullptr;           // exact sums of the CG, [slot][scal_rhs][kBins]
   int partial_stride = 0;          // blocks a reduction may have
   int counter_stride = 0;          // ticket counters per right-hand side
   int scal_rhs = 0;
@@ -407,6 +408,7 @@ int ensure_reduce(dwf_ctx* h, int nrhs) {
     cudaFree(h->scal);
     cudaFree(h->partial);
     cudaFree(h->counter);
+    cudaFree(h->bins);
     cudaFreeHost(h->pinned);
   }
   h->scal_rhs = std::max(nrhs, 1);
@@ -420,6 +422,7 @@ int ensure_reduce(dwf_ctx* h, int nrhs) {
   const size_t cbytes = sizeof(unsigned int) * (size_t)h->counter_stride * h->scal_rhs * 4;
   CUCHK(h, cudaMalloc(&h->counter, cbytes));
   CUCHK(h, cudaMemset(h->counter, 0, cbytes));
+  CUCHK(h, cudaMalloc(&h->bins, sizeof(bin_t) * kBins * h->scal_rhs * 3));
   CUCHK(h, cudaMemset(h->scal, 0, sizeof(double) * kScal * h->scal_rhs));
   CUCHK(h, cudaMallocHost(&h->pinned, sizeof(double) * (kScal * h->scal_rhs + 1)));
   return DWF_OK;
@@ -435,8 +438,21 @@ Reduce make_reduce(dwf_ctx* h, int slot, int which) {
   r.partial_stride = slots;
   r.counter_stride = h->counter_stride;
   r.result_stride = kScal;
+  r.bins = nullptr;
   return r;
 }
+
+// Bins of exact sum slot k (0..2) and the Reduce / SumIn that write and read them.
+enum { BIN_ZZ = 0, BIN_WW = 1, BIN_RR = 2 };
+bin_t* bins_of(dwf_ctx* h, int k) { return h->bins + (size_t)k * h->scal_rhs * kBins; }
+Reduce bin_reduce(dwf_ctx* h, int k) {
+  Reduce r{};
+  r.bins = bins_of(h, k);
+  return r;
+}
+SumIn bin_sum(dwf_ctx* h, int k, double* val) { return SumIn{val, bins_of(h, k), kScal}; }
+// the tree's result (or a value of the host's), as it stands in memory
+SumIn plain_sum(double* val) { return SumIn{val, nullptr, kScal}; }
 
 const void* gauge_for(dwf_ctx* h, int prec) {
   return prec == P64 ? h->gauge[0] : (prec == P32 ? h->gauge[1] : h->gauge[2]);
@@ -492,7 +508,7 @@ void set_coef(HopLaunch& L, const CoefView& cv) {
 }
 
 int apply_dbb_bp(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* p, const void* bp,
-                 void* tmp, int nrhs, const Reduce* norm, cudaStream_t s);
+                 void* tmp, int nrhs, const Reduce* norm, cudaStream_t s, bin_t* zero0 = nullptr);
 
 // out = PROG in, site-local, FP64 (B, I, K or I^-1), by the tuned kernels (cv.tuned(P64)).
 // in and out may be the same field.
@@ -572,13 +588,14 @@ int apply_dbb(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* i
 // out = D_bb p given bp = B p (the fused CG forms B p with p): pass A hops bp
 // without the B pre-multiplication, pass B as in apply_dbb.
 int apply_dbb_bp(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* p, const void* bp,
-                 void* tmp, int nrhs, const Reduce* norm, cudaStream_t s) {
+                 void* tmp, int nrhs, const Reduce* norm, cudaStream_t s, bin_t* zero0) {
   const MatSet& ms = *cv.layout;
   const int black = h->opt.rb_parity, red = 1 - black;
   const size_t st = field_bytes(h->g, prec);
   HopLaunch A = base_hop(h, prec, red, nrhs, st);
   A.out = tmp;
   A.v = bp;
+  A.zero[0] = zero0;
   A.post = cv.ptr(prec, ms.mat_off(MatSet::K));
   A.post_prog = hop2::PR_K;
   A.chain = cv.chain(prec);
@@ -621,15 +638,19 @@ int apply_hat(dwf_ctx* h, const CoefView& cv, int prec, void* hat, const void* i
   return DWF_OK;
 }
 
-// out = D_bb^+ in given hat = I^-T gamma5 in.  tmp_red: red field(s).
+// out = D_bb^+ in given hat = I^-T gamma5 in.  tmp_red: red field(s).  zero0, zero1: bins
+// that pass A sets to zero.
 int apply_dbb_dag_hat(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* in,
-                      const void* hat, void* tmp_red, int nrhs, const Reduce* norm, cudaStream_t s) {
+                      const void* hat, void* tmp_red, int nrhs, const Reduce* norm, cudaStream_t s,
+                      bin_t* zero0 = nullptr, bin_t* zero1 = nullptr) {
   const MatSet& ms = *cv.layout;
   const int black = h->opt.rb_parity, red = 1 - black;
   const size_t st = field_bytes(h->g, prec);
   HopLaunch A = base_hop(h, prec, red, nrhs, st);
   A.out = tmp_red;
   A.v = hat;
+  A.zero[0] = zero0;
+  A.zero[1] = zero1;
   A.post = cv.ptr(prec, ms.mat_off(MatSet::KT));
   A.post_prog = hop2::PR_KT;
   A.chain = cv.chain(prec);
@@ -936,6 +957,10 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
   // replacements r = r_64 - D x_lo in FP32, where r_64 is the FP64 residual of the
   // last FP64 replacement and x_lo (FP32) the solution accumulated since; its
   // error is ~1e-6 |r_64|, small against |r| while |r| > tier_eta |r_64|.
+  // With B p the norms of the iteration are exact sums in bins, which the next kernel reads;
+  // pass A of D^+ clears those of |w|^2 and |r|^2, pass A of D those of |z|^2.
+  const Reduce bin_zz = bin_reduce(h, BIN_ZZ), bin_ww = bin_reduce(h, BIN_WW), bin_rr = bin_reduce(h, BIN_RR);
+  if (with_bp) CUCHK(h, cudaMemsetAsync(bins_of(h, BIN_ZZ), 0, sizeof(bin_t) * kBins * nb, s));
   const bool tiered = (prec == P16 || prec == PB16) && form == DWF_SCHUR_PRECOND && h->tier_eta > 0;
   if (with_bp) CUCHK(h, cudaMemsetAsync(W.p2, 0, fi * nb, s));
 
@@ -950,7 +975,9 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
     double* zz_old = h->scal + (cur ? S_ZZ1 : S_ZZ0);
     int r;
     if ((r = mark(first, true, 1))) return r;
-    if ((r = apply_dbb_dag_hat(h, cv, prec, W.z, W.r, W.tb, W.tr, nb, &red_zz[nxt], s))) return r;
+    if ((r = apply_dbb_dag_hat(h, cv, prec, W.z, W.r, W.tb, W.tr, nb, with_bp ? &bin_zz : &red_zz[nxt], s,
+                               with_bp ? bins_of(h, BIN_WW) : nullptr, with_bp ? bins_of(h, BIN_RR) : nullptr)))
+      return r;
     if ((r = mark(first, false, 1))) return r;
     void* pcur = W.p;
     if (with_bp) {
@@ -959,7 +986,7 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
       void* pold = cur ? W.p2 : W.p;
       pcur = cur ? W.p : W.p2;
       KLAUNCH(h, launch_pxb_update(h->g, prec, xprec, W.xlo, pold, pcur, W.bp, W.z, h->scal + S_A,
-                                   zz_new, zz_old, kScal, nb, fx, fi,
+                                   bin_sum(h, BIN_ZZ, zz_new), zz_old, kScal, nb, fx, fi,
                                    cv.ptr(prec, cv.layout->bdiag_off()),
                                    cv.ptr(prec, cv.layout->boff_off()), cv.cstride, s, h->d_active,
                                    first ? 0 : 1));
@@ -971,7 +998,7 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
     }
     if ((r = mark(first, true, 0))) return r;
     if (with_bp) {
-      if ((r = apply_dbb_bp(h, cv, prec, W.w, pcur, W.bp, W.tr, nb, &red_ww, s))) return r;
+      if ((r = apply_dbb_bp(h, cv, prec, W.w, pcur, W.bp, W.tr, nb, &bin_ww, s, bins_of(h, BIN_ZZ)))) return r;
     } else if ((r = apply_dbb(h, cv, prec, W.w, W.p, W.tr, nb, &red_ww, s))) {
       return r;
     }
@@ -986,15 +1013,16 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
     U.chain = cv.chain(prec);
     U.cstride = cv.cstride;
     U.num = zz_new;
-    U.den = h->scal + S_WW;
+    U.den = with_bp ? bin_sum(h, BIN_WW, h->scal + S_WW) : plain_sum(h->scal + S_WW);
     U.a_out = h->scal + S_A;
     U.sstride = kScal;
-    U.red = &red_rr;
+    U.red = with_bp ? &bin_rr : &red_rr;
     U.active = h->d_active;
     KLAUNCH(h, launch_rupdate(h->g, U, s));
     return DWF_OK;
   };
   auto flush_x = [&]() -> int {
+    if (with_bp) KLAUNCH(h, launch_finish_sum(bin_sum(h, BIN_RR, h->scal + S_RR), nb, s, h->d_active));
     if (fused)
       KLAUNCH(h, launch_x_update(h->g, prec, xprec, W.xlo, W.p, h->scal + S_A, kScal, nb, fx, fi, s,
                                  h->d_active));
@@ -1301,10 +1329,12 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
   // 8^3x16, Ls = 8, FP32 inner: action and gradient 88.9 -> 63.5 ms (two solves).
   const bool fused = h->fused_cg && cv.tuned(prec) && (prec == P32 || prec == P64);
   auto slot = [&](int k) { return h->scal + (k ? S_ZZ1 : S_ZZ0); };
+  // |w|^2 and |r|^2 are exact sums in bins; pass A of D clears them
+  const Reduce bin_ww = bin_reduce(h, BIN_WW), bin_rr = bin_reduce(h, BIN_RR);
   auto enqueue_fused = [&](int c, bool first, cudaStream_t q) -> int {
     const int n = 1 - c, black = h->opt.rb_parity;
     KLAUNCH(h, launch_pxb_update(h->g, prec, xprec, W.xlo, c ? W.p2 : W.p, c ? W.p : W.p2, W.bp, W.r,
-                                 h->scal + S_A, slot(c), slot(n), kScal, 1, fx, fi,
+                                 h->scal + S_A, first ? plain_sum(slot(c)) : bin_sum(h, BIN_RR, slot(c)), slot(n), kScal, 1, fx, fi,
                                  cv.ptr(prec, ms.bdiag_off()), cv.ptr(prec, ms.boff_off()), 0, q, nullptr,
                                  first ? 0 : 1));
     void* p = c ? W.p : W.p2;
@@ -1314,6 +1344,8 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
     L.v = W.bp;
     L.post_prog = hop2::PR_K;
     L.post = cv.ptr(prec, ms.mat_off(MatSet::K));
+    L.zero[0] = bins_of(h, BIN_WW);
+    L.zero[1] = bins_of(h, BIN_RR);
     KLAUNCH(h, launch_hop(h->g, L, q));
     HopLaunch B = base_hop(h, prec, black, 1, fi);
     B.chain = cv.chain(prec);
@@ -1324,11 +1356,12 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
     B.loc = LOC_ID;
     B.c_hop = -0.25;
     B.c_loc = 1.0;
-    B.red = &red_ww;
+    B.red = &bin_ww;
     B.extra = hop2::EX_HAT;
     B.out2 = W.tb;
     KLAUNCH(h, launch_hop(h->g, B, q));
     L.v = W.tb;
+    L.zero[0] = L.zero[1] = nullptr;
     L.post_prog = hop2::PR_KT;
     L.post = cv.ptr(prec, ms.mat_off(MatSet::KT));
     KLAUNCH(h, launch_hop(h->g, L, q));
@@ -1336,11 +1369,11 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
     B.w = W.w;
     B.post_prog = hop2::PR_BT;
     B.g5out = 1;
-    B.red = &red_rr[n];
+    B.red = &bin_rr;
     B.extra = hop2::EX_RUPD;
     B.out2 = W.r;
     B.num = slot(c);
-    B.den = h->scal + S_WW;
+    B.den = bin_sum(h, BIN_WW, h->scal + S_WW);
     B.a_out = h->scal + S_A;
     B.sstride = kScal;
     KLAUNCH(h, launch_hop(h->g, B, q));
@@ -1352,6 +1385,7 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
     int c = 0, e;
     for (int k = 0; k < n; k++, c = 1 - c)
       if ((e = enqueue_fused(c, k == 0, q))) return e;
+    KLAUNCH(h, launch_finish_sum(bin_sum(h, BIN_RR, slot(c)), 1, q, nullptr));
     KLAUNCH(h, launch_x_update(h->g, prec, xprec, W.xlo, c ? W.p2 : W.p, h->scal + S_A, kScal, 1, fx, fi, q,
                                nullptr));
     return DWF_OK;
@@ -1558,7 +1592,7 @@ int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_ou
     if (h->env_tma) tiles = {0};  // the staged variant has one tile
     else if (h->env_tile < 0 && (prec == P16 || prec == PB16 ||
                                  !hop2::split_directions(Ls, h->g.Vh, nrhs, prec == P64)))
-      tiles = {128, 64, 32};  // all of the same bits
+      tiles = {128, 64};  // of the same bits
   }
   double best = 1e300;
   int best_nb = ok.front(), best_tma = tmas.front(), best_tile = 0;
@@ -1770,6 +1804,7 @@ int dwf_destroy(dwf_handle h) {
     cudaFree(h->scal);
     cudaFree(h->partial);
     cudaFree(h->counter);
+    cudaFree(h->bins);
     cudaFreeHost(h->pinned);
   }
   delete h;

@@ -293,6 +293,17 @@ __global__ void extract_z1_kernel(const Geom g, double* prop, const void* p0, co
 // ---- BLAS-1 -------------------------------------------------------------------
 // One thread per slice pair m (two 5D sites), vector loads of the pair layout.
 
+// *num / *den, divided by one warp of the CTA (see sum_in); every thread calls it.
+__device__ __forceinline__ double quotient(const double* num, const double* den) {
+  __shared__ double q;
+  if (threadIdx.x < 32) {
+    const double v = *num / *den;
+    if (threadIdx.x == 0) q = v;
+  }
+  __syncthreads();
+  return q;
+}
+
 template <class SPX, class SP>
 __global__ void __launch_bounds__(kBlasThreads) xr_update_kernel(
     const Geom g, void* x, void* r, const void* p, const void* w, const double* num,
@@ -302,7 +313,7 @@ __global__ void __launch_bounds__(kBlasThreads) xr_update_kernel(
   const int rhs = blockIdx.y;
   if (active && !active[rhs]) return;
   const size_t off = rhs * stride, offx = rhs * stride_x;
-  const double ad = num[rhs * sstride] / den[rhs * sstride];
+  const double ad = quotient(num + (size_t)rhs * sstride, den + (size_t)rhs * sstride);
   const T a = (T)ad;
   const TX ax = (TX)ad;
   const int NP = g.N5 >> 1;
@@ -336,7 +347,7 @@ __global__ void __launch_bounds__(kBlasThreads) p_update_kernel(
   const int rhs = blockIdx.y;
   if (active && !active[rhs]) return;
   const size_t off = rhs * stride;
-  const T beta = (T)(num[rhs * sstride] / den[rhs * sstride]);
+  const T beta = (T)quotient(num + (size_t)rhs * sstride, den + (size_t)rhs * sstride);
   const int NP = g.N5 >> 1;
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < NP; m += gridDim.x * blockDim.x) {
     Spinor<T> pv[2], zv[2];
@@ -362,7 +373,7 @@ __global__ void __launch_bounds__(kBlasThreads) px_update_kernel(
   if (active && !active[rhs]) return;
   const size_t off = rhs * stride, offx = rhs * stride_x;
   const TX a = (TX)a_ptr[(size_t)rhs * sstride];
-  const T beta = do_p ? (T)(num[(size_t)rhs * sstride] / den[(size_t)rhs * sstride]) : (T)0;
+  const T beta = do_p ? (T)quotient(num + (size_t)rhs * sstride, den + (size_t)rhs * sstride) : (T)0;
   const int NP = g.N5 >> 1;
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < NP; m += gridDim.x * blockDim.x) {
     Spinor<T> pv[2];
@@ -392,22 +403,15 @@ __global__ void __launch_bounds__(kBlasThreads) px_update_kernel(
 // slice pair m of site h, t = m mod (Ls/2), plus bp = B p_new: B is cyclic
 // bidiagonal per chirality (Eq. mobius1 with D_w -> 1),
 //   (B v)+(s) = d+(s) v+(s) + o+(s) v+(s-1),  (B v)-(s) = d-(s) v-(s) + o-(s) v-(s+1),
-// so v+ of slice 2t-1 (pair below) and v- of slice 2t+2 (pair above) are formed
-// from z and p of those pairs as well.  Used by the CG on the tuned path, whose
-// D_bb pass A then hops B p directly.  p_old and p_new are different buffers
-// (neighbouring pairs of p_old are read while p_new is written).
-// FP32 fields: two CTAs per SM (128 registers, 48 bytes spilled) so that one
-// CTA's loads overlap the other's stores; the other combinations would spill
-// hundreds of bytes at that cap and keep one CTA per SM.
+// so v+ of slice 2t-1 (pair below) and v- of slice 2t+2 (pair above) enter as well: they are
+// in the registers of the neighbouring lanes (a warp takes the pairs of 32 / (Ls/2) whole
+// sites).  Used by the CG on the tuned path, whose D_bb pass A then hops B p directly.
+// HBM bound: 6 half-field passes.  Forming the neighbours' slices again from loads of
+// their own (48 words a thread) kept 16^3x32, Ls = 16, FP32 at 99 us, against 90 (cold, under ncu).
 template <class SPX, class SP>
-constexpr int pxb_min_blocks() {
-  return SP::kPrec == P32 && SPX::kPrec == P32 ? 2 : 1;
-}
-
-template <class SPX, class SP>
-__global__ void __launch_bounds__(kBlasThreads, (pxb_min_blocks<SPX, SP>())) pxb_update_kernel(
+__global__ void __launch_bounds__(kBlasThreads, 2) pxb_update_kernel(
     const Geom g, void* x, const void* p, void* pnew, void* bp, const void* z, const double* a_ptr,
-    const double* num, const double* den, int sstride, size_t stride_x, size_t stride,
+    const SumIn num, const double* den, int sstride, size_t stride_x, size_t stride,
     const typename SP::T* bdiag, const typename SP::T* boff, size_t cstride, const int* active,
     int do_x) {
   using T = typename SP::T;
@@ -415,28 +419,42 @@ __global__ void __launch_bounds__(kBlasThreads, (pxb_min_blocks<SPX, SP>())) pxb
   const int rhs = blockIdx.y;
   if (active && !active[rhs]) return;
   const size_t off = rhs * stride, offx = rhs * stride_x;
-  const TX a = do_x ? (TX)a_ptr[(size_t)rhs * sstride] : (TX)0;
-  const T beta = (T)(num[(size_t)rhs * sstride] / den[(size_t)rhs * sstride]);
+  __shared__ T beta_sh;
+  bool have_beta = false;
+  T beta = 0;
   const int NP = g.N5 >> 1, half = g.Ls >> 1;
+  const int per = 32 / half * half;  // pairs of a warp
+  const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const T* bd = bdiag + (size_t)rhs * cstride;
   const T* bo = boff + (size_t)rhs * cstride;
   const char* pb = reinterpret_cast<const char*>(p) + off;
   const char* zb = reinterpret_cast<const char*>(z) + off;
-  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < NP; m += gridDim.x * blockDim.x) {
-    const int t = m % half, base = m - t;
-    const int mp = base + (t == 0 ? half - 1 : t - 1), mn = base + (t + 1 == half ? 0 : t + 1);
-    // the slice below the pair (lane 1 of pair mp) enters through its v+ half,
-    // the slice above (lane 0 of pair mn) through its v- half; 16-bit storage
-    // loads all 12 components of those slices (the scale of their stored p_new)
-    const int n_below = 2 * mp + 1, n_above = 2 * mn;
-    Spinor<T> pv[2], zv[2], pl, zl, pu, zu;
+  // whole blocks go round the loop, for the barrier and the shuffles
+  for (int m0 = blockIdx.x * warps * per; m0 < NP; m0 += gridDim.x * warps * per) {
+    const int mt = m0 + (threadIdx.x >> 5) * per + lane;
+    const bool mine = lane < per && mt < NP;
+    const int m = mine ? mt : NP - 1;
+    const int t = m % half;
+    const int below = t == 0 ? lane + half - 1 : lane - 1, above = t + 1 == half ? lane - t : lane + 1;
+    Spinor<T> pv[2], q[2];
     SP::load_pair(pb, m, NP, pv[0], pv[1]);
-    SP::load_pair(zb, m, NP, zv[0], zv[1]);
-    SP::load_chir(pb, n_below, g.N5, 0, pl);
-    SP::load_chir(zb, n_below, g.N5, 0, zl);
-    SP::load_chir(pb, n_above, g.N5, 1, pu);
-    SP::load_chir(zb, n_above, g.N5, 1, zu);
-    if (do_x) {
+    SP::load_pair(zb, m, NP, q[0], q[1]);
+    if (!have_beta) {  // by one warp, while the loads are on their way
+      if (threadIdx.x < 32) {
+        const double b = sum_in(num, rhs, blockIdx.x == 0) / den[(size_t)rhs * sstride];
+        if (threadIdx.x == 0) beta_sh = (T)b;
+      }
+      __syncthreads();
+      beta = beta_sh;
+      have_beta = true;
+    }
+#pragma unroll
+    for (int l = 0; l < 2; l++)
+#pragma unroll
+      for (int k = 0; k < 12; k++)
+        q[l].c[k] = cmake(fma(beta, pv[l].c[k].re, q[l].c[k].re), fma(beta, pv[l].c[k].im, q[l].c[k].im));
+    if (do_x && mine) {
+      const TX a = (TX)a_ptr[(size_t)rhs * sstride];
       Spinor<TX> xv[2];
       SPX::load_pair(reinterpret_cast<const char*>(x) + offx, m, NP, xv[0], xv[1]);
 #pragma unroll
@@ -446,32 +464,11 @@ __global__ void __launch_bounds__(kBlasThreads, (pxb_min_blocks<SPX, SP>())) pxb
           xv[l].c[k] = cmake(fma(a, (TX)pv[l].c[k].re, xv[l].c[k].re), fma(a, (TX)pv[l].c[k].im, xv[l].c[k].im));
       SPX::store_pair(reinterpret_cast<char*>(x) + offx, m, NP, xv[0], xv[1]);
     }
-    // p_new on the pair, v+ of the slice below and v- of the slice above
-    Spinor<T> q[2], qb, qa;
-#pragma unroll
-    for (int k = 0; k < 12; k++) {
-#pragma unroll
-      for (int l = 0; l < 2; l++)
-        q[l].c[k] = cmake(fma(beta, pv[l].c[k].re, zv[l].c[k].re), fma(beta, pv[l].c[k].im, zv[l].c[k].im));
-      if (SP::kScaled || k < 6)
-        qb.c[k] = cmake(fma(beta, pl.c[k].re, zl.c[k].re), fma(beta, pl.c[k].im, zl.c[k].im));
-      if (SP::kScaled || k >= 6)
-        qa.c[k] = cmake(fma(beta, pu.c[k].re, zu.c[k].re), fma(beta, pu.c[k].im, zu.c[k].im));
-    }
-    SP::store_pair(reinterpret_cast<char*>(pnew) + off, m, NP, q[0], q[1]);
+    if (mine) SP::store_pair(reinterpret_cast<char*>(pnew) + off, m, NP, q[0], q[1]);
     if constexpr (SP::kScaled) {
-      // 16-bit storage: B acts on the stored (rounded) p_new, as pass B's local
-      // term sees it; the slices below and above round with their own scales
+      // 16-bit storage: B acts on the stored (rounded) p_new, as pass B's local term sees it
       SP::quantize(q[0]);
       SP::quantize(q[1]);
-      SP::quantize(qb);
-      SP::quantize(qa);
-    }
-    cplx<T> below[6], above[6];
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-      below[k] = qb.c[k];
-      above[k] = qa.c[6 + k];
     }
     const int s0 = 2 * t;
     const T dp0 = bd[s0], dp1 = bd[s0 + 1], op0 = bo[s0], op1 = bo[s0 + 1];
@@ -479,14 +476,17 @@ __global__ void __launch_bounds__(kBlasThreads, (pxb_min_blocks<SPX, SP>())) pxb
     Spinor<T> b[2];
 #pragma unroll
     for (int k = 0; k < 6; k++) {
-      b[0].c[k] = cmake(fma(op0, below[k].re, dp0 * q[0].c[k].re), fma(op0, below[k].im, dp0 * q[0].c[k].im));
+      const cplx<T> lo = cmake(__shfl_sync(0xffffffffu, q[1].c[k].re, below),
+                               __shfl_sync(0xffffffffu, q[1].c[k].im, below));
+      const cplx<T> up = cmake(__shfl_sync(0xffffffffu, q[0].c[6 + k].re, above),
+                               __shfl_sync(0xffffffffu, q[0].c[6 + k].im, above));
+      b[0].c[k] = cmake(fma(op0, lo.re, dp0 * q[0].c[k].re), fma(op0, lo.im, dp0 * q[0].c[k].im));
       b[1].c[k] = cmake(fma(op1, q[0].c[k].re, dp1 * q[1].c[k].re), fma(op1, q[0].c[k].im, dp1 * q[1].c[k].im));
       b[0].c[6 + k] = cmake(fma(om0, q[1].c[6 + k].re, dm0 * q[0].c[6 + k].re),
                             fma(om0, q[1].c[6 + k].im, dm0 * q[0].c[6 + k].im));
-      b[1].c[6 + k] = cmake(fma(om1, above[k].re, dm1 * q[1].c[6 + k].re),
-                            fma(om1, above[k].im, dm1 * q[1].c[6 + k].im));
+      b[1].c[6 + k] = cmake(fma(om1, up.re, dm1 * q[1].c[6 + k].re), fma(om1, up.im, dm1 * q[1].c[6 + k].im));
     }
-    SP::store_pair(reinterpret_cast<char*>(bp) + off, m, NP, b[0], b[1]);
+    if (mine) SP::store_pair(reinterpret_cast<char*>(bp) + off, m, NP, b[0], b[1]);
   }
 }
 
@@ -634,6 +634,12 @@ __global__ void __launch_bounds__(kBlasThreads) dot_re64_kernel(const Geom g, co
         acc = fma(x[l].c[k].re, y[l].c[k].re, fma(x[l].c[k].im, y[l].c[k].im, acc));
   }
   block_sum_to(acc, red, rhs, gridDim.x, blockIdx.x);
+}
+
+__global__ void finish_sum_kernel(const SumIn in, const int* active) {
+  const int rhs = blockIdx.x;
+  if (active && !active[rhs]) return;
+  sum_in(in, rhs, true);
 }
 
 // Launch shape of n elements, one per thread up to 16 CTAs of kBlasThreads per SM.  Below
@@ -818,11 +824,14 @@ cudaError_t launch_x_update(const Geom& g, int prec, int xprec, void* x, const v
 }
 
 cudaError_t launch_pxb_update(const Geom& g, int prec, int xprec, void* x, const void* p,
-                              void* pnew, void* bp, const void* z, const double* a_ptr, const double* num,
+                              void* pnew, void* bp, const void* z, const double* a_ptr, const SumIn& num,
                               const double* den, int sstride, int nrhs, size_t sx, size_t sp,
                               const void* bdiag, const void* boff, size_t cstride, cudaStream_t s,
                               const int* active, int do_x) {
-  const Shape sh = elementwise((size_t)g.N5 / 2);
+  // threads for whole sites per warp
+  const int half = g.Ls / 2, per = 32 / half * half;
+  if (half > 16) return cudaErrorInvalidValue;
+  const Shape sh = elementwise(((size_t)g.N5 / 2 + per - 1) / per * 32);
   const dim3 grid(sh.blocks, nrhs);
   if (prec == P32 && xprec == P32) {
     pxb_update_kernel<Store32, Store32><<<grid, sh.threads, 0, s>>>(
@@ -847,6 +856,11 @@ cudaError_t launch_pxb_update(const Geom& g, int prec, int xprec, void* x, const
   } else {
     return cudaErrorInvalidValue;
   }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_finish_sum(const SumIn& in, int nrhs, cudaStream_t s, const int* active) {
+  finish_sum_kernel<<<nrhs, 32, 0, s>>>(in, active);
   return cudaGetLastError();
 }
 

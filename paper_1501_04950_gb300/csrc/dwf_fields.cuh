@@ -324,20 +324,66 @@ __device__ __forceinline__ double warp_sum_of(const double* part, int n, int lan
   return warp_sum(acc);
 }
 
-__device__ __forceinline__ void block_sum_to(double v, const Reduce& red, int rhs, int nblocks,
-                                             int bid) {
-  __shared__ double wsum[32];
-  const int nth = blockDim.x * blockDim.y;
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
-  const int nw = (nth + 31) >> 5;
-  v = warp_sum(v, lane, nth - (warp << 5));
-  if (nw > 1) {
-    if (lane == 0) wsum[warp] = v;
-    __syncthreads();
-    if (warp > 0) return;
-    v = warp_sum(lane < nw ? wsum[lane] : 0.0);
+// ---------------------------------------------------------------------------
+// Bins: an exact, order-independent sum of non-negative doubles as fixed-point words.  A
+// summand m 2^(E - 1074) adds the 32-bit pieces of its shifted significand to the words
+// E / 32 .. E / 32 + 2, so the sum is the words' value, sum_k word_k 2^(32 k - 1074), whatever
+// the order, and 2^32 summands fit.  Word kBinFlag marks a summand that is not finite.
+// The adds return nothing and need no fence: the kernel that reads the words comes after
+// this one in its stream.  In the CG this takes the place of the tree above, whose fence and
+// ticket keep a CTA's registers for about 2 us after its last store (8^3x16, Ls = 8: pass B
+// 15.1 us with the tree, 8.8 with the bins and the integer warp sums below).
+// ---------------------------------------------------------------------------
+constexpr int kBinFlag = 71;
+__device__ __forceinline__ void bins_add(bin_t* bins, bin_t m, int E) {  // m 2^(E - 1074)
+  const int k = E >> 5, sh = E & 31;
+  const bin_t lo = m << sh, hi = sh ? m >> (64 - sh) : 0ull;
+  if (lo & 0xffffffffull) atomicAdd(bins + k, lo & 0xffffffffull);
+  if (lo >> 32) atomicAdd(bins + k + 1, lo >> 32);
+  if (hi) atomicAdd(bins + k + 2, hi);
+}
+__device__ __forceinline__ void bins_add(bin_t* bins, double v) {
+  const bin_t bits = (bin_t)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  const int e = (int)(bits >> 52);
+  if (e == 0x7ff) {
+    atomicOr(bins + kBinFlag, 1ull);
+    return;
   }
+  bins_add(bins, (bits & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull), e ? e - 1 : 0);
+}
+// The value of the words, to every lane of a full warp.
+__device__ __forceinline__ double bins_value(const bin_t* bins) {
+  const int lane = (threadIdx.y * blockDim.x + threadIdx.x) & 31;
+  double acc = 0.0;
+  bool bad = false;
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    const int k = lane + 32 * i;
+    if (k < kBins) {
+      const bin_t w = __ldcg(bins + k);
+      if (k == kBinFlag) bad = w != 0;
+      else if (w) acc += scalbn((double)w, 32 * k - 1074);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return __any_sync(0xffffffffu, bad) ? __longlong_as_double(0x7ff8000000000000ll) : acc;
+}
+// num[rhs] / den and the like, once per CTA: FP64 arithmetic runs at 64 cycles a warp
+// instruction, and a division in every warp of an update of 16^3x32, Ls = 16 was 20 us of
+// each sub-partition's FP64 pipe.  One warp calls it; the first block of a right-hand side
+// (first) stores the sum that it read from bins.
+__device__ __forceinline__ double sum_in(const SumIn& in, int rhs, bool first) {
+  double* val = in.val + (size_t)rhs * in.stride;
+  if (!in.bins) return *val;
+  const double v = bins_value(in.bins + (size_t)rhs * kBins);
+  if (first && ((threadIdx.y * blockDim.x + threadIdx.x) & 31) == 0) *val = v;
+  return v;
+}
+
+// The block's sum v (lane 0 of its first warp, all of whose lanes call) into the tree.
+__device__ __forceinline__ void publish_sum(double v, const Reduce& red, int rhs, int nblocks, int bid,
+                                            int lane) {
   double* part = red.partial + (size_t)rhs * red.partial_stride;
   unsigned int* count = red.counter + (size_t)rhs * red.counter_stride;
   const int ngroups = reduce_groups(nblocks), group = bid / kReduceGroup;
@@ -364,6 +410,84 @@ __device__ __forceinline__ void block_sum_to(double v, const Reduce& red, int rh
     if (lane == 0) count[0] = 0u;
   }
   if (lane == 0) red.result[(size_t)rhs * red.result_stride] = acc;
+}
+
+// The sum of two non-negative floats per lane over a full warp as t 2^(e - 182), in integer
+// arithmetic (the FP64 pipe would need 8 instructions of 64 cycles a warp): the
+// significands are aligned to the warp's largest exponent with 32 bits below it, so
+// that summands within 2^32 of the largest are exact and the others are cut at 2^-56 of it.
+struct FixedSum {
+  bin_t t;
+  int e;  // 255: a summand is not finite
+};
+__device__ __forceinline__ FixedSum warp_fixed_sum(float x, float y) {
+  const unsigned bx = __float_as_uint(x), by = __float_as_uint(y);
+  const int ex = max((int)((bx >> 23) & 255u), 1), ey = max((int)((by >> 23) & 255u), 1);
+  const int e = __reduce_max_sync(0xffffffffu, max(ex, ey));
+  const bin_t mx = (bx & 0x7fffffu) | (bx & 0x7f800000u ? 0x800000u : 0u);
+  const bin_t my = (by & 0x7fffffu) | (by & 0x7f800000u ? 0x800000u : 0u);
+  const bin_t s = ((mx << 32) >> min(e - ex, 63)) + ((my << 32) >> min(e - ey, 63));  // < 2^57
+  const unsigned m19 = 0x7ffffu;
+  const bin_t a = __reduce_add_sync(0xffffffffu, (unsigned)s & m19);
+  const bin_t b = __reduce_add_sync(0xffffffffu, (unsigned)(s >> 19) & m19);
+  const bin_t c = __reduce_add_sync(0xffffffffu, (unsigned)(s >> 38));
+  return FixedSum{a + (b << 19) + (c << 38), e};
+}
+
+// block_sum_to of the squares of FP32 slice pairs, r = (slice 0, slice 1): full warps, at
+// most 4 of them.
+__device__ __forceinline__ void block_sum_pair(float2 r, const Reduce& red, int rhs, int nblocks, int bid) {
+  __shared__ FixedSum wsum[4];
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x, lane = tid & 31;
+  const int nw = (blockDim.x * blockDim.y) >> 5;
+  FixedSum f = warp_fixed_sum(r.x, r.y);
+  if (nw > 1) {
+    if (lane == 0) wsum[tid >> 5] = f;
+    __syncthreads();
+    if (tid >= 32) return;
+    int e = f.e;
+    for (int w = 1; w < nw; w++) e = max(e, wsum[w].e);
+    f.t >>= min(e - f.e, 63);
+    for (int w = 1; w < nw; w++) f.t += wsum[w].t >> min(e - wsum[w].e, 63);  // < 2^64
+    f.e = e;
+  }
+  if (red.bins) {
+    bin_t* bins = red.bins + (size_t)rhs * kBins;
+    if (lane == 0) {
+      if (f.e == 255) atomicOr(bins + kBinFlag, 1ull);
+      else bins_add(bins, f.t, f.e - 182 + 1074);
+    }
+    return;
+  }
+  const double v = f.e == 255 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn((double)f.t, f.e - 182);
+  publish_sum(v, red, rhs, nblocks, bid, lane);
+}
+__device__ __forceinline__ void block_sum_pair(double2 r, const Reduce& red, int rhs, int nblocks, int bid);
+
+__device__ __forceinline__ void block_sum_to(double v, const Reduce& red, int rhs, int nblocks,
+                                             int bid) {
+  __shared__ double wsum[32];
+  const int nth = blockDim.x * blockDim.y;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
+  const int nw = (nth + 31) >> 5;
+  v = warp_sum(v, lane, nth - (warp << 5));
+  if (nw > 1) {
+    if (lane == 0) wsum[warp] = v;
+    __syncthreads();
+    if (warp > 0) return;
+    v = warp_sum(lane < nw ? wsum[lane] : 0.0);
+  }
+  if (red.bins) {
+    if (lane == 0) bins_add(red.bins + (size_t)rhs * kBins, v);
+    return;
+  }
+  publish_sum(v, red, rhs, nblocks, bid, lane);
+}
+
+
+__device__ __forceinline__ void block_sum_pair(double2 r, const Reduce& red, int rhs, int nblocks, int bid) {
+  block_sum_to(r.x + r.y, red, rhs, nblocks, bid);
 }
 
 // ---------------------------------------------------------------------------

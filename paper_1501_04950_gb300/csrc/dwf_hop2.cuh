@@ -282,14 +282,24 @@ struct Args {
   size_t cstride;       // elements between right-hand sides of bdiag, boff, chain
   const int* active;    // per right-hand side: 0 skips it (nullptr: all active)
   int* err;             // set to 1 when a bounded wait gives up (staged variant)
-  // EX_HAT: out2 = I^-T gamma5 out.  EX_RUPD: r = out2 is updated, r -= a out, a = *num / *den
+  // EX_HAT: out2 = I^-T gamma5 out.  EX_RUPD: r = out2 is updated, r -= a out, a = *num / den
   // (stored to a_out, one per right-hand side sstride apart), and out itself is not stored.
   void* out2;
   const double* num;
-  const double* den;
+  SumIn den;
   double* a_out;
   int sstride;
+  bin_t* zero[2];       // bins that the right-hand side's first block sets to zero
 };
+
+template <typename T>
+__device__ __forceinline__ void zero_bins(const Args<T>& a, int rhs, int tid, int nth) {
+  if (blockIdx.x == 0)
+#pragma unroll
+    for (int i = 0; i < 2; i++)
+      if (a.zero[i])
+        for (int k = tid; k < kBins; k += nth) a.zero[i][(size_t)rhs * kBins + k] = 0ull;
+}
 
 // h = P_+ - dir A P_- in place into P: the half spinor of (1 - DIR gamma_mu).
 template <typename T, int MU, int DIR>
@@ -613,19 +623,18 @@ __device__ __forceinline__ void get(const T* site, int t, SpinP<typename Pr<T>::
   }
 }
 
+// squares of the two slices
 template <typename V>
-__device__ __forceinline__ double sqr(const SpinP<V>& a) {
-  V r = a.re[0];
-  r.x *= r.x;
-  r.y *= r.y;
-  using A = Pr<decltype(r.x)>;
+__device__ __forceinline__ V sqr(const SpinP<V>& a) {
+  using A = Pr<decltype(a.re[0].x)>;
+  V r = A::mul(a.re[0], a.re[0]);
   r = A::fma(a.im[0], a.im[0], r);
 #pragma unroll
   for (int c = 1; c < 12; c++) {
     r = A::fma(a.re[c], a.re[c], r);
     r = A::fma(a.im[c], a.im[c], r);
   }
-  return (double)r.x + (double)r.y;
+  return r;
 }
 
 template <typename V>
@@ -651,6 +660,25 @@ __device__ __forceinline__ void add(SpinP<V>& a, const SpinP<V>& b) {
 
 template <typename T>
 constexpr int min_blocks() { return sizeof(T) == 8 ? 2 : 4; }
+
+// The step a = *num / den of EX_RUPD, computed by the first warp of a CTA at its start
+// (later barriers of the kernel make it visible).
+template <typename T>
+__device__ __forceinline__ T& rupd_scalar() {
+  __shared__ T a;
+  return a;
+}
+template <typename T>
+__device__ __forceinline__ void start_rupd(const Args<T>& a, int rhs, int tid) {
+  if (tid < 32) {
+    const bool first = blockIdx.x == 0;
+    const double ad = a.num[(size_t)rhs * a.sstride] / sum_in(a.den, rhs, first);
+    if (tid == 0) {
+      rupd_scalar<T>() = (T)ad;
+      if (first) a.a_out[(size_t)rhs * a.sstride] = ad;
+    }
+  }
+}
 
 // Steps of the CG on D_bb^+ D_bb that end a hopping pass (HopLaunch.extra).
 enum { EX_NONE = 0, EX_HAT = 1, EX_RUPD = 2 };
@@ -700,10 +728,8 @@ __device__ __forceinline__ void epilogue_g(const Args<typename SP::T>& a, const 
     }
   }
   if constexpr (EX == EX_RUPD) {
-    const double ad = a.num[(size_t)rhs * a.sstride] / a.den[(size_t)rhs * a.sstride];
-    if (blockIdx.x == 0 && tid == 0) a.a_out[(size_t)rhs * a.sstride] = ad;
     if (active) {
-      const V na = A::dup(-(T)ad);
+      const V na = A::dup(-rupd_scalar<T>());
       char* r = reinterpret_cast<char*>(a.out2) + off;
       SpinP<V> x;
       load_spin<SP>(r, m, NP, x);
@@ -719,7 +745,7 @@ __device__ __forceinline__ void epilogue_g(const Args<typename SP::T>& a, const 
   }
   if constexpr (EX == EX_HAT) {
     static_assert(!SP::kScaled && NORM, "the fused hat is for FP32 and FP64 fields");
-    const double nrm = active ? sqr(acc) : 0.0;
+    const V nrm = active ? sqr(acc) : A::dup((T)0);
 #pragma unroll
     for (int c = 6; c < 12; c++) {
       acc.re[c] = A::neg(acc.re[c]);
@@ -735,9 +761,9 @@ __device__ __forceinline__ void epilogue_g(const Args<typename SP::T>& a, const 
       get<T, LS, PR_ITINV>(site, t, acc);
       PairIO<SP>::store(reinterpret_cast<char*>(a.out2) + off, m, NP, acc);
     }
-    block_sum_to(nrm, a.red, rhs, gridDim.x, blockIdx.x);
+    block_sum_pair(nrm, a.red, rhs, gridDim.x, blockIdx.x);
   } else if (NORM) {
-    double v = 0.0;
+    V v = A::dup((T)0);
     if (active) {
       if constexpr (SP::kScaled) {
         // 16-bit storage rounds: the norm follows the stored values
@@ -748,7 +774,7 @@ __device__ __forceinline__ void epilogue_g(const Args<typename SP::T>& a, const 
         v = sqr(acc);
       }
     }
-    block_sum_to(v, a.red, rhs, gridDim.x, blockIdx.x);
+    block_sum_pair(v, a.red, rhs, gridDim.x, blockIdx.x);
   }
 }
 
@@ -781,6 +807,8 @@ __global__ void __launch_bounds__(128, MINB) hop_kernel(const Geom g, const Args
   const size_t co = (size_t)rhs * a.cstride;
   const size_t NP = (size_t)g.N5 >> 1;
   const int s0 = 2 * t;
+  zero_bins(a, rhs, tid, nth);
+  if (EX == EX_RUPD) start_rupd(a, rhs, tid);
   load_coefs<T, LS, POST>(coef, a.chain + co, tid, nth);
   if (EX == EX_HAT) load_coefs<T, LS, PR_ITINV>(coef + prog_coefs(LS, POST), a.chain + co, tid, nth);
   const char* vb = reinterpret_cast<const char*>(a.v) + rhs * a.stride;
@@ -900,6 +928,8 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
   if (a.active && !a.active[rhs]) return;
   const size_t co = (size_t)rhs * a.cstride;
   const size_t NP = (size_t)g.N5 >> 1;
+  zero_bins(a, rhs, tid, 128);
+  if (EX == EX_RUPD) start_rupd(a, rhs, tid);
   load_coefs<T, LS, POST>(coef, a.chain + co, tid, 128);
   if (EX == EX_HAT) load_coefs<T, LS, PR_ITINV>(coef + prog_coefs(LS, POST), a.chain + co, tid, 128);
   const char* vb = reinterpret_cast<const char*>(a.v) + rhs * a.stride;
@@ -953,15 +983,9 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
   const T* p = sbuf + j * SST + (rev ? G - 1 - t : t) * kPairStride + 4 * c0;
   const T f = G5 && chir == 1 ? -a.c_hop : a.c_hop;
   V re[3], im[3];
-  double nrm = 0.0;
-  T na = 0;
-  if (EX == EX_RUPD) {
-    const double ad = a.num[(size_t)rhs * a.sstride] / a.den[(size_t)rhs * a.sstride];
-    if (blockIdx.x == 0 && tid == 0) a.a_out[(size_t)rhs * a.sstride] = ad;
-    na = -(T)ad;
-  }
+  const T na = EX == EX_RUPD ? -rupd_scalar<T>() : (T)0;
+  V n2 = A::dup((T)0);
   if (active) {
-    V n2 = A::dup((T)0);
 #pragma unroll
     for (int k = 0; k < 3; k++) {
       const Coef4<T> v = coef4(p + 4 * k);
@@ -978,7 +1002,6 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
       n2 = A::fma(re[k], re[k], n2);
       n2 = A::fma(im[k], im[k], n2);
     }
-    nrm = (double)n2.x + (double)n2.y;
   }
   if (EX == EX_HAT) {
     const bool hrev = prog_reversed(PR_ITINV, 1) == (chir == 1);
@@ -1007,7 +1030,7 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
       }
     }
   }
-  if (NORM) block_sum_to(nrm, a.red, rhs, gridDim.x, blockIdx.x);
+  if (NORM) block_sum_pair(n2, a.red, rhs, gridDim.x, blockIdx.x);
 }
 
 // out = c * PROG(gamma5^g5in in), site-local, two slices per thread.
@@ -1199,6 +1222,8 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   a.den = L.den;
   a.a_out = L.a_out;
   a.sstride = L.sstride;
+  a.zero[0] = L.zero[0];
+  a.zero[1] = L.zero[1];
   if constexpr (tma_ls(LS) && POST != PR_NONE && EX == EX_NONE) {
     if (L.use_tma) return run_tma<SP, LS, PRE, POST, LOC, G5, NORM>(g, L, a, st);
   }
@@ -1325,7 +1350,7 @@ template <class SP, int LS>
 __global__ void __launch_bounds__(128) rupdate_kernel(const Geom g, void* r, void* rhat,
                                                       const void* w, size_t stride,
                                                       const typename SP::T* chain, size_t cstride,
-                                                      const double* num, const double* den,
+                                                      const double* num, const SumIn den,
                                                       double* a_out, int sstride, Reduce red,
                                                       const int* rhs_on) {
   using T = typename SP::T;
@@ -1342,19 +1367,30 @@ __global__ void __launch_bounds__(128) rupdate_kernel(const Geom g, void* r, voi
   const int rhs = blockIdx.z;
   if (rhs_on && !rhs_on[rhs]) return;
   const size_t NP = (size_t)g.N5 >> 1;
-  const double ad = num[(size_t)rhs * sstride] / den[(size_t)rhs * sstride];
-  if (blockIdx.x == 0 && tid == 0) a_out[(size_t)rhs * sstride] = ad;
-  const V na = A::dup(-(T)ad);
   load_coefs<T, LS, PR_ITINV>(coef, chain + (size_t)rhs * cstride, tid, nth);
   const size_t off = rhs * stride;
   const size_t m = (size_t)h * G + t;
   SpinP<V> x;
   zero(x);
-  double nrm = 0.0;
+  V nrm = A::dup((T)0);
+  SpinP<V> wv;
+  zero(wv);
   if (active) {
-    SpinP<V> wv;
     load_spin<SP>(reinterpret_cast<const char*>(r) + off, m, NP, x);
     load_spin<SP>(reinterpret_cast<const char*>(w) + off, m, NP, wv);
+  }
+  // a by one warp, while the loads are on their way
+  __shared__ T a_sh;
+  if (tid < 32) {
+    const double ad = num[(size_t)rhs * sstride] / sum_in(den, rhs, blockIdx.x == 0);
+    if (tid == 0) {
+      a_sh = (T)ad;
+      if (blockIdx.x == 0) a_out[(size_t)rhs * sstride] = ad;
+    }
+  }
+  __syncthreads();
+  const V na = A::dup(-a_sh);
+  if (active) {
 #pragma unroll
     for (int k = 0; k < 12; k++) {
       x.re[k] = A::fma(na, wv.re[k], x.re[k]);
@@ -1379,7 +1415,7 @@ __global__ void __launch_bounds__(128) rupdate_kernel(const Geom g, void* r, voi
     get<T, LS, PR_ITINV>(site, t, x);
     PairIO<SP>::store(reinterpret_cast<char*>(rhat) + off, m, NP, x);
   }
-  block_sum_to(nrm, red, rhs, gridDim.x, blockIdx.x);
+  block_sum_pair(nrm, red, rhs, gridDim.x, blockIdx.x);
 }
 
 template <class SP, int LS>

@@ -255,6 +255,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  zero_bins(a, rhs, tid, kTmaThreads);
   load_coefs<T, LS, POST>(coef, a.chain + co, tid, kTmaThreads);
   __syncthreads();
   SpinP<V> acc;

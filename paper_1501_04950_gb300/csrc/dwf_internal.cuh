@@ -47,6 +47,11 @@ constexpr int kReduceGroup = 128;
 __host__ __device__ constexpr int reduce_groups(int nblocks) {
   return (nblocks + kReduceGroup - 1) / kReduceGroup;
 }
+//
+// With bins set the sum goes there instead, to be read by the next kernel: see Bins in
+// dwf_fields.cuh.
+constexpr int kBins = 72;  // 64-bit words of one sum
+typedef unsigned long long bin_t;
 struct Reduce {
   double* partial;
   unsigned int* counter;
@@ -54,7 +59,16 @@ struct Reduce {
   int partial_stride;
   int counter_stride;
   int result_stride;
+  bin_t* bins;  // [right-hand side][kBins], or nullptr
 };
+// A sum of the kernel before: val[rhs * stride], or, with bins, the bins' value, which the
+// reader also stores to val.
+struct SumIn {
+  double* val;
+  const bin_t* bins;  // [right-hand side][kBins], or nullptr
+  int stride;
+};
+
 
 // ---- the generic hopping pass -------------------------------------------------
 //   acc(x,s)  = sum_mu [ (1-g_mu) U_mu(x) v'(x+mu,s) + (1+g_mu) U_mu(x-mu)^+ v'(x-mu,s) ]
@@ -107,9 +121,10 @@ struct HopLaunch {
   int extra;
   void* out2;
   const double* num;
-  const double* den;
+  SumIn den;
   double* a_out;
   int sstride;
+  bin_t* zero[2];           // tuned path: bins to set to zero (nullptr: none)
 };
 // Tries the tuned kernel first, then the generic one (which has no extra steps).
 cudaError_t launch_hop(const Geom& g, const HopLaunch& a, cudaStream_t s);
@@ -144,7 +159,7 @@ struct RUpdateLaunch {
   const void* chain;
   size_t cstride;
   const double* num;
-  const double* den;
+  SumIn den;
   double* a_out;
   int sstride;
   const Reduce* red;
@@ -160,13 +175,15 @@ cudaError_t launch_px_update(const Geom& g, int prec, int xprec, void* x, void* 
 // per right-hand side coefficients bdiag/boff [2][Ls] in prec's compute type with
 // stride cstride); with do_x also the deferred x += a_prev p.  p and pnew are
 // different buffers; 16-bit storage applies B to the stored (rounded) p_new.
-// Ls even; prec FP32 (x FP32 or FP64), FP64, or FP16/BF16 with x in FP32.
+// Ls even, at most 32; prec FP32 (x FP32 or FP64), FP64, or FP16/BF16 with x in FP32.
 cudaError_t launch_pxb_update(const Geom& g, int prec, int xprec, void* x, const void* p, void* pnew,
                               void* bp,
-                              const void* z, const double* a_ptr, const double* num,
+                              const void* z, const double* a_ptr, const SumIn& num,
                               const double* den, int sstride, int nrhs, size_t stride_x,
                               size_t stride, const void* bdiag, const void* boff, size_t cstride,
                               cudaStream_t s, const int* active, int do_x);
+// val[rhs * stride] = the bins' value.
+cudaError_t launch_finish_sum(const SumIn& in, int nrhs, cudaStream_t s, const int* active);
 // x += a p, a = *a_ptr (flush of the deferred solution update).
 cudaError_t launch_x_update(const Geom& g, int prec, int xprec, void* x, const void* p,
                             const double* a_ptr, int sstride, int nrhs, size_t stride_x,

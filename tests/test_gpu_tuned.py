@@ -140,3 +140,31 @@ def test_force_matches_oracle(L, Ls, black, bc_t):
     op.force(G, Xd, Xd, projected=False)
     ref = torch.from_numpy(O.force_gradient(sysm, X, X)).cuda()
     assert _rel(G, ref) <= 1e-12
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+@pytest.mark.parametrize("L,Ls,scale", [((4, 4, 4, 4), 8, 1e-14), ((2, 6, 2, 4), 8, 1e14), ((4, 2, 6, 2), 12, 1.0),
+                                        ((8, 8, 8, 8), 16, 1.0)])
+def test_cg_sums_match_unfused(L, Ls, scale, prec, monkeypatch):
+    """The exact sums of the fused CG (norms of 1e-28 .. 1e28 times the field's, a point
+    source, whose slices differ by many orders of magnitude, ragged CTAs, one and four warps a
+    site) against the unfused CG with its tree sums: the same iteration count to one poll
+    (the recurrences differ by FP32 rounding only) and the same propagator to 1e-7."""
+    from synthetic import point_source4d
+    sysm = make_case(L, Ls, "mobius", alpha=1.2, m=0.1)
+    src = torch.from_numpy(scale * point_source4d(L, 1, 2)).cuda()
+    res = []
+    for unfused in (True, False):
+        if unfused:
+            monkeypatch.setenv("DWF_UNFUSED_CG", "1")
+        else:
+            monkeypatch.delenv("DWF_UNFUSED_CG")
+        op = _op(sysm, precision_inner=prec, check_every=2)
+        prop = torch.empty_like(src)
+        st = op.cgne_solve(src, prop)[0]
+        assert st["true_resid"] <= 1e-10
+        res.append((st["iterations"], prop))
+        op.close()
+    slack = 4 if prec == 1 else 40   # 16-bit recurrences part ways at their replacements
+    assert abs(res[0][0] - res[1][0]) <= slack
+    assert _rel(res[1][1], res[0][1]) <= 1e-7

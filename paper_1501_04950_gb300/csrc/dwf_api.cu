@@ -487,6 +487,7 @@ struct CoefView {
   const int* active;
   bool chain_ok;  // of every right-hand side's set
   int rule_nrhs;  // HopLaunch.rule_nrhs
+  bool ahead;     // HopLaunch.ahead
   const void* ptr(int prec, size_t off) const {
     const int f = prec == P64 ? 0 : 1;
     return reinterpret_cast<const char*>(dev[f]) + off * (f == 0 ? 8 : 4);
@@ -498,17 +499,28 @@ struct CoefView {
   }
 };
 CoefView view_of(const MatSet& ms) {
-  return CoefView{&ms, {ms.dev[0], ms.dev[1]}, 0, nullptr, ms.chain_ok, 0};
+  return CoefView{&ms, {ms.dev[0], ms.dev[1]}, 0, nullptr, ms.chain_ok, 0, false};
 }
 
 void set_coef(HopLaunch& L, const CoefView& cv) {
   L.cstride = cv.cstride;
   L.active = cv.active;
   L.rule_nrhs = cv.rule_nrhs;
+  L.ahead = cv.ahead;
 }
 
 int apply_dbb_bp(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* p, const void* bp,
                  void* tmp, int nrhs, const Reduce* norm, cudaStream_t s, bin_t* zero0 = nullptr);
+
+// Whether the kernels of a CG iteration start ahead (launch_ahead): where each of them fills
+// the GPU more than once (16 warps per SM), so that the next one's CTAs take the place of
+// finished ones.  FP32 solves, with / without: 12^4, Ls 16 (2592 warps)
+// 67.6 / 71.5 ms a solve, 12^3x24, Ls 12 110.0 / 114.6, 16^3x32, Ls 16 434.5 / 439.1, 24 FP16
+// sources on 8^4 340 / 350.  Below that the CTAs that come early crowd the SMs that have room
+// (8^3x16, Ls 16, 1024 warps: 52.7 / 41.0), most of all with FP64 fields (805 / 428).
+bool ahead_rule(const Geom& g, int prec, int nrhs) {
+  return prec != P64 && (long long)g.N5 / 64 * nrhs >= 152 * 16;
+}
 
 // out = PROG in, site-local, FP64 (B, I, K or I^-1), by the tuned kernels (cv.tuned(P64)).
 // in and out may be the same field.
@@ -969,13 +981,15 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
   auto mark = [&](bool first, bool start, int kind) -> int {
     return first ? timer_mark(h, s, start, kind) : DWF_OK;
   };
+  CoefView cva = cv;  // of the iteration's kernels
+  cva.ahead = ahead_rule(h->g, prec, nb);
   auto enqueue_fused = [&](int cur, bool first) -> int {
     const int nxt = 1 - cur;
     double* zz_new = h->scal + (nxt ? S_ZZ1 : S_ZZ0);
     double* zz_old = h->scal + (cur ? S_ZZ1 : S_ZZ0);
     int r;
     if ((r = mark(first, true, 1))) return r;
-    if ((r = apply_dbb_dag_hat(h, cv, prec, W.z, W.r, W.tb, W.tr, nb, with_bp ? &bin_zz : &red_zz[nxt], s,
+    if ((r = apply_dbb_dag_hat(h, cva, prec, W.z, W.r, W.tb, W.tr, nb, with_bp ? &bin_zz : &red_zz[nxt], s,
                                with_bp ? bins_of(h, BIN_WW) : nullptr, with_bp ? bins_of(h, BIN_RR) : nullptr)))
       return r;
     if ((r = mark(first, false, 1))) return r;
@@ -989,7 +1003,7 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
                                    bin_sum(h, BIN_ZZ, zz_new), zz_old, kScal, nb, fx, fi,
                                    cv.ptr(prec, cv.layout->bdiag_off()),
                                    cv.ptr(prec, cv.layout->boff_off()), cv.cstride, s, h->d_active,
-                                   first ? 0 : 1));
+                                   first ? 0 : 1, cva.ahead));
     } else if (first) {
       KLAUNCH(h, launch_p_update(h->g, prec, W.p, W.z, zz_new, zz_old, kScal, nb, fi, s, h->d_active));
     } else {
@@ -998,8 +1012,8 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
     }
     if ((r = mark(first, true, 0))) return r;
     if (with_bp) {
-      if ((r = apply_dbb_bp(h, cv, prec, W.w, pcur, W.bp, W.tr, nb, &bin_ww, s, bins_of(h, BIN_ZZ)))) return r;
-    } else if ((r = apply_dbb(h, cv, prec, W.w, W.p, W.tr, nb, &red_ww, s))) {
+      if ((r = apply_dbb_bp(h, cva, prec, W.w, pcur, W.bp, W.tr, nb, &bin_ww, s, bins_of(h, BIN_ZZ)))) return r;
+    } else if ((r = apply_dbb(h, cva, prec, W.w, W.p, W.tr, nb, &red_ww, s))) {
       return r;
     }
     if ((r = mark(first, false, 0))) return r;
@@ -1018,6 +1032,7 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
     U.sstride = kScal;
     U.red = with_bp ? &bin_rr : &red_rr;
     U.active = h->d_active;
+    U.ahead = cva.ahead;
     KLAUNCH(h, launch_rupdate(h->g, U, s));
     return DWF_OK;
   };
@@ -1331,14 +1346,16 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
   auto slot = [&](int k) { return h->scal + (k ? S_ZZ1 : S_ZZ0); };
   // |w|^2 and |r|^2 are exact sums in bins; pass A of D clears them
   const Reduce bin_ww = bin_reduce(h, BIN_WW), bin_rr = bin_reduce(h, BIN_RR);
+  const bool ahead = ahead_rule(h->g, prec, 1);
   auto enqueue_fused = [&](int c, bool first, cudaStream_t q) -> int {
     const int n = 1 - c, black = h->opt.rb_parity;
     KLAUNCH(h, launch_pxb_update(h->g, prec, xprec, W.xlo, c ? W.p2 : W.p, c ? W.p : W.p2, W.bp, W.r,
                                  h->scal + S_A, first ? plain_sum(slot(c)) : bin_sum(h, BIN_RR, slot(c)), slot(n), kScal, 1, fx, fi,
                                  cv.ptr(prec, ms.bdiag_off()), cv.ptr(prec, ms.boff_off()), 0, q, nullptr,
-                                 first ? 0 : 1));
+                                 first ? 0 : 1, ahead));
     void* p = c ? W.p : W.p2;
     HopLaunch L = base_hop(h, prec, 1 - black, 1, fi);
+    L.ahead = ahead;
     L.chain = cv.chain(prec);
     L.out = W.tr;
     L.v = W.bp;
@@ -1348,6 +1365,7 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
     L.zero[1] = bins_of(h, BIN_RR);
     KLAUNCH(h, launch_hop(h->g, L, q));
     HopLaunch B = base_hop(h, prec, black, 1, fi);
+    B.ahead = ahead;
     B.chain = cv.chain(prec);
     B.out = W.w;
     B.v = W.tr;
@@ -2133,7 +2151,7 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
       KLAUNCH(h, launch_hop(g, Hs, st));
     }
     std::vector<dwf_stats> sk(n);
-    CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr, true, nrhs};
+    CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr, true, nrhs, false};
     for (int r = 0; r < n; r++) cv.chain_ok = cv.chain_ok && ms[blk + r]->chain_ok;
     rc = cgnr_batched(h, cv, prec, h->opt.rel_tol, h->opt.maxiter, delta, restart, W, n, sk.data(), st);
     if (rc && rc != DWF_ERR_NOT_CONVERGED && rc != DWF_ERR_BREAKDOWN) return rc;

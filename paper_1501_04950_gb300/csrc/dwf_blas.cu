@@ -417,8 +417,10 @@ __global__ void __launch_bounds__(kBlasThreads, 2) pxb_update_kernel(
   using T = typename SP::T;
   using TX = typename SPX::T;
   const int rhs = blockIdx.y;
+  ahead_trigger();
   if (active && !active[rhs]) return;
   const size_t off = rhs * stride, offx = rhs * stride_x;
+  ahead_wait();
   __shared__ T beta_sh;
   bool have_beta = false;
   T beta = 0;
@@ -827,36 +829,38 @@ cudaError_t launch_pxb_update(const Geom& g, int prec, int xprec, void* x, const
                               void* pnew, void* bp, const void* z, const double* a_ptr, const SumIn& num,
                               const double* den, int sstride, int nrhs, size_t sx, size_t sp,
                               const void* bdiag, const void* boff, size_t cstride, cudaStream_t s,
-                              const int* active, int do_x) {
+                              const int* active, int do_x, bool ahead) {
   // threads for whole sites per warp
   const int half = g.Ls / 2, per = 32 / half * half;
   if (half > 16) return cudaErrorInvalidValue;
   const Shape sh = elementwise(((size_t)g.N5 / 2 + per - 1) / per * 32);
   const dim3 grid(sh.blocks, nrhs);
   if (prec == P32 && xprec == P32) {
-    pxb_update_kernel<Store32, Store32><<<grid, sh.threads, 0, s>>>(
-        g, x, p, pnew, bp, z, a_ptr, num, den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
-        reinterpret_cast<const float*>(boff), cstride, active, do_x);
-  } else if (prec == P32 && xprec == P64) {
-    pxb_update_kernel<Store64, Store32><<<grid, sh.threads, 0, s>>>(
-        g, x, p, pnew, bp, z, a_ptr, num, den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
-        reinterpret_cast<const float*>(boff), cstride, active, do_x);
-  } else if (prec == P64 && xprec == P64) {
-    pxb_update_kernel<Store64, Store64><<<grid, sh.threads, 0, s>>>(
-        g, x, p, pnew, bp, z, a_ptr, num, den, sstride, sx, sp, reinterpret_cast<const double*>(bdiag),
-        reinterpret_cast<const double*>(boff), cstride, active, do_x);
-  } else if (prec == P16 && xprec == P32) {
-    pxb_update_kernel<Store32, Store16<false>><<<grid, sh.threads, 0, s>>>(
-        g, x, p, pnew, bp, z, a_ptr, num, den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
-        reinterpret_cast<const float*>(boff), cstride, active, do_x);
-  } else if (prec == PB16 && xprec == P32) {
-    pxb_update_kernel<Store32, Store16<true>><<<grid, sh.threads, 0, s>>>(
-        g, x, p, pnew, bp, z, a_ptr, num, den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
-        reinterpret_cast<const float*>(boff), cstride, active, do_x);
-  } else {
-    return cudaErrorInvalidValue;
+    return launch_ahead(ahead, pxb_update_kernel<Store32, Store32>, grid, sh.threads, 0, s, g, x, p, pnew, bp, z, a_ptr, num,
+                        den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
+                        reinterpret_cast<const float*>(boff), cstride, active, do_x);
   }
-  return cudaGetLastError();
+  if (prec == P32 && xprec == P64) {
+    return launch_ahead(ahead, pxb_update_kernel<Store64, Store32>, grid, sh.threads, 0, s, g, x, p, pnew, bp, z, a_ptr, num,
+                        den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
+                        reinterpret_cast<const float*>(boff), cstride, active, do_x);
+  }
+  if (prec == P64 && xprec == P64) {
+    return launch_ahead(ahead, pxb_update_kernel<Store64, Store64>, grid, sh.threads, 0, s, g, x, p, pnew, bp, z, a_ptr, num,
+                        den, sstride, sx, sp, reinterpret_cast<const double*>(bdiag),
+                        reinterpret_cast<const double*>(boff), cstride, active, do_x);
+  }
+  if (prec == P16 && xprec == P32) {
+    return launch_ahead(ahead, pxb_update_kernel<Store32, Store16<false>>, grid, sh.threads, 0, s, g, x, p, pnew, bp, z, a_ptr, num,
+                        den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
+                        reinterpret_cast<const float*>(boff), cstride, active, do_x);
+  }
+  if (prec == PB16 && xprec == P32) {
+    return launch_ahead(ahead, pxb_update_kernel<Store32, Store16<true>>, grid, sh.threads, 0, s, g, x, p, pnew, bp, z, a_ptr, num,
+                        den, sstride, sx, sp, reinterpret_cast<const float*>(bdiag),
+                        reinterpret_cast<const float*>(boff), cstride, active, do_x);
+  }
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_finish_sum(const SumIn& in, int nrhs, cudaStream_t s, const int* active) {

@@ -705,6 +705,33 @@ __device__ __forceinline__ void su3_mul(const Link<T>& U, const cplx<T> h0[3], c
 }
 
 // ---------------------------------------------------------------------------
+// Launch that may begin while the kernel before it in the stream still runs (programmatic
+// dependent launch), for the chain of small kernels of a CG iteration: a kernel lets the
+// next one be scheduled at once (ahead_trigger), reads what no kernel of the chain
+// writes (coefficients, neighbour table), and waits for the one before it to be complete
+// and visible (ahead_wait) before its first access to fields, sums or scalars.  Without
+// the launch attribute both are no-ops.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void ahead_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void ahead_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_ahead(bool ahead, void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                         A&&... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &a;
+  c.numAttrs = ahead ? 1 : 0;
+  return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // The tuned kernels (dwf_hop2.cuh): the Ls they are compiled for (the others take the
 // generic kernels) are the Ls of the alpha study, of the benchmark and of the Mobius /
 // Zolotarev comparison.  With 16-bit storage (scaled) only the Ls of the benchmark

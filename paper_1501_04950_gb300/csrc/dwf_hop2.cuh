@@ -803,22 +803,24 @@ __global__ void __launch_bounds__(128, MINB) hop_kernel(const Geom g, const Args
   const bool part = warp_groups(LS) || (BYWARP ? jl < 32 / G : j < S);
   const bool active = part && h < g.Vh;
   const int rhs = blockIdx.z;
+  ahead_trigger();
   if (a.active && !a.active[rhs]) return;
   const size_t co = (size_t)rhs * a.cstride;
   const size_t NP = (size_t)g.N5 >> 1;
   const int s0 = 2 * t;
-  zero_bins(a, rhs, tid, nth);
-  if (EX == EX_RUPD) start_rupd(a, rhs, tid);
   load_coefs<T, LS, POST>(coef, a.chain + co, tid, nth);
   if (EX == EX_HAT) load_coefs<T, LS, PR_ITINV>(coef + prog_coefs(LS, POST), a.chain + co, tid, nth);
+  const int hl = BYWARP ? min(h, g.Vh - 1) : (active ? h : 0);
+  const int4 nb0 = __ldg(a.nbr + 2 * hl), nb1 = __ldg(a.nbr + 2 * hl + 1);
+  ahead_wait();
+  zero_bins(a, rhs, tid, nth);
+  if (EX == EX_RUPD) start_rupd(a, rhs, tid);
   const char* vb = reinterpret_cast<const char*>(a.v) + rhs * a.stride;
   SpinP<V> acc;
   zero(acc);
   // whole warps take part in the shuffles of the B pre-multiplication: threads past the
   // last site compute it again and store nothing
   if (BYWARP || active) {
-    const int hl = BYWARP ? min(h, g.Vh - 1) : h;
-    const int4 nb0 = __ldg(a.nbr + 2 * hl), nb1 = __ldg(a.nbr + 2 * hl + 1);
     T bd[2][2] = {{0, 0}, {0, 0}}, bo[2][2] = {{0, 0}, {0, 0}};
     if (PRE == PRE_B) {
 #pragma unroll
@@ -925,20 +927,22 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
   const bool part = warp_groups(LS) || j < S;
   const bool active = part && h < g.Vh;
   const int rhs = blockIdx.z;
+  ahead_trigger();
   if (a.active && !a.active[rhs]) return;
   const size_t co = (size_t)rhs * a.cstride;
   const size_t NP = (size_t)g.N5 >> 1;
-  zero_bins(a, rhs, tid, 128);
-  if (EX == EX_RUPD) start_rupd(a, rhs, tid);
   load_coefs<T, LS, POST>(coef, a.chain + co, tid, 128);
   if (EX == EX_HAT) load_coefs<T, LS, PR_ITINV>(coef + prog_coefs(LS, POST), a.chain + co, tid, 128);
+  constexpr bool WHOLE = PRE == PRE_B;  // its shuffles need whole warps
+  const int hl = WHOLE ? min(h, g.Vh - 1) : (active ? h : 0);
+  const int2 nb = __ldg(reinterpret_cast<const int2*>(a.nbr) + (size_t)hl * 4 + mu);
+  ahead_wait();
+  zero_bins(a, rhs, tid, 128);
+  if (EX == EX_RUPD) start_rupd(a, rhs, tid);
   const char* vb = reinterpret_cast<const char*>(a.v) + rhs * a.stride;
   SpinP<V> acc;
   zero(acc);
-  constexpr bool WHOLE = PRE == PRE_B;  // its shuffles need whole warps
   if (WHOLE || active) {
-    const int hl = WHOLE ? min(h, g.Vh - 1) : h;
-    const int2 nb = __ldg(reinterpret_cast<const int2*>(a.nbr) + (size_t)hl * 4 + mu);
     T bd[2][2] = {{0, 0}, {0, 0}}, bo[2][2] = {{0, 0}, {0, 0}};
     if (PRE == PRE_B) {
 #pragma unroll
@@ -1235,8 +1239,7 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
       static std::atomic<bool> attr{false};
       cudaError_t e = smem_limit_once(k, smem, attr);
       if (e != cudaSuccess) return e;
-      k<<<dim3((g.Vh + S - 1) / S, 1, L.nrhs), 128, smem, st>>>(g, a);
-      return cudaGetLastError();
+      return launch_ahead(L.ahead, k, dim3((g.Vh + S - 1) / S, 1, L.nrhs), 128, smem, st, g, a);
     }
   }
   const int nt = L.block_threads ? L.block_threads : tile_threads(LS, g.Vh, L.nrhs, sizeof(T) == 8);
@@ -1247,8 +1250,7 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   static std::atomic<bool> attr{false};
   cudaError_t e = smem_limit_once(k, smem_of(128), attr);
   if (e != cudaSuccess) return e;
-  k<<<grid, nt, smem_of(nt), st>>>(g, a);
-  return cudaGetLastError();
+  return launch_ahead(L.ahead, k, grid, nt, smem_of(nt), st, g, a);
 }
 
 // The hot combinations of the CG; anything else returns cudaErrorNotSupported
@@ -1365,9 +1367,11 @@ __global__ void __launch_bounds__(128) rupdate_kernel(const Geom g, void* r, voi
   const int h = blockIdx.x * S + j;
   const bool active = j < S && h < g.Vh;
   const int rhs = blockIdx.z;
+  ahead_trigger();
   if (rhs_on && !rhs_on[rhs]) return;
   const size_t NP = (size_t)g.N5 >> 1;
   load_coefs<T, LS, PR_ITINV>(coef, chain + (size_t)rhs * cstride, tid, nth);
+  ahead_wait();
   const size_t off = rhs * stride;
   const size_t m = (size_t)h * G + t;
   SpinP<V> x;
@@ -1427,9 +1431,9 @@ cudaError_t run_rupdate(const Geom& g, const RUpdateLaunch& L, cudaStream_t st) 
   cudaError_t e = smem_limit_once(k, smem_bytes(LS, 128 / (LS / 2), sizeof(T), PR_ITINV), attr);
   if (e != cudaSuccess) return e;
   dim3 grid((g.Vh + S - 1) / S, 1, L.nrhs);
-  k<<<grid, nt, smem_bytes(LS, S, sizeof(T), PR_ITINV), st>>>(g, L.r, L.rhat, L.w, L.stride, reinterpret_cast<const T*>(L.chain),
-                               L.cstride, L.num, L.den, L.a_out, L.sstride, *L.red, L.active);
-  return cudaGetLastError();
+  return launch_ahead(L.ahead, k, grid, nt, smem_bytes(LS, S, sizeof(T), PR_ITINV), st, g, L.r, L.rhat, L.w,
+                      L.stride, reinterpret_cast<const T*>(L.chain), L.cstride, L.num, L.den, L.a_out, L.sstride,
+                      *L.red, L.active);
 }
 
 template <class SP, int GROUP>

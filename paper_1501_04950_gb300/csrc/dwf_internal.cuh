@@ -125,6 +125,7 @@ struct HopLaunch {
   double* a_out;
   int sstride;
   bin_t* zero[2];           // tuned path: bins to set to zero (nullptr: none)
+  bool ahead;               // tuned path: may start while the kernel before it ends (launch_ahead)
 };
 // Tries the tuned kernel first, then the generic one (which has no extra steps).
 cudaError_t launch_hop(const Geom& g, const HopLaunch& a, cudaStream_t s);
@@ -164,6 +165,7 @@ struct RUpdateLaunch {
   int sstride;
   const Reduce* red;
   const int* active;
+  bool ahead;               // as HopLaunch.ahead
 };
 cudaError_t launch_rupdate(const Geom& g, const RUpdateLaunch& a, cudaStream_t s);
 // x += a_prev p; p = z + beta p (a_prev = *a_ptr, beta = num / den); x in xprec.
@@ -181,7 +183,7 @@ cudaError_t launch_pxb_update(const Geom& g, int prec, int xprec, void* x, const
                               const void* z, const double* a_ptr, const SumIn& num,
                               const double* den, int sstride, int nrhs, size_t stride_x,
                               size_t stride, const void* bdiag, const void* boff, size_t cstride,
-                              cudaStream_t s, const int* active, int do_x);
+                              cudaStream_t s, const int* active, int do_x, bool ahead);
 // val[rhs * stride] = the bins' value.
 cudaError_t launch_finish_sum(const SumIn& in, int nrhs, cudaStream_t s, const int* active);
 // x += a p, a = *a_ptr (flush of the deferred solution update).

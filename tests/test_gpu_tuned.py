@@ -143,12 +143,13 @@ def test_force_matches_oracle(L, Ls, black, bc_t):
 
 
 @pytest.mark.parametrize("prec", [1, 2])
-@pytest.mark.parametrize("L,Ls,scale", [((4, 4, 4, 4), 8, 1e-14), ((2, 6, 2, 4), 8, 1e14), ((4, 2, 6, 2), 12, 1.0),
+@pytest.mark.parametrize("L,Ls,scale", [((4, 4, 4, 4), 8, 1e-8), ((2, 6, 2, 4), 8, 1e14), ((4, 2, 6, 2), 12, 1.0),
                                         ((8, 8, 8, 8), 16, 1.0)])
 def test_cg_sums_match_unfused(L, Ls, scale, prec, monkeypatch):
-    """The exact sums of the fused CG (norms of 1e-28 .. 1e28 times the field's, a point
-    source, whose slices differ by many orders of magnitude, ragged CTAs, one and four warps a
-    site) against the unfused CG with its tree sums: the same iteration count to one poll
+    """The exact sums of the fused CG (norms of 1e-16 .. 1e28 times the field's, down to 1e-36
+    at convergence, near the end of FP32's range, in which the squares of a slice are formed;
+    a point source, whose slices differ by many orders of magnitude; ragged CTAs; one and four
+    warps a site) against the unfused CG with its tree sums: the same iteration count to one poll
     (the recurrences differ by FP32 rounding only) and the same propagator to 1e-7."""
     from synthetic import point_source4d
     sysm = make_case(L, Ls, "mobius", alpha=1.2, m=0.1)

@@ -166,7 +166,8 @@ int dwf_unpack_half(dwf_handle h, double* dst_canonical, const void* src_interna
 
 /* out = D_bb in (Sec. 3, Eq. redblack) on nrhs internal black half-fields of
  * precision prec.  Two kernels: u = K H_rb (B in) on red sites, then
- * out = in - 1/4 I^-1 H_br u on black sites (D_rb = -1/2 H_rb B, K = B I^-1).
+ * out = in - 1/4 I^-1 H_br u on black sites (D_rb = -1/2 H_rb B, K = B I^-1);
+ * with FP64 fields B in is formed first (in out), by a third.
  * in and out must not overlap. */
 int dwf_apply_Dbb(dwf_handle h, void* out, const void* in, int prec, int nrhs, dwf_stream s);
 
@@ -202,10 +203,9 @@ int dwf_apply_dalpha(dwf_handle h, double* out_full, const double* in_full, doub
  * sides that share every kernel launch (each with its own alpha, scalars and
  * convergence; converged ones are masked off).  With rhs_block = 0 a built-in
  * autotuner times the batched D_bb apply for block sizes that fit in free
- * device memory, for the two CTA tiles of the hop kernels and for the two
- * neighbour staging variants, and keeps the fastest per right-hand side
- * (cached per lattice, Ls, precision and nrhs in the handle, and in the file
- * named by DWF_AUTOTUNE_CACHE if set).  The CG
+ * device memory and for the CTA shapes of the hop kernels, and keeps the
+ * fastest per right-hand side (cached per lattice, Ls, precision and nrhs in
+ * the handle, and in the file named by DWF_AUTOTUNE_CACHE if set).  The CG
  * iterations between two convergence polls (check_every, rounded up to even)
  * are captured once as a CUDA graph and replayed.  All solver work runs on a
  * stream owned by the handle; the call first waits for the caller's stream. */

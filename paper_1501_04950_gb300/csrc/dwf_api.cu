@@ -223,7 +223,7 @@ struct dwf_ctx {
   void* gauge[3] = {nullptr, nullptr, nullptr};  // FP64, FP32, FP16
   int* nbr = nullptr;                            // [2][Vh][8] neighbour table
   int* dev_err = nullptr;                        // set by a kernel whose bounded wait gave up
-  int use_tma = 0;                               // tensor-copy staged tuned kernels (autotuned)
+  int use_tma = 0;                               // tensor-copy staged tuned kernels
   int env_tma = 0;                               // DWF_TMA set: staging fixed to tensor copies
   long long wait_budget = 0;                     // DWF_WAIT_BUDGET: clock cycles per bounded wait
   int skip_hop = -1;                             // DWF_TEST_SKIP_HOP: the first staged launch
@@ -260,8 +260,8 @@ struct dwf_ctx {
     int nb, tma, tile;  // right-hand-side block, staging variant, threads per CTA (0: by size)
   };
   std::map<std::string, Tuned> tune;  // autotuned launch shapes
-  int tile = 0;                      // threads per CTA of the tuned hop kernels (0: by size)
-  int env_tile = -1;                 // DWF_HOP_TILE set: tile fixed (-1: autotuned)
+  int tile = 0;                      // tuned threads per CTA of the last solve's inner applies (0: by size)
+  int env_tile = -1;                 // DWF_HOP_TILE set: threads fixed (-1: autotuned)
   double tier_eta = 1e-3;            // 16-bit solves: FP64 replacement once |r| < eta |r_64|
                                      // (DWF_TIER_ETA; <= 0: every replacement in FP64)
 };
@@ -399,7 +399,7 @@ int get_ws(dwf_ctx* h, const std::string& name, size_t bytes, void** out) {
 int ensure_reduce(dwf_ctx* h, int nrhs) {
   int need_blocks = std::max(hop_grid_blocks(h->g, P64),
                              std::max(hop_grid_blocks(h->g, P32), blas_grid_blocks(h->g)));
-  if (hop2::tuned_ls(h->Ls, false)) {  // the smallest tile of the tuned kernels (32 threads a site)
+  if (hop2::tuned_ls(h->Ls, false)) {  // the smallest CTAs of the tuned kernels (32 threads)
     const int S = 32 / (h->Ls / 2);
     need_blocks = std::max(need_blocks, (h->g.Vh + S - 1) / S);
   }
@@ -471,7 +471,7 @@ HopLaunch base_hop(dwf_ctx* h, int prec, int p, int nrhs, size_t stride) {
   L.nbr = h->nbr;
   L.err = h->dev_err;
   L.use_tma = h->use_tma;
-  L.block_threads = h->tile;
+  L.block_threads = std::max(h->env_tile, 0);
   L.wait_budget = h->wait_budget;
   L.skip_hop = &h->skip_hop;  // one-shot test hook, consumed by the first staged launch
   return L;
@@ -488,6 +488,7 @@ struct CoefView {
   bool chain_ok;  // of every right-hand side's set
   int rule_nrhs;  // HopLaunch.rule_nrhs
   bool ahead;     // HopLaunch.ahead
+  int tile, tile_prec;  // HopLaunch.block_threads of the kernels of precision tile_prec (0: by size)
   const void* ptr(int prec, size_t off) const {
     const int f = prec == P64 ? 0 : 1;
     return reinterpret_cast<const char*>(dev[f]) + off * (f == 0 ? 8 : 4);
@@ -499,7 +500,7 @@ struct CoefView {
   }
 };
 CoefView view_of(const MatSet& ms) {
-  return CoefView{&ms, {ms.dev[0], ms.dev[1]}, 0, nullptr, ms.chain_ok, 0, false};
+  return CoefView{&ms, {ms.dev[0], ms.dev[1]}, 0, nullptr, ms.chain_ok, 0, false, 0, P64};
 }
 
 void set_coef(HopLaunch& L, const CoefView& cv) {
@@ -507,6 +508,7 @@ void set_coef(HopLaunch& L, const CoefView& cv) {
   L.active = cv.active;
   L.rule_nrhs = cv.rule_nrhs;
   L.ahead = cv.ahead;
+  if (cv.tile && L.prec == cv.tile_prec) L.block_threads = cv.tile;
 }
 
 int apply_dbb_bp(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* p, const void* bp,
@@ -1538,13 +1540,15 @@ int solver_params(dwf_ctx* h, int* prec, double* delta, bool* restart) {
 
 // Autotuner of the launch shapes of the solver: times the (batched) D_bb apply
 // of the inner precision for every right-hand-side block size that fits in free
-// device memory (batched solves), every CTA tile of the tuned hop kernels
-// (default and small) and both neighbour staging variants (direct loads,
-// tensor-copy staging), and keeps the fastest per right-hand side (within 3%,
-// the larger block).  Results are cached per (lattice, Ls, precision, nrhs) in
-// the handle and, if DWF_AUTOTUNE_CACHE names a file, there as
+// device memory (batched solves) and for the tuned hop kernels' CTAs of 128 and 64
+// threads (where the choice by size takes the direction-split kernel, only that: the
+// other shapes all give the same bits, which a timing may therefore choose among),
+// and keeps the fastest per right-hand side (within 3%, the larger block).  The
+// tensor-copy staged variant was slower at every size it was tried on (FP16, 24 sources
+// on 8^4, Ls = 16: 278 us a pass against 52 to 74) and is not tried.  Results are cached per (lattice,
+// Ls, precision, nrhs) in the handle and, if DWF_AUTOTUNE_CACHE names a file, there as
 // "key nb staging tile" lines.  An explicit rhs_block option fixes the block;
-// DWF_TMA (set at dwf_create) fixes the staging.
+// DWF_TMA (set at dwf_create) fixes the staging, DWF_HOP_TILE the CTA.
 int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_out) {
   const int Ls = h->g.Ls;
   const bool tuned = !g_disable_tuned && hop2::tuned_ls(Ls, prec == P16 || prec == PB16);
@@ -1567,7 +1571,7 @@ int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_ou
     std::string k;
     int nb, tma, tile;
     while (in >> k >> nb >> tma >> tile)
-      if (k == key.str()) h->tune[k] = dwf_ctx::Tuned{nb, tma, tile};
+      if (k == key.str()) h->tune[k] = dwf_ctx::Tuned{nb, tma, tile == 64 || tile == 128 ? tile : 0};
     it = h->tune.find(key.str());
   }
   if (it != h->tune.end()) {
@@ -1601,6 +1605,7 @@ int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_ou
   if ((rc = build_matset(h, h->alpha, h->m, &ms))) return rc;
   CoefView tv = view_of(*ms);
   tv.rule_nrhs = nrhs;
+  tv.tile_prec = prec;
   cudaEvent_t e0, e1;
   CUCHK(h, cudaEventCreate(&e0));
   CUCHK(h, cudaEventCreate(&e1));
@@ -1621,7 +1626,7 @@ int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_ou
     for (int tma : tmas)
       for (int tile : tiles) {
         h->use_tma = tma;
-        h->tile = tile;
+        tv.tile = tile;
         if ((rc = apply_dbb(h, tv, prec, y, x, t, nb, nullptr, st))) return rc;
         // best of two timed passes of 3 applies (one slow pass does not decide)
         double per_rhs = 1e300;
@@ -1728,7 +1733,6 @@ int dwf_create(dwf_handle* out, const int lattice[4], int Ls, double M5, double 
   // DWF_HOP_TILE=small|default fixes the CTA tile of the tuned hop kernels
   if (const char* e = std::getenv("DWF_HOP_TILE")) {
     h->env_tile = std::string(e) == "small" ? 64 : 128;
-    h->tile = h->env_tile;
   }
   h->bp_fused = std::getenv("DWF_NO_BP_FUSED") == nullptr;
   if (const char* e = std::getenv("DWF_TIER_ETA")) h->tier_eta = std::atof(e);
@@ -2151,7 +2155,7 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
       KLAUNCH(h, launch_hop(g, Hs, st));
     }
     std::vector<dwf_stats> sk(n);
-    CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr, true, nrhs, false};
+    CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr, true, nrhs, false, h->tile, prec};
     for (int r = 0; r < n; r++) cv.chain_ok = cv.chain_ok && ms[blk + r]->chain_ok;
     rc = cgnr_batched(h, cv, prec, h->opt.rel_tol, h->opt.maxiter, delta, restart, W, n, sk.data(), st);
     if (rc && rc != DWF_ERR_NOT_CONVERGED && rc != DWF_ERR_BREAKDOWN) return rc;

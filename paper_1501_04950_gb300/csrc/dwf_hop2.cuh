@@ -1095,19 +1095,20 @@ __global__ void __launch_bounds__(128) local_kernel(const Geom g, void* out, con
 namespace dwf {
 namespace hop2 {
 
-// Threads per CTA (HopLaunch.block_threads; 0: by the rule of tile_threads).
-constexpr int kTileThreads[3] = {128, 64, 32};
-
-// The largest CTA that still gives every SM four of them (FP64: eight, its pipe wants the
-// warps spread evenly over the sub-partitions); 64 threads at most where a site's threads
-// straddle warps and the CTA's tail of unused lanes counts (FP32, Ls = 10, 12^3x24, D_bb +
-// D_bb^+: 103.6 us at 64, 107.4 at 128).  All of them give the same bits.
+// Threads per CTA (HopLaunch.block_threads; 0: by this rule).
+// FP32 and 16-bit: 128 threads, or 64 where a site's threads straddle warps and the CTA's
+// tail of unused lanes counts (FP32, Ls = 12, 12^2x8x12, D_bb + D_bb^+, CUDA graph: 43.0 us at
+// 64, 46.6 at 128); CTAs of one warp load the coefficients and pass the barriers once per
+// warp (BF16, Ls = 16, 8^2x4^2: 30.8 us at 32, 28.6 at 64, 26.2 at 128).
+// FP64: the largest CTA that still gives every SM eight of them: its pipe wants the warps
+// spread evenly over the sub-partitions (Ls = 8, 12^2x8x12: 439 us at 64, 548 at 128).
+// All of them give the same bits.
 inline int tile_threads(int Ls, int Vh, int nrhs, bool f64) {
-  for (int nt : kTileThreads) {
-    if (nt == 128 && !f64 && !warp_groups(Ls)) continue;
+  if (!f64) return warp_groups(Ls) ? 128 : 64;
+  for (int nt : {128, 64}) {
     const int S = nt / (Ls / 2);
     const long long blocks = (long long)((Vh + S - 1) / S) * nrhs;
-    if (blocks >= 152 * (f64 ? 8 : 4) * 128 / nt) return nt;
+    if (blocks >= 152 * 8 * 128 / nt) return nt;
   }
   return 32;
 }

@@ -435,9 +435,11 @@ __device__ __forceinline__ FixedSum warp_fixed_sum(float x, float y) {
 }
 
 // block_sum_to of the squares of FP32 slice pairs, r = (slice 0, slice 1): full warps, at
-// most 4 of them.
+// most kPairSumWarps of them (the four of the tuned kernels' largest CTA and the producer
+// warp of the staged one, which adds zero: the sum of four warps' t < 2^62 still fits 64 bits).
+constexpr int kPairSumWarps = 5;
 __device__ __forceinline__ void block_sum_pair(float2 r, const Reduce& red, int rhs, int nblocks, int bid) {
-  __shared__ FixedSum wsum[4];
+  __shared__ FixedSum wsum[kPairSumWarps];
   const int tid = threadIdx.y * blockDim.x + threadIdx.x, lane = tid & 31;
   const int nw = (blockDim.x * blockDim.y) >> 5;
   FixedSum f = warp_fixed_sum(r.x, r.y);

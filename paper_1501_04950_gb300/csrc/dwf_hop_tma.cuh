@@ -22,6 +22,7 @@ namespace hop2 {
 
 constexpr int kTmaConsumers = 128;
 constexpr int kTmaThreads = kTmaConsumers + 32;
+static_assert(kTmaThreads <= 32 * kPairSumWarps, "the fused norm has room for every warp of the CTA");
 // the Ls with a staged variant
 __host__ __device__ constexpr bool tma_ls(int Ls) { return Ls == 8 || Ls == 12 || Ls == 16; }
 

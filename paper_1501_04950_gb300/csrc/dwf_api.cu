@@ -230,6 +230,7 @@ struct dwf_ctx {
                                                  // issues no copies for this hop (timeout test)
   bool fused_cg = true;                          // DWF_UNFUSED_CG unset: fused CG BLAS steps
   bool bp_fused = true;                          // DWF_NO_BP_FUSED unset: p update forms B p
+  bool ahead = true;                             // DWF_NO_AHEAD unset: CG kernels may start ahead
   int check = 16;                                // effective iterations between polls
   bool gauge_loaded = false;
   std::vector<void*> allocs;
@@ -984,7 +985,7 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
     return first ? timer_mark(h, s, start, kind) : DWF_OK;
   };
   CoefView cva = cv;  // of the iteration's kernels
-  cva.ahead = ahead_rule(h->g, prec, nb);
+  cva.ahead = h->ahead && ahead_rule(h->g, prec, nb);
   auto enqueue_fused = [&](int cur, bool first) -> int {
     const int nxt = 1 - cur;
     double* zz_new = h->scal + (nxt ? S_ZZ1 : S_ZZ0);
@@ -1348,7 +1349,7 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
   auto slot = [&](int k) { return h->scal + (k ? S_ZZ1 : S_ZZ0); };
   // |w|^2 and |r|^2 are exact sums in bins; pass A of D clears them
   const Reduce bin_ww = bin_reduce(h, BIN_WW), bin_rr = bin_reduce(h, BIN_RR);
-  const bool ahead = ahead_rule(h->g, prec, 1);
+  const bool ahead = h->ahead && ahead_rule(h->g, prec, 1);
   auto enqueue_fused = [&](int c, bool first, cudaStream_t q) -> int {
     const int n = 1 - c, black = h->opt.rb_parity;
     KLAUNCH(h, launch_pxb_update(h->g, prec, xprec, W.xlo, c ? W.p2 : W.p, c ? W.p : W.p2, W.bp, W.r,
@@ -1735,6 +1736,7 @@ int dwf_create(dwf_handle* out, const int lattice[4], int Ls, double M5, double 
     h->env_tile = std::string(e) == "small" ? 64 : 128;
   }
   h->bp_fused = std::getenv("DWF_NO_BP_FUSED") == nullptr;
+  h->ahead = std::getenv("DWF_NO_AHEAD") == nullptr;
   if (const char* e = std::getenv("DWF_TIER_ETA")) h->tier_eta = std::atof(e);
   if (const char* e = std::getenv("DWF_WAIT_BUDGET")) h->wait_budget = std::atoll(e);
   if (const char* e = std::getenv("DWF_TEST_SKIP_HOP")) h->skip_hop = std::atoi(e);

@@ -73,6 +73,12 @@ __host__ __device__ __forceinline__ int site5(int h, int s, int Ls) { return h *
 //              then float scale[N5] (index n)                      52 B / site
 // load/store move one 5D site n (scalar lanes; the generic kernels and the
 // conversions); load_pair/store_pair move the two sites of pair m.
+//
+// load_pair (and PairIO::load6 of dwf_hop2.cuh) reads with ordinary loads, not __ldg: that
+// one is only for memory that nothing writes while the kernel lives, may be moved across
+// the wait of a kernel that starts ahead (launch_ahead), whose life overlaps the writes of
+// the kernel before it, and the updates in place write what they read.  __ldg stays for the
+// links, the coefficients and the neighbour table.
 // ---------------------------------------------------------------------------
 struct Store64 {
   using T = double;
@@ -108,7 +114,7 @@ struct Store64 {
     const double2* p = reinterpret_cast<const double2*>(base);
 #pragma unroll
     for (int k = 0; k < 12; k++) {
-      const double2 re = __ldg(p + ((size_t)k * NP + m) * 2), im = __ldg(p + ((size_t)k * NP + m) * 2 + 1);
+      const double2 re = p[((size_t)k * NP + m) * 2], im = p[((size_t)k * NP + m) * 2 + 1];
       a.c[k] = cmake(re.x, im.x);
       b.c[k] = cmake(re.y, im.y);
     }
@@ -157,7 +163,7 @@ struct Store32 {
     const float4* p = reinterpret_cast<const float4*>(base);
 #pragma unroll
     for (int k = 0; k < 12; k++) {
-      const float4 v = __ldg(p + (size_t)k * NP + m);
+      const float4 v = p[(size_t)k * NP + m];
       a.c[k] = cmake(v.x, v.z);
       b.c[k] = cmake(v.y, v.w);
     }
@@ -255,10 +261,10 @@ struct Store16 {
   }
   __device__ static void load_pair(const void* base, int m, int NP, Spinor<float>& a, Spinor<float>& b) {
     const uint4* p = reinterpret_cast<const uint4*>(base);
-    const float2 sc = __ldg(reinterpret_cast<const float2*>(p + (size_t)6 * NP) + m);
+    const float2 sc = reinterpret_cast<const float2*>(p + (size_t)6 * NP)[m];
 #pragma unroll
     for (int j = 0; j < 6; j++) {
-      const uint4 v = __ldg(p + (size_t)j * NP + m);
+      const uint4 v = p[(size_t)j * NP + m];
       const float2 r0 = to_f2(v.x), i0 = to_f2(v.y), r1 = to_f2(v.z), i1 = to_f2(v.w);
       a.c[2 * j] = cmake(sc.x * r0.x, sc.x * i0.x);
       b.c[2 * j] = cmake(sc.y * r0.y, sc.y * i0.y);

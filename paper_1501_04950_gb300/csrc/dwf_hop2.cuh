@@ -123,6 +123,7 @@ struct SpinP {
 // ---------------------------------------------------------------------------
 // Pair access to the half-field layouts of dwf_fields.cuh (pair m, NP pairs).
 // load6: components c0 .. c0 + 5 (c0 = 0: P_+ spins, 6: P_- spins), unscaled.
+// Ordinary loads (see load_pair there): these kernels may start ahead of the end of the one before.
 // ---------------------------------------------------------------------------
 template <class SP>
 struct PairIO;
@@ -135,7 +136,7 @@ struct PairIO<Store32> {
     const float4* p = reinterpret_cast<const float4*>(base) + (size_t)c0 * NP + m;
 #pragma unroll
     for (int k = 0; k < 6; k++) {
-      const float4 v = __ldg(p + (size_t)k * NP);
+      const float4 v = p[(size_t)k * NP];
       re[k] = make_float2(v.x, v.y);
       im[k] = make_float2(v.z, v.w);
     }
@@ -158,8 +159,8 @@ struct PairIO<Store64> {
     const double2* p = reinterpret_cast<const double2*>(base) + ((size_t)c0 * NP + m) * 2;
 #pragma unroll
     for (int k = 0; k < 6; k++) {
-      re[k] = __ldg(p + (size_t)k * NP * 2);
-      im[k] = __ldg(p + (size_t)k * NP * 2 + 1);
+      re[k] = p[(size_t)k * NP * 2];
+      im[k] = p[(size_t)k * NP * 2 + 1];
     }
   }
   static __device__ __forceinline__ V scale(const void*, size_t, size_t) { return make_double2(1.0, 1.0); }
@@ -183,7 +184,7 @@ struct PairIO<Store16<BF>> {
     const uint4* p = reinterpret_cast<const uint4*>(base) + (size_t)(c0 >> 1) * NP + m;
 #pragma unroll
     for (int j = 0; j < 3; j++) {
-      const uint4 v = __ldg(p + (size_t)j * NP);
+      const uint4 v = p[(size_t)j * NP];
       re[2 * j] = S::to_f2(v.x);
       im[2 * j] = S::to_f2(v.y);
       re[2 * j + 1] = S::to_f2(v.z);
@@ -191,7 +192,7 @@ struct PairIO<Store16<BF>> {
     }
   }
   static __device__ __forceinline__ V scale(const void* base, size_t m, size_t NP) {
-    return __ldg(reinterpret_cast<const float2*>(reinterpret_cast<const uint4*>(base) + 6 * NP) + m);
+    return reinterpret_cast<const float2*>(reinterpret_cast<const uint4*>(base) + 6 * NP)[m];
   }
   static __device__ __forceinline__ float2 scales_of(const SpinP<V>& a) {
     float mx = 0.f, my = 0.f;
@@ -848,14 +849,14 @@ __global__ void __launch_bounds__(128, MINB) hop_kernel(const Geom g, const Args
 
 // One component of a slice pair (FP32 and FP64 fields).
 __device__ __forceinline__ void load_comp(const float* base, size_t m, size_t NP, int c, float2& re, float2& im) {
-  const float4 v = __ldg(reinterpret_cast<const float4*>(base) + (size_t)c * NP + m);
+  const float4 v = reinterpret_cast<const float4*>(base)[(size_t)c * NP + m];
   re = make_float2(v.x, v.y);
   im = make_float2(v.z, v.w);
 }
 __device__ __forceinline__ void load_comp(const double* base, size_t m, size_t NP, int c, double2& re, double2& im) {
   const double2* p = reinterpret_cast<const double2*>(base) + ((size_t)c * NP + m) * 2;
-  re = __ldg(p);
-  im = __ldg(p + 1);
+  re = p[0];
+  im = p[1];
 }
 __device__ __forceinline__ void store_comp(float* base, size_t m, size_t NP, int c, float2 re, float2 im) {
   reinterpret_cast<float4*>(base)[(size_t)c * NP + m] = make_float4(re.x, re.y, im.x, im.y);

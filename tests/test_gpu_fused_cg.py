@@ -3,7 +3,7 @@ other launches (all comparisons bitwise unless a tolerance is stated)."""
 import pytest
 import torch
 
-from synthetic import gaussian_source4d
+from synthetic import gaussian_half5d, gaussian_source4d
 
 from gpu_common import make_case
 
@@ -42,3 +42,42 @@ def test_staged_solve_matches_direct_loads(prec, monkeypatch):
     staged = _solve(sysm, src, precision_inner=prec)
     assert staged[1] == direct[1]
     assert torch.equal(torch.view_as_real(staged[0]), torch.view_as_real(direct[0]))
+
+
+@pytest.mark.parametrize("L,prec,nrhs,zeros", [((12, 12, 12, 12), 1, 1, ()), ((8, 8, 8, 8), 2, 24, range(2, 22)),
+                                               ((8, 8, 8, 8), 1, 6, (0, 3))])
+def test_kernels_that_start_ahead_match_plain_launches(L, prec, nrhs, zeros, monkeypatch):
+    """Solves whose CG kernels start ahead of the end of the one before (2592, 12288 and 3072
+    warps an iteration, above the 2432 of the rule) against launches one after the other.  Zero
+    sources are converged from the start: their CTAs leave at once, down to 4 active sources of
+    24, whose CTAs fill the GPU less than once."""
+    sysm = make_case(L, 16, "mobius", alpha=1.2, m=0.1)
+    src = torch.stack([torch.from_numpy(gaussian_source4d(L, seed=1 + k)) for k in range(nrhs)]).cuda()
+    for k in zeros:
+        src[k].zero_()
+    monkeypatch.setenv("DWF_HOP_TILE", "default")
+    kw = dict(precision_inner=prec, rhs_block=nrhs)
+    ahead = _solve(sysm, src, nrhs, **kw)
+    monkeypatch.setenv("DWF_NO_AHEAD", "1")
+    plain = _solve(sysm, src, nrhs, **kw)
+    assert ahead[1] == plain[1]
+    assert torch.equal(torch.view_as_real(ahead[0]), torch.view_as_real(plain[0]))
+
+
+def test_normal_solve_ahead_matches_plain_launches(monkeypatch):
+    """The same for the CG on D_bb^+ D_bb (12^4, Ls = 16: 2592 warps)."""
+    L, Ls = (12, 12, 12, 12), 16
+    sysm = make_case(L, Ls, "mobius", alpha=1.2, m=0.1)
+    phi = torch.from_numpy(gaussian_half5d(L, Ls, seed=3)).cuda()
+    res = []
+    for plain in (False, True):
+        if plain:
+            monkeypatch.setenv("DWF_NO_AHEAD", "1")
+        op = _op(sysm, rel_tol=1e-8)
+        x = torch.empty_like(phi)
+        st = op.solve_normal(x, phi)
+        torch.cuda.synchronize()
+        res.append((st["iterations"], st["true_resid"], x))
+        op.close()
+    assert res[0][:2] == res[1][:2]
+    assert torch.equal(torch.view_as_real(res[0][2]), torch.view_as_real(res[1][2]))

@@ -390,7 +390,8 @@ cudaError_t tuned(const Geom& g, const Launch& L, cudaStream_t st) {
 cudaError_t launch_hop(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   const cudaError_t e = tuned(g, L, st);
   if (e != cudaErrorNotSupported) return e;
-  if (L.extra) return cudaErrorInvalidValue;
+  // the generic kernel has neither the extra steps nor the clearing of bins
+  if (L.extra || L.zero[0] || L.zero[1] || (L.red && L.red->bins)) return cudaErrorInvalidValue;
   switch (L.prec) {
     case P64: return dispatch_hop<Store64>(g, L, st);
     case P32: return dispatch_hop<Store32>(g, L, st);

@@ -1182,7 +1182,6 @@ template <class SP, int LS, int PRE, int POST, int LOC, bool G5, bool NORM>
 cudaError_t run_tma(const Geom& g, const HopLaunch& L, const Args<typename SP::T>& a, cudaStream_t st) {
   constexpr int NST = tma_stages<SP, LS>();
   constexpr int S = kTmaConsumers / (LS / 2);
-  if (((reinterpret_cast<uintptr_t>(L.v) | L.stride) & 15) != 0) return cudaErrorNotSupported;
   CUtensorMap map;
   cudaError_t e = encode_field_map<SP, LS>(&map, g, L.v, L.stride, L.nrhs);
   if (e != cudaSuccess) return e;
@@ -1231,7 +1230,11 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   a.zero[0] = L.zero[0];
   a.zero[1] = L.zero[1];
   if constexpr (tma_ls(LS) && POST != PR_NONE && EX == EX_NONE) {
-    if (L.use_tma) return run_tma<SP, LS, PRE, POST, LOC, G5, NORM>(g, L, a, st);
+    if (L.use_tma) {
+      if (((reinterpret_cast<uintptr_t>(L.v) | L.stride) & 15) != 0) return cudaErrorNotSupported;
+      const cudaError_t e = run_tma<SP, LS, PRE, POST, LOC, G5, NORM>(g, L, a, st);
+      if (e != cudaErrorNotSupported) return e;  // no tensor map to be had: direct loads
+    }
   }
   if constexpr (!SP::kScaled) {
     if (L.block_threads == 0 && split_directions(LS, g.Vh, std::max(L.nrhs, L.rule_nrhs), sizeof(T) == 8)) {

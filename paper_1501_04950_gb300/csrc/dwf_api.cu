@@ -563,7 +563,7 @@ int apply_hop64(dwf_ctx* h, const CoefView& cv, int p, void* out, const void* v,
 int apply_dbb(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* in, void* tmp, int nrhs,
               const Reduce* norm, cudaStream_t s) {
   const MatSet& ms = *cv.layout;
-  if (prec == P64 && cv.tuned(P64)) {
+  if (prec == P64 && cv.tuned(P64) && fields_aligned(out, in)) {
     // FP64 is bound by the FP64 pipe: B folded into the 8 hops of pass A is 384 of
     // its ~1370 operations per 5D site, formed once it is 48.  out holds B in until
     // pass B overwrites it.  16^3x32, Ls = 16:

@@ -52,8 +52,41 @@ size_t tile_bytes(int Ls, int sites, size_t ts, int nfields) {
   return (size_t)sites * Ls * (kTileStride * ts + sizeof(float)) * nfields;
 }
 
+// 16 bytes of an internal field by one access (WIDE), or by accesses of one element for a
+// caller's field that does not start on a 16-byte boundary.
+template <bool WIDE>
+__device__ __forceinline__ void put16(void* p, uint4 v) {
+  if (WIDE) {
+    *reinterpret_cast<uint4*>(p) = v;
+  } else {
+    uint32_t* q = reinterpret_cast<uint32_t*>(p);
+    q[0] = v.x; q[1] = v.y; q[2] = v.z; q[3] = v.w;
+  }
+}
+template <bool WIDE>
+__device__ __forceinline__ void put16(void* p, double2 v) {
+  if (WIDE) {
+    *reinterpret_cast<double2*>(p) = v;
+  } else {
+    reinterpret_cast<double*>(p)[0] = v.x;
+    reinterpret_cast<double*>(p)[1] = v.y;
+  }
+}
+template <bool WIDE>
+__device__ __forceinline__ uint4 get16(const uint4* p) {
+  if (WIDE) return __ldg(p);
+  const uint32_t* q = reinterpret_cast<const uint32_t*>(p);
+  return make_uint4(__ldg(q), __ldg(q + 1), __ldg(q + 2), __ldg(q + 3));
+}
+template <bool WIDE>
+__device__ __forceinline__ double2 get16(const double2* p) {
+  if (WIDE) return __ldg(p);
+  const double* q = reinterpret_cast<const double*>(p);
+  return make_double2(__ldg(q), __ldg(q + 1));
+}
+
 // Tile -> internal half-field (n5 = 5D sites of the tile, first one at n0; both even).
-template <class SP>
+template <class SP, bool WIDE>
 __device__ __forceinline__ void tile_store(void* dst, const typename SP::T* tile, float* scale, int n0,
                                            int n5, int N5, int tid, int nth) {
   using T = typename SP::T;
@@ -72,9 +105,9 @@ __device__ __forceinline__ void tile_store(void* dst, const typename SP::T* tile
       const T* a = tile + 2 * m * kTileStride + 4 * j;
       const T* b = a + kTileStride;
       const float ia = 1.f / scale[2 * m], ib = 1.f / scale[2 * m + 1];
-      reinterpret_cast<uint4*>(dst)[j * NP + m0 + m] =
-          make_uint4(SP::from_f2(make_float2(a[0] * ia, b[0] * ib)), SP::from_f2(make_float2(a[1] * ia, b[1] * ib)),
-                     SP::from_f2(make_float2(a[2] * ia, b[2] * ib)), SP::from_f2(make_float2(a[3] * ia, b[3] * ib)));
+      put16<WIDE>(reinterpret_cast<uint4*>(dst) + j * NP + m0 + m,
+                  make_uint4(SP::from_f2(make_float2(a[0] * ia, b[0] * ib)), SP::from_f2(make_float2(a[1] * ia, b[1] * ib)),
+                             SP::from_f2(make_float2(a[2] * ia, b[2] * ib)), SP::from_f2(make_float2(a[3] * ia, b[3] * ib))));
     }
     for (int n = tid; n < n5; n += nth) const_cast<float*>(SP::scales(dst, N5))[n0 + n] = scale[n];
   } else {
@@ -84,17 +117,18 @@ __device__ __forceinline__ void tile_store(void* dst, const typename SP::T* tile
       const T* b = a + kTileStride;
       if constexpr (sizeof(T) == 8) {
         double2* o = reinterpret_cast<double2*>(dst) + (c * NP + m0 + m) * 2;
-        o[0] = make_double2(a[0], b[0]);
-        o[1] = make_double2(a[1], b[1]);
+        put16<WIDE>(o, make_double2(a[0], b[0]));
+        put16<WIDE>(o + 1, make_double2(a[1], b[1]));
       } else {
-        reinterpret_cast<float4*>(dst)[c * NP + m0 + m] = make_float4(a[0], b[0], a[1], b[1]);
+        put16<WIDE>(reinterpret_cast<uint4*>(dst) + c * NP + m0 + m,
+                    make_uint4(__float_as_uint(a[0]), __float_as_uint(b[0]), __float_as_uint(a[1]), __float_as_uint(b[1])));
       }
     }
   }
 }
 
 // Internal half-field -> tile.
-template <class SP>
+template <class SP, bool WIDE>
 __device__ __forceinline__ void tile_load(typename SP::T* tile, const void* src, int n0, int n5, int N5,
                                           int tid, int nth) {
   using T = typename SP::T;
@@ -103,7 +137,7 @@ __device__ __forceinline__ void tile_load(typename SP::T* tile, const void* src,
   if constexpr (SP::kScaled) {
     for (int i = tid; i < 6 * np; i += nth) {
       const int j = i / np, m = i - j * np;
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(src) + j * NP + m0 + m);
+      const uint4 v = get16<WIDE>(reinterpret_cast<const uint4*>(src) + j * NP + m0 + m);
       const float* sc = SP::scales(src, N5) + n0 + 2 * m;
       const float sa = __ldg(sc), sb = __ldg(sc + 1);
       T* a = tile + 2 * m * kTileStride + 4 * j;
@@ -123,18 +157,18 @@ __device__ __forceinline__ void tile_load(typename SP::T* tile, const void* src,
       T* b = a + kTileStride;
       if constexpr (sizeof(T) == 8) {
         const double2* q = reinterpret_cast<const double2*>(src) + (c * NP + m0 + m) * 2;
-        const double2 re = __ldg(q), im = __ldg(q + 1);
+        const double2 re = get16<WIDE>(q), im = get16<WIDE>(q + 1);
         a[0] = re.x; b[0] = re.y; a[1] = im.x; b[1] = im.y;
       } else {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(src) + c * NP + m0 + m);
-        a[0] = v.x; b[0] = v.y; a[1] = v.z; b[1] = v.w;
+        const uint4 v = get16<WIDE>(reinterpret_cast<const uint4*>(src) + c * NP + m0 + m);
+        a[0] = __uint_as_float(v.x); b[0] = __uint_as_float(v.y); a[1] = __uint_as_float(v.z); b[1] = __uint_as_float(v.w);
       }
     }
   }
 }
 
 // Canonical half-field(s) [nrhs][Ls][Vh][12] <-> internal, `sites` sites per CTA.
-template <class SP, bool PACK>
+template <class SP, bool PACK, bool WIDE>
 __global__ void __launch_bounds__(kBlasThreads) half_kernel(const Geom g, void* field, double* canon,
                                                             size_t stride, int sites, int tiles) {
   using T = typename SP::T;
@@ -147,7 +181,7 @@ __global__ void __launch_bounds__(kBlasThreads) half_kernel(const Geom g, void* 
   double2* c = reinterpret_cast<double2*>(canon) + (size_t)rhs * g.N5 * 12;
   const int run = nh * 12;  // components of one slice of the tile
   if (!PACK) {
-    tile_load<SP>(tile, f, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
+    tile_load<SP, WIDE>(tile, f, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
     __syncthreads();
   }
   for (int i = tid; i < run * g.Ls; i += nth) {
@@ -164,7 +198,7 @@ __global__ void __launch_bounds__(kBlasThreads) half_kernel(const Geom g, void* 
   }
   if (PACK) {
     __syncthreads();
-    tile_store<SP>(f, tile, scale, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
+    tile_store<SP, WIDE>(f, tile, scale, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
   }
 }
 
@@ -188,8 +222,8 @@ __global__ void __launch_bounds__(kBlasThreads) full_kernel(const Geom g, void* 
   const int run = 2 * nh * 12;
   const size_t V = (size_t)g.Vh * 2;
   if (!SPLIT) {
-    tile_load<Store64>(tile, p0, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
-    tile_load<Store64>(tile + per, p1, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
+    tile_load<Store64, true>(tile, p0, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
+    tile_load<Store64, true>(tile + per, p1, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
     __syncthreads();
   }
   for (int i = tid; i < run * g.Ls; i += nth) {
@@ -207,8 +241,8 @@ __global__ void __launch_bounds__(kBlasThreads) full_kernel(const Geom g, void* 
   }
   if (SPLIT) {
     __syncthreads();
-    tile_store<Store64>(p0, tile, nullptr, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
-    tile_store<Store64>(p1, tile + per, nullptr, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
+    tile_store<Store64, true>(p0, tile, nullptr, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
+    tile_store<Store64, true>(p1, tile + per, nullptr, h0 * g.Ls, nh * g.Ls, g.N5, tid, nth);
   }
 }
 
@@ -695,8 +729,8 @@ void run_half(const Geom& g, void* field, double* canon, int nrhs, size_t stride
   const size_t ts = sizeof(typename SP::T);
   const int sites = tile_sites(g.Ls, ts, 1);
   const int tiles = (g.Vh + sites - 1) / sites;
-  half_kernel<SP, PACK><<<(unsigned)tiles * nrhs, kBlasThreads, tile_bytes(g.Ls, sites, ts, 1), s>>>(
-      g, field, canon, stride, sites, tiles);
+  auto k = (reinterpret_cast<uintptr_t>(field) & 15) == 0 ? half_kernel<SP, PACK, true> : half_kernel<SP, PACK, false>;
+  k<<<(unsigned)tiles * nrhs, kBlasThreads, tile_bytes(g.Ls, sites, ts, 1), s>>>(g, field, canon, stride, sites, tiles);
 }
 
 cudaError_t launch_pack_half(const Geom& g, int prec, void* dst, const double* src, int nrhs,

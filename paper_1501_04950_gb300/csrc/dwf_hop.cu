@@ -373,9 +373,15 @@ cudaError_t tuned_of(const Geom& g, const Launch& L, cudaStream_t st) {
     default: return hop2::dispatch<SP, 3>(g, L, st);
   }
 }
+// The tuned kernels move 16 bytes an access: a caller's field that starts elsewhere takes the
+// generic ones, whose accesses are single elements.
+bool aligned(const HopLaunch& L) { return fields_aligned(L.out, L.v) && fields_aligned(L.w, L.out2); }
+bool aligned(const LocalLaunch& L) { return fields_aligned(L.out, L.in); }
+bool aligned(const RUpdateLaunch&) { return true; }  // fields of the solver's own
+
 template <class Launch>
 cudaError_t tuned(const Geom& g, const Launch& L, cudaStream_t st) {
-  if (g_disable_tuned) return cudaErrorNotSupported;
+  if (g_disable_tuned || !aligned(L)) return cudaErrorNotSupported;
   switch (L.prec) {
     case P64: return tuned_of<Store64>(g, L, st);
     case P32: return tuned_of<Store32>(g, L, st);
@@ -406,6 +412,7 @@ cudaError_t launch_rupdate(const Geom& g, const RUpdateLaunch& L, cudaStream_t s
 cudaError_t launch_local(const Geom& g, const LocalLaunch& L, cudaStream_t st) {
   const cudaError_t e = tuned(g, L, st);
   if (e != cudaErrorNotSupported) return e;
+  if (!L.m) return cudaErrorInvalidValue;  // no dense matrix for the generic kernel
   switch (L.prec) {
     case P64: return run_local<Store64>(g, L, st);
     case P32: return run_local<Store32>(g, L, st);

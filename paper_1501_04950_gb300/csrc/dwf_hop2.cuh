@@ -1231,7 +1231,6 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   a.zero[1] = L.zero[1];
   if constexpr (tma_ls(LS) && POST != PR_NONE && EX == EX_NONE) {
     if (L.use_tma) {
-      if (((reinterpret_cast<uintptr_t>(L.v) | L.stride) & 15) != 0) return cudaErrorNotSupported;
       const cudaError_t e = run_tma<SP, LS, PRE, POST, LOC, G5, NORM>(g, L, a, st);
       if (e != cudaErrorNotSupported) return e;  // no tensor map to be had: direct loads
     }

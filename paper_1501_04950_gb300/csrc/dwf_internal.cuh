@@ -191,6 +191,11 @@ cudaError_t launch_x_update(const Geom& g, int prec, int xprec, void* x, const v
                             const double* a_ptr, int sstride, int nrhs, size_t stride_x,
                             size_t stride, cudaStream_t s, const int* active);
 
+// Whether both fields (nullptr: none) start on the 16-byte boundary that the tuned kernels need.
+inline bool fields_aligned(const void* a, const void* b) {
+  return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
+}
+
 // Set to 1 to force the generic kernels (tests compare both paths).
 extern int g_disable_tuned;
 

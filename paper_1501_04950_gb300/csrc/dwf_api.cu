@@ -717,15 +717,16 @@ int apply_local_dense(dwf_ctx* h, const CoefView& cv, int prec, int which, void*
 }
 
 // (out0, out1) = D_alpha(ms) (in0, in1) = I in - 1/2 H (B in), FP64 internal halves by parity.
-int apply_dalpha_halves(dwf_ctx* h, const MatSet& ms, void* out[2], const void* in[2], cudaStream_t s) {
+// bv: a half-field of scratch (B in; tuned kernels only); a solve, which runs on the handle's stream, passes one of
+// its own, so that it does not meet a caller's D_alpha on another stream.
+int apply_dalpha_halves(dwf_ctx* h, const MatSet& ms, void* out[2], const void* in[2], void* bv,
+                        cudaStream_t s) {
   const CoefView cv = view_of(ms);
   if (cv.tuned(P64)) {
     // I and B as recurrences (144 flops a 5D site each), once per site: folded into the
     // hops and as a dense contraction they were 384 + 24 Ls of the ~1270 FP64
     // operations of a site at Ls = 16
-    void* bv;
-    int rc = get_ws(h, "da_b", field_bytes(h->g, P64), &bv);
-    if (rc) return rc;
+    int rc;
     for (int p = 0; p < 2; p++)
       if ((rc = apply_prog64(h, cv, hop2::PR_B, bv, in[1 - p], 1, s)) ||
           (rc = apply_prog64(h, cv, hop2::PR_I, out[p], in[p], 1, s)) ||
@@ -1909,14 +1910,15 @@ int dwf_apply_dalpha(dwf_handle h, double* out_full, const double* in_full, doub
   int rc = build_matset(h, alpha, m, &ms);
   if (rc) return rc;
   const size_t f64 = field_bytes(h->g, P64);
-  void *i0, *i1, *o0, *o1;
+  void *i0, *i1, *o0, *o1, *bv = nullptr;
   if ((rc = get_ws(h, "da_i0", f64, &i0)) || (rc = get_ws(h, "da_i1", f64, &i1)) ||
-      (rc = get_ws(h, "da_o0", f64, &o0)) || (rc = get_ws(h, "da_o1", f64, &o1)))
+      (rc = get_ws(h, "da_o0", f64, &o0)) || (rc = get_ws(h, "da_o1", f64, &o1)) ||
+      (view_of(*ms).tuned(P64) && (rc = get_ws(h, "da_b", f64, &bv))))
     return rc;
   KLAUNCH(h, launch_split_full(h->g, i0, i1, in_full, st));
   void* outs[2] = {o0, o1};
   const void* ins[2] = {i0, i1};
-  if ((rc = apply_dalpha_halves(h, *ms, outs, ins, st))) return rc;
+  if ((rc = apply_dalpha_halves(h, *ms, outs, ins, bv, st))) return rc;
   KLAUNCH(h, launch_merge_full(h->g, out_full, o0, o1, st));
   return DWF_OK;
 }
@@ -2112,7 +2114,7 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
     }
     KLAUNCH(h, launch_source_pb(g, pb[0], pb[1], src_k, st));
     const void* pbc[2] = {pb[0], pb[1]};
-    return apply_dalpha_halves(h, *rhs_set, rhs, pbc, st);
+    return apply_dalpha_halves(h, *rhs_set, rhs, pbc, W.t64, st);
   };
   int result = DWF_OK;
   for (int blk = 0; blk < nrhs; blk += nb) {
@@ -2200,7 +2202,7 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
       if (sol5d) KLAUNCH(h, launch_merge_full(g, sol5d + (size_t)k * g.N5 * 2 * 24, psi[0], psi[1], st));
       // full 5D residual |rhs - D_alpha psi| / |rhs|
       const void* psic[2] = {psi[0], psi[1]};
-      if ((rc = apply_dalpha_halves(h, m, tmp5, psic, st))) return rc;
+      if ((rc = apply_dalpha_halves(h, m, tmp5, psic, W.t64, st))) return rc;
       Reduce r0 = make_reduce(h, 0, S_T0), r1 = make_reduce(h, 1, S_T1);
       Reduce n0 = make_reduce(h, 2, S_T2), n1 = make_reduce(h, 3, S_ZZ0);
       KLAUNCH(h, launch_sub64_norm(g, tmp5[0], rhs[0], tmp5[0], 1, f64, &r0, st));

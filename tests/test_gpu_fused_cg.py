@@ -81,3 +81,27 @@ def test_normal_solve_ahead_matches_plain_launches(monkeypatch):
         op.close()
     assert res[0][:2] == res[1][:2]
     assert torch.equal(torch.view_as_real(res[0][2]), torch.view_as_real(res[1][2]))
+
+
+def test_dalpha_on_another_stream_than_a_solve():
+    """D_alpha on a caller's stream while a solve of the same handle runs on the handle's: no
+    workspace in common (both form B v), so both give what they give one after the other."""
+    L, Ls = (8, 8, 8, 8), 8
+    sysm = make_case(L, Ls, "mobius", alpha=1.2, m=0.3)
+    op = _op(sysm, rhs_block=1)
+    src = torch.stack([torch.from_numpy(gaussian_source4d(L, seed=1 + k)) for k in range(4)]).cuda()
+    g = torch.Generator(device="cuda").manual_seed(1)
+    full = torch.view_as_complex(torch.randn(Ls, *L[::-1], 4, 3, 2, dtype=torch.float64, device="cuda", generator=g))
+    prop, prop_ref, ref = torch.empty_like(src), torch.empty_like(src), torch.empty_like(full)
+    op.apply_dalpha(ref, full, 0.8, 0.2)
+    op.cgne_solve(src, prop_ref, nrhs=4)
+    torch.cuda.synchronize()
+    outs = [torch.empty_like(full) for _ in range(300)]
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        for out in outs:   # about 0.3 ms each: they are under way while the solve forms its right-hand sides
+            op.apply_dalpha(out, full, 0.8, 0.2)
+    op.cgne_solve(src, prop, nrhs=4)
+    torch.cuda.synchronize()
+    assert torch.equal(torch.view_as_real(prop), torch.view_as_real(prop_ref))
+    assert all(torch.equal(torch.view_as_real(out), torch.view_as_real(ref)) for out in outs)

@@ -326,8 +326,31 @@ __device__ __forceinline__ void project_half(HalfP<typename Pr<T>::V>& P, const 
   }
 }
 
-// chi_k = U' h_k, acc_upper(k) += f chi_k, acc_lower(pk) += f rs (i) chi_k for the half
-// spinor h = P; U' = U (dir > 0) or U^+ (dir < 0).
+// Component a of chi_k = U' h_k for the half spinor h = P; U' = U (dir > 0) or U^+ (dir < 0).
+template <typename T, int DIR>
+__device__ __forceinline__ void link_row(const HalfP<typename Pr<T>::V>& P, const Link<T>& U, int k, int a,
+                                         typename Pr<T>::V& cr, typename Pr<T>::V& ci) {
+  using A = Pr<T>;
+  using V = typename A::V;
+#pragma unroll
+  for (int b = 0; b < 3; b++) {
+    const cplx<T> u = DIR > 0 ? U.u[3 * a + b] : U.u[3 * b + a];
+    const V ur = A::dup(u.re);
+    const V ui = A::dup(DIR > 0 ? u.im : -u.im);
+    const V hr = P.re[3 * k + b], hi = P.im[3 * k + b];
+    if (b == 0) {
+      cr = A::mul(ur, hr);
+      ci = A::mul(ur, hi);
+    } else {
+      cr = A::fma(ur, hr, cr);
+      ci = A::fma(ur, hi, ci);
+    }
+    cr = A::fma(A::neg(ui), hi, cr);
+    ci = A::fma(ui, hr, ci);
+  }
+}
+
+// chi_k = U' h_k, acc_upper(k) += f chi_k, acc_lower(pk) += f rs (i) chi_k.
 template <class SP, int MU, int DIR>
 __device__ __forceinline__ void mul_acc(const HalfP<typename Pr<typename SP::T>::V>& P,
                                         const Link<typename SP::T>& U,
@@ -337,7 +360,6 @@ __device__ __forceinline__ void mul_acc(const HalfP<typename Pr<typename SP::T>:
   using A = Pr<T>;
   using V = typename A::V;
   const V fn = A::neg(f);
-  // chi_k = U' h_k; acc_upper(k) += f chi_k; acc_lower(pk) += f rs (i) chi_k
 #pragma unroll
   for (int k = 0; k < 2; k++) {
     const int q = partner(MU, k);  // lower row fed by chi_k
@@ -345,22 +367,7 @@ __device__ __forceinline__ void mul_acc(const HalfP<typename Pr<typename SP::T>:
 #pragma unroll
     for (int a = 0; a < 3; a++) {
       V cr, ci;
-#pragma unroll
-      for (int b = 0; b < 3; b++) {
-        const cplx<T> u = DIR > 0 ? U.u[3 * a + b] : U.u[3 * b + a];
-        const V ur = A::dup(u.re);
-        const V ui = A::dup(DIR > 0 ? u.im : -u.im);
-        const V hr = P.re[3 * k + b], hi = P.im[3 * k + b];
-        if (b == 0) {
-          cr = A::mul(ur, hr);
-          ci = A::mul(ur, hi);
-        } else {
-          cr = A::fma(ur, hr, cr);
-          ci = A::fma(ur, hi, ci);
-        }
-        cr = A::fma(A::neg(ui), hi, cr);
-        ci = A::fma(ui, hr, ci);
-      }
+      link_row<T, DIR>(P, U, k, a, cr, ci);
       acc.re[3 * k + a] = A::fma(f, cr, acc.re[3 * k + a]);
       acc.im[3 * k + a] = A::fma(f, ci, acc.im[3 * k + a]);
       const int l = 6 + 3 * q + a;
@@ -377,6 +384,14 @@ __device__ __forceinline__ void mul_acc(const HalfP<typename Pr<typename SP::T>:
 
 // 32 / G sites fill a warp.
 __host__ __device__ constexpr bool warp_groups(int Ls) { return 32 % (Ls / 2) == 0; }
+
+// v or -v by its sign bit (the FP64 pipe takes no part)
+__device__ __forceinline__ float signed_by(bool neg, float v) {
+  return __uint_as_float(__float_as_uint(v) ^ (neg ? 0x80000000u : 0u));
+}
+__device__ __forceinline__ double signed_by(bool neg, double v) {
+  return __hiloint2double(__double2hiint(v) ^ (neg ? (int)0x80000000u : 0), __double2loint(v));
+}
 
 __device__ __forceinline__ float lane_of(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 __device__ __forceinline__ double lane_of(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
@@ -400,8 +415,9 @@ struct MemSrc {
 
 // acc += f (1 - dir gamma_mu) U' v'(x +- mu) for the two slices of a thread,
 // U' = U_mu(x) (dir > 0) or U_mu(x - mu)^+ (dir < 0).  With PRE_B the G threads of a site
-// are neighbouring lanes and every thread of the warp calls it.
-template <class SP, int LS, int PRE, int MU, int DIR, class Src>
+// are neighbouring lanes and every thread of the warp calls it.  With CHI the hop's f chi
+// goes to components 0 .. 5 (dir > 0) or 6 .. 11 of acc instead of being added up.
+template <class SP, int LS, int PRE, int MU, int DIR, bool CHI, class Src>
 __device__ __forceinline__ void hop_from(const Src& src, bool neg, int t, const typename SP::T (&bd)[2][2],
                                          const typename SP::T (&bo)[2][2],
                                          SpinP<typename Pr<typename SP::T>::V>& acc) {
@@ -441,11 +457,25 @@ __device__ __forceinline__ void hop_from(const Src& src, bool neg, int t, const 
   Link<T> U;
   src.template link<MU>(U);
   project_half<T, MU, DIR>(P, M);
-  mul_acc<SP, MU, DIR>(P, U, f, acc);
+  if constexpr (CHI) {
+    static_assert(!SP::kScaled, "f is a sign here");
+#pragma unroll
+    for (int k = 0; k < 2; k++)
+#pragma unroll
+      for (int a = 0; a < 3; a++) {
+        V cr, ci;
+        link_row<T, DIR>(P, U, k, a, cr, ci);
+        const int c = (DIR > 0 ? 0 : 6) + 3 * k + a;
+        acc.re[c] = A::mk(signed_by(neg, cr.x), signed_by(neg, cr.y));
+        acc.im[c] = A::mk(signed_by(neg, ci.x), signed_by(neg, ci.y));
+      }
+  } else {
+    mul_acc<SP, MU, DIR>(P, U, f, acc);
+  }
 }
 
 // The same from memory: neighbour entry nb of site h.
-template <class SP, int LS, int PRE, int MU, int DIR>
+template <class SP, int LS, int PRE, int MU, int DIR, bool CHI = false>
 __device__ __forceinline__ void hop_dir(int nb, int h, int t, size_t NP,
                                         const typename SP::T (&bd)[2][2],
                                         const typename SP::T (&bo)[2][2], const void* v,
@@ -453,7 +483,7 @@ __device__ __forceinline__ void hop_dir(int nb, int h, int t, size_t NP,
                                         SpinP<typename Pr<typename SP::T>::V>& acc) {
   const int hn = nb & 0x7fffffff;
   const MemSrc<SP> src{v, (size_t)hn * (LS / 2) + t, NP, DIR > 0 ? gp : gq, DIR > 0 ? h : hn};
-  hop_from<SP, LS, PRE, MU, DIR>(src, nb < 0, t, bd, bo, acc);
+  hop_from<SP, LS, PRE, MU, DIR, CHI>(src, nb < 0, t, bd, bo, acc);
 }
 
 // One step's coefficients (4-vector) of a sweep.
@@ -646,16 +676,6 @@ __device__ __forceinline__ void zero(SpinP<V>& a) {
     a.re[c].y = 0;
     a.im[c].x = 0;
     a.im[c].y = 0;
-  }
-}
-
-template <typename V>
-__device__ __forceinline__ void add(SpinP<V>& a, const SpinP<V>& b) {
-  using A = Pr<decltype(a.re[0].x)>;
-#pragma unroll
-  for (int c = 0; c < 12; c++) {
-    a.re[c] = A::add(a.re[c], b.re[c]);
-    a.im[c] = A::add(a.im[c], b.im[c]);
   }
 }
 
@@ -867,29 +887,82 @@ __device__ __forceinline__ void store_comp(double* base, size_t m, size_t NP, in
   p[1] = im;
 }
 
-// run_prog for 128 threads on nsites <= 32 / (LS / 2) sites whose input is the sum of
-// NPART blocks, `part_stride` apart; the result replaces the first block.
-template <typename T, int LS, int PROG, int NPART>
-__device__ __forceinline__ void run_prog_sum(T* sbuf, int part_stride, const T* coef, int tid, int nsites) {
-  constexpr int NIT = (12 * (32 / (LS / 2)) + 63) / 64;
+// Where hop_split_kernel adds up the hops of a site.  FP32: on the way into the sweeps, direction
+// x's warp having added up its own two (they come first in the order of the sum), which leaves
+// one block less to read.  FP64 (sum_lanes): by the lanes of all four warps in a step of its own,
+// 96 additions a thread; the sweeps fill few lanes (Ls = 32: 24 of 64), and an instruction of the
+// FP64 pipe costs the same however many lanes are on.  D_bb + D_bb^+ (CUDA graph), by lanes / on
+// the way into the sweeps: FP64 4^3x8, Ls = 32 115 / 132 us, 8x4x4x8, Ls = 10 105 / 110; FP32
+// 8^3x16, Ls = 8 30.7 / 25.8, 8^4, Ls = 16 26.2 / 25.0.
+template <typename T>
+__host__ __device__ constexpr bool sums_in_sweeps() { return sizeof(T) == 4; }
+
+// The sweep of component R of chirality CH from what the four warps left of the eight hops of a
+// site (blocks part_stride apart; direction x's sum as put leaves it, then put_hops: f chi of the
+// hop to x + mu, f chi of that to x - mu, pairs in the sweep order of chirality 0).  The hops
+// are added up one after the other as hop_kernel does, so that both kernels give the same bits:
+// the upper rows of (1 -+ gamma_mu) U' v' are chi, the lower ones rs (i) chi of the partner row
+// (mul_acc).
+template <typename T, int LS, int CH>
+__device__ __forceinline__ void sum_hops(T (&V)[LS], const T* site, int part_stride, int R) {
+  using A = Pr<T>;
+  constexpr int G = LS / 2;
+  const int row = R / 6, col = R - 6 * row;  // spin row, 2 colour + (re | im)
+  const T* at[4];
+  T sg[4];
+#pragma unroll
+  for (int mu = 1; mu < 4; mu++) {
+    const int rs = row == 0 ? recon_sign(mu, +1, 0) : recon_sign(mu, +1, 1);
+    // += rs i chi: re takes -rs im, im takes rs re
+    sg[mu] = (T)(imag_mu(mu) && !(col & 1) ? -rs : rs);
+    at[mu] = site + mu * part_stride + 2 * (CH == 0 ? R : 6 * partner(mu, row) + (imag_mu(mu) ? col ^ 1 : col));
+  }
+#pragma unroll
+  for (int k = 0; k < G; k++) {
+    const int o = (CH == 0 ? k : G - 1 - k) * kPairStride;
+    const auto x = pair_at(site + 24 * CH + 2 * R + k * kPairStride);
+    auto v = CH == 0 ? x : A::mk(x.y, x.x);
+#pragma unroll
+    for (int mu = 1; mu < 4; mu++) {
+      const auto f = pair_at(at[mu] + o), b = pair_at(at[mu] + o + 24);
+      v = CH == 0 ? A::add(v, f) : A::fma(A::dup(sg[mu]), f, v);
+      v = CH == 0 ? A::add(v, b) : A::fma(A::dup(-sg[mu]), b, v);
+    }
+    V[2 * k] = CH == 0 ? v.x : v.y;
+    V[2 * k + 1] = CH == 0 ? v.y : v.x;
+  }
+}
+
+// run_prog for 128 threads on nsites <= 32 / (LS / 2) sites, with HOPS on the sums of sum_hops.
+// The result goes to the first block, in the layout of put.
+template <typename T, int LS, int PROG, bool HOPS>
+__device__ __forceinline__ void run_prog_split(T* sbuf, int part_stride, const T* coef, int tid, int nsites) {
+  using A = Pr<T>;
+  constexpr int G = LS / 2;
+  constexpr int NIT = (12 * (32 / G) + 63) / 64;
   const int ch = tid >> 6;
   T V[NIT][LS];
 #pragma unroll
   for (int q = 0; q < NIT; q++) {
-    const int i = (tid & 63) + 64 * q, site = i / 12;
-    const T* p = sbuf + site * site_stride(LS) + 24 * ch + 2 * (i - 12 * site);
+    const int i = (tid & 63) + 64 * q, site = i / 12, R = i - 12 * site;
+    const T* p = sbuf + site * site_stride(LS);
+    if (i >= 12 * nsites) {
 #pragma unroll
-    for (int k = 0; k < LS / 2; k++) {
-      V[q][2 * k] = V[q][2 * k + 1] = (T)0;
-      if (i < 12 * nsites) {
-        auto v = pair_at(p + k * kPairStride);
+      for (int k = 0; k < LS; k++) V[q][k] = (T)0;
+    } else if (!HOPS) {
 #pragma unroll
-        for (int b = 1; b < NPART; b++) v = Pr<T>::add(v, pair_at(p + b * part_stride + k * kPairStride));
+      for (int k = 0; k < G; k++) {
+        const auto v = pair_at(p + 24 * ch + 2 * R + k * kPairStride);
         V[q][2 * k] = v.x;
         V[q][2 * k + 1] = v.y;
       }
+    } else if (ch == 0) {
+      sum_hops<T, LS, 0>(V[q], p, part_stride, R);
+    } else {
+      sum_hops<T, LS, 1>(V[q], p, part_stride, R);
     }
   }
+  // the result overwrites the first block, where a thread has read only what it writes
 #pragma unroll
   for (int i = 0; i < prog_len(PROG); i++) {
     const T* c = coef + (2 * i + ch) * chain_stride(LS);
@@ -902,13 +975,65 @@ __device__ __forceinline__ void run_prog_sum(T* sbuf, int part_stride, const T* 
     T* p = sbuf + site * site_stride(LS) + 24 * ch + 2 * (i - 12 * site);
     if (i < 12 * nsites)
 #pragma unroll
-      for (int k = 0; k < LS / 2; k++)
-        *reinterpret_cast<typename Pr<T>::V*>(p + k * kPairStride) = Pr<T>::mk(V[q][2 * k], V[q][2 * k + 1]);
+      for (int k = 0; k < G; k++)
+        *reinterpret_cast<typename A::V*>(p + k * kPairStride) = A::mk(V[q][2 * k], V[q][2 * k + 1]);
+  }
+}
+
+// Slice pair t of a site into shared memory, all components in the sweep order of PROG's chirality 0.
+template <typename T, int LS, int PROG>
+__device__ __forceinline__ void put_hops(T* site, int t, const SpinP<typename Pr<T>::V>& a) {
+  static_assert(prog_reversed(PROG, 0) != prog_reversed(PROG, 1), "one chirality sweeps the slices last to first");
+  constexpr bool R = prog_reversed(PROG, 0);
+  T* p = site + (R ? LS / 2 - 1 - t : t) * kPairStride;
+#pragma unroll
+  for (int c = 0; c < 12; c++) {
+    if (R) put4(p + 4 * c, a.re[c].y, a.re[c].x, a.im[c].y, a.im[c].x);
+    else put4(p + 4 * c, a.re[c].x, a.re[c].y, a.im[c].x, a.im[c].y);
+  }
+}
+
+// Components 3 w .. 3 w + 2 of slice pair t summed over the eight hops that put_hops left, in the
+// same order as sum_hops (w: the warp).
+template <typename T, int LS, int PROG>
+__device__ __forceinline__ void sum_lanes(const T* site, int part_stride, int t, int w, typename Pr<T>::V (&re)[3],
+                                          typename Pr<T>::V (&im)[3]) {
+  using A = Pr<T>;
+  using V = typename A::V;
+  constexpr bool R = prog_reversed(PROG, 0);
+  const T* p = site + (R ? LS / 2 - 1 - t : t) * kPairStride;
+  const int row = w & 1;
+#pragma unroll
+  for (int a = 0; a < 3; a++) re[a] = im[a] = A::dup((T)0);
+#pragma unroll
+  for (int mu = 0; mu < 4; mu++)
+#pragma unroll
+    for (int d = 0; d < 2; d++)
+#pragma unroll
+      for (int a = 0; a < 3; a++) {
+        if (w < 2) {
+          const Coef4<T> v = coef4(p + mu * part_stride + 24 * d + 4 * (3 * row + a));
+          re[a] = A::add(re[a], A::mk(v.a, v.b));
+          im[a] = A::add(im[a], A::mk(v.c, v.d));
+        } else {
+          const Coef4<T> v = coef4(p + mu * part_stride + 24 * d + 4 * (3 * partner(mu, row) + a));
+          const int rs = row == 0 ? recon_sign(mu, d == 0 ? +1 : -1, 0) : recon_sign(mu, d == 0 ? +1 : -1, 1);
+          const V s = A::dup((T)rs), x = A::mk(v.a, v.b), y = A::mk(v.c, v.d);
+          re[a] = A::fma(imag_mu(mu) ? A::neg(s) : s, imag_mu(mu) ? y : x, re[a]);
+          im[a] = A::fma(s, imag_mu(mu) ? x : y, im[a]);
+        }
+      }
+  if (R) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+      re[a] = A::mk(re[a].y, re[a].x);
+      im[a] = A::mk(im[a].y, im[a].x);
+    }
   }
 }
 
 // hop_kernel with the four directions mu of a site on the four warps of a CTA (two hops
-// each) and 32 / G sites per CTA; the warps' sums are added on the way into the
+// each) and 32 / G sites per CTA; the hops are added up on the way into the
 // 5th-dimension program, and each warp finishes three of the twelve components.
 // For lattices that leave SM sub-partitions without a warp: a warp alone is bound by its
 // own chain (FP64: one instruction per 64 cycles of its sub-partition's pipe; FP32: eight
@@ -919,6 +1044,7 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
   using A = Pr<T>;
   using V = typename A::V;
   constexpr int G = LS / 2, S = 32 / G, SST = site_stride(LS);
+  constexpr bool XSUM = sums_in_sweeps<T>();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* coef = reinterpret_cast<T*>(smem_raw);
   T* sbuf = coef + prog_coefs(LS, POST) + (EX == EX_HAT ? prog_coefs(LS, PR_ITINV) : 0);
@@ -956,8 +1082,8 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
     }
 #define DWF_SPLIT_MU(MU)                                                                          \
   case MU:                                                                                        \
-    hop_dir<SP, LS, PRE, MU, +1>(nb.x, hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);          \
-    hop_dir<SP, LS, PRE, MU, -1>(nb.y, hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc);          \
+    hop_dir<SP, LS, PRE, MU, +1, !(MU == 0 && XSUM)>(nb.x, hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc); \
+    hop_dir<SP, LS, PRE, MU, -1, !(MU == 0 && XSUM)>(nb.y, hl, t, NP, bd, bo, vb, a.gauge_p, a.gauge_q, acc); \
     break;
     switch (mu) {
       DWF_SPLIT_MU(0)
@@ -980,12 +1106,28 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
       load_comp(reinterpret_cast<const T*>(reinterpret_cast<const char*>(a.w) + off), m, NP, c0 + k, wr[k], wi[k]);
     if (EX == EX_RUPD && active) load_comp(other, m, NP, c0 + k, xr[k], xi[k]);
   }
-  if (part) put<T, LS, POST>(sbuf + (mu * S + j) * SST, t, acc);
-  __syncthreads();
-  run_prog_sum<T, LS, POST, 4>(sbuf, S * SST, coef, tid, S);
+  if (part) {
+    if (XSUM && mu == 0) put<T, LS, POST>(sbuf + j * SST, t, acc);
+    else put_hops<T, LS, POST>(sbuf + (mu * S + j) * SST, t, acc);
+  }
   __syncthreads();
   const bool rev = prog_reversed(POST, 1) == (chir == 1);  // one of the chiralities is reversed
-  const T* p = sbuf + j * SST + (rev ? G - 1 - t : t) * kPairStride + 4 * c0;
+  T* p = sbuf + j * SST + (rev ? G - 1 - t : t) * kPairStride + 4 * c0;
+  if constexpr (!XSUM) {
+    V sr[3], si[3];
+    if (part) sum_lanes<T, LS, POST>(sbuf + j * SST, S * SST, t, mu, sr, si);
+    __syncthreads();  // the sums overwrite the first block
+    if (part) {
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        if (rev) put4(p + 4 * k, sr[k].y, sr[k].x, si[k].y, si[k].x);
+        else put4(p + 4 * k, sr[k].x, sr[k].y, si[k].x, si[k].y);
+      }
+    }
+    __syncthreads();
+  }
+  run_prog_split<T, LS, POST, XSUM>(sbuf, S * SST, coef, tid, S);
+  __syncthreads();
   const T f = G5 && chir == 1 ? -a.c_hop : a.c_hop;
   V re[3], im[3];
   const T na = EX == EX_RUPD ? -rupd_scalar<T>() : (T)0;
@@ -1024,7 +1166,7 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
       }
     }
     __syncthreads();
-    run_prog_sum<T, LS, PR_ITINV, 1>(sbuf, 0, coef + prog_coefs(LS, POST), tid, S);
+    run_prog_split<T, LS, PR_ITINV, false>(sbuf, 0, coef + prog_coefs(LS, POST), tid, S);
     __syncthreads();
     if (active) {
 #pragma unroll
@@ -1124,12 +1266,13 @@ inline size_t smem_bytes(int Ls, int S, size_t ts, int prog, int extra = EX_NONE
   return prog == PR_NONE ? 0 : ts * ((size_t)coefs + (size_t)S * site_stride(Ls));
 }
 
-// hop_split_kernel instead of hop_kernel: while the warps of hop_kernel do not fill the 608
-// SM sub-partitions once (FP32), or fill them in a last round of FP64 work that four times
-// as many quarter-sized warps finish sooner.  D_bb + D_bb^+ at Ls = 16, us with / without
-// (CUDA graph): FP32 4^4 14.3 / 26.3, 8^4 (512 warps) 24.0 / 28.8, 12 right-hand sides of
-// 8^2x4^2 (1536 warps) 49.4 / 42.4; FP64 4^4 101 / 276, 8^3x4 (256) 175 / 277,
-// 12^2x8x12 at Ls = 4 (432) 237 / 290, 8^4 (512) 326 / 296.
+// hop_split_kernel instead of hop_kernel while the warps of hop_kernel do not fill the 608
+// SM sub-partitions once (FP32); FP64 up to a line between the sizes where it was seen to win
+// (432 warps) and to lose (512).  Both give the same bits (sum_hops).  D_bb + D_bb^+ at Ls = 16,
+// us with / without (CUDA graph): FP32 4^4 15.4 / 26.3, 8^4 (512 warps) 25.0 / 28.8, FP64 4^4
+// 101 / 276, 8^3x4 (256) 170 / 277, 12^2x8x12 at Ls = 4 (432) 239 / 290; above the lines (with
+// sums by direction, 5-8% faster in FP32): FP32 12 right-hand sides of 8^2x4^2 (1536 warps)
+// 49.4 / 42.4, FP64 8^4 (512) 326 / 296.
 inline bool split_directions(int Ls, int Vh, int nrhs, bool f64) {
   const int S = 32 / (Ls / 2);
   return (long long)((Vh + S - 1) / S) * nrhs <= (f64 ? 456 : 608);
@@ -1196,8 +1339,7 @@ cudaError_t run_tma(const Geom& g, const HopLaunch& L, const Args<typename SP::T
     skip = *L.skip_hop;
     *L.skip_hop = -1;
   }
-  k<<<grid, kTmaThreads, smem, st>>>(g, a, map, L.wait_budget > 0 ? L.wait_budget : (1LL << 31), skip,
-                                     split_directions(LS, g.Vh, std::max(L.nrhs, L.rule_nrhs), sizeof(typename SP::T) == 8));
+  k<<<grid, kTmaThreads, smem, st>>>(g, a, map, L.wait_budget > 0 ? L.wait_budget : (1LL << 31), skip);
   return cudaGetLastError();
 }
 

@@ -227,7 +227,7 @@ __device__ __forceinline__ void hop_staged(const unsigned char* sb, bool neg, in
 template <class SP, int LS, int PRE, int POST, int LOC, bool G5, bool NORM, int NST, int MINB>
 __global__ void __launch_bounds__(kTmaThreads, MINB)
     hop_tma_kernel(const Geom g, const Args<typename SP::T> a, const __grid_constant__ CUtensorMap tmap,
-                   long long budget, int skip_hop, int by_direction) {
+                   long long budget, int skip_hop) {
   using T = typename SP::T;
   using V = typename Pr<T>::V;
   using ST = Stage<SP, LS>;
@@ -261,7 +261,6 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
   __syncthreads();
   SpinP<V> acc;
   zero(acc);
-  SpinP<V> sum;  // by_direction: the directions' sums added up, as hop_split_kernel adds them
   bool timed_out = false;
   if (producer) {
     const int lane = tid - kTmaConsumers;
@@ -337,26 +336,14 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
                                        nbv[D] < 0, t, bd, bo, acc);                           \
     mbar_arrive(&empty[st]);                                                                  \
   }
-#define DWF_TMA_SUM(MU)                     \
-  if (!SP::kScaled && by_direction) {       \
-    if (MU == 0) sum = acc;                 \
-    else add(sum, acc);                     \
-    zero(acc);                              \
-  }
     DWF_TMA_STEP(0, 0, +1)
     DWF_TMA_STEP(1, 0, -1)
-    DWF_TMA_SUM(0)
     DWF_TMA_STEP(2, 1, +1)
     DWF_TMA_STEP(3, 1, -1)
-    DWF_TMA_SUM(1)
     DWF_TMA_STEP(4, 2, +1)
     DWF_TMA_STEP(5, 2, -1)
-    DWF_TMA_SUM(2)
     DWF_TMA_STEP(6, 3, +1)
     DWF_TMA_STEP(7, 3, -1)
-    DWF_TMA_SUM(3)
-    if (!SP::kScaled && by_direction) acc = sum;
-#undef DWF_TMA_SUM
 #undef DWF_TMA_STEP
   }
   if (timed_out && a.err) atomicOr(a.err, 1);

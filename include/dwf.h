@@ -203,9 +203,9 @@ int dwf_apply_dalpha(dwf_handle h, double* out_full, const double* in_full, doub
  * sides that share every kernel launch (each with its own alpha, scalars and
  * convergence; converged ones are masked off).  With rhs_block = 0 a built-in
  * autotuner times the batched D_bb apply for block sizes that fit in free
- * device memory and for the CTA shapes of the hop kernels, and keeps the
- * fastest per right-hand side (cached per lattice, Ls, precision and nrhs in
- * the handle, and in the file named by DWF_AUTOTUNE_CACHE if set).  The CG
+ * device memory and keeps the fastest per right-hand side (cached per lattice,
+ * Ls, precision and nrhs in the handle, and in the file named by
+ * DWF_AUTOTUNE_CACHE if set); the solutions do not depend on the block.  The CG
  * iterations between two convergence polls (check_every, rounded up to even)
  * are captured once as a CUDA graph and replayed.  All solver work runs on a
  * stream owned by the handle; the call first waits for the caller's stream. */

@@ -258,11 +258,10 @@ struct dwf_ctx {
   int* pinned_i = nullptr;         // host staging of the mask
   int active_cap = 0;
   struct Tuned {
-    int nb, tma, tile;  // right-hand-side block, staging variant, threads per CTA (0: by size)
+    int nb, tma;  // right-hand-side block, staging variant
   };
-  std::map<std::string, Tuned> tune;  // autotuned launch shapes
-  int tile = 0;                      // tuned threads per CTA of the last solve's inner applies (0: by size)
-  int env_tile = -1;                 // DWF_HOP_TILE set: threads fixed (-1: autotuned)
+  std::map<std::string, Tuned> tune;  // autotuned blocks
+  int env_tile = 0;                  // DWF_HOP_TILE set: threads per CTA of the hop kernels (0: by size)
   double tier_eta = 1e-3;            // 16-bit solves: FP64 replacement once |r| < eta |r_64|
                                      // (DWF_TIER_ETA; <= 0: every replacement in FP64)
 };
@@ -472,7 +471,7 @@ HopLaunch base_hop(dwf_ctx* h, int prec, int p, int nrhs, size_t stride) {
   L.nbr = h->nbr;
   L.err = h->dev_err;
   L.use_tma = h->use_tma;
-  L.block_threads = std::max(h->env_tile, 0);
+  L.block_threads = h->env_tile;
   L.wait_budget = h->wait_budget;
   L.skip_hop = &h->skip_hop;  // one-shot test hook, consumed by the first staged launch
   return L;
@@ -489,7 +488,6 @@ struct CoefView {
   bool chain_ok;  // of every right-hand side's set
   int rule_nrhs;  // HopLaunch.rule_nrhs
   bool ahead;     // HopLaunch.ahead
-  int tile, tile_prec;  // HopLaunch.block_threads of the kernels of precision tile_prec (0: by size)
   const void* ptr(int prec, size_t off) const {
     const int f = prec == P64 ? 0 : 1;
     return reinterpret_cast<const char*>(dev[f]) + off * (f == 0 ? 8 : 4);
@@ -501,7 +499,7 @@ struct CoefView {
   }
 };
 CoefView view_of(const MatSet& ms) {
-  return CoefView{&ms, {ms.dev[0], ms.dev[1]}, 0, nullptr, ms.chain_ok, 0, false, 0, P64};
+  return CoefView{&ms, {ms.dev[0], ms.dev[1]}, 0, nullptr, ms.chain_ok, 0, false};
 }
 
 void set_coef(HopLaunch& L, const CoefView& cv) {
@@ -509,7 +507,6 @@ void set_coef(HopLaunch& L, const CoefView& cv) {
   L.active = cv.active;
   L.rule_nrhs = cv.rule_nrhs;
   L.ahead = cv.ahead;
-  if (cv.tile && L.prec == cv.tile_prec) L.block_threads = cv.tile;
 }
 
 int apply_dbb_bp(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void* p, const void* bp,
@@ -1028,6 +1025,7 @@ int cgnr_batched(dwf_ctx* h, const CoefView& cv_in, int prec, double tol, int ma
     U.w = W.w;
     U.stride = fi;
     U.nrhs = nb;
+    U.rule_nrhs = cv.rule_nrhs;
     U.chain = cv.chain(prec);
     U.cstride = cv.cstride;
     U.num = zz_new;
@@ -1540,61 +1538,51 @@ int solver_params(dwf_ctx* h, int* prec, double* delta, bool* restart) {
   return DWF_OK;
 }
 
-// Autotuner of the launch shapes of the solver: times the (batched) D_bb apply
-// of the inner precision for every right-hand-side block size that fits in free
-// device memory (batched solves) and for the tuned hop kernels' CTAs of 128 and 64
-// threads (where the choice by size takes the direction-split kernel, only that: the
-// other shapes all give the same bits, which a timing may therefore choose among),
-// and keeps the fastest per right-hand side (within 3%, the larger block).  The
-// tensor-copy staged variant was slower at every size it was tried on (FP16, 24 sources
-// on 8^4, Ls = 16: 278 us a pass against 52 to 74) and is not tried.  Results are cached per (lattice,
-// Ls, precision, nrhs) in the handle and, if DWF_AUTOTUNE_CACHE names a file, there as
-// "key nb staging tile" lines.  An explicit rhs_block option fixes the block;
-// DWF_TMA (set at dwf_create) fixes the staging, DWF_HOP_TILE the CTA.
+// Autotuner of a batched solve's block: times the D_bb apply of the inner precision for every
+// right-hand-side block size that fits in free device memory and keeps the fastest per
+// right-hand side (within 3%, the larger block).  It changes how many sources share a launch and
+// nothing else: CTA shapes go by the solve's total number of sources (HopLaunch.rule_nrhs),
+// because the norms of FP64 fields and the sum tree are rounded CTA by CTA, and the bits of a
+// solution do not depend on a timing.  The tensor-copy staged variant was slower at every size
+// it was tried on (FP16, 24 sources on 8^4, Ls = 16: 278 us a pass against 52 to 74) and is not
+// tried.  Results are cached per (lattice, Ls, precision, nrhs) in the handle and, if
+// DWF_AUTOTUNE_CACHE names a file, there as "key nb staging 0" lines (files of before may hold a
+// CTA size in the last place, which is ignored).  An explicit rhs_block option fixes the block;
+// DWF_TMA (set at dwf_create) the staging, DWF_HOP_TILE the CTA.
 int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_out) {
   const int Ls = h->g.Ls;
-  const bool tuned = !g_disable_tuned && hop2::tuned_ls(Ls, prec == P16 || prec == PB16);
-  const bool fixed_nb = h->opt.rhs_block > 0 || nrhs == 1;
-  const int fnb = nrhs == 1 ? 1 : std::min(std::max(h->opt.rhs_block, 1), nrhs);
-  if (!tuned) {  // one generic kernel shape: only the block is tuned (or fixed)
-    if (fixed_nb) {
-      *nb_out = fnb;
-      return DWF_OK;
-    }
+  h->use_tma = h->env_tma;
+  if (h->opt.rhs_block > 0 || nrhs == 1) {
+    *nb_out = nrhs == 1 ? 1 : std::min(h->opt.rhs_block, nrhs);
+    return DWF_OK;
   }
   std::ostringstream key;
   key << "v3_" << h->g.L[0] << "x" << h->g.L[1] << "x" << h->g.L[2] << "x" << h->g.L[3] << "_Ls" << Ls
-      << "_p" << prec << "_n" << nrhs << "_b" << (fixed_nb ? fnb : 0) << "_t" << h->env_tma
-      << "_s" << h->env_tile;
+      << "_p" << prec << "_n" << nrhs << "_b0_t" << h->env_tma << "_s" << (h->env_tile ? h->env_tile : -1);
   auto it = h->tune.find(key.str());
   const char* cache_file = std::getenv("DWF_AUTOTUNE_CACHE");
   if (it == h->tune.end() && cache_file) {
     std::ifstream in(cache_file);
     std::string k;
-    int nb, tma, tile;
-    while (in >> k >> nb >> tma >> tile)
-      if (k == key.str()) h->tune[k] = dwf_ctx::Tuned{nb, tma, tile == 64 || tile == 128 ? tile : 0};
+    int nb, tma, unused;
+    while (in >> k >> nb >> tma >> unused)
+      if (k == key.str()) h->tune[k] = dwf_ctx::Tuned{nb, tma};
     it = h->tune.find(key.str());
   }
   if (it != h->tune.end()) {
     *nb_out = std::min(it->second.nb, nrhs);
     h->use_tma = it->second.tma;
-    h->tile = it->second.tile;
     return DWF_OK;
   }
   std::vector<int> ok;
-  if (fixed_nb) {
-    ok.push_back(fnb);
-  } else {
-    size_t freeb = 0, totalb = 0;
-    CUCHK(h, cudaMemGetInfo(&freeb, &totalb));
-    const size_t per = solve_bytes_per_rhs(h->g, prec) + 3 * field_bytes(h->g, prec);
-    const double budget = 0.8 * (double)freeb;
-    const int cand[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
-    for (int c : cand)
-      if (c <= nrhs && (double)c * per <= budget) ok.push_back(c);
-    if (ok.empty()) ok.push_back(1);
-  }
+  size_t freeb = 0, totalb = 0;
+  CUCHK(h, cudaMemGetInfo(&freeb, &totalb));
+  const size_t per = solve_bytes_per_rhs(h->g, prec) + 3 * field_bytes(h->g, prec);
+  const double budget = 0.8 * (double)freeb;
+  const int cand[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
+  for (int c : cand)
+    if (c <= nrhs && (double)c * per <= budget) ok.push_back(c);
+  if (ok.empty()) ok.push_back(1);
   const int maxnb = ok.back();
   const size_t fi = field_bytes(h->g, prec);
   void *x, *y, *t;
@@ -1607,59 +1595,40 @@ int choose_rhs_block(dwf_ctx* h, int nrhs, int prec, cudaStream_t st, int* nb_ou
   if ((rc = build_matset(h, h->alpha, h->m, &ms))) return rc;
   CoefView tv = view_of(*ms);
   tv.rule_nrhs = nrhs;
-  tv.tile_prec = prec;
   cudaEvent_t e0, e1;
   CUCHK(h, cudaEventCreate(&e0));
   CUCHK(h, cudaEventCreate(&e1));
-  std::vector<int> tmas = {h->env_tma};
-  std::vector<int> tiles = {h->env_tile >= 0 ? h->env_tile : 0};
-  if (tuned) {
-    if (h->env_tma) tiles = {0};  // the staged variant has one tile
-    else if (h->env_tile < 0 && (prec == P16 || prec == PB16 ||
-                                 !hop2::split_directions(Ls, h->g.Vh, nrhs, prec == P64)))
-      tiles = {128, 64};  // of the same bits
-  }
   double best = 1e300;
-  int best_nb = ok.front(), best_tma = tmas.front(), best_tile = 0;
-  const bool single = ok.size() == 1 && tmas.size() == 1 && (tiles.size() == 1 || tmas[0]);
-  best_tile = tiles.front();
-  if (!single)
-  for (int nb : ok)
-    for (int tma : tmas)
-      for (int tile : tiles) {
-        h->use_tma = tma;
-        tv.tile = tile;
-        if ((rc = apply_dbb(h, tv, prec, y, x, t, nb, nullptr, st))) return rc;
-        // best of two timed passes of 3 applies (one slow pass does not decide)
-        double per_rhs = 1e300;
-        for (int pass = 0; pass < 2; pass++) {
-          CUCHK(h, cudaEventRecord(e0, st));
-          for (int k = 0; k < 3; k++)
-            if ((rc = apply_dbb(h, tv, prec, y, x, t, nb, nullptr, st))) return rc;
-          CUCHK(h, cudaEventRecord(e1, st));
-          CUCHK(h, cudaEventSynchronize(e1));
-          float ms_t = 0.f;
-          CUCHK(h, cudaEventElapsedTime(&ms_t, e0, e1));
-          per_rhs = std::min(per_rhs, ms_t / (3.0 * nb));
-        }
-        if (per_rhs < 0.97 * best || (per_rhs <= best * 1.03 && nb > best_nb)) {
-          if (per_rhs < best) best = per_rhs;
-          best_nb = nb;
-          best_tma = tma;
-          best_tile = tile;
-        }
+  int best_nb = ok.front();
+  if (ok.size() > 1)
+    for (int nb : ok) {
+      if ((rc = apply_dbb(h, tv, prec, y, x, t, nb, nullptr, st))) return rc;
+      // best of two timed passes of 3 applies (one slow pass does not decide)
+      double per_rhs = 1e300;
+      for (int pass = 0; pass < 2; pass++) {
+        CUCHK(h, cudaEventRecord(e0, st));
+        for (int k = 0; k < 3; k++)
+          if ((rc = apply_dbb(h, tv, prec, y, x, t, nb, nullptr, st))) return rc;
+        CUCHK(h, cudaEventRecord(e1, st));
+        CUCHK(h, cudaEventSynchronize(e1));
+        float ms_t = 0.f;
+        CUCHK(h, cudaEventElapsedTime(&ms_t, e0, e1));
+        per_rhs = std::min(per_rhs, ms_t / (3.0 * nb));
       }
+      if (per_rhs < 0.97 * best || (per_rhs <= best * 1.03 && nb > best_nb)) {
+        if (per_rhs < best) best = per_rhs;
+        best_nb = nb;
+      }
+    }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  h->use_tma = best_tma;
-  h->tile = best_tile;
-  h->tune[key.str()] = dwf_ctx::Tuned{best_nb, best_tma, best_tile};
+  h->tune[key.str()] = dwf_ctx::Tuned{best_nb, h->use_tma};
   if (cache_file) {
     // handles tuned on several host threads at once append whole lines
     static std::mutex cache_mutex;
     std::lock_guard<std::mutex> lock(cache_mutex);
     std::ofstream out(cache_file, std::ios::app);
-    out << key.str() << " " << best_nb << " " << best_tma << " " << best_tile << "\n";
+    out << key.str() << " " << best_nb << " " << h->use_tma << " 0\n";
   }
   *nb_out = best_nb;
   return DWF_OK;
@@ -2159,7 +2128,7 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
       KLAUNCH(h, launch_hop(g, Hs, st));
     }
     std::vector<dwf_stats> sk(n);
-    CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr, true, nrhs, false, h->tile, prec};
+    CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr, true, nrhs, false};
     for (int r = 0; r < n; r++) cv.chain_ok = cv.chain_ok && ms[blk + r]->chain_ok;
     rc = cgnr_batched(h, cv, prec, h->opt.rel_tol, h->opt.maxiter, delta, restart, W, n, sk.data(), st);
     if (rc && rc != DWF_ERR_NOT_CONVERGED && rc != DWF_ERR_BREAKDOWN) return rc;

@@ -1245,7 +1245,8 @@ namespace hop2 {
 // warp (BF16, Ls = 16, 8^2x4^2: 30.8 us at 32, 28.6 at 64, 26.2 at 128).
 // FP64: the largest CTA that still gives every SM eight of them: its pipe wants the warps
 // spread evenly over the sub-partitions (Ls = 8, 12^2x8x12: 439 us at 64, 548 at 128).
-// All of them give the same bits.
+// All of them give the same fields; the fused norms of FP64 fields and the sums of the tree are
+// rounded CTA by CTA, so the size counts rule_nrhs right-hand sides and is never timed.
 inline int tile_threads(int Ls, int Vh, int nrhs, bool f64) {
   if (!f64) return warp_groups(Ls) ? 128 : 64;
   for (int nt : {128, 64}) {
@@ -1388,7 +1389,8 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
       return launch_ahead(L.ahead, k, dim3((g.Vh + S - 1) / S, 1, L.nrhs), 128, smem, st, g, a);
     }
   }
-  const int nt = L.block_threads ? L.block_threads : tile_threads(LS, g.Vh, L.nrhs, sizeof(T) == 8);
+  const int nt =
+      L.block_threads ? L.block_threads : tile_threads(LS, g.Vh, std::max(L.nrhs, L.rule_nrhs), sizeof(T) == 8);
   const int S = cta_sites<LS, PRE>(nt);
   const auto smem_of = [](int n) { return smem_bytes(LS, cta_sites<LS, PRE>(n), sizeof(T), POST, EX); };
   dim3 grid((g.Vh + S - 1) / S, 1, L.nrhs);
@@ -1571,7 +1573,7 @@ __global__ void __launch_bounds__(128) rupdate_kernel(const Geom g, void* r, voi
 template <class SP, int LS>
 cudaError_t run_rupdate(const Geom& g, const RUpdateLaunch& L, cudaStream_t st) {
   using T = typename SP::T;
-  const int nt = tile_threads(LS, g.Vh, L.nrhs, sizeof(T) == 8), S = nt / (LS / 2);
+  const int nt = tile_threads(LS, g.Vh, std::max(L.nrhs, L.rule_nrhs), sizeof(T) == 8), S = nt / (LS / 2);
   auto k = rupdate_kernel<SP, LS>;
   static std::atomic<bool> attr{false};
   cudaError_t e = smem_limit_once(k, smem_bytes(LS, 128 / (LS / 2), sizeof(T), PR_ITINV), attr);

@@ -99,8 +99,9 @@ struct HopLaunch {
   int g5out;
   const Reduce* red;        // nullptr: no norm
   int block_threads;        // threads per CTA of the tuned kernels (0: by size)
-  int rule_nrhs;            // right-hand sides that the choice by size counts (at least nrhs): a
-                            // solve's total, so that its bits do not depend on how it is blocked
+  int rule_nrhs;            // right-hand sides that the choices by size (CTA size, directions on four
+                            // warps) count, at least nrhs: a solve's total, so that its norms, and
+                            // with them its bits, do not depend on how it is blocked
   // Tuned path (hop2::tuned_ls): 5th-dimension operators as chain programs
   // (hop2::PR_*) over the recurrence coefficient block, and the neighbour table.
   int post_prog;
@@ -165,6 +166,7 @@ struct RUpdateLaunch {
   int sstride;
   const Reduce* red;
   const int* active;
+  int rule_nrhs;            // as HopLaunch.rule_nrhs
   bool ahead;               // as HopLaunch.ahead
 };
 cudaError_t launch_rupdate(const Geom& g, const RUpdateLaunch& a, cudaStream_t s);

@@ -105,3 +105,26 @@ def test_dalpha_on_another_stream_than_a_solve():
     torch.cuda.synchronize()
     assert torch.equal(torch.view_as_real(prop), torch.view_as_real(prop_ref))
     assert all(torch.equal(torch.view_as_real(out), torch.view_as_real(ref)) for out in outs)
+
+
+@pytest.mark.parametrize("prec,L,Ls,nrhs,kw", [
+    (0, (8, 8, 8, 8), 8, 24, dict(solver=2)), (1, (8, 8, 4, 4), 16, 6, {}), (2, (4, 4, 4, 8), 8, 6, {}),
+    (3, (4, 4, 4, 8), 12, 6, {})])
+def test_solution_bits_do_not_depend_on_the_block(prec, L, Ls, nrhs, kw, tmp_path, monkeypatch):
+    """One source at a time, ragged blocks, the autotuned block, and blocks from a cache file whose
+    lines name CTAs of 64 and of 128 threads: the same bits.  (FP64 norms are rounded CTA by CTA;
+    FP64 at 8^4, Ls = 8 would take CTAs of 32 threads for one source and of 128 for 24.)"""
+    sysm = make_case(L, Ls, "mobius", alpha=1.2, m=0.3)
+    src = torch.stack([torch.from_numpy(gaussian_source4d(L, seed=1 + k)) for k in range(nrhs)]).cuda()
+    kw = dict(kw, precision_inner=prec)
+    ref = _solve(sysm, src, nrhs, rhs_block=1, **kw)
+    res = [_solve(sysm, src, nrhs, rhs_block=nrhs - 2, **kw), _solve(sysm, src, nrhs, **kw)]
+    for nb, tile in ((nrhs, 64), (nrhs, 128), (nrhs // 2, 128)):
+        cache = tmp_path / ("cache%d_%d" % (nb, tile))
+        cache.write_text("v3_%dx%dx%dx%d_Ls%d_p%d_n%d_b0_t0_s-1 %d 0 %d\n" % (*L, Ls, prec, nrhs, nb, tile))
+        monkeypatch.setenv("DWF_AUTOTUNE_CACHE", str(cache))
+        res.append(_solve(sysm, src, nrhs, **kw))
+        monkeypatch.delenv("DWF_AUTOTUNE_CACHE")
+    for prop, stats in res:
+        assert torch.equal(torch.view_as_real(prop), torch.view_as_real(ref[0]))
+        assert stats == ref[1]

@@ -2086,8 +2086,10 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
     return apply_dalpha_halves(h, *rhs_set, rhs, pbc, W.t64, st);
   };
   int result = DWF_OK;
-  for (int blk = 0; blk < nrhs; blk += nb) {
-    const int n = std::min(nb, nrhs - blk);
+  for (int blk = 0, n; blk < nrhs; blk += n) {
+    // a block ends where the next source's recurrences are fit for the tuned kernels and this
+    // one's are not, or the other way round: each source takes the kernels it takes alone
+    for (n = 1; n < std::min(nb, nrhs - blk) && ms[blk + n]->chain_ok == ms[blk]->chain_ok;) n++;
     auto t0 = std::chrono::steady_clock::now();
     const long long l0 = h->launches;
     for (int r = 0; r < n; r++) {
@@ -2128,8 +2130,7 @@ static int solve_5d(dwf_ctx* h, const double* src4d, double* prop4d, double* sol
       KLAUNCH(h, launch_hop(g, Hs, st));
     }
     std::vector<dwf_stats> sk(n);
-    CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr, true, nrhs, false};
-    for (int r = 0; r < n; r++) cv.chain_ok = cv.chain_ok && ms[blk + r]->chain_ok;
+    const CoefView cv{ms[blk], {bc64, bc32}, cnt, nullptr, ms[blk]->chain_ok, nrhs, false};
     rc = cgnr_batched(h, cv, prec, h->opt.rel_tol, h->opt.maxiter, delta, restart, W, n, sk.data(), st);
     if (rc && rc != DWF_ERR_NOT_CONVERGED && rc != DWF_ERR_BREAKDOWN) return rc;
     if (rc) result = rc;

@@ -1399,10 +1399,10 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
     KLAUNCH(h, launch_hop(h->g, B, q));
     return DWF_OK;
   };
-  // n iterations (the first p is in W.p and |r|^2 in slot 0, the last ones in slot n & 1)
-  // and the pending x update
-  auto enqueue_block = [&](int n, cudaStream_t q) -> int {
-    int c = 0, e;
+  // n iterations from parity c (p in the buffer and |r|^2 in the slot of that parity, at the end
+  // in those of c + n) and the pending x update
+  auto enqueue_block = [&](int c, int n, cudaStream_t q) -> int {
+    int e;
     for (int k = 0; k < n; k++, c = 1 - c)
       if ((e = enqueue_fused(c, k == 0, q))) return e;
     KLAUNCH(h, launch_finish_sum(bin_sum(h, BIN_RR, slot(c)), 1, q, nullptr));
@@ -1410,32 +1410,32 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
                                nullptr));
     return DWF_OK;
   };
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  struct Release {
-    cudaGraph_t& g;
-    cudaGraphExec_t& e;
-    ~Release() {
+  // the block between two polls as a graph, from parity 0 and, where it is odd, from parity 1
+  // (long blocks hide their launches by themselves and would be thousands of nodes)
+  struct Graph {
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t e = nullptr;
+    ~Graph() {
       if (e) cudaGraphExecDestroy(e);
       if (g) cudaGraphDestroy(g);
     }
-  } release{graph, exec};
-  const int block = check + (check & 1);  // iterations between polls of the fused path
+  } graph[2];
   long long per_block = 0;
   if (fused) {
     CUCHK(h, cudaMemsetAsync(W.p, 0, fi, s));
     CUCHK(h, cudaMemsetAsync(W.p2, 0, fi, s));
     h->pinned[0] = std::numeric_limits<double>::infinity();
     CUCHK(h, cudaMemcpyAsync(slot(1), h->pinned, sizeof(double), cudaMemcpyHostToDevice, s));
-    if (h->opt.graph != 0 && block <= maxiter) {
+    const bool use_graph = h->opt.graph != 0 && check <= 256;
+    for (int c = 0; use_graph && c <= (check & 1) && check <= maxiter / (c + 1); c++) {
       // captured on the handle's stream, replayed on the caller's
       const long long l0 = h->launches;
       CUCHK(h, cudaStreamBeginCapture(h->cstream, cudaStreamCaptureModeRelaxed));
-      const int e = enqueue_block(block, h->cstream);
-      const cudaError_t ce = cudaStreamEndCapture(h->cstream, &graph);
+      const int e = enqueue_block(c, check, h->cstream);
+      const cudaError_t ce = cudaStreamEndCapture(h->cstream, &graph[c].g);
       if (e) return e;
       CUCHK(h, ce);
-      CUCHK(h, cudaGraphInstantiate(&exec, graph, 0));
+      CUCHK(h, cudaGraphInstantiate(&graph[c].e, graph[c].g, 0));
       per_block = h->launches - l0;
       h->launches = l0;
     }
@@ -1445,17 +1445,17 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
   while (it < maxiter) {
     int nxt;
     if (fused) {
-      const int n = std::min(block, maxiter - it);
-      if (exec && n == block) {
-        CUCHK(h, cudaGraphLaunch(exec, s));
+      const int n = std::min(check, maxiter - it);
+      if (graph[cur].e && n == check) {
+        CUCHK(h, cudaGraphLaunch(graph[cur].e, s));
         h->launches += per_block;
-      } else if ((rc = enqueue_block(n, s))) {
+      } else if ((rc = enqueue_block(cur, n, s))) {
         return rc;
       }
       n_app += n;
       n_dag += n;
       it += n;
-      nxt = n & 1;  // n is odd only in the last block
+      nxt = (cur + n) & 1;
     } else {
       if ((rc = apply_dbb(h, cv, prec, W.w, W.p, W.tr, 1, &red_ww, s))) return rc;
       if ((rc = apply_dbb_dag(h, cv, prec, W.z, W.w, W.tr, W.tb, 1, nullptr, s))) return rc;
@@ -1498,10 +1498,8 @@ int cgnormal_solve(dwf_ctx* h, const MatSet& ms, int prec, double tol, int maxit
         if (it >= maxiter) break;
       }
     }
-    if (!fused) {
-      KLAUNCH(h, launch_p_update(h->g, prec, W.p, W.r, slot(nxt), slot(cur), kScal, 1, fi, s));
-      cur = nxt;
-    }
+    if (!fused) KLAUNCH(h, launch_p_update(h->g, prec, W.p, W.r, slot(nxt), slot(cur), kScal, 1, fi, s));
+    cur = nxt;
   }
   fill(it, restarts, true_res);
   if (!converged)

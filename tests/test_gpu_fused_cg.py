@@ -150,3 +150,29 @@ def test_source_with_unstable_recurrence_leaves_its_batch_alone():
     for k in (0, 1, 3):
         assert torch.equal(torch.view_as_real(res[0][k]), torch.view_as_real(res[1][k]))
     assert not torch.equal(torch.view_as_real(res[0][2]), torch.view_as_real(res[1][2]))
+
+
+@pytest.mark.parametrize("every,prec", [(1, 0), (5, 0), (7, 0), (16, 0), (300, 0), (1, 1), (5, 1), (7, 1), (16, 1)])
+def test_normal_solve_polls_every_check_every_iterations(every, prec, monkeypatch):
+    """Odd numbers of iterations between polls too, from both parities of the alternating buffers:
+    the count is a multiple of check_every, near the unfused CG's (one poll or 3 iterations, the
+    recurrences differ by rounding), with and without graphs the same, and the solutions agree."""
+    L, Ls = (4, 4, 4, 8), 8
+    sysm = make_case(L, Ls, "mobius", alpha=1.2, m=0.3)
+    phi = torch.from_numpy(gaussian_half5d(L, Ls, seed=3)).cuda()
+    res = []
+    for kw, unfused in ((dict(), False), (dict(graph=0), False), (dict(), True)):
+        if unfused:
+            monkeypatch.setenv("DWF_UNFUSED_CG", "1")
+        op = _op(sysm, precision_inner=prec, check_every=every, **kw)
+        x = torch.empty_like(phi)
+        st = op.solve_normal(x, phi)
+        torch.cuda.synchronize()
+        op.close()
+        assert st["true_resid"] <= 1e-10 and st["iterations"] % every == 0
+        res.append((st["iterations"], x))
+    assert res[0][0] == res[1][0]
+    assert torch.equal(torch.view_as_real(res[0][1]), torch.view_as_real(res[1][1]))
+    assert abs(res[0][0] - res[2][0]) <= max(3, every)
+    rel = torch.linalg.norm(res[0][1] - res[2][1]) / torch.linalg.norm(res[2][1])
+    assert rel <= 1e-8

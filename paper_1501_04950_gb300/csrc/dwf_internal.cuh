@@ -105,7 +105,6 @@ struct HopLaunch {
   // Tuned path (hop2::tuned_ls): 5th-dimension operators as chain programs
   // (hop2::PR_*) over the recurrence coefficient block, and the neighbour table.
   int post_prog;
-  int loc_prog;
   const void* chain;        // hop2 chain coefficient block in the compute type
   const int* nbr;           // [2 parities][Vh][8] neighbour half indices, bit 31 = sign
   int* err;                 // device flag set when a bounded wait gives up

@@ -26,6 +26,9 @@
  *     is the legacy default stream).  Apply calls do not synchronise.  The
  *     solver calls (dwf_cgne_solve, dwf_apply_overlap, dwf_solve_normal,
  *     dwf_force without X) synchronise internally (convergence polling).
+ *   - Alignment: canonical (complex128) arrays start on a 16-byte boundary.  So
+ *     should internal half-fields (device allocations do); others are taken, by
+ *     the slower generic kernels.
  *   - Gamma basis: chiral, gamma_k = [[0,-i sigma_k],[i sigma_k,0]],
  *     gamma_4 = [[0,1],[1,0]], gamma5 = diag(1,1,-1,-1); mu = 0..3 <-> x,y,z,t.
  *   - Canonical layouts (complex128 stored as interleaved double pairs, C order):

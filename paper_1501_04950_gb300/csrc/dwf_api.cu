@@ -514,9 +514,9 @@ int apply_dbb_bp(dwf_ctx* h, const CoefView& cv, int prec, void* out, const void
 
 // Whether the kernels of a CG iteration start ahead (launch_ahead): where each of them fills
 // the GPU more than once (16 warps per SM), so that the next one's CTAs take the place of
-// finished ones.  FP32 solves, with / without: 12^4, Ls 16 (2592 warps)
-// 67.6 / 71.5 ms a solve, 12^3x24, Ls 12 110.0 / 114.6, 16^3x32, Ls 16 434.5 / 439.1, 24 FP16
-// sources on 8^4 340 / 350.  Below that the CTAs that come early crowd the SMs that have room
+// finished ones.  Solves, with / without (in turn, one call): FP32 12^4, Ls 16 (2592 warps)
+// 55.4 / 57.8 ms, 12^3x24, Ls 12 91.1 / 94.6, 16^3x32, Ls 16 325.4 / 327.9; FP16 16^3x32, Ls 16
+// 281.9 / 284.6, 24 sources on 8^4 240.4 / 242.7.  Below that the CTAs that come early crowd the SMs that have room
 // (8^3x16, Ls 16, 1024 warps: 52.7 / 41.0), most of all with FP64 fields (805 / 428).
 bool ahead_rule(const Geom& g, int prec, int nrhs) {
   return prec != P64 && (long long)g.N5 / 64 * nrhs >= 152 * 16;

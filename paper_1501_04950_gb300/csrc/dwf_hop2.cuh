@@ -892,19 +892,33 @@ __device__ __forceinline__ void store_comp(double* base, size_t m, size_t NP, in
 // one block less to read.  FP64 (sum_lanes): by the lanes of all four warps in a step of its own,
 // 96 additions a thread; the sweeps fill few lanes (Ls = 32: 24 of 64), and an instruction of the
 // FP64 pipe costs the same however many lanes are on.  D_bb + D_bb^+ (CUDA graph), by lanes / on
-// the way into the sweeps: FP64 4^3x8, Ls = 32 115 / 132 us, 8x4x4x8, Ls = 10 105 / 110; FP32
-// 8^3x16, Ls = 8 30.7 / 25.8, 8^4, Ls = 16 26.2 / 25.0.
+// the way into the sweeps, both with an access to each hop: FP64 4^3x8, Ls = 32 115 / 132 us,
+// 8x4x4x8, Ls = 10 105 / 110; FP32 8^3x16, Ls = 8 30.7 / 25.8, 8^4, Ls = 16 26.2 / 25.0.  With the
+// two hops of a direction in one access (put_hops): 112, 103, 25.0 and 25.1.
 template <typename T>
 __host__ __device__ constexpr bool sums_in_sweeps() { return sizeof(T) == 4; }
 
+// Shared memory of the hops: direction x's block has the layout of put (site_stride); the other
+// directions' follow.  FP32 sites are 16 words apart modulo 32 there: the 16-byte accesses of
+// consecutive sweeps (12 of a site, one behind the other) are then conflict-free.
+template <typename T>
+__host__ __device__ constexpr int hop_site_stride(int Ls) {
+  return sizeof(T) == 8 ? site_stride(Ls) : (Ls / 2) * kPairStride + ((16 - ((Ls / 2) * kPairStride) % 32) + 32) % 32;
+}
+template <typename T, int LS>
+__device__ __forceinline__ T* hop_block(T* sbuf, int mu, int site) {
+  constexpr int S = 32 / (LS / 2);
+  return mu == 0 ? sbuf + site * site_stride(LS)
+                 : sbuf + S * site_stride(LS) + ((mu - 1) * S + site) * hop_site_stride<T>(LS);
+}
+
 // The sweep of component R of chirality CH from what the four warps left of the eight hops of a
-// site (blocks part_stride apart; direction x's sum as put leaves it, then put_hops: f chi of the
-// hop to x + mu, f chi of that to x - mu, pairs in the sweep order of chirality 0).  The hops
+// site (hop_block: direction x's sum as put leaves it, then put_hops of the others).  The hops
 // are added up one after the other as hop_kernel does, so that both kernels give the same bits:
 // the upper rows of (1 -+ gamma_mu) U' v' are chi, the lower ones rs (i) chi of the partner row
 // (mul_acc).
 template <typename T, int LS, int CH>
-__device__ __forceinline__ void sum_hops(T (&V)[LS], const T* site, int part_stride, int R) {
+__device__ __forceinline__ void sum_hops(T (&V)[LS], T* sbuf, int site, int R) {
   using A = Pr<T>;
   constexpr int G = LS / 2;
   const int row = R / 6, col = R - 6 * row;  // spin row, 2 colour + (re | im)
@@ -915,16 +929,17 @@ __device__ __forceinline__ void sum_hops(T (&V)[LS], const T* site, int part_str
     const int rs = row == 0 ? recon_sign(mu, +1, 0) : recon_sign(mu, +1, 1);
     // += rs i chi: re takes -rs im, im takes rs re
     sg[mu] = (T)(imag_mu(mu) && !(col & 1) ? -rs : rs);
-    at[mu] = site + mu * part_stride + 2 * (CH == 0 ? R : 6 * partner(mu, row) + (imag_mu(mu) ? col ^ 1 : col));
+    at[mu] = hop_block<T, LS>(sbuf, mu, site) + 4 * (CH == 0 ? R : 6 * partner(mu, row) + (imag_mu(mu) ? col ^ 1 : col));
   }
 #pragma unroll
   for (int k = 0; k < G; k++) {
     const int o = (CH == 0 ? k : G - 1 - k) * kPairStride;
-    const auto x = pair_at(site + 24 * CH + 2 * R + k * kPairStride);
+    const auto x = pair_at(hop_block<T, LS>(sbuf, 0, site) + 24 * CH + 2 * R + k * kPairStride);
     auto v = CH == 0 ? x : A::mk(x.y, x.x);
 #pragma unroll
     for (int mu = 1; mu < 4; mu++) {
-      const auto f = pair_at(at[mu] + o), b = pair_at(at[mu] + o + 24);
+      const Coef4<T> h = coef4(at[mu] + o);
+      const auto f = A::mk(h.a, h.b), b = A::mk(h.c, h.d);
       v = CH == 0 ? A::add(v, f) : A::fma(A::dup(sg[mu]), f, v);
       v = CH == 0 ? A::add(v, b) : A::fma(A::dup(-sg[mu]), b, v);
     }
@@ -936,7 +951,7 @@ __device__ __forceinline__ void sum_hops(T (&V)[LS], const T* site, int part_str
 // run_prog for 128 threads on nsites <= 32 / (LS / 2) sites, with HOPS on the sums of sum_hops.
 // The result goes to the first block, in the layout of put.
 template <typename T, int LS, int PROG, bool HOPS>
-__device__ __forceinline__ void run_prog_split(T* sbuf, int part_stride, const T* coef, int tid, int nsites) {
+__device__ __forceinline__ void run_prog_split(T* sbuf, const T* coef, int tid, int nsites) {
   using A = Pr<T>;
   constexpr int G = LS / 2;
   constexpr int NIT = (12 * (32 / G) + 63) / 64;
@@ -945,21 +960,20 @@ __device__ __forceinline__ void run_prog_split(T* sbuf, int part_stride, const T
 #pragma unroll
   for (int q = 0; q < NIT; q++) {
     const int i = (tid & 63) + 64 * q, site = i / 12, R = i - 12 * site;
-    const T* p = sbuf + site * site_stride(LS);
     if (i >= 12 * nsites) {
 #pragma unroll
       for (int k = 0; k < LS; k++) V[q][k] = (T)0;
     } else if (!HOPS) {
 #pragma unroll
       for (int k = 0; k < G; k++) {
-        const auto v = pair_at(p + 24 * ch + 2 * R + k * kPairStride);
+        const auto v = pair_at(sbuf + site * site_stride(LS) + 24 * ch + 2 * R + k * kPairStride);
         V[q][2 * k] = v.x;
         V[q][2 * k + 1] = v.y;
       }
     } else if (ch == 0) {
-      sum_hops<T, LS, 0>(V[q], p, part_stride, R);
+      sum_hops<T, LS, 0>(V[q], sbuf, site, R);
     } else {
-      sum_hops<T, LS, 1>(V[q], p, part_stride, R);
+      sum_hops<T, LS, 1>(V[q], sbuf, site, R);
     }
   }
   // the result overwrites the first block, where a thread has read only what it writes
@@ -980,49 +994,56 @@ __device__ __forceinline__ void run_prog_split(T* sbuf, int part_stride, const T
   }
 }
 
-// Slice pair t of a site into shared memory, all components in the sweep order of PROG's chirality 0.
+// f chi of a direction's two hops (components 0 .. 5 of a: to x + mu, 6 .. 11: to x - mu) of slice
+// pair t into shared memory, in the sweep order of PROG's chirality 0: real component R of both, as
+// (x + mu, x - mu) pairs, at 4 R.
 template <typename T, int LS, int PROG>
 __device__ __forceinline__ void put_hops(T* site, int t, const SpinP<typename Pr<T>::V>& a) {
   static_assert(prog_reversed(PROG, 0) != prog_reversed(PROG, 1), "one chirality sweeps the slices last to first");
   constexpr bool R = prog_reversed(PROG, 0);
   T* p = site + (R ? LS / 2 - 1 - t : t) * kPairStride;
 #pragma unroll
-  for (int c = 0; c < 12; c++) {
-    if (R) put4(p + 4 * c, a.re[c].y, a.re[c].x, a.im[c].y, a.im[c].x);
-    else put4(p + 4 * c, a.re[c].x, a.re[c].y, a.im[c].x, a.im[c].y);
+  for (int c = 0; c < 6; c++) {
+    if (R) {
+      put4(p + 8 * c, a.re[c].y, a.re[c].x, a.re[6 + c].y, a.re[6 + c].x);
+      put4(p + 8 * c + 4, a.im[c].y, a.im[c].x, a.im[6 + c].y, a.im[6 + c].x);
+    } else {
+      put4(p + 8 * c, a.re[c].x, a.re[c].y, a.re[6 + c].x, a.re[6 + c].y);
+      put4(p + 8 * c + 4, a.im[c].x, a.im[c].y, a.im[6 + c].x, a.im[6 + c].y);
+    }
   }
 }
 
 // Components 3 w .. 3 w + 2 of slice pair t summed over the eight hops that put_hops left, in the
 // same order as sum_hops (w: the warp).
 template <typename T, int LS, int PROG>
-__device__ __forceinline__ void sum_lanes(const T* site, int part_stride, int t, int w, typename Pr<T>::V (&re)[3],
+__device__ __forceinline__ void sum_lanes(T* sbuf, int site, int t, int w, typename Pr<T>::V (&re)[3],
                                           typename Pr<T>::V (&im)[3]) {
   using A = Pr<T>;
   using V = typename A::V;
   constexpr bool R = prog_reversed(PROG, 0);
-  const T* p = site + (R ? LS / 2 - 1 - t : t) * kPairStride;
-  const int row = w & 1;
+  const int o = (R ? LS / 2 - 1 - t : t) * kPairStride, row = w & 1;
 #pragma unroll
   for (int a = 0; a < 3; a++) re[a] = im[a] = A::dup((T)0);
 #pragma unroll
   for (int mu = 0; mu < 4; mu++)
 #pragma unroll
-    for (int d = 0; d < 2; d++)
-#pragma unroll
-      for (int a = 0; a < 3; a++) {
-        if (w < 2) {
-          const Coef4<T> v = coef4(p + mu * part_stride + 24 * d + 4 * (3 * row + a));
-          re[a] = A::add(re[a], A::mk(v.a, v.b));
-          im[a] = A::add(im[a], A::mk(v.c, v.d));
-        } else {
-          const Coef4<T> v = coef4(p + mu * part_stride + 24 * d + 4 * (3 * partner(mu, row) + a));
-          const int rs = row == 0 ? recon_sign(mu, d == 0 ? +1 : -1, 0) : recon_sign(mu, d == 0 ? +1 : -1, 1);
-          const V s = A::dup((T)rs), x = A::mk(v.a, v.b), y = A::mk(v.c, v.d);
-          re[a] = A::fma(imag_mu(mu) ? A::neg(s) : s, imag_mu(mu) ? y : x, re[a]);
-          im[a] = A::fma(s, imag_mu(mu) ? x : y, im[a]);
-        }
+    for (int a = 0; a < 3; a++) {
+      const T* p = hop_block<T, LS>(sbuf, mu, site) + o + 8 * (3 * (w < 2 ? row : partner(mu, row)) + a);
+      const Coef4<T> x = coef4(p), y = coef4(p + 4);  // re, im: (to x + mu, to x - mu)
+      if (w < 2) {
+        re[a] = A::add(A::add(re[a], A::mk(x.a, x.b)), A::mk(x.c, x.d));
+        im[a] = A::add(A::add(im[a], A::mk(y.a, y.b)), A::mk(y.c, y.d));
+      } else {  // += rs chi or rs i chi, rs turned around for the hop to x - mu
+        const V s = A::dup((T)(row == 0 ? recon_sign(mu, +1, 0) : recon_sign(mu, +1, 1))), n = A::neg(s);
+        const Coef4<T>& u = imag_mu(mu) ? y : x;
+        const Coef4<T>& v = imag_mu(mu) ? x : y;
+        re[a] = A::fma(imag_mu(mu) ? n : s, A::mk(u.a, u.b), re[a]);
+        re[a] = A::fma(imag_mu(mu) ? s : n, A::mk(u.c, u.d), re[a]);
+        im[a] = A::fma(s, A::mk(v.a, v.b), im[a]);
+        im[a] = A::fma(n, A::mk(v.c, v.d), im[a]);
       }
+    }
   if (R) {
 #pragma unroll
     for (int a = 0; a < 3; a++) {
@@ -1108,14 +1129,14 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
   }
   if (part) {
     if (XSUM && mu == 0) put<T, LS, POST>(sbuf + j * SST, t, acc);
-    else put_hops<T, LS, POST>(sbuf + (mu * S + j) * SST, t, acc);
+    else put_hops<T, LS, POST>(hop_block<T, LS>(sbuf, mu, j), t, acc);
   }
   __syncthreads();
   const bool rev = prog_reversed(POST, 1) == (chir == 1);  // one of the chiralities is reversed
   T* p = sbuf + j * SST + (rev ? G - 1 - t : t) * kPairStride + 4 * c0;
   if constexpr (!XSUM) {
     V sr[3], si[3];
-    if (part) sum_lanes<T, LS, POST>(sbuf + j * SST, S * SST, t, mu, sr, si);
+    if (part) sum_lanes<T, LS, POST>(sbuf, j, t, mu, sr, si);
     __syncthreads();  // the sums overwrite the first block
     if (part) {
 #pragma unroll
@@ -1126,7 +1147,7 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
     }
     __syncthreads();
   }
-  run_prog_split<T, LS, POST, XSUM>(sbuf, S * SST, coef, tid, S);
+  run_prog_split<T, LS, POST, XSUM>(sbuf, coef, tid, S);
   __syncthreads();
   const T f = G5 && chir == 1 ? -a.c_hop : a.c_hop;
   V re[3], im[3];
@@ -1166,7 +1187,7 @@ __global__ void __launch_bounds__(128, MINB) hop_split_kernel(const Geom g, cons
       }
     }
     __syncthreads();
-    run_prog_split<T, LS, PR_ITINV, false>(sbuf, 0, coef + prog_coefs(LS, POST), tid, S);
+    run_prog_split<T, LS, PR_ITINV, false>(sbuf, coef + prog_coefs(LS, POST), tid, S);
     __syncthreads();
     if (active) {
 #pragma unroll
@@ -1257,9 +1278,10 @@ inline int tile_threads(int Ls, int Vh, int nrhs, bool f64) {
   return 32;
 }
 
-constexpr size_t split_smem(int Ls, size_t ts, int prog, int extra) {
-  return ts * ((size_t)prog_coefs(Ls, prog) + (extra == EX_HAT ? prog_coefs(Ls, PR_ITINV) : 0) +
-               4 * (size_t)(32 / (Ls / 2)) * site_stride(Ls));
+template <typename T>
+constexpr size_t split_smem(int Ls, int prog, int extra) {
+  return sizeof(T) * ((size_t)prog_coefs(Ls, prog) + (extra == EX_HAT ? prog_coefs(Ls, PR_ITINV) : 0) +
+                      (size_t)(32 / (Ls / 2)) * (site_stride(Ls) + 3 * hop_site_stride<T>(Ls)));
 }
 
 inline size_t smem_bytes(int Ls, int S, size_t ts, int prog, int extra = EX_NONE) {
@@ -1270,9 +1292,9 @@ inline size_t smem_bytes(int Ls, int S, size_t ts, int prog, int extra = EX_NONE
 // hop_split_kernel instead of hop_kernel while the warps of hop_kernel do not fill the 608
 // SM sub-partitions once (FP32); FP64 up to a line between the sizes where it was seen to win
 // (432 warps) and to lose (512).  Both give the same bits (sum_hops).  D_bb + D_bb^+ at Ls = 16,
-// us with / without (CUDA graph): FP32 4^4 15.4 / 26.3, 8^4 (512 warps) 25.0 / 28.8, FP64 4^4
-// 101 / 276, 8^3x4 (256) 170 / 277, 12^2x8x12 at Ls = 4 (432) 239 / 290; above the lines (with
-// sums by direction, 5-8% faster in FP32): FP32 12 right-hand sides of 8^2x4^2 (1536 warps)
+// us with / without (CUDA graph): FP32 4^4 15.3 / 26.3, 8^4 (512 warps) 25.1 / 28.8, FP64 4^4
+// 99 / 276, 8^3x4 (256) 167 / 277, 12^2x8x12 at Ls = 4 (432) 234 / 290; above the lines (with
+// sums by direction, 2-8% faster in FP32): FP32 12 right-hand sides of 8^2x4^2 (1536 warps)
 // 49.4 / 42.4, FP64 8^4 (512) 326 / 296.
 inline bool split_directions(int Ls, int Vh, int nrhs, bool f64) {
   const int S = 32 / (Ls / 2);
@@ -1381,7 +1403,7 @@ cudaError_t run(const Geom& g, const HopLaunch& L, cudaStream_t st) {
   if constexpr (!SP::kScaled) {
     if (L.block_threads == 0 && split_directions(LS, g.Vh, std::max(L.nrhs, L.rule_nrhs), sizeof(T) == 8)) {
       constexpr int S = 32 / (LS / 2);
-      constexpr size_t smem = split_smem(LS, sizeof(T), POST, EX);
+      constexpr size_t smem = split_smem<T>(LS, POST, EX);
       auto k = hop_split_kernel<SP, LS, PRE, POST, LOC, G5, NORM, min_blocks<T>(), EX>;
       static std::atomic<bool> attr{false};
       cudaError_t e = smem_limit_once(k, smem, attr);
